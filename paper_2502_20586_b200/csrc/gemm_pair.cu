@@ -210,11 +210,14 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
                             tc_cp_32x128b_warpx4_pair(sfb_t + 8 * c + 4 * j, make_smem_desc(sf_s + kSfaB + (2 * j + c) * kSfTile, 0, 128, 0));
                     }
                 }
-                if (kt == 0) {                                                   // the copies above did not need the accumulator
+                if (!(ok = mbar_wait_spin(&turn[me], (n & 1) ^ me ^ 1, abort_flag))) break;   // the step before mine is issued
+                // The copies above did not need the accumulator.  Waited for under the baton: with one K-step per tile the
+                // two threads alternate between tiles, and a thread that waited before its turn could see the hand-back of
+                // two tiles ago as its own (a phase parity only tells neighbouring phases apart).
+                if (kt == 0) {
                     if (!(ok = mbar_wait(tmem_empty, (tile_i & 1) ^ 1, abort_flag))) break;
                     tc_fence_after_sync();
                 }
-                if (!(ok = mbar_wait_spin(&turn[me], (n & 1) ^ me ^ 1, abort_flag))) break;   // the step before mine is issued
                 const uint32_t hi2 = 2u << 30;
                 const bool last = kt == num_kt - 1;
                 auto D = [&](uint32_t lo) { return ((uint64_t)desc_hi << 32) | lo; };
