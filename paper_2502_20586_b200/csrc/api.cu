@@ -199,39 +199,45 @@ void attach_input_map(QuantArgs& a) {
 }
 
 // Tensor map over the output C [M, N] for the pair kernel's stores: box = 64 bytes of a row x 32 rows, 64-byte swizzle.
-bool make_output_map(CUtensorMap* map, void* C, int64_t M, int64_t N, int64_t ldc, bool fp32) {
+// (C is 16-byte aligned and its pitch a multiple of 16 bytes: checked at the entry points.)
+mxfp4_status make_output_map(CUtensorMap* map, void* C, int64_t M, int64_t N, int64_t ldc, bool fp32) {
     const int64_t es = fp32 ? 4 : 2;
-    if ((reinterpret_cast<uintptr_t>(C) & 15u) != 0 || (ldc * es) % 16 != 0 || M > 0x7FFFFFFF || N > 0x7FFFFFFF) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)N, (cuuint64_t)M};
     const cuuint64_t strides[1] = {(cuuint64_t)(ldc * es)};
     const cuuint32_t box[2] = {(cuuint32_t)(64 / es), 32};
     const cuuint32_t elem_strides[2] = {1, 1};
-    const CUresult r = g_rt.encode(map, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, C, dims, strides,
-                                   box, elem_strides, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
-                                   CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS;
+    return encode_status(g_rt.encode(map, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, C, dims, strides,
+                                     box, elem_strides, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                                     CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE), "output");
+}
+
+// Tensor map over the native scale tiles of an operand [rows, K]: 512 bytes per tile, tiles along K fastest; box = two tiles.
+mxfp4_status make_scales_map(CUtensorMap* map, const uint8_t* scales, int64_t rows, int64_t K) {
+    const cuuint64_t dims[2] = {128, (cuuint64_t)(((rows + 127) / 128) * ((K + 127) / 128))};
+    const cuuint64_t strides[1] = {512};
+    const cuuint32_t box[2] = {128, 2};
+    const cuuint32_t elem_strides[2] = {1, 1};
+    return encode_status(g_rt.encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<uint8_t*>(scales), dims, strides, box, elem_strides,
+                                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE), "scales");
 }
 
 // Everything a GEMM launch needs (tensor maps included), built without touching the device.
 mxfp4_status gemm_prepare(GemmArgs& a, const uint8_t* A_codes, const uint8_t* A_scales, const uint8_t* B_codes, const uint8_t* B_scales,
                           int64_t M, int64_t N, int64_t K, float alpha, void* C, int64_t ldc, int out_dtype, int accumulate) {
-    mxfp4_status st = make_codes_map(&a.tmap_a, A_codes, M, K, mx::kGemmBM);
-    if (st != MXFP4_OK) return st;
-    st = make_codes_map(&a.tmap_b, B_codes, N, K, mx::kGemmBN);
-    if (st != MXFP4_OK) return st;
     a.sfa = A_scales; a.sfb = B_scales;
     a.M = M; a.N = N; a.K = K;
     a.alpha = alpha; a.C = C; a.ldc = ldc; a.out_fp32 = out_dtype == MXFP4_OUT_FP32;
     a.accumulate = accumulate;
     a.use_pair = g_rt.gemm_pair && M > 128;                   // one 128-row tile gives a pair nothing to share
-    a.has_tmap_c = false;
     a.lite = a.use_pair && force_lite();
-    if (a.use_pair) {
-        st = make_codes_map(&a.tmap_b_half, B_codes, N, K, 128);
-        if (st != MXFP4_OK) return st;
-        a.has_tmap_c = make_output_map(&a.tmap_c, C, M, N, ldc, a.out_fp32 != 0);
-    }
-    return MXFP4_OK;
+    mxfp4_status st = make_codes_map(&a.tmap_a, A_codes, M, K, mx::kGemmBM);
+    if (st != MXFP4_OK) return st;
+    if (!a.use_pair) return make_codes_map(&a.tmap_b, B_codes, N, K, mx::kGemmBN);
+    if ((st = make_codes_map(&a.tmap_b, B_codes, N, K, 128)) != MXFP4_OK) return st;           // each CTA of a pair loads half a B tile
+    if ((st = make_scales_map(&a.tmap_sfa, A_scales, M, K)) != MXFP4_OK) return st;
+    if ((st = make_scales_map(&a.tmap_sfb, B_scales, N, K)) != MXFP4_OK) return st;
+    return make_output_map(&a.tmap_c, C, M, N, ldc, a.out_fp32 != 0);
 }
 
 mxfp4_status gemm_launch(const GemmArgs& a, cudaStream_t stream) {
@@ -404,7 +410,8 @@ mxfp4_status quantize_operands_impl(const void* dY, const void* X, const void* W
     };
     bool all_tc = true;
     for (int i = 0; i < 4; ++i) {
-        attach_input_map(q[i]);
+        if (i == 2) { q[2].tmap_x = q[0].tmap_x; q[2].has_tmap = q[0].has_tmap; }   // the same tensor; both reduce lengths are multiples of 128
+        else attach_input_map(q[i]);
         all_tc = all_tc && mx::quant_tc_eligible(q[i]);
     }
     if (ov != nullptr && ov->first >= 0 && all_tc && g != 256) {

@@ -9,18 +9,25 @@
 //
 // Roles per CTA (12 warps in three warp groups), all waits bounded as in gemm.cu:
 //   warp 0       TMA producer: own A rows, own half of B (completion counted on the LEADER's barrier);
-//   warp 3       scale loader: own A-row scale tiles and the scale tiles of all 256 B rows, bulk copies into ring slot
-//                s of stage s (free again when the step's MMAs, and with them its scale copies, have completed);
+//   warp 3       scale loader: own A-row scale tiles and the scale tiles of all 256 B rows, tiled copies into ring slot
+//                s of stage s, counted on the same leader barrier as the operands, so the issuer waits once per step;
 //   warps 1, 2   MMA issuers, leader CTA only, taking the K-steps in turn under a baton.  Per step: six tcgen05.cp
 //                carry the step's scale tiles from the ring into TMEM slot s of BOTH CTAs (the copy itself replicates
 //                them to the four lane quadrants and reads shared memory once; they are issued while the other
 //                thread still issues its MMAs), then four K = 64 pair-MMAs; ONE multicast tcgen05.commit per step
 //                frees operand stage, ring slot and TMEM scale slot in both CTAs;
-//   warp 8       forwards "this CTA's scale tiles of step i have landed" to the leader's full barrier of the stage,
-//                the same one the operand bytes complete, so the issuer waits once (warps 9..11 only fill the group);
-//   warps 4..7   epilogue of the CTA's own 128 x 256 half tile: accumulator -> registers (packed bf16) -> hand the
-//                accumulator back -> swizzled staging -> TMA stores (or reduce-adds when accumulating).
+//   warps 4..11  epilogue of the CTA's own 128 x 256 half tile, a warp 32 rows x 128 columns: accumulator -> registers
+//                (all 128 columns in flight) -> hand the accumulator back -> scale, convert -> swizzled staging -> TMA
+//                stores (or reduce-adds when accumulating).
 // A-row scales are per CTA; every CTA needs the scales of all 256 B rows.
+//
+// What the second epilogue group is for: TMEM has no room for a second 256-column accumulator beside the scale slots, so
+// the tensor pipe stands still from a tile's last MMA until the accumulator is in registers.  With eight warps that
+// hold it unconverted (in place of four that had to convert the first half before reading the second, and for fp32
+// stored every 32 columns before reading the next) a tile costs 0.42 us per K-step + 0.8 us.  Back to back, before ->
+// now: 16384 x 8192 x 2048 bf16 125 -> 115 us, fp32 197 -> 143; 16384 x 4096 x 4096 111 -> 105; 16384 x 4096 x 16384
+// 391 -> 388.  The fp32 store is then bound by writing (537 MB in 140 us); a second staging buffer, stores without the
+// evict-first hint, and 32-byte stores straight from the registers (175 us; 113 us at K = 4096) gained nothing.
 #include <cuda_bf16.h>
 
 #include <cstdlib>
@@ -38,8 +45,8 @@ constexpr uint32_t kSfaB = 2 * kSfTile;                     // own 128 A rows, 2
 constexpr uint32_t kSfbB = 2 * 2 * kSfTile;                 // all 256 B rows
 constexpr uint32_t kStageB = 2 * kAB;                       // 32 KB: A rows + B half
 constexpr uint32_t kSfSlotB = kSfaB + kSfbB;                // 3 KB
-constexpr uint32_t kEpiBuf = 2048;                          // epilogue staging: 32 rows x 64 B, two buffers per epilogue warp (4 warps)
-constexpr uint32_t kEpiB = 4 * 2 * kEpiBuf;
+constexpr uint32_t kEpiBuf = 2048;                          // epilogue staging: 32 rows x 64 B, one buffer per epilogue warp (8 warps)
+constexpr uint32_t kEpiB = 8 * kEpiBuf;
 constexpr uint32_t kBarB = 256;
 constexpr uint32_t kSfSlotColsP = 24;
 constexpr int kThreadsP = 12 * 32;
@@ -51,29 +58,26 @@ constexpr int kThreadsP = 12 * 32;
 template <bool LITE>
 struct PairCfg {
     static constexpr int kStages = LITE ? 4 : 6;
-    static constexpr int kSfSlots = kStages;                // scale ring: shared-memory slot i feeds TMEM slot i; same ring
-                                                            // index as the operand stages so ONE commit frees both
+    // scale ring: shared-memory slot i feeds TMEM slot i; same ring index as the operand stages so ONE commit frees both
     // The dynamic shared-memory window is at least 256-byte aligned, so rounding its base up to 1024 costs at most 768 bytes.
-    static constexpr uint32_t kSmem = kStages * kStageB + kSfSlots * kSfSlotB + kEpiB + kBarB + 768;
-    // Register hand-over (setmaxnreg) between the three warp groups (kRegsFwd: the forwarder's group); an increase can only
+    static constexpr uint32_t kSmem = kStages * (kStageB + kSfSlotB) + kEpiB + kBarB + 768;
+    // Register hand-over (setmaxnreg) between warp group 0 and the two epilogue groups; an increase can only
     // draw on what the CTA holds at launch (threads x registers per thread), which gemm_pair_init checks: an increase
     // that cannot be met waits forever.
-    static constexpr int kRegsLight = 56, kRegsFwd = LITE ? 24 : 64, kRegsEpi = 232;
+    static constexpr int kRegsLight = LITE ? 56 : 72, kRegsEpi = LITE ? 128 : 216;
+    static constexpr int kBatch = LITE ? 2 : 4;             // 32-column accumulator loads an epilogue warp keeps in flight
     static constexpr int kLaunchRegs = LITE ? 104 : 168;    // registers per thread the CTA is given at launch
     static_assert(kSmem <= 232448, "over the 227 KB shared-memory limit");
-    static_assert(kSfSlots * kSfSlotColsP <= (LITE ? 128 : 256), "scale slots do not fit their TMEM allocation");
-    static_assert(kThreadsP * kLaunchRegs >= 128 * (kRegsLight + kRegsFwd + kRegsEpi), "warp groups ask for more registers than the CTA holds");
+    static_assert(kStages * kSfSlotColsP <= (LITE ? 128 : 256), "scale slots do not fit their TMEM allocation");
+    static_assert(kThreadsP * kLaunchRegs >= 128 * (kRegsLight + 2 * kRegsEpi), "warp groups ask for more registers than the CTA holds");
 };
 
 struct ParamsP {
-    const uint8_t* sfa;
-    const uint8_t* sfb;
     void* C;
     int64_t M, N, K, ldc;
     float alpha;
     int out_fp32;
     int m_tiles, n_tiles;                                   // in pair tiles
-    int c_tma;                                              // C goes out through tmap_c (else plain stores)
     int accumulate;                                         // fp32 output only: C += instead of C =
     int group_m;                                            // rasterisation: this many pair-tile rows share the B tiles in L2 (launch_gemm_pair)
 };
@@ -89,19 +93,18 @@ __device__ __forceinline__ void tile_coords_p(int t, int m_tiles, int n_tiles, i
 }
 
 template <bool LITE>
-__device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const CUtensorMap& tmap_b, const CUtensorMap& tmap_c, const ParamsP& p) {
+__device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const CUtensorMap& tmap_b, const CUtensorMap& tmap_sfa, const CUtensorMap& tmap_sfb,
+                                               const CUtensorMap& tmap_c, const ParamsP& p) {
     using Cfg = PairCfg<LITE>;
-    constexpr int kStagesP = Cfg::kStages, kSfSlotsP = Cfg::kSfSlots;
+    constexpr int kStagesP = Cfg::kStages;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* sf_ring = smem + kStagesP * kStageB;
-    uint8_t* epi_ring = sf_ring + kSfSlotsP * kSfSlotB;
+    uint8_t* epi_ring = sf_ring + kStagesP * kSfSlotB;
     uint64_t* bars = reinterpret_cast<uint64_t*>(epi_ring + kEpiB);
     uint64_t* full_bar = bars;                              // [kStagesP] leader: operands and scale tiles of both CTAs landed
-                                                            //            (1 expect_tx arrival + 1 forwarder per CTA)
     uint64_t* empty_bar = full_bar + kStagesP;              // [kStagesP] per CTA: stage and scale slot free (pair commit)
-    uint64_t* sfl_full = empty_bar + kStagesP;              // [kSfSlotsP] per CTA: scale tiles landed in the ring slot
-    uint64_t* turn = sfl_full + kSfSlotsP;                 // [2] leader: baton between the two MMA issuers
+    uint64_t* turn = empty_bar + kStagesP;                  // [2] leader: baton between the two MMA issuers
     uint64_t* tmem_full = turn + 2;                         // per CTA: accumulator complete (pair commit)
     uint64_t* tmem_empty = tmem_full + 1;                   // leader: both CTAs drained their accumulators
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tmem_empty + 1);   // [2] base columns of the TMEM allocation(s)
@@ -117,16 +120,17 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
     const uint32_t total = my_tiles * (uint32_t)num_kt;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStagesP; ++s) { mbar_init(&full_bar[s], 1 + 2); mbar_init(&empty_bar[s], 1); }
-        for (int s = 0; s < kSfSlotsP; ++s) mbar_init(&sfl_full[s], 1);
+        for (int s = 0; s < kStagesP; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
         mbar_init(&turn[0], 1); mbar_init(&turn[1], 1);
         mbar_init(tmem_full, 1);
-        mbar_init(tmem_empty, 8);
+        mbar_init(tmem_empty, 16);
         *abort_flag = 0;
         mbar_fence_init();
         prefetch_tensormap(&tmap_a);
         prefetch_tensormap(&tmap_b);
-        if (p.c_tma) prefetch_tensormap(&tmap_c);
+        prefetch_tensormap(&tmap_sfa);
+        prefetch_tensormap(&tmap_sfb);
+        prefetch_tensormap(&tmap_c);
     }
     if (warp == 1) {
         if (LITE) {                                         // accumulator and scale slots as two allocations: 128 columns stay free
@@ -143,8 +147,8 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
     tc_fence_after_sync();
     const uint32_t tmem_acc = tmem_slot[0];                 // 256 accumulator columns
     const uint32_t tmem_sf = LITE ? tmem_slot[1] : tmem_slot[0] + 256;   // scale slots of 24 columns
-    // Warp group 0 (producer, issuers, scale loader) and warp group 2 (forwarder) need few registers; the epilogue
-    // group takes them to hold half an accumulator row and four TMEM loads in flight.
+    // Warp group 0 (producer, issuers, scale loader) needs few registers; the epilogue groups take them to hold 128 columns
+    // of the accumulator each.
     // Each warp group (four warps) sets its register limit once, at the head of its own branch: all four warps must
     // execute the same setmaxnreg, and the limit must dominate the code that relies on it.
     pdl_launch_dependents();                                // the next kernel of the stream may set itself up behind this one
@@ -166,7 +170,7 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
                     const int s = it % kStagesP;
                     if (!(ok = mbar_wait(&empty_bar[s], ((it / kStagesP) & 1) ^ 1, abort_flag))) break;
                     uint8_t* st = smem + s * kStageB;
-                    if (rank == 0) mbar_expect_tx(&full_bar[s], 4 * kAB);       // two loads from each CTA
+                    if (rank == 0) mbar_expect_tx(&full_bar[s], 2 * (kStageB + kSfSlotB));   // operands and scales of both CTAs
                     tma_load_2d_pair(st, &tmap_a, &full_bar[s], kt * kGemmBKBytes, a_rt * 128);
                     tma_load_2d_pair(st + kAB, &tmap_b, &full_bar[s], kt * kGemmBKBytes, nt * PN + (int)rank * 128);
                 }
@@ -240,64 +244,40 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
         }
     } else {
         // ------------------------------------------------------------------ scale loader (both CTAs)
+        // One box = the two 512-byte scale tiles of a 128-row tile for this K-step (box rows past the operand read zeros; a
+        // box that runs over the end of an odd K reads the next row tile's first, which no MMA uses).
         if (lane == 0) {
             uint32_t it = 0;
             bool ok = true;
             for (uint32_t tl = 0; tl < my_tiles && ok; ++tl) {
                 int mt, nt;
                 tile_coords_p((int)(pair + tl * num_pairs), p.m_tiles, p.n_tiles, p.group_m, mt, nt);
-                const int a_rt = 2 * mt + (int)rank;
-                const bool has_a = (int64_t)a_rt * 128 < p.M;
-                const int n_row_tiles = min(2, (int)((p.N - (int64_t)nt * PN + 127) >> 7));
+                const int32_t a_row = (2 * mt + (int)rank) * nkc, b_row = nt * 2 * nkc;
                 for (int kt = 0; kt < num_kt; ++kt, ++it) {
-                    const int slot = it % kSfSlotsP;
-                    // the ring slot is free once the MMAs of the step that used it (and their scale copies) have completed
-                    if (!(ok = mbar_wait(&empty_bar[slot], ((it / kSfSlotsP) & 1) ^ 1, abort_flag))) break;
-                    uint8_t* dst = sf_ring + slot * kSfSlotB;
-                    const int nch = min(2, nkc - 2 * kt);
-                    mbar_expect_tx(&sfl_full[slot], (uint32_t)nch * kSfTile * ((has_a ? 1u : 0u) + (uint32_t)n_row_tiles));
-                    if (has_a) bulk_load(dst, p.sfa + ((int64_t)a_rt * nkc + 2 * kt) * kSfTile, nch * kSfTile, &sfl_full[slot]);
-                    for (int j = 0; j < n_row_tiles; ++j)
-                        bulk_load(dst + kSfaB + j * 2 * kSfTile, p.sfb + ((int64_t)(nt * 2 + j) * nkc + 2 * kt) * kSfTile,
-                                  nch * kSfTile, &sfl_full[slot]);
+                    const int s = it % kStagesP;
+                    if (!(ok = mbar_wait(&empty_bar[s], ((it / kStagesP) & 1) ^ 1, abort_flag))) break;
+                    uint8_t* dst = sf_ring + s * kSfSlotB;
+                    tma_load_2d_pair(dst, &tmap_sfa, &full_bar[s], 0, a_row + 2 * kt);
+                    tma_load_2d_pair(dst + kSfaB, &tmap_sfb, &full_bar[s], 0, b_row + 2 * kt);
+                    tma_load_2d_pair(dst + kSfaB + 2 * kSfTile, &tmap_sfb, &full_bar[s], 0, b_row + nkc + 2 * kt);
                 }
             }
             if (!ok) *abort_flag = 1;
         }
     }
-    } else if (warp >= 8) {
-        // ============================ warp group 2: scale forwarder (warp 8)
-        reg_dealloc<Cfg::kRegsFwd>();
-        // The scale copies run in both CTAs on the leader's instruction, so the leader has to know that the peer's tiles
-        // have landed too: one thread per CTA passes its ring's completions on to the leader's full barrier.
-        bool ok = true;
-        if (warp == 8 && lane == 0) {
-            for (uint32_t it = 0; it < total; ++it) {
-                const int slot = it % kSfSlotsP;
-                if (!(ok = mbar_wait(&sfl_full[slot], (it / kSfSlotsP) & 1, abort_flag))) break;
-                mbar_arrive_cluster(&full_bar[slot], 0);
-            }
-        }
-        if (!ok && lane == 0) *abort_flag = 1;
     } else {
         // ------------------------------------------------------------------ epilogue (both CTAs, own 128 rows)
-        reg_alloc<Cfg::kRegsEpi>();                                  // warp group 1 takes the registers the others gave up
-        // TMEM -> registers -> (alpha, convert) -> shared memory -> TMA store.  Each warp owns the 32 accumulator
-        // lanes of its quadrant and two 2 KB staging buffers (32 rows x 64 bytes, 64-byte swizzle, so the row-per-lane
-        // writes are conflict-free); the accumulator is handed back as soon as its last column is in registers.
-        const int q = warp & 3;
-        uint8_t* stage0 = epi_ring + q * 2 * kEpiBuf;
-        uint32_t n_stores = 0;                                  // bulk groups this warp committed so far
+        reg_alloc<Cfg::kRegsEpi>();                                  // the epilogue groups take the registers the others gave up
+        const int q = warp & 3, half = (warp - 4) >> 2;              // TMEM lane quadrant; columns 128 half .. 128 half + 127 of the tile
+        uint8_t* stage = epi_ring + (warp - 4) * kEpiBuf;
         const uint64_t pol_c = l2_policy_evict_first();         // the output is not read again here: let the operands keep L2
         bool ok = true;
-        // One staged block: 16 registers = 64 bytes of this lane's row, columns [col, col + 64 B).
+        // One staged block: 16 registers = 64 bytes of this lane's row, columns [col, col + 64 B), into this warp's buffer
+        // (64-byte swizzle: the row-per-lane writes are conflict-free) and out by TMA.
         auto put = [&](const uint32_t (&w)[16], int32_t col, int32_t row0, bool in_range) {
-            uint8_t* buf = stage0 + (n_stores & 1) * kEpiBuf;
-            if (n_stores >= 2) {                                // the store that last read this buffer must be done with it
-                if (lane == 0) bulk_wait_group_read<1>();
-                __syncwarp();
-            }
-            uint4* dst = reinterpret_cast<uint4*>(buf + lane * 64);
+            if (lane == 0) bulk_wait_group_read<0>();           // the store before this one must have left the buffer
+            __syncwarp();
+            uint4* dst = reinterpret_cast<uint4*>(stage + lane * 64);
             const int sw = (lane >> 1) & 3;
 #pragma unroll
             for (int j = 0; j < 4; ++j) dst[j ^ sw] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
@@ -305,12 +285,11 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
             __syncwarp();
             if (lane == 0) {
                 if (in_range) {
-                    if (p.accumulate) tma_reduce_add_2d(&tmap_c, buf, col, row0);
-                    else tma_store_2d_hint(&tmap_c, buf, col, row0, pol_c);
+                    if (p.accumulate) tma_reduce_add_2d(&tmap_c, stage, col, row0);
+                    else tma_store_2d_hint(&tmap_c, stage, col, row0, pol_c);
                 }
                 bulk_commit_group();
             }
-            ++n_stores;
         };
         for (uint32_t tl = 0; tl < my_tiles; ++tl) {
             int mt, nt;
@@ -320,103 +299,39 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
             if (!ok) break;
             tc_fence_after_sync();
             const int64_t row0 = (int64_t)mt * PM + (int64_t)rank * 128 + q * 32;
-            const int64_t row = row0 + lane;
-            const int64_t col0 = (int64_t)nt * PN;
-            int n_chunks = PN / 32;
-            if (p.c_tma && !p.out_fp32) {
-                // bf16: drain the whole accumulator into registers first (packed pairs), hand it back, then store.
-                uint32_t out[PN / 2];
+            const uint32_t taddr = tmem_acc + ((uint32_t)(q * 32) << 16) + half * 128;
 #pragma unroll
-                for (int hb = 0; hb < 2; ++hb) {                // two batches of four 32-column loads in flight together
-                    uint32_t r[4][32];
+            for (int hb = 0; hb < 4 / Cfg::kBatch; ++hb) {
+                uint32_t r[Cfg::kBatch][32];
 #pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        tmem_ld_32x32b_x32(tmem_acc + ((uint32_t)(q * 32) << 16) + (4 * hb + c) * 32, r[c]);
-                    tmem_ld_wait();
-                    if (hb == 1) {                              // the accumulator is in registers: hand it back before converting
-                        tc_fence_before_sync();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive_cluster(tmem_empty, 0);
-                    }
-#pragma unroll
-                    for (int c = 0; c < 4; ++c)
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(r[c][2 * j]) * p.alpha,
-                                                                           __uint_as_float(r[c][2 * j + 1]) * p.alpha);
-                            out[16 * (4 * hb + c) + j] = *reinterpret_cast<const uint32_t*>(&h);
-                        }
-                }
-#pragma unroll
-                for (int c = 0; c < PN / 32; ++c) {
-                    uint32_t w[16];
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) w[j] = out[16 * c + j];
-                    const int64_t col = col0 + c * 32;
-                    put(w, (int32_t)col, (int32_t)row0, row0 < p.M && col < p.N);
-                }
-                n_chunks = 0;
-            }
-#pragma unroll 1
-            for (int c = 0; c < n_chunks; ++c) {
-                uint32_t r[32];
-                tmem_ld_32x32b_x32(tmem_acc + ((uint32_t)(q * 32) << 16) + c * 32, r);
+                for (int c = 0; c < Cfg::kBatch; ++c) tmem_ld_32x32b_x32(taddr + (hb * Cfg::kBatch + c) * 32, r[c]);
                 tmem_ld_wait();
-                if (c == n_chunks - 1) {                        // accumulator drained: the next tile's MMAs may start
+                if (hb == 4 / Cfg::kBatch - 1) {                // the accumulator is in registers: the next tile's MMAs may start
                     tc_fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive_cluster(tmem_empty, 0);
                 }
-                const int64_t col = col0 + c * 32;
-                if (p.c_tma) {
+                const int64_t colb = (int64_t)nt * PN + half * 128 + hb * Cfg::kBatch * 32;
+#pragma unroll
+                for (int c = 0; c < Cfg::kBatch; ++c) {
+                    const int64_t col = colb + c * 32;
                     const bool in_range = row0 < p.M && col < p.N;
+                    uint32_t w[16];
                     if (p.out_fp32) {
-                        uint32_t w[16];
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) w[j] = __float_as_uint(__uint_as_float(r[16 * h + j]) * p.alpha);
+                            for (int j = 0; j < 16; ++j) w[j] = __float_as_uint(__uint_as_float(r[c][16 * h + j]) * p.alpha);
                             put(w, (int32_t)col + 16 * h, (int32_t)row0, in_range && col + 16 * h < p.N);
                         }
                     } else {
-                        uint32_t w[16];
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
-                            const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(r[2 * j]) * p.alpha,
-                                                                           __uint_as_float(r[2 * j + 1]) * p.alpha);
+                            const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(r[c][2 * j]) * p.alpha,
+                                                                           __uint_as_float(r[c][2 * j + 1]) * p.alpha);
                             w[j] = *reinterpret_cast<const uint32_t*>(&h);
                         }
                         put(w, (int32_t)col, (int32_t)row0, in_range);
-                    }
-                    } else if (row < p.M && col < p.N) {
-                    const int nvalid = (int)min((int64_t)32, p.N - col);      // multiple of 8
-                    if (p.out_fp32) {
-                        float* dst = static_cast<float*>(p.C) + row * p.ldc + col;
-#pragma unroll
-                        for (int v = 0; v < 8; ++v)
-                            if (4 * v < nvalid) {
-                                float4 o = p.accumulate ? reinterpret_cast<const float4*>(dst)[v] : make_float4(0.f, 0.f, 0.f, 0.f);
-                                // product rounded first, then one add: the same two roundings as the TMA-reduce path (no fused multiply-add)
-                                o.x = __fadd_rn(o.x, __fmul_rn(__uint_as_float(r[4 * v]), p.alpha));
-                                o.y = __fadd_rn(o.y, __fmul_rn(__uint_as_float(r[4 * v + 1]), p.alpha));
-                                o.z = __fadd_rn(o.z, __fmul_rn(__uint_as_float(r[4 * v + 2]), p.alpha));
-                                o.w = __fadd_rn(o.w, __fmul_rn(__uint_as_float(r[4 * v + 3]), p.alpha));
-                                reinterpret_cast<float4*>(dst)[v] = o;
-                            }
-                    } else {
-                        __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(p.C) + row * p.ldc + col;
-#pragma unroll
-                        for (int v = 0; v < 4; ++v)
-                            if (8 * v < nvalid) {
-                                uint32_t w[4];
-#pragma unroll
-                                for (int j = 0; j < 4; ++j) {
-                                    const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(r[8 * v + 2 * j]) * p.alpha,
-                                                                                   __uint_as_float(r[8 * v + 2 * j + 1]) * p.alpha);
-                                    w[j] = *reinterpret_cast<const uint32_t*>(&h);
-                                }
-                                reinterpret_cast<uint4*>(dst)[v] = make_uint4(w[0], w[1], w[2], w[3]);
-                            }
                     }
                 }
             }
@@ -445,15 +360,17 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsP, 1)
 gemm_mxf4_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
+                      const __grid_constant__ CUtensorMap tmap_sfa, const __grid_constant__ CUtensorMap tmap_sfb,
                       const __grid_constant__ CUtensorMap tmap_c, const ParamsP p) {
-    gemm_pair_body<false>(tmap_a, tmap_b, tmap_c, p);
+    gemm_pair_body<false>(tmap_a, tmap_b, tmap_sfa, tmap_sfb, tmap_c, p);
 }
 
 // The small-footprint build (see PairCfg): same roles, same arithmetic, same accumulation order.
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(PairCfg<true>::kLaunchRegs)
 gemm_mxf4_pair_lite_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
+                           const __grid_constant__ CUtensorMap tmap_sfa, const __grid_constant__ CUtensorMap tmap_sfb,
                            const __grid_constant__ CUtensorMap tmap_c, const ParamsP p) {
-    gemm_pair_body<true>(tmap_a, tmap_b, tmap_c, p);
+    gemm_pair_body<true>(tmap_a, tmap_b, tmap_sfa, tmap_sfb, tmap_c, p);
 }
 
 }  // namespace
@@ -472,7 +389,7 @@ static cudaError_t pair_kernel_init(K kernel) {
     cudaFuncAttributes fa;
     e = cudaFuncGetAttributes(&fa, kernel);
     if (e != cudaSuccess) return e;
-    if (fa.numRegs * kThreadsP < 128 * (Cfg::kRegsLight + Cfg::kRegsFwd + Cfg::kRegsEpi)) return cudaErrorLaunchOutOfResources;
+    if (fa.numRegs * kThreadsP < 128 * (Cfg::kRegsLight + 2 * Cfg::kRegsEpi)) return cudaErrorLaunchOutOfResources;
     return cudaSuccess;
 }
 
@@ -483,7 +400,7 @@ cudaError_t gemm_pair_init() {
 
 cudaError_t launch_gemm_pair(const GemmArgs& a, cudaStream_t stream) {
     ParamsP p;
-    p.sfa = a.sfa; p.sfb = a.sfb; p.C = a.C;
+    p.C = a.C;
     p.M = a.M; p.N = a.N; p.K = a.K; p.ldc = a.ldc;
     p.alpha = a.alpha; p.out_fp32 = a.out_fp32;
     p.m_tiles = (int)((a.M + PM - 1) / PM);
@@ -495,7 +412,6 @@ cudaError_t launch_gemm_pair(const GemmArgs& a, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     const int tiles = p.m_tiles * p.n_tiles;
     const int pairs = tiles < sms / 2 ? tiles : sms / 2;
-    p.c_tma = a.has_tmap_c ? 1 : 0;
     p.accumulate = a.accumulate;
     // Tile order: groups of group_m pair-tile rows x all n-tiles.  Inside a group the A rows stay in L2 and B streams
     // through once; B is fetched from DRAM once for the whole launch only if it survives in L2 from one group to the
@@ -518,7 +434,7 @@ cudaError_t launch_gemm_pair(const GemmArgs& a, cudaStream_t stream) {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, a.lite ? gemm_mxf4_pair_lite_kernel : gemm_mxf4_pair_kernel, a.tmap_a, a.tmap_b_half, a.tmap_c, p);
+    return cudaLaunchKernelEx(&cfg, a.lite ? gemm_mxf4_pair_lite_kernel : gemm_mxf4_pair_kernel, a.tmap_a, a.tmap_b, a.tmap_sfa, a.tmap_sfb, a.tmap_c, p);
 }
 
 }  // namespace mx
