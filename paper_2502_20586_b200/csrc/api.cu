@@ -73,9 +73,8 @@ mxfp4_status runtime_init() {
     return g_rt.dev_status[dev];
 }
 
-// Side stream and events for running the two independent GEMMs of a backward call side by side (fork / join around
-// the caller's stream): the second GEMM's CTAs move onto SMs as the first one's last wave drains.  One set per host
-// thread, created at its first large call and kept; on any failure the call simply stays on the caller's stream.
+// Side stream and events of the overlapped form of a backward call (fork / join around the caller's stream).  One set per
+// host thread, created at its first such call and kept; on any failure the call simply stays on the caller's stream.
 struct ForkJoin {
     bool tried = false, ok = false;
     int device = -1;
@@ -222,34 +221,52 @@ mxfp4_status make_scales_map(CUtensorMap* map, const uint8_t* scales, int64_t ro
                                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE), "scales");
 }
 
-// Everything a GEMM launch needs (tensor maps included), built without touching the device.
-mxfp4_status gemm_prepare(GemmArgs& a, const uint8_t* A_codes, const uint8_t* A_scales, const uint8_t* B_codes, const uint8_t* B_scales,
-                          int64_t M, int64_t N, int64_t K, float alpha, void* C, int64_t ldc, int out_dtype, int accumulate) {
-    a.sfa = A_scales; a.sfb = B_scales;
-    a.M = M; a.N = N; a.K = K;
-    a.alpha = alpha; a.C = C; a.ldc = ldc; a.out_fp32 = out_dtype == MXFP4_OUT_FP32;
-    a.accumulate = accumulate;
-    a.use_pair = g_rt.gemm_pair && M > 128;                   // one 128-row tile gives a pair nothing to share
-    a.lite = a.use_pair && force_lite();
-    mxfp4_status st = make_codes_map(&a.tmap_a, A_codes, M, K, mx::kGemmBM);
-    if (st != MXFP4_OK) return st;
-    if (!a.use_pair) return make_codes_map(&a.tmap_b, B_codes, N, K, mx::kGemmBN);
-    if ((st = make_codes_map(&a.tmap_b, B_codes, N, K, 128)) != MXFP4_OK) return st;           // each CTA of a pair loads half a B tile
-    if ((st = make_scales_map(&a.tmap_sfa, A_scales, M, K)) != MXFP4_OK) return st;
-    if ((st = make_scales_map(&a.tmap_sfb, B_scales, N, K)) != MXFP4_OK) return st;
-    return make_output_map(&a.tmap_c, C, M, N, ldc, a.out_fp32 != 0);
-}
-
-mxfp4_status gemm_launch(const GemmArgs& a, cudaStream_t stream) {
-    return cuda_status(a.use_pair ? mx::launch_gemm_pair(a, stream) : mx::launch_gemm(a, stream), a.use_pair ? "pair GEMM launch" : "GEMM launch");
-}
+// One or two independent products, C = alpha A B^T: everything their launches need, built without touching the device
+// (two products that both run on the CTA-pair kernel go out as one launch).
+struct GemmPlan {
+    GemmArgs g[2];
+    const uint8_t *A[2], *B[2];
+    int n = 0, tile_n = 256;
+    void add(const uint8_t* A_codes, const uint8_t* A_scales, const uint8_t* B_codes, const uint8_t* B_scales, int64_t M, int64_t N, int64_t K,
+             float alpha, void* C, int64_t ldc, int out_dtype, int accumulate) {
+        GemmArgs& a = g[n];
+        A[n] = A_codes; B[n] = B_codes;
+        a.sfa = A_scales; a.sfb = B_scales;
+        a.M = M; a.N = N; a.K = K;
+        a.alpha = alpha; a.C = C; a.ldc = ldc; a.out_fp32 = out_dtype == MXFP4_OUT_FP32;
+        a.accumulate = accumulate;
+        a.use_pair = g_rt.gemm_pair && M > 128;                   // one 128-row tile gives a pair nothing to share
+        a.lite = a.use_pair && force_lite();
+        ++n;
+    }
+    bool one_launch() const { return n == 2 && g[0].use_pair && g[1].use_pair && !g[0].lite; }
+    mxfp4_status encode(bool together) {
+        tile_n = together ? mx::gemm_pair_tile_n(g, 2) : n == 1 && g[0].use_pair ? mx::gemm_pair_tile_n(g, 1) : 256;
+        for (int i = 0; i < n; ++i) {
+            GemmArgs& a = g[i];
+            mxfp4_status st = make_codes_map(&a.tmap_a, A[i], a.M, a.K, mx::kGemmBM);
+            if (st != MXFP4_OK) return st;
+            if ((st = make_codes_map(&a.tmap_b, B[i], a.N, a.K, a.use_pair ? tile_n / 2 : mx::kGemmBN)) != MXFP4_OK) return st;
+            if (!a.use_pair) continue;
+            if ((st = make_scales_map(&a.tmap_sfa, a.sfa, a.M, a.K)) != MXFP4_OK) return st;
+            if ((st = make_scales_map(&a.tmap_sfb, a.sfb, a.N, a.K)) != MXFP4_OK) return st;
+            if ((st = make_output_map(&a.tmap_c, a.C, a.M, a.N, a.ldc, a.out_fp32 != 0)) != MXFP4_OK) return st;
+        }
+        return MXFP4_OK;
+    }
+    mxfp4_status launch_one(int i, cudaStream_t stream) const {
+        return g[i].use_pair ? cuda_status(mx::launch_gemm_pair(&g[i], 1, tile_n, stream), "pair GEMM launch")
+                             : cuda_status(mx::launch_gemm(g[i], stream), "GEMM launch");
+    }
+    mxfp4_status launch_both(cudaStream_t stream) const { return cuda_status(mx::launch_gemm_pair(g, 2, tile_n, stream), "pair GEMM launch (two products)"); }
+};
 
 mxfp4_status gemm_impl(const uint8_t* A_codes, const uint8_t* A_scales, const uint8_t* B_codes, const uint8_t* B_scales, int64_t M,
-                       int64_t N, int64_t K, float alpha, void* C, int64_t ldc, int out_dtype, cudaStream_t stream,
-                       int accumulate = 0) {
-    GemmArgs a;
-    const mxfp4_status st = gemm_prepare(a, A_codes, A_scales, B_codes, B_scales, M, N, K, alpha, C, ldc, out_dtype, accumulate);
-    return st != MXFP4_OK ? st : gemm_launch(a, stream);
+                       int64_t N, int64_t K, float alpha, void* C, int64_t ldc, int out_dtype, cudaStream_t stream) {
+    GemmPlan plan;
+    plan.add(A_codes, A_scales, B_codes, B_scales, M, N, K, alpha, C, ldc, out_dtype, 0);
+    const mxfp4_status st = plan.encode(false);
+    return st != MXFP4_OK ? st : plan.launch_one(0, stream);
 }
 
 // C = alpha Q(RHT(A)) deq(B)^T with A = x (reduce_dim 1) or x^T (reduce_dim 0) quantised inside the GEMM kernel.
@@ -484,52 +501,49 @@ mxfp4_status linear_backward_impl(const void* dY, const void* X, const void* W, 
     for (int i = 0; i < 4; ++i) { c[i] = base + ws.codes[i]; s[i] = base + ws.scales[i]; }
     // lines 7-11: two MXFP4 GEMMs; the 16/9 un-does the two 3/4 pre-scales of Algorithm 2.
     const float alpha = rounding != MXFP4_ROUND_RN ? 16.0f / 9.0f : 1.0f;       // both SR modes carry the 3/4 pre-scale
-    // Every tensor map is encoded before the first launch, so an encoding failure leaves nothing enqueued.
-    GemmArgs gx, gw;
-    if ((st = gemm_prepare(gx, c[0], s[0], c[1], s[1], b, n, m, alpha, dX, n, out_dtype, 0)) != MXFP4_OK) return st;   // dX is never accumulated
-    if ((st = gemm_prepare(gw, c[2], s[2], c[3], s[3], m, n, b, alpha, dW, n, out_dtype, accumulate)) != MXFP4_OK) return st;
-    const int64_t waves_dx = ((b + 255) / 256) * ((n + 255) / 256), waves_dw = ((m + 255) / 256) * ((n + 255) / 256);
-    // Large problems (never the ones the fixed-scratch variant accepts) use a side stream.
-    ForkJoin* fj = ws.total > (size_t)MXFP4_STATIC_WORKSPACE_BYTES && waves_dx >= 74 && waves_dw >= 74 ? fork_join() : nullptr;
+    GemmPlan plan;
+    plan.add(c[0], s[0], c[1], s[1], b, n, m, alpha, dX, n, out_dtype, 0);               // dX is never accumulated
+    plan.add(c[2], s[2], c[3], s[3], m, n, b, alpha, dW, n, out_dtype, accumulate);
     // Overlapped form (Section 3.2: the transform need not cost GEMM time): quantise the operands of one product, then
     // run that product's GEMM while the other product's operands are quantised on the same SMs (small builds of both
     // kernels share an SM: the GEMM keeps the FP4 pipe, the quantiser takes the idle issue slots and ALUs), then the
     // second GEMM.  The product whose operands are the smaller half goes first, so that more of the quantiser work hides.
+    const int64_t waves_dx = ((b + 255) / 256) * ((n + 255) / 256), waves_dw = ((m + 255) / 256) * ((n + 255) / 256);
     const int overlap_mode = overlap_setting();
-    Overlap ov{-1, fj};
-    if (fj != nullptr && overlap_mode != 0 && gx.use_pair && gw.use_pair && g != 0 && g != 256) {
+    Overlap ov{-1, nullptr};
+    // large problems only (never the ones the fixed-scratch variant accepts): it needs a side stream
+    if (overlap_mode != 0 && ws.total > (size_t)MXFP4_STATIC_WORKSPACE_BYTES && waves_dx >= 74 && waves_dw >= 74 && plan.g[0].use_pair &&
+        plan.g[1].use_pair && g != 0 && g != 256 && (ov.fj = fork_join()) != nullptr) {
         const int64_t head_dx = b * m + n * m, head_dw = m * b + n * b;       // elements quantised before the first GEMM can start
         ov.first = overlap_mode == 2 ? 0 : overlap_mode == 3 ? 1 : (head_dx <= head_dw ? 0 : 1);
     }
+    // Otherwise both products go out as one launch: they do not depend on each other.
+    const bool together = ov.first < 0 && plan.one_launch();
+    // Every tensor map is encoded before the first launch, so an encoding failure leaves nothing enqueued.
+    if ((st = plan.encode(together)) != MXFP4_OK) return st;
     float* bias_partial = db != nullptr ? reinterpret_cast<float*>(base + bias_off) : nullptr;
     bool bias_fused = false;
     if ((st = quantize_operands_impl(dY, X, W, b, m, n, g, rounding, seed, c, s, stream, &ov, bias_partial, &bias_fused)) != MXFP4_OK) {
-        if (ov.forked && (cudaEventRecord(fj->join, fj->side) != cudaSuccess || cudaStreamWaitEvent(stream, fj->join, 0) != cudaSuccess)) return MXFP4_ERR_CUDA;
+        if (ov.forked && (cudaEventRecord(ov.fj->join, ov.fj->side) != cudaSuccess || cudaStreamWaitEvent(stream, ov.fj->join, 0) != cudaSuccess)) return MXFP4_ERR_CUDA;
         return st;
     }
     if (ov.first >= 0) {
-        GemmArgs& g1 = ov.first == 0 ? gx : gw;
-        GemmArgs& g2 = ov.first == 0 ? gw : gx;
-        g1.lite = true;                              // shares its SMs with the small quantiser running on the side stream
-        st = gemm_launch(g1, stream);
-        const bool joined = cudaEventRecord(fj->join, fj->side) == cudaSuccess && cudaStreamWaitEvent(stream, fj->join, 0) == cudaSuccess;
+        plan.g[ov.first].lite = true;                // shares its SMs with the small quantiser running on the side stream
+        st = plan.launch_one(ov.first, stream);
+        const bool joined = cudaEventRecord(ov.fj->join, ov.fj->side) == cudaSuccess && cudaStreamWaitEvent(stream, ov.fj->join, 0) == cudaSuccess;
         if (!joined) return MXFP4_ERR_CUDA;
-        if (st == MXFP4_OK) st = gemm_launch(g2, stream);
-        fj = nullptr;                                // joined already
+        if (st == MXFP4_OK) st = plan.launch_one(1 - ov.first, stream);
+    } else if (together) {
+        st = plan.launch_both(stream);
     } else {
-        if (fj != nullptr && (cudaEventRecord(fj->fork, stream) != cudaSuccess || cudaStreamWaitEvent(fj->side, fj->fork, 0) != cudaSuccess))
-            fj = nullptr;                            // the side stream was not given anything yet: stay on the caller's stream
-        st = gemm_launch(gx, stream);
-        if (st == MXFP4_OK) st = gemm_launch(gw, fj != nullptr ? fj->side : stream);
+        st = plan.launch_one(0, stream);
+        if (st == MXFP4_OK) st = plan.launch_one(1, stream);
     }
     // dL/db = 1 dL/dy (problem statement): column sums of dY, after the GEMMs on the caller's stream
     // (when the dual-view quantiser launch has already summed every 128-row band of dY, only the bands remain to be added)
     if (st == MXFP4_OK && db != nullptr)
         st = bias_fused ? cuda_status(mx::launch_bias_finish(bias_partial, m, (int)(b / 128), accumulate, db, stream), "bias gradient launch")
                         : cuda_status(mx::launch_bias_grad(dY, b, m, m, accumulate, db, bias_partial, stream), "bias gradient launch");
-    // The join is made whatever happened after the fork, so that the side stream never runs unordered with the caller's.
-    if (fj != nullptr && (cudaEventRecord(fj->join, fj->side) != cudaSuccess || cudaStreamWaitEvent(stream, fj->join, 0) != cudaSuccess))
-        return MXFP4_ERR_CUDA;
     return st;
 }
 }  // namespace

@@ -38,26 +38,29 @@
 namespace mx {
 namespace {
 
-constexpr int PM = 256, PN = 256;                           // pair tile
-constexpr uint32_t kAB = 128 * kGemmBKBytes;                // 16 KB: 128 rows x 128 B, for A and for the B half
+constexpr int PM = 256;                                     // rows of a pair tile
+constexpr uint32_t kAB = 128 * kGemmBKBytes;                // 16 KB: 128 A rows x 128 B
 constexpr uint32_t kSfTile = 512;
 constexpr uint32_t kSfaB = 2 * kSfTile;                     // own 128 A rows, 2 tiles (8 K-blocks) per stage
-constexpr uint32_t kSfbB = 2 * 2 * kSfTile;                 // all 256 B rows
-constexpr uint32_t kStageB = 2 * kAB;                       // 32 KB: A rows + B half
-constexpr uint32_t kSfSlotB = kSfaB + kSfbB;                // 3 KB
 constexpr uint32_t kEpiBuf = 2048;                          // epilogue staging: 32 rows x 64 B, one buffer per epilogue warp (8 warps)
 constexpr uint32_t kEpiB = 8 * kEpiBuf;
 constexpr uint32_t kBarB = 256;
-constexpr uint32_t kSfSlotColsP = 24;
 constexpr int kThreadsP = 12 * 32;
 
-// Two builds of the kernel.  FULL owns its SMs: six operand stages (all 227 KB of shared memory), one 512-column TMEM
-// allocation, every register of the SM.  LITE leaves room for a second, independent kernel on the same SM (the
-// tensor-core quantiser's small build, quantize_tc.cu, which quantises the OTHER product's operands meanwhile): four
-// stages, TMEM taken as 256 + 128 columns, 112 registers per thread at launch.
-template <bool LITE>
+// Three builds of the kernel.  PN = 256 (256 x 256 pair tile): six operand stages (all 227 KB of shared memory), one
+// 512-column TMEM allocation, every register of the SM.  PN = 128 (256 x 128): eight stages, and TMEM room for two
+// accumulators, so that a tile's MMAs run while the tile before is taken out; see tile_width() for when it is the better
+// one.  LITE (PN = 256) leaves room for a second, independent kernel on the same SM (the tensor-core quantiser's small
+// build, quantize_tc.cu, which quantises the OTHER product's operands meanwhile): four stages, TMEM taken as 256 + 128
+// columns, 104 registers per thread at launch.
+template <bool LITE, int PN>
 struct PairCfg {
-    static constexpr int kStages = LITE ? 4 : 6;
+    static constexpr int kAccBufs = 256 / PN;
+    static constexpr int kStages = LITE ? 4 : PN == 128 ? 8 : 6;
+    static constexpr uint32_t kBB = PN / 2 * kGemmBKBytes;  // half of the B tile
+    static constexpr uint32_t kStageB = kAB + kBB;
+    static constexpr uint32_t kSfSlotB = kSfaB + PN / 128 * 2 * kSfTile;   // A rows and all PN B rows
+    static constexpr uint32_t kSfCols = kSfSlotB / 128;     // TMEM columns of a slot: 4 per 512-byte tile
     // scale ring: shared-memory slot i feeds TMEM slot i; same ring index as the operand stages so ONE commit frees both
     // The dynamic shared-memory window is at least 256-byte aligned, so rounding its base up to 1024 costs at most 768 bytes.
     static constexpr uint32_t kSmem = kStages * (kStageB + kSfSlotB) + kEpiB + kBarB + 768;
@@ -67,19 +70,34 @@ struct PairCfg {
     static constexpr int kRegsLight = LITE ? 56 : 72, kRegsEpi = LITE ? 128 : 216;
     static constexpr int kBatch = LITE ? 2 : 4;             // 32-column accumulator loads an epilogue warp keeps in flight
     static constexpr int kLaunchRegs = LITE ? 104 : 168;    // registers per thread the CTA is given at launch
+    static_assert(!LITE || PN == 256, "the small build has one 256-column accumulator");
     static_assert(kSmem <= 232448, "over the 227 KB shared-memory limit");
-    static_assert(kStages * kSfSlotColsP <= (LITE ? 128 : 256), "scale slots do not fit their TMEM allocation");
+    static_assert((2 * kStages + 2 + 2 * kAccBufs) * 8 + 16 <= kBarB, "barriers");
+    static_assert(kStages * kSfCols <= (LITE ? 128 : 256), "scale slots do not fit their TMEM allocation");
     static_assert(kThreadsP * kLaunchRegs >= 128 * (kRegsLight + 2 * kRegsEpi), "warp groups ask for more registers than the CTA holds");
 };
 
-struct ParamsP {
-    void* C;
-    int64_t M, N, K, ldc;
+struct ProblemP {                                           // one product of a launch
+    int64_t M, N;
+    int nkc, num_kt;                                        // 128-element scale tiles along K; 256-element pipeline steps
+    int m_tiles, n_tiles;                                   // in pair tiles
+    int group_m;                                            // rasterisation: this many pair-tile rows share the B tiles in L2 (fill_problem)
     float alpha;
     int out_fp32;
-    int m_tiles, n_tiles;                                   // in pair tiles
     int accumulate;                                         // fp32 output only: C += instead of C =
-    int group_m;                                            // rasterisation: this many pair-tile rows share the B tiles in L2 (launch_gemm_pair)
+};
+
+// A launch runs one product, or two that do not depend on each other (the two GEMMs of a backward call) with the one of
+// the longer K first.  Every pair knows its own tiles without asking: the first product's n0 tiles go round-robin; the
+// n0 mod P = `rest` pairs that got one more of them sit out while the others take `early` tiles of the second product
+// each; what is left of that goes round-robin over all, the others first.
+struct ParamsP {
+    ProblemP prob[2];
+    int n0, n1;                                             // tiles of the two products
+    int rest, early;
+};
+struct MapsP {
+    CUtensorMap a[2], b[2], sfa[2], sfb[2], c[2];
 };
 
 __device__ __forceinline__ void tile_coords_p(int t, int m_tiles, int n_tiles, int kGroupMP, int& mt, int& nt) {
@@ -92,11 +110,35 @@ __device__ __forceinline__ void tile_coords_p(int t, int m_tiles, int n_tiles, i
     nt = r / gm;
 }
 
-template <bool LITE>
-__device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const CUtensorMap& tmap_b, const CUtensorMap& tmap_sfa, const CUtensorMap& tmap_sfb,
-                                               const CUtensorMap& tmap_c, const ParamsP& p) {
-    using Cfg = PairCfg<LITE>;
-    constexpr int kStagesP = Cfg::kStages;
+// The tiles of one pair (see ParamsP).
+struct TileWalk {
+    int pair, pairs, n_first, n_early, order;               // order: this pair's place among the takers of the second product's late tiles
+    uint32_t count;
+    __device__ __forceinline__ TileWalk(const ParamsP& p, int pair_, int pairs_) : pair(pair_), pairs(pairs_) {
+        const int others = pairs - p.rest;
+        const bool extra = pair < p.rest;
+        n_first = p.n0 / pairs + (extra ? 1 : 0);
+        n_early = extra ? 0 : p.early;
+        order = extra ? pair + others : pair - p.rest;
+        const int late = p.n1 - p.early * others;
+        count = (uint32_t)(n_first + n_early + (late > order ? (late - order + pairs - 1) / pairs : 0));
+    }
+    // tile tl (< count) of this pair: the product it belongs to and its coordinates there
+    __device__ __forceinline__ int locate(const ParamsP& p, uint32_t tl, int& mt, int& nt) const {
+        const int x = (int)tl - n_first, others = pairs - p.rest;
+        const int which = x < 0 ? 0 : 1;
+        const int t = x < 0 ? (int)tl * pairs + pair : x < n_early ? x * others + order : p.early * others + (x - n_early) * pairs + order;
+        const ProblemP& q = p.prob[which];
+        tile_coords_p(t, q.m_tiles, q.n_tiles, q.group_m, mt, nt);
+        return which;
+    }
+};
+
+template <bool LITE, int PN>
+__device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP& p) {
+    using Cfg = PairCfg<LITE, PN>;
+    constexpr int kStagesP = Cfg::kStages, kAccBufs = Cfg::kAccBufs;
+    constexpr uint32_t kStageB = Cfg::kStageB, kSfSlotB = Cfg::kSfSlotB;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* sf_ring = smem + kStagesP * kStageB;
@@ -105,32 +147,28 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
     uint64_t* full_bar = bars;                              // [kStagesP] leader: operands and scale tiles of both CTAs landed
     uint64_t* empty_bar = full_bar + kStagesP;              // [kStagesP] per CTA: stage and scale slot free (pair commit)
     uint64_t* turn = empty_bar + kStagesP;                  // [2] leader: baton between the two MMA issuers
-    uint64_t* tmem_full = turn + 2;                         // per CTA: accumulator complete (pair commit)
-    uint64_t* tmem_empty = tmem_full + 1;                   // leader: both CTAs drained their accumulators
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tmem_empty + 1);   // [2] base columns of the TMEM allocation(s)
+    uint64_t* tmem_full = turn + 2;                         // [kAccBufs] per CTA: accumulator complete (pair commit)
+    uint64_t* tmem_empty = tmem_full + kAccBufs;            // [kAccBufs] leader: both CTAs drained the accumulator
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tmem_empty + kAccBufs);   // [2] base columns of the TMEM allocation(s)
     volatile uint32_t* abort_flag = tmem_slot + 2;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();                // 0 = leader
-    const uint32_t pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
-    const int num_tiles = p.m_tiles * p.n_tiles;
-    const int nkc = (int)(p.K >> 7);                        // 128-element scale tiles along K
-    const int num_kt = (nkc + 1) >> 1;                      // 256-element pipeline steps
-    const uint32_t my_tiles = pair < (uint32_t)num_tiles ? ((uint32_t)num_tiles - pair + num_pairs - 1) / num_pairs : 0u;
-    const uint32_t total = my_tiles * (uint32_t)num_kt;
+    const TileWalk walk(p, (int)(blockIdx.x >> 1), (int)(gridDim.x >> 1));
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStagesP; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
         mbar_init(&turn[0], 1); mbar_init(&turn[1], 1);
-        mbar_init(tmem_full, 1);
-        mbar_init(tmem_empty, 16);
+        for (int b = 0; b < kAccBufs; ++b) { mbar_init(&tmem_full[b], 1); mbar_init(&tmem_empty[b], 16 / kAccBufs); }
         *abort_flag = 0;
         mbar_fence_init();
-        prefetch_tensormap(&tmap_a);
-        prefetch_tensormap(&tmap_b);
-        prefetch_tensormap(&tmap_sfa);
-        prefetch_tensormap(&tmap_sfb);
-        prefetch_tensormap(&tmap_c);
+        for (int i = 0; i < (p.n1 > 0 ? 2 : 1); ++i) {
+            prefetch_tensormap(&maps.a[i]);
+            prefetch_tensormap(&maps.b[i]);
+            prefetch_tensormap(&maps.sfa[i]);
+            prefetch_tensormap(&maps.sfb[i]);
+            prefetch_tensormap(&maps.c[i]);
+        }
     }
     if (warp == 1) {
         if (LITE) {                                         // accumulator and scale slots as two allocations: 128 columns stay free
@@ -146,7 +184,7 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
     cluster_sync_all();                                     // both CTAs' barriers exist before anyone signals across
     tc_fence_after_sync();
     const uint32_t tmem_acc = tmem_slot[0];                 // 256 accumulator columns
-    const uint32_t tmem_sf = LITE ? tmem_slot[1] : tmem_slot[0] + 256;   // scale slots of 24 columns
+    const uint32_t tmem_sf = LITE ? tmem_slot[1] : tmem_slot[0] + 256;   // scale slots of kSfCols columns
     // Warp group 0 (producer, issuers, scale loader) needs few registers; the epilogue groups take them to hold 128 columns
     // of the accumulator each.
     // Each warp group (four warps) sets its register limit once, at the head of its own branch: all four warps must
@@ -162,17 +200,19 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
         if (lane == 0) {
             uint32_t it = 0;
             bool ok = true;
-            for (uint32_t tl = 0; tl < my_tiles && ok; ++tl) {
+            for (uint32_t tl = 0; tl < walk.count && ok; ++tl) {
                 int mt, nt;
-                tile_coords_p((int)(pair + tl * num_pairs), p.m_tiles, p.n_tiles, p.group_m, mt, nt);
+                const int w = walk.locate(p, tl, mt, nt);
+                const int num_kt = p.prob[w].num_kt;
+                const CUtensorMap *map_a = &maps.a[w], *map_b = &maps.b[w];
                 const int a_rt = 2 * mt + (int)rank;                            // this CTA's 128-row tile of A
                 for (int kt = 0; kt < num_kt; ++kt, ++it) {
                     const int s = it % kStagesP;
                     if (!(ok = mbar_wait(&empty_bar[s], ((it / kStagesP) & 1) ^ 1, abort_flag))) break;
                     uint8_t* st = smem + s * kStageB;
                     if (rank == 0) mbar_expect_tx(&full_bar[s], 2 * (kStageB + kSfSlotB));   // operands and scales of both CTAs
-                    tma_load_2d_pair(st, &tmap_a, &full_bar[s], kt * kGemmBKBytes, a_rt * 128);
-                    tma_load_2d_pair(st + kAB, &tmap_b, &full_bar[s], kt * kGemmBKBytes, nt * PN + (int)rank * 128);
+                    tma_load_2d_pair(st, map_a, &full_bar[s], kt * kGemmBKBytes, a_rt * 128);
+                    tma_load_2d_pair(st + kAB, map_b, &full_bar[s], kt * kGemmBKBytes, nt * PN + (int)rank * (PN / 2));
                 }
             }
             if (!ok) *abort_flag = 1;
@@ -190,18 +230,18 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
             const uint64_t desc0 = make_smem_desc(smem_u32(smem), 16, 1024, 2);
             const uint32_t desc_hi = (uint32_t)(desc0 >> 32);
             const uint32_t a_lo0 = (uint32_t)desc0;
-            const bool k_tail = (nkc & 1) != 0;                               // last step holds 128 elements only
-            const uint32_t acc = tmem_acc;
             const uint32_t me = warp == 1 ? 0u : 1u;
             uint32_t s = me % kStagesP, ph = 0, tile_i = 0, n = 0;
-            int kt = (int)me;
-            while (kt >= num_kt) { kt -= num_kt; ++tile_i; }
+            auto steps_of = [&](uint32_t tile) { return p.prob[(int)tile < walk.n_first ? 0 : 1].num_kt; };
+            int kt = (int)me, num_kt = steps_of(0);
+            while (tile_i < walk.count && kt >= num_kt) { kt -= num_kt; num_kt = steps_of(++tile_i); }
             bool ok = true;
-            for (uint32_t it = me; it < total; it += 2, ++n) {
+            for (; tile_i < walk.count; ++n) {
                 if (!(ok = mbar_wait(&full_bar[s], ph, abort_flag))) break;
                 tc_fence_after_sync();
                 const uint32_t a_lo = a_lo0 + s * (kStageB >> 4), b_lo = a_lo + (kAB >> 4);
-                const uint32_t sfa_t = tmem_sf + s * kSfSlotColsP, sfb_t = sfa_t + 8;
+                const uint32_t sfa_t = tmem_sf + s * Cfg::kSfCols, sfb_t = sfa_t + 8;
+                constexpr uint32_t kSfbChunk = PN / 32;      // TMEM columns of one 128-element chunk's B scales
                 {   // the step's scales: shared memory -> TMEM of both CTAs, replicated to the four lane quadrants by the copy;
                     // issued while the other thread still issues its MMAs (a different TMEM slot), ordered before this
                     // thread's MMAs by program order
@@ -210,16 +250,17 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
                     for (int c = 0; c < 2; ++c) {
                         tc_cp_32x128b_warpx4_pair(sfa_t + 4 * c, make_smem_desc(sf_s + c * kSfTile, 0, 128, 0));
 #pragma unroll
-                        for (int j = 0; j < 2; ++j)
-                            tc_cp_32x128b_warpx4_pair(sfb_t + 8 * c + 4 * j, make_smem_desc(sf_s + kSfaB + (2 * j + c) * kSfTile, 0, 128, 0));
+                        for (int j = 0; j < PN / 128; ++j)
+                            tc_cp_32x128b_warpx4_pair(sfb_t + kSfbChunk * c + 4 * j, make_smem_desc(sf_s + kSfaB + (2 * j + c) * kSfTile, 0, 128, 0));
                     }
                 }
                 if (!(ok = mbar_wait_spin(&turn[me], (n & 1) ^ me ^ 1, abort_flag))) break;   // the step before mine is issued
                 // The copies above did not need the accumulator.  Waited for under the baton: with one K-step per tile the
-                // two threads alternate between tiles, and a thread that waited before its turn could see the hand-back of
-                // two tiles ago as its own (a phase parity only tells neighbouring phases apart).
+                // two threads alternate between tiles, and a thread that waited before its turn could see an earlier tile's
+                // hand-back as its own (a phase parity only tells neighbouring phases apart).
+                const uint32_t buf = tile_i % kAccBufs, acc = tmem_acc + buf * PN;
                 if (kt == 0) {
-                    if (!(ok = mbar_wait(tmem_empty, (tile_i & 1) ^ 1, abort_flag))) break;
+                    if (!(ok = mbar_wait(&tmem_empty[buf], ((tile_i / kAccBufs) & 1) ^ 1, abort_flag))) break;
                     tc_fence_after_sync();
                 }
                 const uint32_t hi2 = 2u << 30;
@@ -227,18 +268,19 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
                 auto D = [&](uint32_t lo) { return ((uint64_t)desc_hi << 32) | lo; };
                 tc_mma_mxf4_pair(acc, D(a_lo), D(b_lo), idesc0, sfa_t, sfb_t, kt != 0 ? 1u : 0u);
                 tc_mma_mxf4_pair(acc, D(a_lo + 2), D(b_lo + 2), idesc1, sfa_t | hi2, sfb_t | hi2, 1u);
-                if (!(last && k_tail)) {
-                    tc_mma_mxf4_pair(acc, D(a_lo + 4), D(b_lo + 4), idesc0, sfa_t + 4, sfb_t + 8, 1u);
-                    tc_mma_mxf4_pair(acc, D(a_lo + 6), D(b_lo + 6), idesc1, (sfa_t + 4) | hi2, (sfb_t + 8) | hi2, 1u);
+                // an odd number of 128-element chunks: the last step holds one only
+                if (!(last && (p.prob[(int)tile_i < walk.n_first ? 0 : 1].nkc & 1) != 0)) {
+                    tc_mma_mxf4_pair(acc, D(a_lo + 4), D(b_lo + 4), idesc0, sfa_t + 4, sfb_t + kSfbChunk, 1u);
+                    tc_mma_mxf4_pair(acc, D(a_lo + 6), D(b_lo + 6), idesc1, (sfa_t + 4) | hi2, (sfb_t + kSfbChunk) | hi2, 1u);
                 }
                 tc_fence_before_sync();
                 mbar_arrive(&turn[me ^ 1]);                                    // pass the baton
                 tc_commit_pair(&empty_bar[s]);                                 // frees the operand stage and the scale slot
-                if (last) tc_commit_pair(tmem_full);
+                if (last) tc_commit_pair(&tmem_full[buf]);
                 s += 2;
                 if (s >= (uint32_t)kStagesP) { s -= kStagesP; ph ^= 1; }
                 kt += 2;
-                while (kt >= num_kt) { kt -= num_kt; ++tile_i; }
+                while (tile_i < walk.count && kt >= num_kt) { kt -= num_kt; num_kt = steps_of(++tile_i); }
             }
             if (!ok) *abort_flag = 1;
         }
@@ -249,17 +291,20 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
         if (lane == 0) {
             uint32_t it = 0;
             bool ok = true;
-            for (uint32_t tl = 0; tl < my_tiles && ok; ++tl) {
+            for (uint32_t tl = 0; tl < walk.count && ok; ++tl) {
                 int mt, nt;
-                tile_coords_p((int)(pair + tl * num_pairs), p.m_tiles, p.n_tiles, p.group_m, mt, nt);
-                const int32_t a_row = (2 * mt + (int)rank) * nkc, b_row = nt * 2 * nkc;
+                const int w = walk.locate(p, tl, mt, nt);
+                const int num_kt = p.prob[w].num_kt, nkc = p.prob[w].nkc;
+                const CUtensorMap *map_a = &maps.sfa[w], *map_b = &maps.sfb[w];
+                const int32_t a_row = (2 * mt + (int)rank) * nkc, b_row = nt * (PN / 128) * nkc;
                 for (int kt = 0; kt < num_kt; ++kt, ++it) {
                     const int s = it % kStagesP;
                     if (!(ok = mbar_wait(&empty_bar[s], ((it / kStagesP) & 1) ^ 1, abort_flag))) break;
                     uint8_t* dst = sf_ring + s * kSfSlotB;
-                    tma_load_2d_pair(dst, &tmap_sfa, &full_bar[s], 0, a_row + 2 * kt);
-                    tma_load_2d_pair(dst + kSfaB, &tmap_sfb, &full_bar[s], 0, b_row + 2 * kt);
-                    tma_load_2d_pair(dst + kSfaB + 2 * kSfTile, &tmap_sfb, &full_bar[s], 0, b_row + nkc + 2 * kt);
+                    tma_load_2d_pair(dst, map_a, &full_bar[s], 0, a_row + 2 * kt);
+#pragma unroll
+                    for (int j = 0; j < PN / 128; ++j)
+                        tma_load_2d_pair(dst + kSfaB + j * 2 * kSfTile, map_b, &full_bar[s], 0, b_row + j * nkc + 2 * kt);
                 }
             }
             if (!ok) *abort_flag = 1;
@@ -268,13 +313,15 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
     } else {
         // ------------------------------------------------------------------ epilogue (both CTAs, own 128 rows)
         reg_alloc<Cfg::kRegsEpi>();                                  // the epilogue groups take the registers the others gave up
-        const int q = warp & 3, half = (warp - 4) >> 2;              // TMEM lane quadrant; columns 128 half .. 128 half + 127 of the tile
+        // A warp owns one TMEM lane quadrant.  One accumulator: the second group takes columns 128 .. 255 of every tile; two:
+        // the groups take alternate tiles, each its own accumulator.
+        const int q = warp & 3, half = (warp - 4) >> 2;
         uint8_t* stage = epi_ring + (warp - 4) * kEpiBuf;
         const uint64_t pol_c = l2_policy_evict_first();         // the output is not read again here: let the operands keep L2
         bool ok = true;
         // One staged block: 16 registers = 64 bytes of this lane's row, columns [col, col + 64 B), into this warp's buffer
         // (64-byte swizzle: the row-per-lane writes are conflict-free) and out by TMA.
-        auto put = [&](const uint32_t (&w)[16], int32_t col, int32_t row0, bool in_range) {
+        auto put = [&](const uint32_t (&w)[16], const CUtensorMap* map, bool add, int32_t col, int32_t row0, bool in_range) {
             if (lane == 0) bulk_wait_group_read<0>();           // the store before this one must have left the buffer
             __syncwarp();
             uint4* dst = reinterpret_cast<uint4*>(stage + lane * 64);
@@ -285,16 +332,19 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
             __syncwarp();
             if (lane == 0) {
                 if (in_range) {
-                    if (p.accumulate) tma_reduce_add_2d(&tmap_c, stage, col, row0);
-                    else tma_store_2d_hint(&tmap_c, stage, col, row0, pol_c);
+                    if (add) tma_reduce_add_2d(map, stage, col, row0);
+                    else tma_store_2d_hint(map, stage, col, row0, pol_c);
                 }
                 bulk_commit_group();
             }
         };
-        for (uint32_t tl = 0; tl < my_tiles; ++tl) {
+        for (uint32_t tl = kAccBufs == 2 ? half : 0; tl < walk.count; tl += kAccBufs) {
             int mt, nt;
-            tile_coords_p((int)(pair + tl * num_pairs), p.m_tiles, p.n_tiles, p.group_m, mt, nt);
-            if (lane == 0) ok = mbar_wait(tmem_full, tl & 1, abort_flag);
+            const int w = walk.locate(p, tl, mt, nt);
+            const ProblemP& pr = p.prob[w];
+            const CUtensorMap* map = &maps.c[w];
+            const uint32_t buf = kAccBufs == 2 ? half : 0;
+            if (lane == 0) ok = mbar_wait(&tmem_full[buf], (tl / kAccBufs) & 1, abort_flag);
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok) break;
             tc_fence_after_sync();
@@ -309,29 +359,29 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
                 if (hb == 4 / Cfg::kBatch - 1) {                // the accumulator is in registers: the next tile's MMAs may start
                     tc_fence_before_sync();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive_cluster(tmem_empty, 0);
+                    if (lane == 0) mbar_arrive_cluster(&tmem_empty[buf], 0);
                 }
-                const int64_t colb = (int64_t)nt * PN + half * 128 + hb * Cfg::kBatch * 32;
+                const int64_t colb = (int64_t)nt * PN + (kAccBufs == 1 ? half * 128 : 0) + hb * Cfg::kBatch * 32;
 #pragma unroll
                 for (int c = 0; c < Cfg::kBatch; ++c) {
                     const int64_t col = colb + c * 32;
-                    const bool in_range = row0 < p.M && col < p.N;
-                    uint32_t w[16];
-                    if (p.out_fp32) {
+                    const bool in_range = row0 < pr.M && col < pr.N;
+                    uint32_t o[16];
+                    if (pr.out_fp32) {
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) w[j] = __float_as_uint(__uint_as_float(r[c][16 * h + j]) * p.alpha);
-                            put(w, (int32_t)col + 16 * h, (int32_t)row0, in_range && col + 16 * h < p.N);
+                            for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(r[c][16 * h + j]) * pr.alpha);
+                            put(o, map, pr.accumulate != 0, (int32_t)col + 16 * h, (int32_t)row0, in_range && col + 16 * h < pr.N);
                         }
                     } else {
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
-                            const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(r[c][2 * j]) * p.alpha,
-                                                                           __uint_as_float(r[c][2 * j + 1]) * p.alpha);
-                            w[j] = *reinterpret_cast<const uint32_t*>(&h);
+                            const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(r[c][2 * j]) * pr.alpha,
+                                                                           __uint_as_float(r[c][2 * j + 1]) * pr.alpha);
+                            o[j] = *reinterpret_cast<const uint32_t*>(&h);
                         }
-                        put(w, (int32_t)col, (int32_t)row0, in_range);
+                        put(o, map, false, (int32_t)col, (int32_t)row0, in_range);
                     }
                 }
             }
@@ -358,28 +408,26 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmap_a, const 
     }
 }
 
+template <int PN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsP, 1)
-gemm_mxf4_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
-                      const __grid_constant__ CUtensorMap tmap_sfa, const __grid_constant__ CUtensorMap tmap_sfb,
-                      const __grid_constant__ CUtensorMap tmap_c, const ParamsP p) {
-    gemm_pair_body<false>(tmap_a, tmap_b, tmap_sfa, tmap_sfb, tmap_c, p);
+gemm_mxf4_pair_kernel(const __grid_constant__ MapsP maps, const __grid_constant__ ParamsP p) {
+    gemm_pair_body<false, PN>(maps, p);
 }
 
 // The small-footprint build (see PairCfg): same roles, same arithmetic, same accumulation order.
-__global__ void __cluster_dims__(2, 1, 1) __maxnreg__(PairCfg<true>::kLaunchRegs)
-gemm_mxf4_pair_lite_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
-                           const __grid_constant__ CUtensorMap tmap_sfa, const __grid_constant__ CUtensorMap tmap_sfb,
-                           const __grid_constant__ CUtensorMap tmap_c, const ParamsP p) {
-    gemm_pair_body<true>(tmap_a, tmap_b, tmap_sfa, tmap_sfb, tmap_c, p);
+using LiteCfg = PairCfg<true, 256>;
+__global__ void __cluster_dims__(2, 1, 1) __maxnreg__(LiteCfg::kLaunchRegs)
+gemm_mxf4_pair_lite_kernel(const __grid_constant__ MapsP maps, const __grid_constant__ ParamsP p) {
+    gemm_pair_body<true, 256>(maps, p);
 }
 
 }  // namespace
 
 cudaError_t fetch_gemm_pair_status(unsigned int* word) { return device_status_fetch(word); }
 
-template <bool LITE, typename K>
+template <bool LITE, int PN, typename K>
 static cudaError_t pair_kernel_init(K kernel) {
-    using Cfg = PairCfg<LITE>;
+    using Cfg = PairCfg<LITE, PN>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmem);
     if (e != cudaSuccess) return e;
     // All of the SM's configurable memory as shared memory: two kernels can only share an SM under one carve-out, and
@@ -394,25 +442,50 @@ static cudaError_t pair_kernel_init(K kernel) {
 }
 
 cudaError_t gemm_pair_init() {
-    const cudaError_t e = pair_kernel_init<false>(gemm_mxf4_pair_kernel);
-    return e != cudaSuccess ? e : pair_kernel_init<true>(gemm_mxf4_pair_lite_kernel);
+    cudaError_t e = pair_kernel_init<false, 256>(gemm_mxf4_pair_kernel<256>);
+    if (e == cudaSuccess) e = pair_kernel_init<false, 128>(gemm_mxf4_pair_kernel<128>);
+    return e != cudaSuccess ? e : pair_kernel_init<true, 256>(gemm_mxf4_pair_lite_kernel);
 }
 
-cudaError_t launch_gemm_pair(const GemmArgs& a, cudaStream_t stream) {
-    ParamsP p;
-    p.C = a.C;
-    p.M = a.M; p.N = a.N; p.K = a.K; p.ldc = a.ldc;
-    p.alpha = a.alpha; p.out_fp32 = a.out_fp32;
-    p.m_tiles = (int)((a.M + PM - 1) / PM);
-    p.n_tiles = (int)((a.N + PN - 1) / PN);
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    const int tiles = p.m_tiles * p.n_tiles;
-    const int pairs = tiles < sms / 2 ? tiles : sms / 2;
-    p.accumulate = a.accumulate;
+namespace {
+int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
+
+// How the tiles of one or two products spread over the pairs (see ParamsP), and how long the last pair takes: a tile
+// costs cost[i].  `early` is the best of the numbers around cost[0] / cost[1].
+struct Spread {
+    int rest, early;
+    double time;
+};
+Spread spread_tiles(int n0, int n1, const double (&cost)[2], int pairs) {
+    Spread best{n0 % pairs, 0, 0.0};
+    const int rest = best.rest, others = pairs - rest;
+    const int around = rest != 0 ? (int)(cost[0] / cost[1]) : 0;
+    for (int e = around > 0 ? around - 1 : 0; e <= (rest != 0 ? around + 1 : 0); ++e) {
+        if (e > 0 && e > n1 / others) break;
+        const int late = n1 - e * others, rounds = late / pairs, left = late % pairs;
+        const double t_others = (n0 / pairs) * cost[0] + (e + rounds + (left > 0 ? 1 : 0)) * cost[1];
+        const double t_rest = rest == 0 ? 0.0 : (n0 / pairs + 1) * cost[0] + (rounds + (left > others ? 1 : 0)) * cost[1];
+        const double t = t_others > t_rest ? t_others : t_rest;
+        if (best.time == 0.0 || t < best.time) { best.early = e; best.time = t; }
+    }
+    return best;
+}
+
+// Microseconds a pair spends on one tile.  Measured: both widths take their operands at the rate the L2 gives them (35 KB
+// per CTA and K-step of a 256-wide tile in 0.42 us, 26 KB of a 128-wide one in 0.31); a tile's hand-over is hidden by the
+// second accumulator in part only (the stores remain).
+double tile_cost(int pn, int64_t K) {
+    const double steps = (double)ceil_div(K, 256);
+    return pn == 256 ? 0.42 * steps + 0.8 : 0.31 * steps + 0.45;
+}
+
+void fill_problem(ProblemP& p, const GemmArgs& a, int pn) {
+    p.M = a.M; p.N = a.N;
+    p.nkc = (int)(a.K >> 7);
+    p.num_kt = (p.nkc + 1) >> 1;
+    p.alpha = a.alpha; p.out_fp32 = a.out_fp32; p.accumulate = a.accumulate;
+    p.m_tiles = ceil_div(a.M, PM);
+    p.n_tiles = ceil_div(a.N, pn);
     // Tile order: groups of group_m pair-tile rows x all n-tiles.  Inside a group the A rows stay in L2 and B streams
     // through once; B is fetched from DRAM once for the whole launch only if it survives in L2 from one group to the
     // next, i.e. if a group's A rows + all of B + the group's output fit the part of L2 that behaves as one cache
@@ -420,21 +493,67 @@ cudaError_t launch_gemm_pair(const GemmArgs& a, cudaStream_t stream) {
     // eight rows read 348 MB from DRAM, four 243 MB (operands: 168 MB) at the same speed inside a backward step;
     // groups of two or one row read a little less still but cost 0.3 % / 2.5 % of the step (fewer pairs share a B tile
     // at any moment).
-    {
-        const double b_bytes = (double)a.N * (double)a.K * 0.53125, out_b = a.out_fp32 ? 4.0 : 2.0;
-        int gm = 8.0 * 256.0 * (double)a.K * 0.53125 + b_bytes + 8.0 * 256.0 * (double)a.N * out_b > 48.0 * 1024 * 1024 ? 4 : 8;
-        const char* e = getenv("MXFP4_GEMM_GROUP_M");              // tuning switch: fixed group size (1..64) instead of the rule above
-        if (e != nullptr && atoi(e) >= 1 && atoi(e) <= 64) gm = atoi(e);
-        p.group_m = gm;
+    const double b_bytes = (double)a.N * (double)a.K * 0.53125, out_b = a.out_fp32 ? 4.0 : 2.0;
+    p.group_m = 8.0 * 256.0 * (double)a.K * 0.53125 + b_bytes + 8.0 * 256.0 * (double)a.N * out_b > 48.0 * 1024 * 1024 ? 4 : 8;
+    const char* e = getenv("MXFP4_GEMM_GROUP_M");                  // tuning switch: fixed group size (1..64) instead of the rule above
+    if (e != nullptr && atoi(e) >= 1 && atoi(e) <= 64) p.group_m = atoi(e);
+}
+
+cudaError_t pair_count(int* pairs) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    *pairs = sms / 2;
+    return e;
+}
+}  // namespace
+
+// Columns of a pair tile for a launch of these products (n = 1 or 2): the width with which the last pair is done first.
+// 128 wins where 256-wide tiles leave pairs idle: backward 8192 x 1024 x 1024 (dW has 16 tiles of 32 steps) 36.1 -> 33.2 us,
+// 1024 x 1024 x 8192 alone 17.5 -> 16.2; it loses wherever the chip is full (16384 x 4096 x 4096: 106 -> 162).
+int gemm_pair_tile_n(const GemmArgs* a, int n) {
+    int pairs = 0;
+    if (a[0].lite || pair_count(&pairs) != cudaSuccess) return 256;
+    double time[2];
+    for (int i = 0; i < 2; ++i) {
+        const int pn = i == 0 ? 256 : 128;
+        const int lo = n == 2 && a[1].K > a[0].K ? 1 : 0;
+        const int n0 = ceil_div(a[lo].M, PM) * ceil_div(a[lo].N, pn), n1 = n == 2 ? ceil_div(a[1 - lo].M, PM) * ceil_div(a[1 - lo].N, pn) : 0;
+        const double cost[2] = {tile_cost(pn, a[lo].K), tile_cost(pn, a[n == 2 ? 1 - lo : lo].K)};
+        time[i] = spread_tiles(n0, n1, cost, n0 + n1 < pairs ? n0 + n1 : pairs).time;
     }
+    return time[1] < time[0] ? 128 : 256;
+}
+
+cudaError_t launch_gemm_pair(const GemmArgs* a, int n, int pn, cudaStream_t stream) {
+    if (n < 1 || n > 2 || (pn != 128 && pn != 256) || (a[0].lite && (n != 1 || pn != 256))) return cudaErrorInvalidValue;
+    int pairs = 0;
+    const cudaError_t e = pair_count(&pairs);
+    if (e != cudaSuccess) return e;
+    ParamsP p;
+    MapsP maps;
+    const int first = n == 2 && a[1].K > a[0].K ? 1 : 0;
+    int tiles[2] = {0, 0};
+    double cost[2];
+    for (int i = 0; i < 2; ++i) {
+        const GemmArgs& g = a[n == 2 ? (i == 0 ? first : 1 - first) : 0];
+        fill_problem(p.prob[i], g, pn);
+        maps.a[i] = g.tmap_a; maps.b[i] = g.tmap_b; maps.sfa[i] = g.tmap_sfa; maps.sfb[i] = g.tmap_sfb; maps.c[i] = g.tmap_c;
+        cost[i] = tile_cost(pn, g.K);
+        if (i < n) tiles[i] = p.prob[i].m_tiles * p.prob[i].n_tiles;
+    }
+    if (tiles[0] + tiles[1] < pairs) pairs = tiles[0] + tiles[1];
+    const Spread s = spread_tiles(tiles[0], tiles[1], cost, pairs);
+    p.n0 = tiles[0]; p.n1 = tiles[1]; p.rest = s.rest; p.early = s.early;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * pairs); cfg.blockDim = dim3(kThreadsP); cfg.stream = stream;
-    cfg.dynamicSmemBytes = a.lite ? PairCfg<true>::kSmem : PairCfg<false>::kSmem;
+    cfg.dynamicSmemBytes = a[0].lite ? LiteCfg::kSmem : pn == 128 ? PairCfg<false, 128>::kSmem : PairCfg<false, 256>::kSmem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, a.lite ? gemm_mxf4_pair_lite_kernel : gemm_mxf4_pair_kernel, a.tmap_a, a.tmap_b, a.tmap_sfa, a.tmap_sfb, a.tmap_c, p);
+    void (*kernel)(MapsP, ParamsP) = a[0].lite ? gemm_mxf4_pair_lite_kernel : pn == 128 ? gemm_mxf4_pair_kernel<128> : gemm_mxf4_pair_kernel<256>;
+    return cudaLaunchKernelEx(&cfg, kernel, maps, p);
 }
 
 }  // namespace mx

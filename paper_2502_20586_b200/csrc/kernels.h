@@ -40,7 +40,7 @@ cudaError_t launch_rht_dump(const QuantArgs& a, cudaStream_t stream);
 
 struct GemmArgs {
     CUtensorMap tmap_a;   // codes [M, K/2] bytes, box 128 B x 128 rows, 128-byte swizzle
-    CUtensorMap tmap_b;   // codes [N, K/2] bytes, box 128 B x BN rows (pair kernel: x 128 rows, each CTA loads half a B tile)
+    CUtensorMap tmap_b;   // codes [N, K/2] bytes, box 128 B x BN rows (pair kernel: x tile_n / 2 rows, each CTA loads half a B tile)
     CUtensorMap tmap_sfa; // scale tiles of A as [row tiles * K tiles, 512 bytes]: box = two consecutive tiles (pair kernel)
     CUtensorMap tmap_sfb; // ... of B
     CUtensorMap tmap_c;   // output [M, N] (leading dimension ldc): box 64 bytes x 32 rows, 64-byte swizzle (pair kernel's stores)
@@ -128,7 +128,9 @@ cudaError_t launch_mxint4_quantize(const float* y, int64_t R, int64_t K, int rou
 
 cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t stream);
 cudaError_t gemm_init();            // one-time: opt in to large dynamic shared memory
-cudaError_t launch_gemm_pair(const GemmArgs& a, cudaStream_t stream);
+// One product, or two independent ones in one launch; tile_n = what gemm_pair_tile_n says for them (the B maps' boxes depend on it).
+int gemm_pair_tile_n(const GemmArgs* a, int n);
+cudaError_t launch_gemm_pair(const GemmArgs* a, int n, int tile_n, cudaStream_t stream);
 cudaError_t gemm_pair_init();
 
 }  // namespace mx

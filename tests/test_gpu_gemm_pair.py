@@ -40,3 +40,21 @@ def test_tile_walk(gpu, M, N, K, fp32):
     # fp32 sums of K exact products (16 head-room on the unit roundoff); bf16 output: half a unit in the last place
     tol = 16 * 2.0 ** -24 if fp32 else 2.0 ** -8
     assert torch.all((got.double() - want).abs() <= tol * (a.abs() @ b.abs().t() if fp32 else want.abs()) + 1e-30)
+
+
+# The two products of a backward call go out as one launch: tile counts below and above the number of pairs (74), equal
+# and unequal K, a first product that leaves some pairs with one tile more than the rest, both tile widths, ragged edges.
+@pytest.mark.parametrize("b,n,m", [(256, 512, 512), (384, 8, 256), (8192, 1024, 1024), (8192, 1024, 3072), (4224, 1000, 1408), (1024, 4096, 4096),
+                                   (2048, 2304, 2432), (6400, 520, 128 * 33), (256, 5000, 3840), (10240, 264, 384)])
+def test_two_products_in_one_launch(gpu, b, n, m):
+    import torch
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(b + n + m)
+    dY, X, W = (torch.randn(shape, generator=gen, device="cuda").bfloat16() for shape in ((b, m), (b, n), (m, n)))
+    dX = torch.full((b, n), float("nan"), dtype=torch.float32, device="cuda")
+    dW = torch.full((m, n), float("nan"), dtype=torch.float32, device="cuda")
+    gpu.mxfp4_linear_backward(dY, X, W, 64, 5, gpu.ROUND_SR, gpu.OUT_FP32, dX=dX, dW=dW)
+    q = gpu.mxfp4_quantize_operands(dY, X, W, 64, 5, gpu.ROUND_SR)
+    assert torch.equal(dX, gpu.mxfp4_gemm(*q[0], *q[1], 16.0 / 9.0, gpu.OUT_FP32))
+    assert torch.equal(dW, gpu.mxfp4_gemm(*q[2], *q[3], 16.0 / 9.0, gpu.OUT_FP32))
+    assert gpu.mxfp4_device_status() == 0
