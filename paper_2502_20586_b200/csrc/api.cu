@@ -65,7 +65,7 @@ mxfp4_status runtime_init() {
         if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) st = MXFP4_ERR_CUDA;
         else if (major != 10) st = MXFP4_ERR_DEVICE;
         else if (mx::gemm_init() != cudaSuccess || mx::gemm_pair_init() != cudaSuccess || mx::quant_tc_init() != cudaSuccess ||
-                 mx::gemm_fused_init() != cudaSuccess || mx::gemm_f8_init() != cudaSuccess)
+                 mx::gemm_fused_init() != cudaSuccess)
             st = MXFP4_ERR_CUDA;
         g_rt.dev_status[dev] = st;
         g_rt.dev_done[dev] = true;
@@ -210,11 +210,12 @@ mxfp4_status make_output_map(CUtensorMap* map, void* C, int64_t M, int64_t N, in
                                      CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE), "output");
 }
 
-// Tensor map over the native scale tiles of an operand [rows, K]: 512 bytes per tile, tiles along K fastest; box = two tiles.
-mxfp4_status make_scales_map(CUtensorMap* map, const uint8_t* scales, int64_t rows, int64_t K) {
+// Tensor map over the native scale tiles of an operand [rows, K]: 512 bytes per tile, tiles along K fastest; box = the
+// `tiles` of one K-step of the GEMM.
+mxfp4_status make_scales_map(CUtensorMap* map, const uint8_t* scales, int64_t rows, int64_t K, int tiles) {
     const cuuint64_t dims[2] = {128, (cuuint64_t)(((rows + 127) / 128) * ((K + 127) / 128))};
     const cuuint64_t strides[1] = {512};
-    const cuuint32_t box[2] = {128, 2};
+    const cuuint32_t box[2] = {128, (cuuint32_t)tiles};
     const cuuint32_t elem_strides[2] = {1, 1};
     return encode_status(g_rt.encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<uint8_t*>(scales), dims, strides, box, elem_strides,
                                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -248,8 +249,8 @@ struct GemmPlan {
             if (st != MXFP4_OK) return st;
             if ((st = make_codes_map(&a.tmap_b, B[i], a.N, a.K, a.use_pair ? tile_n / 2 : mx::kGemmBN)) != MXFP4_OK) return st;
             if (!a.use_pair) continue;
-            if ((st = make_scales_map(&a.tmap_sfa, a.sfa, a.M, a.K)) != MXFP4_OK) return st;
-            if ((st = make_scales_map(&a.tmap_sfb, a.sfb, a.N, a.K)) != MXFP4_OK) return st;
+            if ((st = make_scales_map(&a.tmap_sfa, a.sfa, a.M, a.K, 2)) != MXFP4_OK) return st;
+            if ((st = make_scales_map(&a.tmap_sfb, a.sfb, a.N, a.K, 2)) != MXFP4_OK) return st;
             if ((st = make_output_map(&a.tmap_c, a.C, a.M, a.N, a.ldc, a.out_fp32 != 0)) != MXFP4_OK) return st;
         }
         return MXFP4_OK;
@@ -635,13 +636,19 @@ namespace {
 mxfp4_status gemm8_impl(const uint8_t* A, const uint8_t* B, const uint8_t* sfa, const uint8_t* sfb, const float* sa, const float* sb,
                         int64_t M, int64_t N, int64_t K, float alpha, void* C, int64_t ldc, int out_dtype, cudaStream_t stream) {
     mx::Gemm8Args a;
+    a.block_scaled = sfa != nullptr;
+    a.scale_a = sa; a.scale_b = sb;
+    a.M = M; a.N = N; a.K = K; a.alpha = alpha; a.C = C; a.ldc = ldc; a.out_fp32 = out_dtype == MXFP4_OUT_FP32;
+    const int tile_n = mx::gemm_f8_tile_n(a);
     mxfp4_status st = make_bytes_map(&a.tmap_a, A, M, K, 128);
     if (st != MXFP4_OK) return st;
-    if ((st = make_bytes_map(&a.tmap_b, B, N, K, 256)) != MXFP4_OK) return st;
-    a.block_scaled = sfa != nullptr;
-    a.sfa = sfa; a.sfb = sfb; a.scale_a = sa; a.scale_b = sb;
-    a.M = M; a.N = N; a.K = K; a.alpha = alpha; a.C = C; a.ldc = ldc; a.out_fp32 = out_dtype == MXFP4_OUT_FP32;
-    return cuda_status(mx::launch_gemm_f8(a, stream), "8-bit GEMM launch");
+    if ((st = make_bytes_map(&a.tmap_b, B, N, K, tile_n / 2)) != MXFP4_OK) return st;
+    if (a.block_scaled) {
+        if ((st = make_scales_map(&a.tmap_sfa, sfa, M, K, 1)) != MXFP4_OK) return st;
+        if ((st = make_scales_map(&a.tmap_sfb, sfb, N, K, 1)) != MXFP4_OK) return st;
+    }
+    if ((st = make_output_map(&a.tmap_c, C, M, N, ldc, a.out_fp32 != 0)) != MXFP4_OK) return st;
+    return cuda_status(mx::launch_gemm_f8(a, tile_n, stream), "8-bit GEMM launch");
 }
 mxfp4_status check_gemm8(const void* A, const void* B, const void* C, int64_t M, int64_t N, int64_t K, int64_t ldc, int out_dtype) {
     if (!A || !B || !C) return MXFP4_ERR_NULL;
@@ -717,7 +724,7 @@ mxfp4_status mxfp4_device_status(void* cuda_stream) {
     if (cudaStreamSynchronize(static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess) return MXFP4_ERR_CUDA;
     unsigned int word = 0;
     cudaError_t (*const fetch[])(unsigned int*) = {mx::fetch_gemm_status, mx::fetch_gemm_pair_status, mx::fetch_quant_tc_status,
-                                                   mx::fetch_fp4_ceiling_status, mx::fetch_gemm_fused_status, mx::fetch_gemm_f8_status};
+                                                   mx::fetch_fp4_ceiling_status, mx::fetch_gemm_fused_status};
     for (auto f : fetch) {
         unsigned int w = 0;
         if (f(&w) != cudaSuccess) return MXFP4_ERR_CUDA;

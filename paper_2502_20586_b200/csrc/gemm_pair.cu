@@ -1,4 +1,4 @@
-// Block-scaled FP4 GEMM, CTA-pair variant (tcgen05 cta_group::2): two CTAs of a 2-CTA cluster share one 256 x 256
+// Block-scaled FP4 GEMM (and 8-bit ones), CTA-pair variant (tcgen05 cta_group::2): two CTAs of a 2-CTA cluster share one 256 x 256
 // output tile.  Each CTA loads 128 rows of A and only HALF of the B tile (128 of its 256 rows); the pair MMA reads
 // both halves, so per MMA a tensor core pulls 4 KB + 4 KB from its own shared memory instead of 4 KB + 8 KB.  The
 // 1-CTA kernel (gemm.cu) is bound by exactly that operand traffic.  Each CTA keeps the accumulator of its own 128
@@ -21,6 +21,11 @@
 //                stores (or reduce-adds when accumulating).
 // A-row scales are per CTA; every CTA needs the scales of all 256 B rows.
 //
+// The 8-bit products (FP8 forward pass, MXINT4; enum Kind) run on the same roles: a one-CTA kernel of 128 x 256 tiles with
+// one accumulator and stores from registers served them before.  E4M3 16384 x 4096 x 4096: 221 -> 174 us (3.2 PFLOP/s,
+// 0.97 of twice the measured bf16 rate), 8192 x 3072 x 1024 50 -> 24, 16 x 4096 x 4096 16.5 -> 13.7; MXINT4
+// 16384 x 4096 x 4096 245 -> 185, 1024 x 1024 x 8192 34 -> 26.
+//
 // What the second epilogue group is for: TMEM has no room for a second 256-column accumulator beside the scale slots, so
 // the tensor pipe stands still from a tile's last MMA until the accumulator is in registers.  With eight warps that
 // hold it unconverted (in place of four that had to convert the first half before reading the second, and for fp32
@@ -40,8 +45,7 @@ namespace {
 
 constexpr int PM = 256;                                     // rows of a pair tile
 constexpr uint32_t kAB = 128 * kGemmBKBytes;                // 16 KB: 128 A rows x 128 B
-constexpr uint32_t kSfTile = 512;
-constexpr uint32_t kSfaB = 2 * kSfTile;                     // own 128 A rows, 2 tiles (8 K-blocks) per stage
+constexpr uint32_t kSfTile = 512;                           // scales of 128 rows x 128 elements
 constexpr uint32_t kEpiBuf = 2048;                          // epilogue staging: 32 rows x 64 B, one buffer per epilogue warp (8 warps)
 constexpr uint32_t kEpiB = 8 * kEpiBuf;
 constexpr uint32_t kBarB = 256;
@@ -53,13 +57,22 @@ constexpr int kThreadsP = 12 * 32;
 // one.  LITE (PN = 256) leaves room for a second, independent kernel on the same SM (the tensor-core quantiser's small
 // build, quantize_tc.cu, which quantises the OTHER product's operands meanwhile): four stages, TMEM taken as 256 + 128
 // columns, 104 registers per thread at launch.
-template <bool LITE, int PN>
+// Operand kinds: E2M1 with one UE8M0 scale per 32 elements (the method's GEMM); E4M3 with one scale per tensor (FP8 forward
+// pass, Section 4.1); E4M3 containers of the integers -7..7 with one UE8M0 scale per 32 elements (MXINT4, Section 3).  A
+// K-step is 128 bytes of every row and four MMAs in all of them.  Without scale slots in TMEM the plain E4M3 build has two
+// 256-column accumulators.
+enum Kind { kMxf4, kF8, kMxf8 };
+
+template <Kind KIND, bool LITE, int PN>
 struct PairCfg {
-    static constexpr int kAccBufs = 256 / PN;
+    static constexpr int kSfTiles = KIND == kMxf4 ? 2 : KIND == kMxf8 ? 1 : 0;   // scale tiles of 128 rows in a K-step
+    static constexpr int kAccBufs = PN == 128 || KIND == kF8 ? 2 : 1;
+    static constexpr int kWarpCols = kAccBufs == 2 ? PN : PN / 2;                // accumulator columns an epilogue warp takes
     static constexpr int kStages = LITE ? 4 : PN == 128 ? 8 : 6;
     static constexpr uint32_t kBB = PN / 2 * kGemmBKBytes;  // half of the B tile
     static constexpr uint32_t kStageB = kAB + kBB;
-    static constexpr uint32_t kSfSlotB = kSfaB + PN / 128 * 2 * kSfTile;   // A rows and all PN B rows
+    static constexpr uint32_t kSfaB = kSfTiles * kSfTile;   // own 128 A rows
+    static constexpr uint32_t kSfSlotB = kSfaB + PN / 128 * kSfaB;               // and all PN B rows
     static constexpr uint32_t kSfCols = kSfSlotB / 128;     // TMEM columns of a slot: 4 per 512-byte tile
     // scale ring: shared-memory slot i feeds TMEM slot i; same ring index as the operand stages so ONE commit frees both
     // The dynamic shared-memory window is at least 256-byte aligned, so rounding its base up to 1024 costs at most 768 bytes.
@@ -70,19 +83,20 @@ struct PairCfg {
     static constexpr int kRegsLight = LITE ? 56 : 72, kRegsEpi = LITE ? 128 : 216;
     static constexpr int kBatch = LITE ? 2 : 4;             // 32-column accumulator loads an epilogue warp keeps in flight
     static constexpr int kLaunchRegs = LITE ? 104 : 168;    // registers per thread the CTA is given at launch
-    static_assert(!LITE || PN == 256, "the small build has one 256-column accumulator");
+    static_assert(!LITE || (KIND == kMxf4 && PN == 256), "the small build has one 256-column accumulator");
     static_assert(kSmem <= 232448, "over the 227 KB shared-memory limit");
     static_assert((2 * kStages + 2 + 2 * kAccBufs) * 8 + 16 <= kBarB, "barriers");
-    static_assert(kStages * kSfCols <= (LITE ? 128 : 256), "scale slots do not fit their TMEM allocation");
+    static_assert(kStages * kSfCols <= (LITE ? 128 : 512 - kAccBufs * PN), "scale slots do not fit their TMEM allocation");
     static_assert(kThreadsP * kLaunchRegs >= 128 * (kRegsLight + 2 * kRegsEpi), "warp groups ask for more registers than the CTA holds");
 };
 
 struct ProblemP {                                           // one product of a launch
     int64_t M, N;
-    int nkc, num_kt;                                        // 128-element scale tiles along K; 256-element pipeline steps
+    int nkc, num_kt;                                        // 128-element scale tiles along K; pipeline steps
     int m_tiles, n_tiles;                                   // in pair tiles
     int group_m;                                            // rasterisation: this many pair-tile rows share the B tiles in L2 (fill_problem)
     float alpha;
+    const float *scale_a, *scale_b;                         // kF8: alpha is 1 / (*scale_a * *scale_b)
     int out_fp32;
     int accumulate;                                         // fp32 output only: C += instead of C =
 };
@@ -134,9 +148,29 @@ struct TileWalk {
     }
 };
 
-template <bool LITE, int PN>
+// Pair MMAs on 8-bit operands, K = 32: E4M3 (formats in the instruction descriptor), and the same with one UE8M0 scale per
+// row and the MMA's 32 elements.
+__device__ __forceinline__ void tc_mma_f8_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+__device__ __forceinline__ void tc_mma_mxf8_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                                 uint32_t sfa_tmem, uint32_t sfb_tmem, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::mxf8f6f4.block_scale.scale_vec::1X [%0], %1, %2, %3, [%5], [%6], p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(sfa_tmem), "r"(sfb_tmem)
+        : "memory");
+}
+
+template <Kind KIND, bool LITE, int PN>
 __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP& p) {
-    using Cfg = PairCfg<LITE, PN>;
+    using Cfg = PairCfg<KIND, LITE, PN>;
     constexpr int kStagesP = Cfg::kStages, kAccBufs = Cfg::kAccBufs;
     constexpr uint32_t kStageB = Cfg::kStageB, kSfSlotB = Cfg::kSfSlotB;
     extern __shared__ uint8_t smem_raw[];
@@ -165,8 +199,10 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
         for (int i = 0; i < (p.n1 > 0 ? 2 : 1); ++i) {
             prefetch_tensormap(&maps.a[i]);
             prefetch_tensormap(&maps.b[i]);
-            prefetch_tensormap(&maps.sfa[i]);
-            prefetch_tensormap(&maps.sfb[i]);
+            if (KIND != kF8) {
+                prefetch_tensormap(&maps.sfa[i]);
+                prefetch_tensormap(&maps.sfb[i]);
+            }
             prefetch_tensormap(&maps.c[i]);
         }
     }
@@ -183,8 +219,8 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
     __syncthreads();
     cluster_sync_all();                                     // both CTAs' barriers exist before anyone signals across
     tc_fence_after_sync();
-    const uint32_t tmem_acc = tmem_slot[0];                 // 256 accumulator columns
-    const uint32_t tmem_sf = LITE ? tmem_slot[1] : tmem_slot[0] + 256;   // scale slots of kSfCols columns
+    const uint32_t tmem_acc = tmem_slot[0];                 // accumulator columns
+    const uint32_t tmem_sf = LITE ? tmem_slot[1] : tmem_slot[0] + kAccBufs * PN;   // scale slots of kSfCols columns
     // Warp group 0 (producer, issuers, scale loader) needs few registers; the epilogue groups take them to hold 128 columns
     // of the accumulator each.
     // Each warp group (four warps) sets its register limit once, at the head of its own branch: all four warps must
@@ -224,8 +260,10 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
         // warp 1, odd steps warp 2): while one issues, the other has already waited for its operands and then
         // commits.  A baton (mbarrier turn[]) keeps the MMAs in step order, so accumulation order is fixed.
         if (rank == 0 && lane == 0) {
-            // instruction descriptor: A, B = E2M1 (1), scale = UE8M0 (1), K-major, N >> 3 at bit 17, M >> 4 at bit 24
-            const uint32_t idesc0 = (1u << 7) | (1u << 10) | ((uint32_t)(PN >> 3) << 17) | (1u << 23) | ((uint32_t)(PM >> 4) << 24);
+            // instruction descriptor: K-major, N >> 3 at bit 17, M >> 4 at bit 24; A, B = E2M1 (1) or E4M3 (0) at bits 7 and 10;
+            // scaled kinds: scale = UE8M0 (bit 23), scale byte ids at bits 4 (B) and 29 (A); plain: D = fp32 (bit 4)
+            const uint32_t idesc0 = ((uint32_t)(PN >> 3) << 17) | ((uint32_t)(PM >> 4) << 24) |
+                                    (KIND == kMxf4 ? (1u << 7) | (1u << 10) | (1u << 23) : KIND == kMxf8 ? 1u << 23 : 1u << 4);
             const uint32_t idesc1 = idesc0 | (2u << 29) | (2u << 4);          // scale bytes 2, 3 of the 32-bit column
             const uint64_t desc0 = make_smem_desc(smem_u32(smem), 16, 1024, 2);
             const uint32_t desc_hi = (uint32_t)(desc0 >> 32);
@@ -240,18 +278,19 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
                 if (!(ok = mbar_wait(&full_bar[s], ph, abort_flag))) break;
                 tc_fence_after_sync();
                 const uint32_t a_lo = a_lo0 + s * (kStageB >> 4), b_lo = a_lo + (kAB >> 4);
-                const uint32_t sfa_t = tmem_sf + s * Cfg::kSfCols, sfb_t = sfa_t + 8;
+                const uint32_t sfa_t = tmem_sf + s * Cfg::kSfCols, sfb_t = sfa_t + 4 * Cfg::kSfTiles;
                 constexpr uint32_t kSfbChunk = PN / 32;      // TMEM columns of one 128-element chunk's B scales
                 {   // the step's scales: shared memory -> TMEM of both CTAs, replicated to the four lane quadrants by the copy;
                     // issued while the other thread still issues its MMAs (a different TMEM slot), ordered before this
                     // thread's MMAs by program order
                     const uint32_t sf_s = smem_u32(sf_ring + s * kSfSlotB);
 #pragma unroll
-                    for (int c = 0; c < 2; ++c) {
+                    for (int c = 0; c < Cfg::kSfTiles; ++c) {
                         tc_cp_32x128b_warpx4_pair(sfa_t + 4 * c, make_smem_desc(sf_s + c * kSfTile, 0, 128, 0));
 #pragma unroll
                         for (int j = 0; j < PN / 128; ++j)
-                            tc_cp_32x128b_warpx4_pair(sfb_t + kSfbChunk * c + 4 * j, make_smem_desc(sf_s + kSfaB + (2 * j + c) * kSfTile, 0, 128, 0));
+                            tc_cp_32x128b_warpx4_pair(sfb_t + kSfbChunk * c + 4 * j,
+                                                      make_smem_desc(sf_s + Cfg::kSfaB + (Cfg::kSfTiles * j + c) * kSfTile, 0, 128, 0));
                     }
                 }
                 if (!(ok = mbar_wait_spin(&turn[me], (n & 1) ^ me ^ 1, abort_flag))) break;   // the step before mine is issued
@@ -266,12 +305,21 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
                 const uint32_t hi2 = 2u << 30;
                 const bool last = kt == num_kt - 1;
                 auto D = [&](uint32_t lo) { return ((uint64_t)desc_hi << 32) | lo; };
-                tc_mma_mxf4_pair(acc, D(a_lo), D(b_lo), idesc0, sfa_t, sfb_t, kt != 0 ? 1u : 0u);
-                tc_mma_mxf4_pair(acc, D(a_lo + 2), D(b_lo + 2), idesc1, sfa_t | hi2, sfb_t | hi2, 1u);
-                // an odd number of 128-element chunks: the last step holds one only
-                if (!(last && (p.prob[(int)tile_i < walk.n_first ? 0 : 1].nkc & 1) != 0)) {
-                    tc_mma_mxf4_pair(acc, D(a_lo + 4), D(b_lo + 4), idesc0, sfa_t + 4, sfb_t + kSfbChunk, 1u);
-                    tc_mma_mxf4_pair(acc, D(a_lo + 6), D(b_lo + 6), idesc1, (sfa_t + 4) | hi2, (sfb_t + kSfbChunk) | hi2, 1u);
+                if constexpr (KIND == kMxf4) {
+                    tc_mma_mxf4_pair(acc, D(a_lo), D(b_lo), idesc0, sfa_t, sfb_t, kt != 0 ? 1u : 0u);
+                    tc_mma_mxf4_pair(acc, D(a_lo + 2), D(b_lo + 2), idesc1, sfa_t | hi2, sfb_t | hi2, 1u);
+                    // an odd number of 128-element chunks: the last step holds one only
+                    if (!(last && (p.prob[(int)tile_i < walk.n_first ? 0 : 1].nkc & 1) != 0)) {
+                        tc_mma_mxf4_pair(acc, D(a_lo + 4), D(b_lo + 4), idesc0, sfa_t + 4, sfb_t + kSfbChunk, 1u);
+                        tc_mma_mxf4_pair(acc, D(a_lo + 6), D(b_lo + 6), idesc1, (sfa_t + 4) | hi2, (sfb_t + kSfbChunk) | hi2, 1u);
+                    }
+                } else {
+#pragma unroll
+                    for (uint32_t kb = 0; kb < 4; ++kb) {        // scale byte kb of the 32-bit column: K-block kb of the step
+                        if (KIND == kF8) tc_mma_f8_pair(acc, D(a_lo + 2 * kb), D(b_lo + 2 * kb), idesc0, (uint32_t)kt | kb ? 1u : 0u);
+                        else tc_mma_mxf8_pair(acc, D(a_lo + 2 * kb), D(b_lo + 2 * kb), idesc0 | (kb << 29) | (kb << 4), sfa_t | (kb << 30), sfb_t | (kb << 30),
+                                              (uint32_t)kt | kb ? 1u : 0u);
+                    }
                 }
                 tc_fence_before_sync();
                 mbar_arrive(&turn[me ^ 1]);                                    // pass the baton
@@ -286,9 +334,9 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
         }
     } else {
         // ------------------------------------------------------------------ scale loader (both CTAs)
-        // One box = the two 512-byte scale tiles of a 128-row tile for this K-step (box rows past the operand read zeros; a
+        // One box = the one or two 512-byte scale tiles of a 128-row tile for this K-step (box rows past the operand read zeros; a
         // box that runs over the end of an odd K reads the next row tile's first, which no MMA uses).
-        if (lane == 0) {
+        if (lane == 0 && KIND != kF8) {
             uint32_t it = 0;
             bool ok = true;
             for (uint32_t tl = 0; tl < walk.count && ok; ++tl) {
@@ -301,10 +349,10 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
                     const int s = it % kStagesP;
                     if (!(ok = mbar_wait(&empty_bar[s], ((it / kStagesP) & 1) ^ 1, abort_flag))) break;
                     uint8_t* dst = sf_ring + s * kSfSlotB;
-                    tma_load_2d_pair(dst, map_a, &full_bar[s], 0, a_row + 2 * kt);
+                    tma_load_2d_pair(dst, map_a, &full_bar[s], 0, a_row + Cfg::kSfTiles * kt);
 #pragma unroll
                     for (int j = 0; j < PN / 128; ++j)
-                        tma_load_2d_pair(dst + kSfaB + j * 2 * kSfTile, map_b, &full_bar[s], 0, b_row + j * nkc + 2 * kt);
+                        tma_load_2d_pair(dst + Cfg::kSfaB * (1 + j), map_b, &full_bar[s], 0, b_row + j * nkc + Cfg::kSfTiles * kt);
                 }
             }
             if (!ok) *abort_flag = 1;
@@ -349,19 +397,21 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
             if (!ok) break;
             tc_fence_after_sync();
             const int64_t row0 = (int64_t)mt * PM + (int64_t)rank * 128 + q * 32;
-            const uint32_t taddr = tmem_acc + ((uint32_t)(q * 32) << 16) + half * 128;
-#pragma unroll
-            for (int hb = 0; hb < 4 / Cfg::kBatch; ++hb) {
+            const uint32_t taddr = tmem_acc + ((uint32_t)(q * 32) << 16) + half * Cfg::kWarpCols;   // (two accumulators: its own, kWarpCols = PN)
+            constexpr int kBatches = Cfg::kWarpCols / 32 / Cfg::kBatch;
+            const float alpha = KIND == kF8 ? 1.0f / (*pr.scale_a * *pr.scale_b) : pr.alpha;
+#pragma unroll 1
+            for (int hb = 0; hb < kBatches; ++hb) {
                 uint32_t r[Cfg::kBatch][32];
 #pragma unroll
                 for (int c = 0; c < Cfg::kBatch; ++c) tmem_ld_32x32b_x32(taddr + (hb * Cfg::kBatch + c) * 32, r[c]);
                 tmem_ld_wait();
-                if (hb == 4 / Cfg::kBatch - 1) {                // the accumulator is in registers: the next tile's MMAs may start
+                if (hb == kBatches - 1) {                // the accumulator is in registers: the next tile's MMAs may start
                     tc_fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive_cluster(&tmem_empty[buf], 0);
                 }
-                const int64_t colb = (int64_t)nt * PN + (kAccBufs == 1 ? half * 128 : 0) + hb * Cfg::kBatch * 32;
+                const int64_t colb = (int64_t)nt * PN + (kAccBufs == 1 ? half * Cfg::kWarpCols : 0) + hb * Cfg::kBatch * 32;
 #pragma unroll
                 for (int c = 0; c < Cfg::kBatch; ++c) {
                     const int64_t col = colb + c * 32;
@@ -371,14 +421,14 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(r[c][16 * h + j]) * pr.alpha);
+                            for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(r[c][16 * h + j]) * alpha);
                             put(o, map, pr.accumulate != 0, (int32_t)col + 16 * h, (int32_t)row0, in_range && col + 16 * h < pr.N);
                         }
                     } else {
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
-                            const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(r[c][2 * j]) * pr.alpha,
-                                                                           __uint_as_float(r[c][2 * j + 1]) * pr.alpha);
+                            const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(r[c][2 * j]) * alpha,
+                                                                           __uint_as_float(r[c][2 * j + 1]) * alpha);
                             o[j] = *reinterpret_cast<const uint32_t*>(&h);
                         }
                         put(o, map, false, (int32_t)col, (int32_t)row0, in_range);
@@ -411,23 +461,27 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
 template <int PN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsP, 1)
 gemm_mxf4_pair_kernel(const __grid_constant__ MapsP maps, const __grid_constant__ ParamsP p) {
-    gemm_pair_body<false, PN>(maps, p);
+    gemm_pair_body<kMxf4, false, PN>(maps, p);
+}
+template <Kind KIND, int PN>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreadsP, 1)
+gemm_8bit_pair_kernel(const __grid_constant__ MapsP maps, const __grid_constant__ ParamsP p) {
+    gemm_pair_body<KIND, false, PN>(maps, p);
 }
 
 // The small-footprint build (see PairCfg): same roles, same arithmetic, same accumulation order.
-using LiteCfg = PairCfg<true, 256>;
+using LiteCfg = PairCfg<kMxf4, true, 256>;
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(LiteCfg::kLaunchRegs)
 gemm_mxf4_pair_lite_kernel(const __grid_constant__ MapsP maps, const __grid_constant__ ParamsP p) {
-    gemm_pair_body<true, 256>(maps, p);
+    gemm_pair_body<kMxf4, true, 256>(maps, p);
 }
 
 }  // namespace
 
 cudaError_t fetch_gemm_pair_status(unsigned int* word) { return device_status_fetch(word); }
 
-template <bool LITE, int PN, typename K>
+template <typename Cfg, typename K>
 static cudaError_t pair_kernel_init(K kernel) {
-    using Cfg = PairCfg<LITE, PN>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmem);
     if (e != cudaSuccess) return e;
     // All of the SM's configurable memory as shared memory: two kernels can only share an SM under one carve-out, and
@@ -442,9 +496,13 @@ static cudaError_t pair_kernel_init(K kernel) {
 }
 
 cudaError_t gemm_pair_init() {
-    cudaError_t e = pair_kernel_init<false, 256>(gemm_mxf4_pair_kernel<256>);
-    if (e == cudaSuccess) e = pair_kernel_init<false, 128>(gemm_mxf4_pair_kernel<128>);
-    return e != cudaSuccess ? e : pair_kernel_init<true, 256>(gemm_mxf4_pair_lite_kernel);
+    cudaError_t e = pair_kernel_init<PairCfg<kMxf4, false, 256>>(gemm_mxf4_pair_kernel<256>);
+    if (e == cudaSuccess) e = pair_kernel_init<PairCfg<kMxf4, false, 128>>(gemm_mxf4_pair_kernel<128>);
+    if (e == cudaSuccess) e = pair_kernel_init<PairCfg<kF8, false, 256>>(gemm_8bit_pair_kernel<kF8, 256>);
+    if (e == cudaSuccess) e = pair_kernel_init<PairCfg<kF8, false, 128>>(gemm_8bit_pair_kernel<kF8, 128>);
+    if (e == cudaSuccess) e = pair_kernel_init<PairCfg<kMxf8, false, 256>>(gemm_8bit_pair_kernel<kMxf8, 256>);
+    if (e == cudaSuccess) e = pair_kernel_init<PairCfg<kMxf8, false, 128>>(gemm_8bit_pair_kernel<kMxf8, 128>);
+    return e != cudaSuccess ? e : pair_kernel_init<LiteCfg>(gemm_mxf4_pair_lite_kernel);
 }
 
 namespace {
@@ -483,7 +541,8 @@ void fill_problem(ProblemP& p, const GemmArgs& a, int pn) {
     p.M = a.M; p.N = a.N;
     p.nkc = (int)(a.K >> 7);
     p.num_kt = (p.nkc + 1) >> 1;
-    p.alpha = a.alpha; p.out_fp32 = a.out_fp32; p.accumulate = a.accumulate;
+    p.alpha = a.alpha; p.scale_a = p.scale_b = nullptr;
+    p.out_fp32 = a.out_fp32; p.accumulate = a.accumulate;
     p.m_tiles = ceil_div(a.M, PM);
     p.n_tiles = ceil_div(a.N, pn);
     // Tile order: groups of group_m pair-tile rows x all n-tiles.  Inside a group the A rows stay in L2 and B streams
@@ -505,6 +564,16 @@ cudaError_t pair_count(int* pairs) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     *pairs = sms / 2;
     return e;
+}
+cudaError_t launch_pairs(void (*kernel)(MapsP, ParamsP), int pairs, uint32_t smem, const MapsP& maps, const ParamsP& p, cudaStream_t stream) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * pairs); cfg.blockDim = dim3(kThreadsP); cfg.stream = stream;
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, maps, p);
 }
 }  // namespace
 
@@ -545,15 +614,48 @@ cudaError_t launch_gemm_pair(const GemmArgs* a, int n, int pn, cudaStream_t stre
     if (tiles[0] + tiles[1] < pairs) pairs = tiles[0] + tiles[1];
     const Spread s = spread_tiles(tiles[0], tiles[1], cost, pairs);
     p.n0 = tiles[0]; p.n1 = tiles[1]; p.rest = s.rest; p.early = s.early;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * pairs); cfg.blockDim = dim3(kThreadsP); cfg.stream = stream;
-    cfg.dynamicSmemBytes = a[0].lite ? LiteCfg::kSmem : pn == 128 ? PairCfg<false, 128>::kSmem : PairCfg<false, 256>::kSmem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    const uint32_t smem = a[0].lite ? LiteCfg::kSmem : pn == 128 ? PairCfg<kMxf4, false, 128>::kSmem : PairCfg<kMxf4, false, 256>::kSmem;
     void (*kernel)(MapsP, ParamsP) = a[0].lite ? gemm_mxf4_pair_lite_kernel : pn == 128 ? gemm_mxf4_pair_kernel<128> : gemm_mxf4_pair_kernel<256>;
-    return cudaLaunchKernelEx(&cfg, kernel, maps, p);
+    return launch_pairs(kernel, pairs, smem, maps, p, stream);
+}
+
+// Columns of a pair tile for an 8-bit product: the width with which the last pair is done first.  Measured per tile: 0.39 us
+// a K-step + 0.2 (256 wide), 0.28 + 0.1 (128 wide).  128 wins where 256-wide tiles leave pairs idle (16 x 4096 x 4096:
+// 15.5 -> 13.7 us), 256 elsewhere (16384 x 4096 x 4096: 174 us against 250).
+int gemm_f8_tile_n(const Gemm8Args& a) {
+    int pairs = 0;
+    if (pair_count(&pairs) != cudaSuccess) return 256;
+    const double steps = (double)(a.K >> 7), cost[2] = {0.39 * steps + 0.2, 0.28 * steps + 0.1};
+    double time[2];
+    for (int i = 0; i < 2; ++i) time[i] = ceil_div((int64_t)ceil_div(a.M, PM) * ceil_div(a.N, i == 0 ? 256 : 128), pairs) * cost[i];
+    return time[1] < time[0] ? 128 : 256;
+}
+
+cudaError_t launch_gemm_f8(const Gemm8Args& a, int pn, cudaStream_t stream) {
+    if (pn != 128 && pn != 256) return cudaErrorInvalidValue;
+    int pairs = 0;
+    const cudaError_t e = pair_count(&pairs);
+    if (e != cudaSuccess) return e;
+    ParamsP p = {};
+    MapsP maps = {};
+    ProblemP& q = p.prob[0];
+    q.M = a.M; q.N = a.N;
+    q.nkc = q.num_kt = (int)(a.K >> 7);
+    q.alpha = a.alpha; q.scale_a = a.scale_a; q.scale_b = a.scale_b;
+    q.out_fp32 = a.out_fp32;
+    q.m_tiles = ceil_div(a.M, PM);
+    q.n_tiles = ceil_div(a.N, pn);
+    q.group_m = 8;
+    p.n0 = q.m_tiles * q.n_tiles;
+    if (p.n0 < pairs) pairs = p.n0;
+    p.rest = p.n0 % pairs;
+    maps.a[0] = a.tmap_a; maps.b[0] = a.tmap_b; maps.c[0] = a.tmap_c;
+    if (a.block_scaled) { maps.sfa[0] = a.tmap_sfa; maps.sfb[0] = a.tmap_sfb; }
+    if (a.block_scaled)
+        return pn == 128 ? launch_pairs(gemm_8bit_pair_kernel<kMxf8, 128>, pairs, PairCfg<kMxf8, false, 128>::kSmem, maps, p, stream)
+                         : launch_pairs(gemm_8bit_pair_kernel<kMxf8, 256>, pairs, PairCfg<kMxf8, false, 256>::kSmem, maps, p, stream);
+    return pn == 128 ? launch_pairs(gemm_8bit_pair_kernel<kF8, 128>, pairs, PairCfg<kF8, false, 128>::kSmem, maps, p, stream)
+                     : launch_pairs(gemm_8bit_pair_kernel<kF8, 256>, pairs, PairCfg<kF8, false, 256>::kSmem, maps, p, stream);
 }
 
 }  // namespace mx

@@ -58,3 +58,43 @@ def test_two_products_in_one_launch(gpu, b, n, m):
     assert torch.equal(dX, gpu.mxfp4_gemm(*q[0], *q[1], 16.0 / 9.0, gpu.OUT_FP32))
     assert torch.equal(dW, gpu.mxfp4_gemm(*q[2], *q[3], 16.0 / 9.0, gpu.OUT_FP32))
     assert gpu.mxfp4_device_status() == 0
+
+
+# The 8-bit products: both tile widths, one and several tiles per pair (alternating accumulators), fewer rows than a CTA
+# owns, ragged edges, one K-step, both output types.
+@pytest.mark.parametrize("M,N,K", [(1, 8, 128), (16, 4096, 256), (129, 264, 128), (1000, 4096, 384), (5120, 4104, 128), (300, 20480, 256)])
+@pytest.mark.parametrize("kind", ["fp8", "int4"])
+@pytest.mark.parametrize("fp32", [False, True])
+def test_eight_bit_products(gpu, M, N, K, kind, fp32):
+    import torch
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(M + N + K)
+    out = gpu.OUT_FP32 if fp32 else gpu.OUT_BF16
+
+    def codes(rows):
+        if kind == "fp8":
+            v = torch.randn((rows, K), generator=gen, device="cuda") * 8
+        else:
+            v = torch.randint(-7, 8, (rows, K), generator=gen, device="cuda").float()
+        c = v.to(torch.float8_e4m3fn)
+        return c.view(torch.uint8), c.double()
+
+    (ca, a), (cb, b) = codes(M), codes(N)
+    if kind == "fp8":
+        sa, sb = (torch.tensor([s, 0.0], device="cuda") for s in (3.0, 0.25))
+        got = gpu.mxfp4_fp8_gemm(ca, sa, cb, sb, out)
+        a = a / 0.75
+    else:
+        _, sa, _ = _operand(gen, M, K)
+        _, sb, _ = _operand(gen, N, K)
+        got = gpu.mxfp4_int4_gemm(ca, sa, cb, sb, 1.0, out)
+
+        def scale(s, rows):
+            t = s.view((rows + 127) // 128, K // 128, 32, 4, 4).permute(0, 3, 2, 1, 4).reshape(-1, K // 32)[:rows].double()
+            return torch.exp2(t - 127.0).repeat_interleave(32, 1)
+        a, b = a * scale(sa, M), b * scale(sb, N)
+    assert gpu.mxfp4_device_status() == 0
+    want, size = a @ b.t(), a.abs() @ b.abs().t()
+    # fp32 sums (and one rounding of the scale and of the product) of K terms; bf16 output: half a unit in the last place more
+    bound = 16 * 2.0 ** -24 * size + (0.0 if fp32 else 2.0 ** -8) * want.abs()
+    assert torch.all((got.double() - want).abs() <= bound + 1e-30)
