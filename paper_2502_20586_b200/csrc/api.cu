@@ -629,7 +629,8 @@ mxfp4_status mxfp4_fp8_quantize(const void* x, int64_t rows, int64_t cols, int64
     if (!aligned16(x) || !aligned16(codes) || (reinterpret_cast<uintptr_t>(scale) & 7u) != 0) return MXFP4_ERR_ALIGN;
     const mxfp4_status st = runtime_init();
     if (st != MXFP4_OK) return st;
-    return cuda_status(mx::launch_fp8_quantize(x, rows, cols, ld, codes, scale, static_cast<cudaStream_t>(cuda_stream)), "FP8 quantiser launch");
+    const mx::Fp8QuantArgs q{x, rows, cols, ld, codes, scale};
+    return cuda_status(mx::launch_fp8_quantize(&q, 1, nullptr, static_cast<cudaStream_t>(cuda_stream)), "FP8 quantiser launch");
 }
 
 namespace {
@@ -671,7 +672,7 @@ mxfp4_status mxfp4_fp8_gemm(const uint8_t* A_codes, const float* A_scale, const 
 
 size_t mxfp4_linear_forward_fp8_workspace(int64_t b, int64_t n, int64_t m) {
     if (b <= 0 || n <= 0 || m <= 0) return 0;
-    return (size_t)(round_up(b * n, 1024) + round_up(m * n, 1024) + 1024);      // codes of x, codes of W, the two scale pairs
+    return (size_t)(round_up(b * n, 1024) + round_up(m * n, 1024) + 1024);      // codes of x, codes of W, the two scale pairs and the partial maxima
 }
 
 mxfp4_status mxfp4_linear_forward_fp8(const void* x, const void* W, int64_t b, int64_t n, int64_t m, void* y, int out_dtype,
@@ -686,9 +687,10 @@ mxfp4_status mxfp4_linear_forward_fp8(const void* x, const void* W, int64_t b, i
     uint8_t* base = static_cast<uint8_t*>(workspace);
     uint8_t* cx = base;
     uint8_t* cw = cx + round_up(b * n, 1024);
-    float* sc = reinterpret_cast<float*>(cw + round_up(m * n, 1024));              // [0..1] x: scale, amax; [2..3] W
-    if ((st = cuda_status(mx::launch_fp8_quantize(x, b, n, n, cx, sc, stream), "FP8 quantiser launch (x)")) != MXFP4_OK) return st;
-    if ((st = cuda_status(mx::launch_fp8_quantize(W, m, n, n, cw, sc + 2, stream), "FP8 quantiser launch (W)")) != MXFP4_OK) return st;
+    float* sc = reinterpret_cast<float*>(cw + round_up(m * n, 1024));              // [0..1] x: scale, amax; [2..3] W; then partial maxima
+    static_assert(16 + mx::kFp8PartialBytes <= 1024, "scales and partial maxima share one kilobyte");
+    const mx::Fp8QuantArgs q[2] = {{x, b, n, n, cx, sc}, {W, m, n, n, cw, sc + 2}};
+    if ((st = cuda_status(mx::launch_fp8_quantize(q, 2, reinterpret_cast<uint16_t*>(sc + 4), stream), "FP8 quantiser launch")) != MXFP4_OK) return st;
     return gemm8_impl(cx, cw, nullptr, nullptr, sc, sc + 2, b, m, n, 1.0f, y, m, out_dtype, stream);
 }
 

@@ -117,9 +117,16 @@ int gemm_f8_tile_n(const Gemm8Args& a);            // from M, N, K
 cudaError_t launch_gemm_f8(const Gemm8Args& a, int tile_n, cudaStream_t stream);
 
 // Element-wise kernels of the extensions (variants.cu).
-// Per-tensor E4M3 quantisation: *scale = 448 / amax(x) (1 for an all-zero tensor), codes = E4M3(x * scale).
-// `scale` doubles as the amax scratch word while the call runs.
-cudaError_t launch_fp8_quantize(const void* x, int64_t rows, int64_t cols, int64_t ld, uint8_t* codes, float* scale, cudaStream_t stream);
+// Per-tensor E4M3 quantisation of one or two tensors: scale[0] = 448 / amax(x) (1 for an all-zero tensor), scale[1] = amax,
+// codes = E4M3(x * scale).  `partial` (kFp8PartialBytes of scratch, may be null) saves the memset of the amax words.
+struct Fp8QuantArgs {
+    const void* x;        // bf16 [rows, cols], leading dimension ld
+    int64_t rows, cols, ld;
+    uint8_t* codes;       // [rows, cols]
+    float* scale;         // [2]
+};
+constexpr size_t kFp8PartialBytes = 2 * 2 * 148;
+cudaError_t launch_fp8_quantize(const Fp8QuantArgs* a, int n, uint16_t* partial, cudaStream_t stream);
 // MXINT4 from fp32 pre-quantisation values y [R, K]: per 32-block E8M0 scale (Algorithm 1 / 2 rule), elements rounded
 // to integers in [-7, 7] (rounding 0: 3/4 pre-scale + stochastic rounding with the path's Philox draws; 1: nearest),
 // stored as E4M3 bytes; scales in the native layout.
