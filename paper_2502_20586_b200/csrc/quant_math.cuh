@@ -77,6 +77,13 @@ __device__ __forceinline__ void sr_draws32(const PhiloxKeys& ks, uint32_t stream
     rw[0] = a.x; rw[1] = a.y; rw[2] = a.z; rw[3] = a.w;
     rw[4] = b.x; rw[5] = b.y; rw[6] = b.z; rw[7] = b.w;
 }
+// The same for MX block `blk` = i0 / 32 of an operand below 2^36 elements.
+__device__ __forceinline__ void sr_draws32_block(const PhiloxKeys& ks, uint32_t stream_tag, uint32_t blk, uint32_t (&rw)[8]) {
+    const uint4 a = philox4x32_10(2u * blk, 0u, stream_tag, 1u, ks);
+    const uint4 b = philox4x32_10(2u * blk | 1u, 0u, stream_tag, 1u, ks);
+    rw[0] = a.x; rw[1] = a.y; rw[2] = a.z; rw[3] = a.w;
+    rw[4] = b.x; rw[5] = b.y; rw[6] = b.z; rw[7] = b.w;
+}
 
 // The SR draws of one operand view share seed and stream tag, and for operands below 2^36 elements the high counter
 // word is zero: the counter is (index, 0, tag, 1).  Everything in the first three rounds that does not depend on the
@@ -113,11 +120,9 @@ __device__ __forceinline__ uint4 philox4x32_10_view(uint32_t x0, const PhiloxVie
     }
     return make_uint4(c0, c1, c2, c3);
 }
-// The 32 draws of elements [i0, i0 + 32), i0 a multiple of 32 below 2^36.
-__device__ __forceinline__ void sr_draws32_view(const PhiloxKeys& ks, const PhiloxViewConsts& v, uint64_t i0, uint32_t (&rw)[8]) {
-    const uint32_t lo = (uint32_t)(i0 >> 4);
-    const uint4 a = philox4x32_10_view(lo, v, ks);
-    const uint4 b = philox4x32_10_view(lo | 1u, v, ks);
+__device__ __forceinline__ void sr_draws32_view(const PhiloxKeys& ks, const PhiloxViewConsts& v, uint32_t blk, uint32_t (&rw)[8]) {
+    const uint4 a = philox4x32_10_view(2u * blk, v, ks);
+    const uint4 b = philox4x32_10_view(2u * blk | 1u, v, ks);
     rw[0] = a.x; rw[1] = a.y; rw[2] = a.z; rw[3] = a.w;
     rw[4] = b.x; rw[5] = b.y; rw[6] = b.z; rw[7] = b.w;
 }
@@ -219,6 +224,16 @@ __device__ __forceinline__ uint32_t cvt_e2m1x4_rs(float v0, float v1, float v2, 
     return d;
 }
 
+// Two products with one factor in one instruction (mul.f32x2): each rounded like the scalar one, toward zero / to nearest.
+__device__ __forceinline__ void mul2_rz(float a0, float a1, float c, float& d0, float& d1) {
+    asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %4};\n\tmul.rz.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+        : "=f"(d0), "=f"(d1) : "f"(a0), "f"(a1), "f"(c));
+}
+__device__ __forceinline__ void mul2_rn(float a0, float a1, float c, float& d0, float& d1) {
+    asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %4};\n\tmul.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+        : "=f"(d0), "=f"(d1) : "f"(a0), "f"(a1), "f"(c));
+}
+
 // (a & ~mask) | (b & mask) in one LOP3.
 __device__ __forceinline__ uint32_t bitselect(uint32_t a, uint32_t b, uint32_t mask) {
     uint32_t d;
@@ -299,8 +314,11 @@ __device__ __forceinline__ void quantize_block32_rw(const float (&y)[32], const 
                 const uint32_t w = rw[2 * q + hh];
                 const uint32_t r_even = w & 0x00FF00FFu;                     // r_i      | r_{i+2} << 16
                 const uint32_t r_odd = __byte_perm(w, 0u, 0x4341);           // r_{i+1}  | r_{i+3} << 16
-                const uint32_t h_even = cvt_f16x2_rz(__fmul_rz(y[i], c), __fmul_rz(y[i + 2], c));
-                const uint32_t h_odd = cvt_f16x2_rz(__fmul_rz(y[i + 1], c), __fmul_rz(y[i + 3], c));
+                float z0, z1, z2, z3;
+                mul2_rz(y[i], y[i + 1], c, z0, z1);
+                mul2_rz(y[i + 2], y[i + 3], c, z2, z3);
+                const uint32_t h_even = cvt_f16x2_rz(z0, z2);
+                const uint32_t h_odd = cvt_f16x2_rz(z1, z3);
                 const uint32_t t_even = h_even * k.eight + (r_even * k.neg16 + 0x0FF80FF8u);   // + 8 (511 - 2r) per lane
                 const uint32_t t_odd = h_odd * k.eight + (r_odd * k.neg16 + 0x0FF80FF8u);
                 u[hh] = bitselect(t_even, h_even, 0x80008000u);              // s ccc .... in the top nibble of each lane
@@ -328,7 +346,7 @@ __device__ __forceinline__ void quantize_block32_rw(const float (&y)[32], const 
             const uint32_t n0 = ~rw[2 * q], n1 = ~rw[2 * q + 1];     // bytes 255 - r of elements i..i+3 and i+4..i+7
             float z[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) z[j] = __fmul_rz(y[i + j], c);
+            for (int j = 0; j < 8; j += 2) mul2_rz(y[i + j], y[i + j + 1], c, z[j], z[j + 1]);
             // random word of a convert: bytes (b3, b2, b1, b0) = (255 - r of position 2, 255 - r of position 0, 0x80, 0x80)
             const uint32_t ca = cvt_e2m1x4_rs(z[0], z[0], z[2], z[2], __byte_perm(n0, 0x80808080u, 0x2044));   // elements i, i+2
             const uint32_t cb = cvt_e2m1x4_rs(z[1], z[1], z[3], z[3], __byte_perm(n0, 0x80808080u, 0x3144));   // elements i+1, i+3
@@ -347,8 +365,11 @@ __device__ __forceinline__ void quantize_block32_rw(const float (&y)[32], const 
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int i = 8 * q;
-            const uint32_t lo = cvt_e2m1x4_rs(__fmul_rz(y[i], c), __fmul_rz(y[i + 1], c), __fmul_rz(y[i + 2], c), __fmul_rz(y[i + 3], c), rw[2 * q]);
-            const uint32_t hi = cvt_e2m1x4_rs(__fmul_rz(y[i + 4], c), __fmul_rz(y[i + 5], c), __fmul_rz(y[i + 6], c), __fmul_rz(y[i + 7], c), rw[2 * q + 1]);
+            float z[8];
+#pragma unroll
+            for (int j = 0; j < 8; j += 2) mul2_rz(y[i + j], y[i + j + 1], c, z[j], z[j + 1]);
+            const uint32_t lo = cvt_e2m1x4_rs(z[0], z[1], z[2], z[3], rw[2 * q]);
+            const uint32_t hi = cvt_e2m1x4_rs(z[4], z[5], z[6], z[7], rw[2 * q + 1]);
             packed[q] = __byte_perm(lo, hi, 0x5410);
         }
     } else {
@@ -363,7 +384,9 @@ __device__ __forceinline__ void quantize_block32_rw(const float (&y)[32], const 
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int i = 8 * q + 2 * j;
-                word |= cvt_e2m1x2_rn(y[i] * inv_x, y[i + 1] * inv_x) << (8 * j);
+                float z0, z1;
+                mul2_rn(y[i], y[i + 1], inv_x, z0, z1);
+                word |= cvt_e2m1x2_rn(z0, z1) << (8 * j);
             }
             packed[q] = word;
         }

@@ -22,8 +22,18 @@
 //   warp 0        TMA producer (two 64-column x 128-row boxes per tile, 128-byte swizzle, 4-stage ring)
 //   warp 1        MMA issuer (8 K=16 MMAs per tile into one of four 128-column TMEM accumulators)
 //   warps 2, 3    idle: they complete warp group 0, which hands registers (setmaxnreg) to the epilogue groups
-//   warps 4..19   epilogue, four groups of four warps on alternate tiles: warp = TMEM lane quadrant, a thread owns one
+//   warps 4..15   epilogue, three groups of four warps on alternate tiles: warp = TMEM lane quadrant, a thread owns one
 //                 output row of the tile: tcgen05.ld 32 columns at a time, scale / SR / pack / store per MX block
+//                 (g = 256: four groups, warps 4..19)
+//
+// What bounds it: the rounding arithmetic of the epilogue warps (10 instructions per element), as long as the issuer
+// keeps up.  It did not: MMAs issued from a lane-0 branch cost 150 cycles each beside busy epilogue warps (descriptors
+// moved to uniform registers every time), 1200 of the 2100 cycles of a tile, and every epilogue warp waited a third of its
+// time for an accumulator.  Warp-uniform issue with one elected lane, 32-bit MX-block arithmetic per tile, two fp32 products
+// per instruction and three groups with a spare accumulator instead of four without one, 16384 x 16384 views, before ->
+// now: SR row-wise 140 -> 123 us, g = 64 133 -> 117, transposing 141 -> 139, g = 256 152 -> 132, SR16 131 -> 111 (6.1 TB/s),
+// RN 112 -> 108; the operands of a backward call, 16384 x 4096 x 16384 341 -> 300, 8192 x 1024 x 4096 56 -> 48, 8192 x 1024
+// x 1024 18.6 -> 16.0.
 // Every mbarrier wait is bounded; on expiry the CTA records a status word and unwinds.
 #include <cuda_bf16.h>
 
@@ -39,35 +49,36 @@ constexpr uint32_t kBoxBytes = 64 * 2 * 128;        // one TMA box: 64 bf16 colu
 constexpr uint32_t kTileBytes = 2 * kBoxBytes;      // 32 KB
 constexpr uint32_t kTBytes = 2 * kBoxBytes;         // transform matrix, 128 x 128 bf16
 
-// Two builds of the kernel.  FULL owns its SM: a 4-stage ring, four TMEM accumulators, four epilogue warp groups on
-// alternate tiles.  LITE is sized to run beside the small build of the pair GEMM (gemm_pair.cu) on the same SM, so that
+// Two builds of the kernel.  FULL owns its SM: a 4-stage ring, four TMEM accumulators, three epilogue warp groups on
+// alternate tiles (g = 256: two teams of two groups, each with its pair of accumulators).  LITE is sized to run beside the small build of the pair GEMM (gemm_pair.cu) on the same SM, so that
 // the operands of one product are quantised while the other product's GEMM keeps the FP4 pipe busy: one 32 KB stage,
 // one accumulator (128 TMEM columns), two epilogue warp groups that share every tile (two MX blocks of each row per
 // group), 64 registers per thread at launch.  g <= 128 only.  Codes and scales are the same bytes in both builds.
-template <bool LITE>
+template <bool LITE, int KW>
 struct QCfg {
     static constexpr int kStages = LITE ? 1 : 4;
     static constexpr int kAccBufs = LITE ? 1 : 4;                        // x 128 TMEM columns
     static constexpr int kTmemCols = LITE ? 128 : 512;
-    static constexpr int kEpiGroups = LITE ? 2 : 4;                      // epilogue warp groups (one warp per TMEM lane quadrant)
+    static constexpr int kEpiGroups = LITE ? 2 : KW == 2 ? 4 : 3;       // epilogue warp groups (one warp per TMEM lane quadrant)
     static constexpr int kEpiWarps = 4 * kEpiGroups;
     static constexpr uint32_t kSmem = kStages * kTileBytes + (LITE ? 1 : 2) * kTBytes + 1024 + 256;   // FULL: two transform matrices for g = 256
     // Register hand-over (setmaxnreg): warp group 0 shrinks to kRegsLight, the epilogue groups grow to kRegsEpi.  The
     // increase can only draw on what the CTA itself holds, i.e. threads x registers-per-thread at launch: the init
     // routine checks that budget against the compiled kernel, because an increase that cannot be met waits forever.
-    static constexpr int kRegsLight = LITE ? 32 : 40, kRegsEpi = LITE ? 80 : 104;
+    static constexpr int kRegsLight = LITE ? 32 : 40, kRegsEpi = LITE ? 80 : kEpiGroups == 3 ? 152 : 104;
     static constexpr int kThreads = (4 + kEpiWarps) * 32;                // warp group 0: producer, MMA issuer, two idle warps; then the epilogue warp groups
-    static constexpr int kLaunchRegs = LITE ? 64 : 96;
+    static constexpr int kLaunchRegs = LITE ? 64 : kEpiGroups == 3 ? 128 : 96;
     static_assert(kThreads * kLaunchRegs >= 128 * kRegsLight + (kThreads - 128) * kRegsEpi, "warp groups ask for more registers than the CTA holds");
 };
 
 struct QView {                 // one operand view: output operand [R, K] read from x [rows, cols]
-    int64_t R, K;
+    uint32_t R, k_blocks;      // output rows; MX blocks of 32 along K (R * k_blocks < 2^31)
     uint32_t r_tiles, k_tiles;
     uint32_t tile_begin;       // first index of this view in the launch's tile list
     uint32_t n_tiles;          // r_tiles * k_tiles
     uint32_t minor_count;      // tiles along the fast direction of the view's tile order (see locate_tile)
-    uint32_t d_major, d_minor; // an epilogue group's stride through the tile list, split by minor_count
+    uint32_t lg_band;          // log2 of the tiles across the fast direction that are walked side by side (TilePos)
+    uint32_t step, d_major, d_minor;   // an epilogue team's stride through the tile list, whole and split by minor_count
     int reduce_dim;            // 1: K runs along x columns (x tile is the K-major operand); 0: along x rows (MN-major)
     uint32_t stream_tag;
     PhiloxViewConsts pv;       // index-independent part of the first three Philox rounds for this view's draws (operands < 2^36 elements)
@@ -92,50 +103,63 @@ struct QMaps {
     CUtensorMap x[kQuantMaxViews];
 };
 
-// Position of a tile in the launch's list: its view and its (row tile, k tile) there.  Tiles of a view with a
-// contiguous reduce dimension run along k first, the transposing ones along the output rows first, so that CTAs
-// working side by side read neighbouring 256-byte row segments of x.
+// Position of a tile in the launch's list: its view and where it lies there.  Tiles of a view with a contiguous reduce
+// dimension run along k first, the transposing ones along the output rows first, so that CTAs working side by side read
+// neighbouring 256-byte row segments of x; across that direction four tiles (two, one where the count is not a multiple)
+// go side by side, so that a transposing view's 64-byte code segments of a row are written as whole lines at nearly the
+// same time (16384 x 16384 transposing: 142 -> 139 us).  major counts bands, minor walks a band.
+// DUAL launches: view 0 (reduce along x columns) and view 1 (reduce along x rows) are the two views of ONE tensor x
+// (dY of Algorithm 3, lines 3 and 5).  A unit is one 128 x 128 tile of x, loaded once, in the same order for both views;
+// it yields two logical tiles, 2 u (view 0) and 2 u + 1 (view 1).
 struct TilePos {
     int v;
-    uint32_t rt, kt;
-    uint32_t local;            // index inside the view
+    uint32_t major, minor;
+    uint32_t local;            // index inside the view (DUAL: the unit)
 };
+template <bool DUAL>
 __device__ __forceinline__ TilePos locate_tile(const QParams& p, uint32_t t) {
-    int v = 0;
-#pragma unroll
-    for (int i = 1; i < kQuantMaxViews; ++i)
-        if (i < p.n_views && t >= p.view[i].tile_begin) v = i;
-    const uint32_t local = t - p.view[v].tile_begin;
     TilePos pos;
-    pos.v = v;
-    pos.local = local;
-    if (p.view[v].reduce_dim == 1) { pos.rt = local / p.view[v].k_tiles; pos.kt = local - pos.rt * p.view[v].k_tiles; }
-    else { pos.kt = local / p.view[v].r_tiles; pos.rt = local - pos.kt * p.view[v].r_tiles; }
+    if (DUAL) {
+        pos.v = (int)(t & 1u);
+        pos.local = t >> 1;
+    } else {
+        pos.v = 0;
+#pragma unroll
+        for (int i = 1; i < kQuantMaxViews; ++i)
+            if (i < p.n_views && t >= p.view[i].tile_begin) pos.v = i;
+        pos.local = t - p.view[pos.v].tile_begin;
+    }
+    pos.major = pos.local / p.view[pos.v].minor_count;
+    pos.minor = pos.local - pos.major * p.view[pos.v].minor_count;
     return pos;
 }
-// The position `stride` tiles further on (stride = the view's d_major * minor_count + d_minor): additions only while
-// the walk stays inside the view.
+__device__ __forceinline__ uint32_t along_minor(const QView& vw, const TilePos& pos) { return pos.minor >> vw.lg_band; }
+__device__ __forceinline__ uint32_t across_minor(const QView& vw, const TilePos& pos) { return (pos.major << vw.lg_band) | (pos.minor & ((1u << vw.lg_band) - 1u)); }
+__device__ __forceinline__ uint32_t row_tile(const QView& vw, const TilePos& pos) { return vw.reduce_dim == 1 ? across_minor(vw, pos) : along_minor(vw, pos); }
+__device__ __forceinline__ uint32_t k_tile(const QView& vw, const TilePos& pos) { return vw.reduce_dim == 1 ? along_minor(vw, pos) : across_minor(vw, pos); }
+// The next tile of an epilogue team (t_next in the list; past its end: any valid position, not used): additions only
+// while the walk stays inside the view.
+template <bool DUAL>
 __device__ __forceinline__ TilePos advance_tile(const QParams& p, const TilePos& cur, uint32_t t_next) {
     const QView& vw = p.view[cur.v];
     TilePos pos = cur;
-    pos.local = cur.local + vw.d_major * vw.minor_count + vw.d_minor;
-    if (pos.local >= vw.n_tiles) return locate_tile(p, t_next);
-    uint32_t major = (vw.reduce_dim == 1 ? cur.rt : cur.kt) + vw.d_major, minor = (vw.reduce_dim == 1 ? cur.kt : cur.rt) + vw.d_minor;
-    if (minor >= vw.minor_count) { minor -= vw.minor_count; ++major; }
-    if (vw.reduce_dim == 1) { pos.rt = major; pos.kt = minor; } else { pos.kt = major; pos.rt = minor; }
-    return pos;
-}
-
-// DUAL launches: view 0 (reduce along x columns) and view 1 (reduce along x rows) are the two views of ONE tensor x
-// (dY of Algorithm 3, lines 3 and 5).  A unit is one 128 x 128 tile of x, loaded once; it yields two logical tiles,
-// 2 u (view 0: rows = x rows) and 2 u + 1 (view 1: rows = x columns).  Units run along x columns first.
-__device__ __forceinline__ TilePos locate_dual(const QParams& p, uint32_t t) {
-    const uint32_t u = t >> 1, xc_tiles = p.view[0].k_tiles;
-    const uint32_t xr = u / xc_tiles, xc = u - xr * xc_tiles;
-    TilePos pos;
-    pos.v = (int)(t & 1u);
-    pos.local = u;
-    if (pos.v == 0) { pos.rt = xr; pos.kt = xc; } else { pos.rt = xc; pos.kt = xr; }
+    if (DUAL) {                               // three tiles on: one or two units, the other view
+        const uint32_t units = cur.v == 0 ? 1u : 2u;
+        pos.local += units * vw.step;
+        if (pos.local >= vw.n_tiles) return locate_tile<DUAL>(p, t_next < p.n_tiles ? t_next : 0u);
+        pos.v = 1 - cur.v;
+        for (uint32_t i = 0; i < units; ++i) {
+            pos.major += vw.d_major;
+            pos.minor += vw.d_minor;
+            if (pos.minor >= vw.minor_count) { pos.minor -= vw.minor_count; ++pos.major; }
+        }
+        return pos;
+    }
+    pos.local += vw.step;
+    if (pos.local >= vw.n_tiles) return locate_tile<DUAL>(p, t_next < p.n_tiles ? t_next : 0u);
+    pos.major += vw.d_major;
+    pos.minor += vw.d_minor;
+    if (pos.minor >= vw.minor_count) { pos.minor -= vw.minor_count; ++pos.major; }
     return pos;
 }
 
@@ -144,18 +168,19 @@ constexpr bool mode_draws(int mode) { return mode == kModeSR || mode == kModeSR1
 // template argument of quantize_block32_rw; the g = 256 kernel (kw = 2) rounds SR through the convert instruction (same codes, fewer registers)
 constexpr int mode_rounding(int mode, int kw) { return mode == kModeSR16 ? 2 : (mode == kModeSR && kw == 2) ? 3 : mode; }
 
-// The 32 draws of a block.  FOLD: with the view's precomputed constants (fewer instructions, five more live values: pays
-// where registers are not the limit, i.e. in the SR16 kernel; the integer SR path and the g = 256 kernel lose with it).
+// The 32 draws of MX block `blk` (of the view: element index / 32).  FOLD: with the view's precomputed constants (fewer
+// instructions, five more live values: pays where registers are not the limit, i.e. in the SR16 kernel; the integer SR
+// path and the g = 256 kernel lose with it).
 template <bool FOLD>
-__device__ __forceinline__ void view_draws32(const PhiloxKeys& ks, uint32_t stream_tag, const PhiloxViewConsts* pv, uint64_t i0, uint32_t (&rw)[8]) {
-    if (FOLD) sr_draws32_view(ks, *pv, i0, rw);
-    else sr_draws32(ks, stream_tag, i0, rw);
+__device__ __forceinline__ void view_draws32(const PhiloxKeys& ks, const QView& vw, uint32_t blk, uint32_t (&rw)[8]) {
+    if (FOLD) sr_draws32_view(ks, vw.pv, blk, rw);
+    else sr_draws32_block(ks, vw.stream_tag, blk, rw);
 }
 
 // KW = 128-wide k-tiles per entry of the tile list: 1, or 2 for g = 256 (a tile then spans one 256-chunk).
 template <int MODE, int KW, bool LITE, bool DUAL>
 __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParams& p) {
-    using Cfg = QCfg<LITE>;
+    using Cfg = QCfg<LITE, KW>;
     static_assert(!DUAL || (KW == 1 && !LITE), "one load for two views: g <= 128, full-size build");
     constexpr int kStagesQ = Cfg::kStages, kAccBufs = Cfg::kAccBufs, kEpiGroups = Cfg::kEpiGroups, kThreadsQ = Cfg::kThreads;
     static_assert(!(LITE && KW == 2), "the small build serves g <= 128");
@@ -170,7 +195,7 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStagesQ + 2 * kAccBufs);
     volatile uint32_t* abort_flag = tmem_slot + 1;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp-uniform, and known to be)
     const uint32_t num_tiles = p.n_tiles;
     constexpr bool kFold = MODE == kModeSR16 && KW == 1;
 
@@ -236,15 +261,15 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
             bool ok = true;
             // DUAL: one load per unit (two logical tiles), in the coordinates of its row-wise view
             for (uint32_t t = DUAL ? 2u * blockIdx.x : blockIdx.x; t < num_tiles && ok; t += (DUAL ? 2u : 1u) * gridDim.x) {
-                const TilePos pos = DUAL ? locate_dual(p, t) : locate_tile(p, t);
+                const TilePos pos = locate_tile<DUAL>(p, t);
                 // x coordinates: (column, row).  reduce_dim 1: output rows = x rows, k = x columns; else swapped.
                 const bool rowwise = p.view[pos.v].reduce_dim == 1;
 #pragma unroll
                 for (int h = 0; h < KW; ++h, ++it) {
                     const int s = it % kStagesQ;
                     if (!(ok = mbar_wait(&empty_bar[s], ((it / kStagesQ) & 1) ^ 1, abort_flag))) break;
-                    const uint32_t kt = pos.kt * KW + h;                 // 128-wide k-tile
-                    const int32_t cx = (int32_t)((rowwise ? kt : pos.rt) * kTile), cy = (int32_t)((rowwise ? pos.rt : kt) * kTile);
+                    const uint32_t rt = row_tile(p.view[pos.v], pos), kt = k_tile(p.view[pos.v], pos) * KW + h;   // 128-wide k-tile
+                    const int32_t cx = (int32_t)((rowwise ? kt : rt) * kTile), cy = (int32_t)((rowwise ? rt : kt) * kTile);
                     uint8_t* st = smem + s * kTileBytes;
                     mbar_expect_tx(&full_bar[s], kTileBytes);
                     tma_load_2d(st, &maps.x[pos.v], &full_bar[s], cx, cy);
@@ -255,43 +280,47 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            // kind::f16 instruction descriptor: D = fp32 (bits 4-5 = 1), A = B = bf16 (bits 7-9, 10-12 = 1),
-            // A major at bit 15 (0 = K-major, 1 = MN-major), B K-major, N >> 3 at bit 17, M >> 4 at bit 24.
-            const uint32_t idesc_k = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTile >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
-            const uint32_t t_addr = smem_u32(smem_t);
-            uint32_t it = 0;
-            bool ok = true;
-            auto transform = [&](uint32_t a_addr, bool rowwise, int h, int b) {      // 8 MMAs: stage -> accumulator b
-                const uint32_t idesc = idesc_k | ((rowwise ? 0u : 1u) << 15);
+        // The whole warp walks the loop and one elected lane issues: with warp-uniform control flow the descriptors live in
+        // uniform registers.
+        // kind::f16 instruction descriptor: D = fp32 (bits 4-5 = 1), A = B = bf16 (bits 7-9, 10-12 = 1),
+        // A major at bit 15 (0 = K-major, 1 = MN-major), B K-major, N >> 3 at bit 17, M >> 4 at bit 24.
+        const uint32_t idesc_k = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTile >> 3) << 17) | ((uint32_t)(kTile >> 4) << 24);
+        const uint32_t t_addr = smem_u32(smem_t), s_addr = smem_u32(smem);
+        uint32_t it = 0;
+        bool ok = true;
+        auto wait = [&](uint64_t* bar, uint32_t parity) { return ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)); };
+        auto transform = [&](uint32_t a_addr, bool rowwise, int h, int b) {      // 8 MMAs (K = 16 each): stage -> accumulator b
+            const uint32_t idesc = idesc_k | ((rowwise ? 0u : 1u) << 15), d = tmem_base + b * kTile;
+            const uint64_t bdesc = make_smem_desc(t_addr + h * kTBytes, 16, 1024, 2);
+            // K-major: box ks/4, 32 bytes of K per step inside the 128-byte swizzle atom; MN-major: 16 k-rows of 128 B per
+            // step, the second 64 output rows sit one box further
+            const uint64_t adesc = rowwise ? make_smem_desc(a_addr, 16, 1024, 2) : make_smem_desc(a_addr, kBoxBytes, 1024, 2);
+            const uint32_t a_half = rowwise ? kBoxBytes >> 4 : 4 * 2048 >> 4, a_step = rowwise ? 32 >> 4 : 2048 >> 4;
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {                           // K = 16 per MMA
-                    uint64_t adesc;
-                    if (rowwise)            // K-major: box ks/4, 32 bytes of K per step inside the 128-byte swizzle atom
-                        adesc = make_smem_desc(a_addr + (ks >> 2) * kBoxBytes + (ks & 3) * 32, 16, 1024, 2);
-                    else                    // MN-major: 16 k-rows of 128 B per step; the second 64 output rows sit one box further
-                        adesc = make_smem_desc(a_addr + ks * 2048, kBoxBytes, 1024, 2);
-                    const uint64_t bdesc = make_smem_desc(t_addr + h * kTBytes + (ks >> 2) * kBoxBytes + (ks & 3) * 32, 16, 1024, 2);
-                    tc_mma_f16(tmem_base + b * kTile, adesc, bdesc, idesc, ks != 0 ? 1u : 0u);
-                }
-            };
-            if (DUAL) {
-                // per unit: the stage is the K-major operand of view 0's transform and the MN-major operand of view 1's
-                uint32_t is = 0;                                             // stage counter (units)
-                for (uint32_t u = blockIdx.x; 2u * u < num_tiles && ok; u += gridDim.x, ++is) {
-                    const int s = is % kStagesQ;
-                    if (!(ok = mbar_wait(&full_bar[s], (is / kStagesQ) & 1, abort_flag))) break;
-                    const uint32_t a_addr = smem_u32(smem + s * kTileBytes);
-                    for (int h = 0; h < 2 && ok; ++h, ++it) {
-                        const int b = it % kAccBufs;
-                        if (!(ok = mbar_wait(&acc_empty[b], ((it / kAccBufs) & 1) ^ 1, abort_flag))) break;
-                        tc_fence_after_sync();
+            for (int ks = 0; ks < 8; ++ks)
+                tc_mma_f16(d, adesc + (ks >> 2) * a_half + (ks & 3) * a_step, bdesc + (ks >> 2) * (kBoxBytes >> 4) + (ks & 3) * (32 >> 4), idesc, ks != 0 ? 1u : 0u);
+        };
+        if (DUAL) {
+            // per unit: the stage is the K-major operand of view 0's transform and the MN-major operand of view 1's
+            uint32_t is = 0;                                             // stage counter (units)
+            for (uint32_t u = blockIdx.x; 2u * u < num_tiles && ok; u += gridDim.x, ++is) {
+                const int s = is % kStagesQ;
+                if (!wait(&full_bar[s], (is / kStagesQ) & 1)) break;
+                const uint32_t a_addr = s_addr + s * kTileBytes;
+#pragma unroll
+                for (int h = 0; h < 2; ++h, ++it) {
+                    const int b = it % kAccBufs;
+                    if (!wait(&acc_empty[b], ((it / kAccBufs) & 1) ^ 1)) break;
+                    tc_fence_after_sync();
+                    if (elect_one()) {
                         transform(a_addr, h == 0, 0, b);
                         tc_commit(&acc_full[b]);
+                        if (h == 1) tc_commit(&empty_bar[s]);            // both transforms have read the stage
                     }
-                    if (ok) tc_commit(&empty_bar[s]);                        // both transforms have read the stage
+                    __syncwarp();
                 }
-            } else
+            }
+        } else {
             for (uint32_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
                 int v = 0;
 #pragma unroll
@@ -301,16 +330,19 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
 #pragma unroll
                 for (int h = 0; h < KW; ++h, ++it) {                       // KW = 2: k-tile h goes through T_h into its own accumulator
                     const int s = it % kStagesQ, b = it % kAccBufs;
-                    if (!(ok = mbar_wait(&acc_empty[b], ((it / kAccBufs) & 1) ^ 1, abort_flag))) break;
-                    if (!(ok = mbar_wait(&full_bar[s], (it / kStagesQ) & 1, abort_flag))) break;
+                    if (!wait(&acc_empty[b], ((it / kAccBufs) & 1) ^ 1)) break;
+                    if (!wait(&full_bar[s], (it / kStagesQ) & 1)) break;
                     tc_fence_after_sync();
-                    transform(smem_u32(smem + s * kTileBytes), rowwise, h, b);
-                    tc_commit(&empty_bar[s]);
-                    tc_commit(&acc_full[b]);
+                    if (elect_one()) {
+                        transform(s_addr + s * kTileBytes, rowwise, h, b);
+                        tc_commit(&empty_bar[s]);
+                        tc_commit(&acc_full[b]);
+                    }
+                    __syncwarp();
                 }
             }
-            if (!ok) *abort_flag = 1;
         }
+        if (!ok && lane == 0) *abort_flag = 1;
     } else if (DUAL && p.col_sums != nullptr) {
         // ------------------------------------------------------------------ warps 2, 3: column sums of the x tile (dL/db = 1 dL/dy)
         // The tile is in shared memory anyway: warp w sums columns 64 w .. 64 w + 63 (one TMA box), a lane two adjacent
@@ -335,8 +367,9 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty_bar[s]);                   // this warp is done with the stage
-            const uint32_t xc_tiles = p.view[0].k_tiles, xr = u / xc_tiles, xc = u - xr * xc_tiles;
-            float* dst = p.col_sums + (int64_t)xr * p.view[0].K + (int64_t)xc * kTile + w * 64 + 2 * lane;
+            const TilePos pos = locate_tile<DUAL>(p, 2u * u);
+            const uint32_t xr = row_tile(p.view[0], pos), xc = k_tile(p.view[0], pos);
+            float* dst = p.col_sums + (int64_t)xr * (32 * (int64_t)p.view[0].k_blocks) + (int64_t)xc * kTile + w * 64 + 2 * lane;
             *reinterpret_cast<float2*>(dst) = make_float2(s0, s1);
         }
         if (!ok && lane == 0) *abort_flag = 1;
@@ -354,14 +387,17 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
         const float cg = p.custom_t != nullptr ? 1.0f : p.g == 32 ? 0.17677669529663687f : p.g == 128 ? 0.08838834764831845f : 1.0f;
         // FULL: the groups take alternate tiles.  LITE: both groups take every tile of the CTA, group 0 the row's MX
         // blocks 0 and 1, group 1 blocks 2 and 3.
-        const uint32_t stride = (LITE ? 1u : (uint32_t)kEpiGroups) * gridDim.x;
+        // A team takes every kTeams-th tile of the CTA.  FULL: a group is a team, a thread handles all four blocks of its row.
+        // LITE: the two groups share every tile, group 0 the row's MX blocks 0 and 1, group 1 blocks 2 and 3.
+        constexpr int kTeams = KW == 2 ? 2 : LITE ? 1 : kEpiGroups;
         constexpr int kBlocksPerThread = LITE ? 2 : 4;
-        const int jb = LITE ? 2 * grp : 0;                          // first MX block of the row this thread handles
+        const uint32_t part = KW == 2 ? 4u * (grp & 1) : LITE ? 2u * grp : 0u;    // first MX block of the row this thread handles
         const uint32_t lane_row = (uint32_t)(q * 32 + lane);
         bool ok = true;
 
-        auto first_elem = [&](const TilePos& pos) -> uint64_t {          // linear index of this thread's first element
-            return (uint64_t)(pos.rt * (uint32_t)kTile + lane_row) * (uint64_t)p.view[pos.v].K + (uint64_t)(pos.kt * (uint32_t)(kTile * KW));
+        auto first_block = [&](const TilePos& pos) -> uint32_t {         // index of this thread's first MX block
+            const QView& vw = p.view[pos.v];
+            return (row_tile(vw, pos) * (uint32_t)kTile + lane_row) * vw.k_blocks + k_tile(vw, pos) * (4u * KW) + part;
         };
 
         // logical tile of this CTA's i-th accumulator: tiles are dealt out round-robin; in a DUAL launch whole units are
@@ -369,11 +405,12 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
         auto tile_of = [&](uint32_t i) -> uint32_t {
             return DUAL ? 2u * (blockIdx.x + (i >> 1) * gridDim.x) + (i & 1u) : blockIdx.x + i * gridDim.x;
         };
-        uint32_t it = LITE ? 0u : (uint32_t)grp;
+        uint32_t it = KW == 2 ? (uint32_t)(grp >> 1) : LITE ? 0u : (uint32_t)grp;
         uint32_t t = tile_of(it);
-        TilePos pos = DUAL ? locate_dual(p, t < num_tiles ? t : 0u) : locate_tile(p, t < num_tiles ? t : 0u);
+        TilePos pos = locate_tile<DUAL>(p, t < num_tiles ? t : 0u);
+        uint32_t blk = first_block(pos);
         uint32_t rw[8];
-        if (mode_draws(MODE)) view_draws32<kFold>(p.keys, p.view[pos.v].stream_tag, &p.view[pos.v].pv, first_elem(pos) + 32u * jb, rw);
+        if (mode_draws(MODE)) view_draws32<kFold>(p.keys, p.view[pos.v], blk, rw);
         if (KW == 2) {
             // g = 256: a tile is one 256-chunk of 128 rows; its two k-tiles went through T_0 and T_1 into the accumulator
             // pair (b0, b0 + 1): u = A_lo T_0, v = A_hi T_1.  The transformed values are y[0..127] = u + v and
@@ -381,30 +418,18 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
             // pr is drained by groups 2 pr (the u + v half) and 2 pr + 1 (the u - v half), so every barrier is used by
             // the same warps each time and its phases alternate for them.
             const int pr = grp >> 1, hh = grp & 1;
-            const uint32_t stride2 = 2u * gridDim.x;
-            it = (uint32_t)pr;
-            t = blockIdx.x + it * gridDim.x;
-            pos = locate_tile(p, t < num_tiles ? t : 0u);
-            if (mode_draws(MODE)) view_draws32<kFold>(p.keys, p.view[pos.v].stream_tag, &p.view[pos.v].pv, first_elem(pos) + 128u * hh, rw);
-            for (; t < num_tiles; t += stride2, it += 2) {
+            for (; t < num_tiles; it += kTeams, t = tile_of(it)) {
                 const int b0 = 2 * pr;
                 const QView& vw = p.view[pos.v];
-                const uint32_t rt = pos.rt, kt = pos.kt;
-                const int64_t K = vw.K;
-                const int64_t row = (int64_t)rt * kTile + lane_row;
-                const int64_t k0 = (int64_t)kt * (2 * kTile) + 128 * hh;        // this group's 128 elements of the row
-                const bool live = row < vw.R;
-                uint8_t* code_dst = vw.codes + row * (K >> 1) + (k0 >> 1);
-                const uint32_t nkb = (uint32_t)(K >> 5), nkc = (nkb + 3) >> 2;
-                uint8_t* scale_dst = vw.scales + (p.sf_native ? ((int64_t)(rt * nkc + 2 * kt + hh) * 512 + lane * 16 + q * 4) : row * nkb + (k0 >> 5));
-                float* y_dst = MODE == kModeDump ? vw.y_out + row * K + k0 : nullptr;
-                const uint64_t i_cur = first_elem(pos) + 128u * hh;
-                const uint32_t tag_cur = vw.stream_tag;
-                const PhiloxViewConsts* pv_cur = &vw.pv;
-                pos = t + stride2 < num_tiles ? advance_tile(p, pos, t + stride2) : locate_tile(p, 0u);
-                const uint64_t i_next = first_elem(pos) + 128u * hh;
-                const uint32_t tag_next = p.view[pos.v].stream_tag;
-            const PhiloxViewConsts* pv_next = &p.view[pos.v].pv;
+                const uint32_t rt = row_tile(vw, pos), kt = k_tile(vw, pos);
+                const bool live = rt * kTile + lane_row < vw.R;
+                const uint32_t blk_cur = blk;
+                uint8_t* code_dst = vw.codes + (uint64_t)blk_cur * 16u;
+                uint8_t* scale_dst = vw.scales + (p.sf_native ? (rt * ((vw.k_blocks + 3) >> 2) + 2 * kt + hh) * 512u + lane * 16 + q * 4 : blk_cur);
+                float* y_dst = MODE == kModeDump ? vw.y_out + (uint64_t)blk_cur * 32u : nullptr;
+                pos = advance_tile<DUAL>(p, pos, tile_of(it + kTeams));
+                blk = first_block(pos);
+                const QView& vw_next = p.view[pos.v];
                 const uint32_t ph = (it >> 1) & 1;                               // this pair's (it / 2)-th use
                 ok = mbar_wait(&acc_full[b0], ph, abort_flag) && mbar_wait(&acc_full[b0 + 1], ph, abort_flag);
                 ok = __all_sync(0xffffffffu, ok);
@@ -432,8 +457,8 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
                         if (lane == 0) { mbar_arrive(&acc_empty[b0]); mbar_arrive(&acc_empty[b0 + 1]); }
                     }
                     if (mode_draws(MODE)) {
-                        if (j < 3) view_draws32<kFold>(p.keys, tag_cur, pv_cur, i_cur + 32 * (j + 1), nx);
-                        else view_draws32<kFold>(p.keys, tag_next, pv_next, i_next, nx);
+                        if (j < 3) view_draws32<kFold>(p.keys, vw, blk_cur + (j + 1), nx);
+                        else view_draws32<kFold>(p.keys, vw_next, blk, nx);
                     }
                     if (MODE == kModeDump) {
                         if (live) {
@@ -454,58 +479,47 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
                 if (MODE != kModeDump && live) *reinterpret_cast<uint32_t*>(scale_dst) = sb_all;
             }
         } else
-        for (; t < num_tiles; it += (LITE ? 1 : kEpiGroups), t = DUAL ? tile_of(it) : t + stride) {
+        for (; t < num_tiles; it += kTeams, t = tile_of(it)) {
             const int b = it % kAccBufs;
             const QView& vw = p.view[pos.v];
-            const uint32_t rt = pos.rt, kt = pos.kt;
-            const int64_t K = vw.K;
-            const int64_t row = (int64_t)rt * kTile + lane_row;                 // output row
-            const int64_t k0 = (int64_t)kt * kTile;
-            const bool live = row < vw.R;
-            uint8_t* code_dst = vw.codes + row * (K >> 1) + (k0 >> 1);
-            const uint32_t nkb = (uint32_t)(K >> 5), nkc = (nkb + 3) >> 2;
-            uint8_t* scale_dst = vw.scales + (p.sf_native ? ((int64_t)(rt * nkc + kt) * 512 + lane * 16 + q * 4) : row * nkb + (k0 >> 5));
-            float* y_dst = MODE == kModeDump ? vw.y_out + row * K + k0 : nullptr;
-            const uint64_t i_cur = first_elem(pos);
-            const uint32_t tag_cur = vw.stream_tag;
-            const PhiloxViewConsts* pv_cur = &vw.pv;
-            // position of the next tile of this group (past the end: computed but not used)
-            if (DUAL) {
-                const uint32_t t_next = tile_of(it + kEpiGroups);
-                pos = locate_dual(p, t_next < num_tiles ? t_next : 0u);
-            } else {
-                pos = t + stride < num_tiles ? advance_tile(p, pos, t + stride) : locate_tile(p, 0u);
-            }
-            const uint64_t i_next = first_elem(pos);
-            const uint32_t tag_next = p.view[pos.v].stream_tag;
-            const PhiloxViewConsts* pv_next = &p.view[pos.v].pv;
+            const uint32_t rt = row_tile(vw, pos), kt = k_tile(vw, pos);
+            const bool live = rt * kTile + lane_row < vw.R;
+            const uint32_t blk_cur = blk;
+            uint8_t* code_dst = vw.codes + (uint64_t)blk_cur * 16u;
+            uint8_t* scale_dst = vw.scales + (p.sf_native ? (rt * ((vw.k_blocks + 3) >> 2) + kt) * 512u + lane * 16 + q * 4 + part : blk_cur);
+            float* y_dst = MODE == kModeDump ? vw.y_out + (uint64_t)blk_cur * 32u : nullptr;
+            // position of the next tile of this team (past the end: computed but not used)
+            pos = advance_tile<DUAL>(p, pos, tile_of(it + kTeams));
+            blk = first_block(pos);
+            const QView& vw_next = p.view[pos.v];
             ok = mbar_wait(&acc_full[b], (it / kAccBufs) & 1, abort_flag);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after_sync();
-            const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + b * kTile;
+            const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + b * kTile + 32 * part;
             uint32_t sb_all = 0;
 #pragma unroll
-            for (int jj = 0; jj < kBlocksPerThread; ++jj) {
-                const int j = jb + jj;                          // MX block of the row
+            for (int j = 0; j < kBlocksPerThread; ++j) {
                 uint32_t raw[32], nx[8], packed[4], sb = 0;
                 float y[32];
                 tmem_ld_32x32b_x32(taddr + 32 * j, raw);
-                tmem_ld_wait();
-                if (jj == kBlocksPerThread - 1) {               // the accumulator is free once it has been read
+                if (mode_draws(MODE)) {                         // while the load is under way
+                    if (j < kBlocksPerThread - 1) view_draws32<kFold>(p.keys, vw, blk_cur + (j + 1), nx);
+                    else view_draws32<kFold>(p.keys, vw_next, blk, nx);
+                    tmem_ld_wait_after(nx);
+                } else {
+                    tmem_ld_wait();
+                }
+                if (j == kBlocksPerThread - 1) {                // the accumulator is free once it has been read
                     tc_fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&acc_empty[b]);
-                }
-                if (mode_draws(MODE)) {
-                    if (jj < kBlocksPerThread - 1) view_draws32<kFold>(p.keys, tag_cur, pv_cur, i_cur + 32 * (j + 1), nx);
-                    else view_draws32<kFold>(p.keys, tag_next, pv_next, i_next + 32u * jb, nx);
                 }
 #pragma unroll
                 for (int i = 0; i < 32; ++i) y[i] = __uint_as_float(raw[i]);
                 if (cg != 1.0f) {                               // g = 32, 128: 1/sqrt(g) is not a power of two (for g = 64 it is folded into T)
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) y[i] *= cg;
+                    for (int i = 0; i < 32; i += 2) mul2_rn(y[i], y[i + 1], cg, y[i], y[i + 1]);
                 }
                 if (MODE == kModeDump) {
                     if (live) {
@@ -516,7 +530,7 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
                 } else {
                     quantize_block32_rw<mode_rounding(MODE, KW)>(y, rw, packed, sb, p.pipe);
                     if (live) *reinterpret_cast<uint4*>(code_dst + 16 * j) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-                    sb_all |= sb << (8 * jj);
+                    sb_all |= sb << (8 * j);
                 }
                 if (mode_draws(MODE)) {
 #pragma unroll
@@ -524,8 +538,9 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
                 }
             }
             if (MODE != kModeDump && live) {
-                if (LITE) *reinterpret_cast<uint16_t*>(scale_dst + jb) = (uint16_t)sb_all;   // this group's two of the row's four scale bytes
-                else *reinterpret_cast<uint32_t*>(scale_dst) = sb_all;                     // four consecutive bytes in either scale layout
+                // this thread's two or four consecutive bytes, in either scale layout
+                if (LITE) *reinterpret_cast<uint16_t*>(scale_dst) = (uint16_t)sb_all;
+                else *reinterpret_cast<uint32_t*>(scale_dst) = sb_all;
             }
         }
         if (!ok && lane == 0) *abort_flag = 1;
@@ -544,21 +559,22 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
 }
 
 template <int MODE, int KW>
-__global__ void __launch_bounds__(QCfg<false>::kThreads, 1)
+__global__ void __launch_bounds__(QCfg<false, KW>::kThreads, 1)
 quantize_tc_kernel(const __grid_constant__ QMaps maps, const __grid_constant__ QParams p) {
     quantize_tc_body<MODE, KW, false, false>(maps, p);
 }
 
 // Both views of one tensor from one read of it (Algorithm 3 lines 3 and 5 use the same dL/dy), g <= 128.
 template <int MODE>
-__global__ void __launch_bounds__(QCfg<false>::kThreads, 1)
+__global__ void __launch_bounds__(QCfg<false, 1>::kThreads, 1)
 quantize_tc_dual_kernel(const __grid_constant__ QMaps maps, const __grid_constant__ QParams p) {
     quantize_tc_body<MODE, 1, false, true>(maps, p);
 }
 
 // The small-footprint build (see QCfg), g <= 128.
+using LiteQCfg = QCfg<true, 1>;
 template <int MODE>
-__global__ void __maxnreg__(QCfg<true>::kLaunchRegs)
+__global__ void __maxnreg__(LiteQCfg::kLaunchRegs)
 quantize_tc_lite_kernel(const __grid_constant__ QMaps maps, const __grid_constant__ QParams p) {
     quantize_tc_body<MODE, 1, true, false>(maps, p);
 }
@@ -576,9 +592,9 @@ bool quant_tc_eligible(const QuantArgs& a) {
 
 cudaError_t fetch_quant_tc_status(unsigned int* word) { return device_status_fetch(word); }
 
-template <bool LITE>
+template <bool LITE, int KW>
 static cudaError_t quant_kernel_init(const void* k) {
-    using Cfg = QCfg<LITE>;
+    using Cfg = QCfg<LITE, KW>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmem);
     if (e != cudaSuccess) return e;
     // all of the SM's configurable memory as shared memory (see gemm_pair.cu: kernels share an SM only under one carve-out)
@@ -597,20 +613,20 @@ cudaError_t quant_tc_init() {
                               (const void*)quantize_tc_kernel<kModeDump, 1>, (const void*)quantize_tc_kernel<kModeSR16, 1>,
                               (const void*)quantize_tc_kernel<kModeSR, 2>, (const void*)quantize_tc_kernel<kModeRN, 2>,
                               (const void*)quantize_tc_kernel<kModeDump, 2>, (const void*)quantize_tc_kernel<kModeSR16, 2>};
-    for (const void* k : kernels) {
-        const cudaError_t e = quant_kernel_init<false>(k);
+    for (int i = 0; i < 8; ++i) {
+        const cudaError_t e = i < 4 ? quant_kernel_init<false, 1>(kernels[i]) : quant_kernel_init<false, 2>(kernels[i]);
         if (e != cudaSuccess) return e;
     }
     const void* dual[3] = {(const void*)quantize_tc_dual_kernel<kModeSR>, (const void*)quantize_tc_dual_kernel<kModeRN>,
                            (const void*)quantize_tc_dual_kernel<kModeSR16>};
     for (const void* k : dual) {
-        const cudaError_t e = quant_kernel_init<false>(k);
+        const cudaError_t e = quant_kernel_init<false, 1>(k);
         if (e != cudaSuccess) return e;
     }
     const void* lite[3] = {(const void*)quantize_tc_lite_kernel<kModeSR>, (const void*)quantize_tc_lite_kernel<kModeRN>,
                            (const void*)quantize_tc_lite_kernel<kModeSR16>};
     for (const void* k : lite) {
-        const cudaError_t e = quant_kernel_init<true>(k);
+        const cudaError_t e = quant_kernel_init<true, 1>(k);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -629,10 +645,10 @@ cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cud
     uint32_t tiles = 0;
     for (int v = 0; v < n; ++v) {
         QView& w = p.view[v];
-        w.R = a[v].reduce_dim == 1 ? a[v].rows : a[v].cols;
-        w.K = a[v].reduce_dim == 1 ? a[v].cols : a[v].rows;
-        w.r_tiles = (uint32_t)((w.R + kTile - 1) / kTile);
-        w.k_tiles = (uint32_t)(w.K / (a[v].g == 256 ? 2 * kTile : kTile));     // g = 256: a tile spans one 256-chunk
+        w.R = (uint32_t)(a[v].reduce_dim == 1 ? a[v].rows : a[v].cols);
+        w.k_blocks = (uint32_t)((a[v].reduce_dim == 1 ? a[v].cols : a[v].rows) / 32);
+        w.r_tiles = (w.R + kTile - 1) / kTile;
+        w.k_tiles = w.k_blocks / (a[v].g == 256 ? 8u : 4u);                    // g = 256: a tile spans one 256-chunk
         w.tile_begin = tiles;
         w.n_tiles = w.r_tiles * w.k_tiles;
         tiles += w.n_tiles;
@@ -667,11 +683,15 @@ cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cud
     const unsigned grid = units < (uint32_t)sms ? units : (unsigned)sms;
     for (int v = 0; v < kQuantMaxViews; ++v) {
         QView& w = p.view[v];
-        w.minor_count = w.reduce_dim == 1 ? w.k_tiles : w.r_tiles;
-        // tiles between two visits of an epilogue group: the groups take alternate tiles (g = 256: in pairs; small build: every tile)
-        const uint32_t step = (lite ? 1u : p.g == 256 ? 2u : (uint32_t)QCfg<false>::kEpiGroups) * grid;
-        w.d_major = step / w.minor_count;
-        w.d_minor = step % w.minor_count;
+        w.lg_band = 0;         // bands of four tiles along the reduce dimension where it runs across the walk
+        const uint32_t across = w.reduce_dim == 1 ? w.r_tiles : w.k_tiles;
+        if (dual || w.reduce_dim == 0) while (w.lg_band < 2 && (across >> w.lg_band) % 2 == 0) ++w.lg_band;
+        w.minor_count = (w.reduce_dim == 1 ? w.k_tiles : w.r_tiles) << w.lg_band;
+        // an epilogue team's stride (kTeams tiles of its CTA; DUAL: one unit, see advance_tile)
+        w.step = (lite || dual ? 1u : p.g == 256 ? 2u : (uint32_t)QCfg<false, 1>::kEpiGroups) * grid;
+        w.d_major = w.step / w.minor_count;
+        w.d_minor = w.step % w.minor_count;
+        if (dual) w.n_tiles = units;
     }
     const bool wide = p.g == 256;
     void (*kernel)(QMaps, QParams);
@@ -683,8 +703,8 @@ cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cud
     else kernel = wide ? quantize_tc_kernel<kModeRN, 2> : quantize_tc_kernel<kModeRN, 1>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid); cfg.stream = stream;
-    cfg.blockDim = dim3(lite ? QCfg<true>::kThreads : QCfg<false>::kThreads);
-    cfg.dynamicSmemBytes = lite ? QCfg<true>::kSmem : QCfg<false>::kSmem;
+    cfg.blockDim = dim3(lite ? LiteQCfg::kThreads : wide ? QCfg<false, 2>::kThreads : QCfg<false, 1>::kThreads);
+    cfg.dynamicSmemBytes = lite ? LiteQCfg::kSmem : QCfg<false, 1>::kSmem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;

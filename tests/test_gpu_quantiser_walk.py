@@ -1,0 +1,56 @@
+"""The tensor-core quantiser's tile walk (bands, teams, several views, both views of one tensor), against the CUDA-core
+quantiser or a walk of another shape: the transform is exact on small integers, so codes and scales are equal bytes."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _small_integers(shape, seed):
+    """Values whose transform is exact in any order of summation; scales differ from block to block."""
+    import torch
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    x = torch.randint(-8, 9, shape, generator=gen, device="cuda").float()
+    return x.bfloat16()
+
+
+# numbers of 128-tiles across the walk that give bands of one, two and four tiles, fewer tiles than CTAs and many more
+@pytest.mark.parametrize("rows,cols", [(128, 128), (128, 1032), (256, 4104), (384, 2056), (512, 8), (1152, 2048), (2048, 5128), (4608, 4096)])
+@pytest.mark.parametrize("g", [64, 256])
+@pytest.mark.parametrize("rounding", [0, 1, 2])
+def test_transposing_view_equals_row_view_of_the_transpose(rows, cols, g, rounding):
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    if rows % g:
+        pytest.skip("reduce length not a multiple of g")
+    x = _small_integers((rows, cols), rows + cols)
+    codes, scales = gpu.mxfp4_rht_sr_quantize(x, 0, g, 3, 2, rounding)
+    want, want_scales = gpu.mxfp4_rht_sr_quantize(x.t().contiguous(), 1, g, 3, 2, rounding)
+    assert torch.equal(codes, want)
+    linear = gpu.mxfp4_rht_sr_quantize(x, 0, g, 3, 2, rounding, gpu.SF_LINEAR)
+    assert torch.equal(linear[0], want)
+    per_tile = scales.view(-1, rows // 128, 32, 4, 4).permute(0, 3, 2, 1, 4).reshape(-1, rows // 32)[:cols]
+    assert torch.equal(linear[1].view(cols, rows // 32), per_tile)
+    assert torch.equal(linear[1], gpu.mxfp4_rht_sr_quantize(x.t().contiguous(), 1, g, 3, 2, rounding, gpu.SF_LINEAR)[1])
+    assert want_scales.numel() == scales.numel() and gpu.mxfp4_device_status() == 0
+
+
+# four views in one launch, and dY's two views from one read of it, against one launch per view
+@pytest.mark.parametrize("b,n,m", [(128, 8, 128), (256, 1000, 384), (1152, 264, 2176), (4096, 512, 8192)])
+@pytest.mark.parametrize("dual", ["0", "2"])
+@pytest.mark.parametrize("rounding", [0, 1, 2])
+def test_views_of_a_layer(b, n, m, dual, rounding, monkeypatch):
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    monkeypatch.setenv("MXFP4_DUAL_DY", dual)
+    dY, X, W = _small_integers((b, m), 1), _small_integers((b, n), 2), _small_integers((m, n), 3)
+    q = gpu.mxfp4_quantize_operands(dY, X, W, 64, 9, rounding)
+    for (codes, scales), (x, dim, tag) in zip(q, ((dY, 1, 1), (W, 0, 2), (dY, 0, 3), (X, 0, 4))):
+        want = gpu.mxfp4_rht_sr_quantize(x, dim, 64, 9, tag, rounding)
+        R = want[0].shape[0]
+        assert torch.equal(codes, want[0])
+        live = torch.arange(want[1].numel(), device="cuda").view(-1, want[0].shape[1] // 64, 32, 4, 4)       # rows beyond R are not written
+        row = (torch.arange(live.shape[0], device="cuda").view(-1, 1, 1, 1, 1) * 128 + torch.arange(4, device="cuda").view(1, 1, 1, 4, 1) * 32
+               + torch.arange(32, device="cuda").view(1, 1, 32, 1, 1)).expand_as(live) < R
+        assert torch.equal(scales.view(live.shape)[row], want[1].view(live.shape)[row])
+    assert gpu.mxfp4_device_status() == 0
