@@ -1,5 +1,5 @@
-// Block-scaled FP4 GEMM (and 8-bit ones), CTA-pair variant (tcgen05 cta_group::2): two CTAs of a 2-CTA cluster share one 256 x 256
-// output tile.  Each CTA loads 128 rows of A and only HALF of the B tile (128 of its 256 rows); the pair MMA reads
+// Block-scaled FP4 GEMM (and 8-bit ones), CTA-pair variant (tcgen05 cta_group::2): two CTAs of a 2-CTA cluster share one
+// 256 x 256 output tile.  Each CTA loads 128 rows of A and only HALF of the B tile (128 of its 256 rows); the pair MMA reads
 // both halves, so per MMA a tensor core pulls 4 KB + 4 KB from its own shared memory instead of 4 KB + 8 KB.  The
 // 1-CTA kernel (gemm.cu) is bound by exactly that operand traffic.  Each CTA keeps the accumulator of its own 128
 // rows (all 256 columns) in its TMEM.
@@ -11,28 +11,35 @@
 //   warp 0       TMA producer: own A rows, own half of B (completion counted on the LEADER's barrier);
 //   warp 3       scale loader: own A-row scale tiles and the scale tiles of all 256 B rows, tiled copies into ring slot
 //                s of stage s, counted on the same leader barrier as the operands, so the issuer waits once per step;
-//   warps 1, 2   MMA issuers, leader CTA only, taking the K-steps in turn under a baton.  Per step: six tcgen05.cp
-//                carry the step's scale tiles from the ring into TMEM slot s of BOTH CTAs (the copy itself replicates
-//                them to the four lane quadrants and reads shared memory once; they are issued while the other
-//                thread still issues its MMAs), then four K = 64 pair-MMAs; ONE multicast tcgen05.commit per step
-//                frees operand stage, ring slot and TMEM scale slot in both CTAs;
+//   warps 1, 2   MMA issuers, leader CTA only, taking the K-steps in turn under a baton, one elected lane each.  Per
+//                step: six tcgen05.cp carry the step's scale tiles from the ring into TMEM slot s of BOTH CTAs (the copy
+//                itself replicates them to the four lane quadrants and reads shared memory once; they are issued while
+//                the other warp still issues its MMAs), then four K = 64 pair-MMAs; ONE multicast tcgen05.commit per
+//                step frees operand stage, ring slot and TMEM scale slot in both CTAs;
 //   warps 4..11  epilogue of the CTA's own 128 x 256 half tile, a warp 32 rows x 128 columns: accumulator -> registers
 //                (all 128 columns in flight) -> hand the accumulator back -> scale, convert -> swizzled staging -> TMA
 //                stores (or reduce-adds when accumulating).
 // A-row scales are per CTA; every CTA needs the scales of all 256 B rows.
 //
-// The 8-bit products (FP8 forward pass, MXINT4; enum Kind) run on the same roles: a one-CTA kernel of 128 x 256 tiles with
-// one accumulator and stores from registers served them before.  E4M3 16384 x 4096 x 4096: 221 -> 174 us (3.2 PFLOP/s,
-// 0.97 of twice the measured bf16 rate), 8192 x 3072 x 1024 50 -> 24, 16 x 4096 x 4096 16.5 -> 13.7; MXINT4
-// 16384 x 4096 x 4096 245 -> 185, 1024 x 1024 x 8192 34 -> 26.
+// What bounds it: the tensor pipe in the steady state (539 cycles a K-step, four MMAs of 137 by their nominal rate)
+// and the board's power (1.36 - 1.57 GHz in a long launch); per tile about 1100 cycles in which the pipe stands still,
+// since TMEM has no room for a second 256-column accumulator beside the scale slots.  Two things got it there:
+//   - issue.  From a lane-0 branch an MMA took its thread 92 cycles, a scale copy 60, a commit 109 (descriptors go to
+//     uniform registers one by one), 660 cycles a step with two threads.  With warp-uniform control flow and an elected
+//     lane the issuers wait for operands instead.  Back to back, before -> now: 16384 x 4096 x 16384 382 -> 349 us (alone
+//     372 -> 333: 6.6 PFLOP/s), 16384 x 4096 x 4096 105 -> 97, 1024 x 1024 x 8192 16.2 -> 12.5.  One issuing warp without
+//     the baton: 376, 103, 16.5;
+//   - the hand-over.  Eight warps take the accumulator out unconverted, in place of four that had to convert the first
+//     half before reading the second, and for fp32 stored every 32 columns before reading the next: 16384 x 8192 x 2048
+//     bf16 125 -> 115 us, fp32 197 -> 143 (537 MB written: the store bounds it; a second staging buffer, stores without
+//     the evict-first hint, and 32-byte stores straight from the registers gained nothing).
+// A 256 x 384 pair tile (two N = 192 MMAs from one A) was slower everywhere: 391 -> 414 us at K = 16384, 106 -> 115 at 4096
+// (before the issue change).
 //
-// What the second epilogue group is for: TMEM has no room for a second 256-column accumulator beside the scale slots, so
-// the tensor pipe stands still from a tile's last MMA until the accumulator is in registers.  With eight warps that
-// hold it unconverted (in place of four that had to convert the first half before reading the second, and for fp32
-// stored every 32 columns before reading the next) a tile costs 0.42 us per K-step + 0.8 us.  Back to back, before ->
-// now: 16384 x 8192 x 2048 bf16 125 -> 115 us, fp32 197 -> 143; 16384 x 4096 x 4096 111 -> 105; 16384 x 4096 x 16384
-// 391 -> 388.  The fp32 store is then bound by writing (537 MB in 140 us); a second staging buffer, stores without the
-// evict-first hint, and 32-byte stores straight from the registers (175 us; 113 us at K = 4096) gained nothing.
+// The 8-bit products (FP8 forward pass, MXINT4; enum Kind) run on the same roles: a one-CTA kernel of 128 x 256 tiles with
+// one accumulator and stores from registers served them before.  E4M3 16384 x 4096 x 4096: 221 -> 168 us (3.3 PFLOP/s,
+// twice the measured bf16 rate), 8192 x 3072 x 1024 50 -> 23, 16 x 4096 x 4096 16.5 -> 11.4; MXINT4
+// 16384 x 4096 x 4096 245 -> 178, 1024 x 1024 x 8192 34 -> 20.
 #include <cuda_bf16.h>
 
 #include <cstdlib>
@@ -53,7 +60,7 @@ constexpr int kThreadsP = 12 * 32;
 
 // Three builds of the kernel.  PN = 256 (256 x 256 pair tile): six operand stages (all 227 KB of shared memory), one
 // 512-column TMEM allocation, every register of the SM.  PN = 128 (256 x 128): eight stages, and TMEM room for two
-// accumulators, so that a tile's MMAs run while the tile before is taken out; see tile_width() for when it is the better
+// accumulators, so that a tile's MMAs run while the tile before is taken out; see gemm_pair_tile_n() for when it is the better
 // one.  LITE (PN = 256) leaves room for a second, independent kernel on the same SM (the tensor-core quantiser's small
 // build, quantize_tc.cu, which quantises the OTHER product's operands meanwhile): four stages, TMEM taken as 256 + 128
 // columns, 104 registers per thread at launch.
@@ -186,7 +193,7 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tmem_empty + kAccBufs);   // [2] base columns of the TMEM allocation(s)
     volatile uint32_t* abort_flag = tmem_slot + 2;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp-uniform, and known to be)
     const uint32_t rank = cluster_ctarank();                // 0 = leader
     const TileWalk walk(p, (int)(blockIdx.x >> 1), (int)(gridDim.x >> 1));
 
@@ -255,11 +262,11 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
         }
     } else if (warp == 1 || warp == 2) {
         // ------------------------------------------------------------------ MMA issuers (leader CTA only)
-        // Issuing one pair MMA occupies its thread for ~90 cycles and a commit for ~100, which is more than the
-        // tensor pipe needs for the four MMAs of a step.  Two threads therefore take the steps in turn (even steps
-        // warp 1, odd steps warp 2): while one issues, the other has already waited for its operands and then
-        // commits.  A baton (mbarrier turn[]) keeps the MMAs in step order, so accumulation order is fixed.
-        if (rank == 0 && lane == 0) {
+        // Two warps take the steps in turn (even steps warp 1, odd steps warp 2): while one issues its MMAs, the other has
+        // already waited for its operands and copied its scales.  A baton (mbarrier turn[]) keeps the MMAs in step order,
+        // so accumulation order is fixed.  The whole warp walks the loop (every wait ends for all lanes or none) and one
+        // elected lane issues.
+        if (rank == 0) {
             // instruction descriptor: K-major, N >> 3 at bit 17, M >> 4 at bit 24; A, B = E2M1 (1) or E4M3 (0) at bits 7 and 10;
             // scaled kinds: scale = UE8M0 (bit 23), scale byte ids at bits 4 (B) and 29 (A); plain: D = fp32 (bit 4)
             const uint32_t idesc0 = ((uint32_t)(PN >> 3) << 17) | ((uint32_t)(PM >> 4) << 24) |
@@ -275,14 +282,15 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
             while (tile_i < walk.count && kt >= num_kt) { kt -= num_kt; num_kt = steps_of(++tile_i); }
             bool ok = true;
             for (; tile_i < walk.count; ++n) {
-                if (!(ok = mbar_wait(&full_bar[s], ph, abort_flag))) break;
+                if (!(ok = __all_sync(0xffffffffu, mbar_wait(&full_bar[s], ph, abort_flag)))) break;
                 tc_fence_after_sync();
                 const uint32_t a_lo = a_lo0 + s * (kStageB >> 4), b_lo = a_lo + (kAB >> 4);
                 const uint32_t sfa_t = tmem_sf + s * Cfg::kSfCols, sfb_t = sfa_t + 4 * Cfg::kSfTiles;
                 constexpr uint32_t kSfbChunk = PN / 32;      // TMEM columns of one 128-element chunk's B scales
-                {   // the step's scales: shared memory -> TMEM of both CTAs, replicated to the four lane quadrants by the copy;
-                    // issued while the other thread still issues its MMAs (a different TMEM slot), ordered before this
-                    // thread's MMAs by program order
+                if (Cfg::kSfTiles != 0 && elect_one()) {
+                    // the step's scales: shared memory -> TMEM of both CTAs, replicated to the four lane quadrants by the copy;
+                    // issued while the other warp still issues its MMAs (a different TMEM slot), ordered before this
+                    // lane's MMAs by program order
                     const uint32_t sf_s = smem_u32(sf_ring + s * kSfSlotB);
 #pragma unroll
                     for (int c = 0; c < Cfg::kSfTiles; ++c) {
@@ -293,44 +301,48 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
                                                       make_smem_desc(sf_s + Cfg::kSfaB + (Cfg::kSfTiles * j + c) * kSfTile, 0, 128, 0));
                     }
                 }
-                if (!(ok = mbar_wait_spin(&turn[me], (n & 1) ^ me ^ 1, abort_flag))) break;   // the step before mine is issued
+                if (!(ok = __all_sync(0xffffffffu, mbar_wait_spin(&turn[me], (n & 1) ^ me ^ 1, abort_flag)))) break;   // the step before mine is issued
                 // The copies above did not need the accumulator.  Waited for under the baton: with one K-step per tile the
                 // two threads alternate between tiles, and a thread that waited before its turn could see an earlier tile's
                 // hand-back as its own (a phase parity only tells neighbouring phases apart).
                 const uint32_t buf = tile_i % kAccBufs, acc = tmem_acc + buf * PN;
                 if (kt == 0) {
-                    if (!(ok = mbar_wait(&tmem_empty[buf], ((tile_i / kAccBufs) & 1) ^ 1, abort_flag))) break;
+                    if (!(ok = __all_sync(0xffffffffu, mbar_wait_spin(&tmem_empty[buf], ((tile_i / kAccBufs) & 1) ^ 1, abort_flag)))) break;
                     tc_fence_after_sync();
                 }
                 const uint32_t hi2 = 2u << 30;
                 const bool last = kt == num_kt - 1;
                 auto D = [&](uint32_t lo) { return ((uint64_t)desc_hi << 32) | lo; };
-                if constexpr (KIND == kMxf4) {
-                    tc_mma_mxf4_pair(acc, D(a_lo), D(b_lo), idesc0, sfa_t, sfb_t, kt != 0 ? 1u : 0u);
-                    tc_mma_mxf4_pair(acc, D(a_lo + 2), D(b_lo + 2), idesc1, sfa_t | hi2, sfb_t | hi2, 1u);
-                    // an odd number of 128-element chunks: the last step holds one only
-                    if (!(last && (p.prob[(int)tile_i < walk.n_first ? 0 : 1].nkc & 1) != 0)) {
-                        tc_mma_mxf4_pair(acc, D(a_lo + 4), D(b_lo + 4), idesc0, sfa_t + 4, sfb_t + kSfbChunk, 1u);
-                        tc_mma_mxf4_pair(acc, D(a_lo + 6), D(b_lo + 6), idesc1, (sfa_t + 4) | hi2, (sfb_t + kSfbChunk) | hi2, 1u);
+                // an odd number of 128-element chunks: the last step holds one only
+                const bool two_chunks = KIND != kMxf4 || !(last && (p.prob[(int)tile_i < walk.n_first ? 0 : 1].nkc & 1) != 0);
+                if (elect_one()) {
+                    if constexpr (KIND == kMxf4) {
+                        tc_mma_mxf4_pair(acc, D(a_lo), D(b_lo), idesc0, sfa_t, sfb_t, kt != 0 ? 1u : 0u);
+                        tc_mma_mxf4_pair(acc, D(a_lo + 2), D(b_lo + 2), idesc1, sfa_t | hi2, sfb_t | hi2, 1u);
+                        if (two_chunks) {
+                            tc_mma_mxf4_pair(acc, D(a_lo + 4), D(b_lo + 4), idesc0, sfa_t + 4, sfb_t + kSfbChunk, 1u);
+                            tc_mma_mxf4_pair(acc, D(a_lo + 6), D(b_lo + 6), idesc1, (sfa_t + 4) | hi2, (sfb_t + kSfbChunk) | hi2, 1u);
+                        }
+                    } else {
+    #pragma unroll
+                        for (uint32_t kb = 0; kb < 4; ++kb) {        // scale byte kb of the 32-bit column: K-block kb of the step
+                            if (KIND == kF8) tc_mma_f8_pair(acc, D(a_lo + 2 * kb), D(b_lo + 2 * kb), idesc0, (uint32_t)kt | kb ? 1u : 0u);
+                            else tc_mma_mxf8_pair(acc, D(a_lo + 2 * kb), D(b_lo + 2 * kb), idesc0 | (kb << 29) | (kb << 4), sfa_t | (kb << 30), sfb_t | (kb << 30),
+                                                  (uint32_t)kt | kb ? 1u : 0u);
+                        }
                     }
-                } else {
-#pragma unroll
-                    for (uint32_t kb = 0; kb < 4; ++kb) {        // scale byte kb of the 32-bit column: K-block kb of the step
-                        if (KIND == kF8) tc_mma_f8_pair(acc, D(a_lo + 2 * kb), D(b_lo + 2 * kb), idesc0, (uint32_t)kt | kb ? 1u : 0u);
-                        else tc_mma_mxf8_pair(acc, D(a_lo + 2 * kb), D(b_lo + 2 * kb), idesc0 | (kb << 29) | (kb << 4), sfa_t | (kb << 30), sfb_t | (kb << 30),
-                                              (uint32_t)kt | kb ? 1u : 0u);
-                    }
+                    tc_fence_before_sync();
+                    mbar_arrive(&turn[me ^ 1]);                                    // pass the baton
+                    tc_commit_pair(&empty_bar[s]);                                 // frees the operand stage and the scale slot
+                    if (last) tc_commit_pair(&tmem_full[buf]);
                 }
-                tc_fence_before_sync();
-                mbar_arrive(&turn[me ^ 1]);                                    // pass the baton
-                tc_commit_pair(&empty_bar[s]);                                 // frees the operand stage and the scale slot
-                if (last) tc_commit_pair(&tmem_full[buf]);
+                __syncwarp();
                 s += 2;
                 if (s >= (uint32_t)kStagesP) { s -= kStagesP; ph ^= 1; }
                 kt += 2;
                 while (tile_i < walk.count && kt >= num_kt) { kt -= num_kt; num_kt = steps_of(++tile_i); }
             }
-            if (!ok) *abort_flag = 1;
+            if (!ok && lane == 0) *abort_flag = 1;
         }
     } else {
         // ------------------------------------------------------------------ scale loader (both CTAs)
@@ -392,8 +404,7 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
             const ProblemP& pr = p.prob[w];
             const CUtensorMap* map = &maps.c[w];
             const uint32_t buf = kAccBufs == 2 ? half : 0;
-            if (lane == 0) ok = mbar_wait(&tmem_full[buf], (tl / kAccBufs) & 1, abort_flag);
-            ok = __shfl_sync(0xffffffffu, ok, 0);
+            ok = __all_sync(0xffffffffu, mbar_wait_spin(&tmem_full[buf], (tl / kAccBufs) & 1, abort_flag));
             if (!ok) break;
             tc_fence_after_sync();
             const int64_t row0 = (int64_t)mt * PM + (int64_t)rank * 128 + q * 32;
@@ -529,12 +540,11 @@ Spread spread_tiles(int n0, int n1, const double (&cost)[2], int pairs) {
     return best;
 }
 
-// Microseconds a pair spends on one tile.  Measured: both widths take their operands at the rate the L2 gives them (35 KB
-// per CTA and K-step of a 256-wide tile in 0.42 us, 26 KB of a 128-wide one in 0.31); a tile's hand-over is hidden by the
-// second accumulator in part only (the stores remain).
+// Microseconds a pair spends on one tile of a launch that does not reach the board's power limit: measured per K-step, and
+// per tile what the hand-over of the accumulator (256) or the stores (128, two accumulators) add.
 double tile_cost(int pn, int64_t K) {
     const double steps = (double)ceil_div(K, 256);
-    return pn == 256 ? 0.42 * steps + 0.8 : 0.31 * steps + 0.45;
+    return pn == 256 ? 0.34 * steps + 0.65 : 0.245 * steps + 0.3;
 }
 
 void fill_problem(ProblemP& p, const GemmArgs& a, int pn) {
@@ -578,8 +588,8 @@ cudaError_t launch_pairs(void (*kernel)(MapsP, ParamsP), int pairs, uint32_t sme
 }  // namespace
 
 // Columns of a pair tile for a launch of these products (n = 1 or 2): the width with which the last pair is done first.
-// 128 wins where 256-wide tiles leave pairs idle: backward 8192 x 1024 x 1024 (dW has 16 tiles of 32 steps) 36.1 -> 33.2 us,
-// 1024 x 1024 x 8192 alone 17.5 -> 16.2; it loses wherever the chip is full (16384 x 4096 x 4096: 106 -> 162).
+// 128 wins where 256-wide tiles leave pairs idle: backward 8192 x 1024 x 1024 (dW has 16 tiles of 32 steps) 31.7 -> 28.3 us,
+// 1024 x 1024 x 8192 alone 15.2 -> 12.3; it loses wherever the chip is full (16384 x 4096 x 4096: 98 -> 124).
 int gemm_pair_tile_n(const GemmArgs* a, int n) {
     int pairs = 0;
     if (a[0].lite || pair_count(&pairs) != cudaSuccess) return 256;
@@ -619,13 +629,13 @@ cudaError_t launch_gemm_pair(const GemmArgs* a, int n, int pn, cudaStream_t stre
     return launch_pairs(kernel, pairs, smem, maps, p, stream);
 }
 
-// Columns of a pair tile for an 8-bit product: the width with which the last pair is done first.  Measured per tile: 0.39 us
-// a K-step + 0.2 (256 wide), 0.28 + 0.1 (128 wide).  128 wins where 256-wide tiles leave pairs idle (16 x 4096 x 4096:
-// 15.5 -> 13.7 us), 256 elsewhere (16384 x 4096 x 4096: 174 us against 250).
+// Columns of a pair tile for an 8-bit product: the width with which the last pair is done first.  Measured per tile: 0.36 us
+// a K-step + 0.1 (256 wide), 0.245 + 0.1 (128 wide).  128 wins where 256-wide tiles leave pairs idle (16 x 4096 x 4096:
+// 15.0 -> 11.4 us, 1024 x 1024 x 8192 26 -> 20), 256 elsewhere (16384 x 4096 x 4096: 168 us against 221).
 int gemm_f8_tile_n(const Gemm8Args& a) {
     int pairs = 0;
     if (pair_count(&pairs) != cudaSuccess) return 256;
-    const double steps = (double)(a.K >> 7), cost[2] = {0.39 * steps + 0.2, 0.28 * steps + 0.1};
+    const double steps = (double)(a.K >> 7), cost[2] = {0.36 * steps + 0.1, 0.245 * steps + 0.1};
     double time[2];
     for (int i = 0; i < 2; ++i) time[i] = ceil_div((int64_t)ceil_div(a.M, PM) * ceil_div(a.N, i == 0 ? 256 : 128), pairs) * cost[i];
     return time[1] < time[0] ? 128 : 256;
