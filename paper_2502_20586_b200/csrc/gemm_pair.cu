@@ -528,9 +528,8 @@ struct Spread {
 Spread spread_tiles(int n0, int n1, const double (&cost)[2], int pairs) {
     Spread best{n0 % pairs, 0, 0.0};
     const int rest = best.rest, others = pairs - rest;
-    const int around = rest != 0 ? (int)(cost[0] / cost[1]) : 0;
-    for (int e = around > 0 ? around - 1 : 0; e <= (rest != 0 ? around + 1 : 0); ++e) {
-        if (e > 0 && e > n1 / others) break;
+    const int most = rest != 0 ? n1 / others : 0, around = (int)(cost[0] / cost[1]) < most ? (int)(cost[0] / cost[1]) : most;
+    for (int e = around > 0 ? around - 1 : 0; e <= around + 1 && e <= most; ++e) {
         const int late = n1 - e * others, rounds = late / pairs, left = late % pairs;
         const double t_others = (n0 / pairs) * cost[0] + (e + rounds + (left > 0 ? 1 : 0)) * cost[1];
         const double t_rest = rest == 0 ? 0.0 : (n0 / pairs + 1) * cost[0] + (rounds + (left > others ? 1 : 0)) * cost[1];
