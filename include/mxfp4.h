@@ -271,7 +271,8 @@ MXFP4_API mxfp4_status mxfp4_linear_forward_fp8(const void* x, const void* W, in
  * mxfp4_int4_quantize: arguments as mxfp4_rht_sr_quantize (same transform, same sign vector, same draws), except:
  *   codes [R, K] is ONE BYTE per element, the integer held as an E4M3 number (the tensor core has no 4-bit integer
  *   type; E4M3 holds -7..7 exactly), scales always in the NATIVE layout, and y_scratch (fp32 [R, K], 16-byte
- *   aligned, caller-owned) receives the transformed values on the way.
+ *   aligned, caller-owned) receives the transformed values on the way.  Scale bytes that only fill the last tiles
+ *   are set to zero.
  * mxfp4_int4_gemm: C [M, N] = alpha sum_k q_A X_A q_B X_B on the tensor cores (tcgen05 kind::mxf8f6f4, one scale per
  *   32 elements); K % 128 == 0, N % 8 == 0; alpha = 16/9 undoes two 3/4 pre-scales as in Algorithm 3.
  */

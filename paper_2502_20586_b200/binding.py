@@ -365,7 +365,7 @@ def mxfp4_int4_quantize(x: torch.Tensor, reduce_dim: int, g: int, seed: int, str
     rows, cols = x.shape
     R, K = (rows, cols) if reduce_dim == 1 else (cols, rows)
     codes = torch.empty((R, K), dtype=torch.uint8, device=x.device)
-    scales = torch.zeros(mxfp4_scale_bytes(R, K, SF_NATIVE), dtype=torch.uint8, device=x.device)
+    scales = torch.empty(mxfp4_scale_bytes(R, K, SF_NATIVE), dtype=torch.uint8, device=x.device)
     y = torch.empty((R, K), dtype=torch.float32, device=x.device)
     _check(_lib.mxfp4_int4_quantize(_ptr(x), rows, cols, x.stride(0), reduce_dim, g, rounding, seed, stream_tag, _ptr(codes), _ptr(scales),
                                     _ptr(y), _stream()))

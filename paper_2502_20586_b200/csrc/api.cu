@@ -704,9 +704,14 @@ mxfp4_status mxfp4_int4_quantize(const void* x, int64_t rows, int64_t cols, int6
     if (!aligned16(codes) || !aligned16(y_scratch)) return MXFP4_ERR_ALIGN;
     if ((st = runtime_init()) != MXFP4_OK) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    // the transform is the MXFP4 path's own (its fp32 output, rounded once); only the element format differs
-    QuantArgs a{x, rows, cols, ld, reduce_dim, g, 0, seed, 0u, nullptr, nullptr, 0, y_scratch};
+    // The transform is the MXFP4 path's own (its fp32 output, rounded once); only the element format differs.  Where it runs
+    // on the tensor cores (g <= 128; a thread then holds a row's four scale bytes, stored as one word) one launch does all.
+    QuantArgs a{x, rows, cols, ld, reduce_dim, g, rounding, seed, stream_tag, codes, scales, 1, y_scratch};
     attach_input_map(a);
+    if (mx::quant_tc_eligible(a) && g != 256 && (reinterpret_cast<uintptr_t>(scales) & 3u) == 0) {
+        a.mxint4 = true;
+        return cuda_status(mx::launch_quantize_tc_group(&a, 1, false, stream), "MXINT4 quantiser launch");
+    }
     if ((st = cuda_status(mx::launch_rht_dump(a, stream), "transform launch")) != MXFP4_OK) return st;
     const int64_t R = reduce_dim == 1 ? rows : cols, K = reduce_dim == 1 ? cols : rows;
     return cuda_status(mx::launch_mxint4_quantize(y_scratch, R, K, rounding, seed, stream_tag, codes, scales, stream), "MXINT4 quantiser launch");

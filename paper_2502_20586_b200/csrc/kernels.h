@@ -21,6 +21,7 @@ struct QuantArgs {
     CUtensorMap tmap_x;   // x as [rows, cols] bf16, box 64 cols x 128 rows, 128-byte swizzle (tensor-core path)
     bool has_tmap;
     const void* custom_t = nullptr;   // bf16 [g, g] row-major: transform matrix given by the caller instead of diag(S) H_g / sqrt(g) (tensor-core path, g <= 128)
+    bool mxint4 = false;    // MXINT4 codes (one byte per element) and y_out in one pass (tensor-core path, g <= 128, rounding 0 or 1, native scales)
 };
 
 // Tensor-core transform path (quantize_tc.cu): g in {32, 64, 128} and reduce length a multiple of 128.

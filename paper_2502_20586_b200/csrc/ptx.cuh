@@ -165,6 +165,17 @@ __device__ __forceinline__ void bulk_wait_group() { asm volatile("cp.async.bulk.
 // Make generic-proxy shared-memory writes visible to the async proxy (TMA store, tcgen05 reads).
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// 32 bytes of a thread: a whole L2 sector in one store where the address is a multiple of 32 (`wide`), else two of 16.
+__device__ __forceinline__ void st_global_32B(void* dst, const uint32_t* w, bool wide) {
+    if (wide) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                     ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+    } else {
+        reinterpret_cast<uint4*>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+        reinterpret_cast<uint4*>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+    }
+}
+
 // ---------------------------------------------------------------- tcgen05 / TMEM
 // Allocate `cols` (power of two >= 32) TMEM columns; the base address is written to *smem_slot.  Warp-collective.
 __device__ __forceinline__ void tmem_alloc(uint32_t* smem_slot, uint32_t cols) {

@@ -92,6 +92,7 @@ struct QParams {
     int n_views;
     uint32_t n_tiles;          // over all views
     int g, sf_native;
+    bool wide_stores;          // y_out (and MXINT4 codes) start on 32-byte boundaries
     const uint16_t* custom_t;  // bf16 [g, g] row-major transform matrix given by the caller, or null (then diag(S) H_g / sqrt(g))
     uint64_t seed;
     float* col_sums;           // DUAL launches: partial column sums [x rows / 128][x cols] of x in fp32 (bias gradient), or null
@@ -163,8 +164,13 @@ __device__ __forceinline__ TilePos advance_tile(const QParams& p, const TilePos&
     return pos;
 }
 
-enum { kModeSR = 0, kModeRN = 1, kModeDump = 2, kModeSR16 = 3 };
-constexpr bool mode_draws(int mode) { return mode == kModeSR || mode == kModeSR16; }
+// kModeInt4*: MXINT4 elements, one byte each, together with the transformed values that were rounded (g <= 128): what a pass
+// of its own over the fp32 values did before.  Bound by writing them; 32-byte stores, since a thread owns a row: 1024 x 8192
+// 37 -> 15.7 us, 16384 x 4096 252 -> 89 (the dump alone 175 -> 72: 402 MB at 5.6 TB/s).
+enum { kModeSR = 0, kModeRN = 1, kModeDump = 2, kModeSR16 = 3, kModeInt4SR = 4, kModeInt4RN = 5 };
+constexpr bool mode_draws(int mode) { return mode == kModeSR || mode == kModeSR16 || mode == kModeInt4SR; }
+constexpr bool mode_int4(int mode) { return mode == kModeInt4SR || mode == kModeInt4RN; }
+constexpr bool mode_keeps_y(int mode) { return mode == kModeDump || mode_int4(mode); }
 // template argument of quantize_block32_rw; the g = 256 kernel (kw = 2) rounds SR through the convert instruction (same codes, fewer registers)
 constexpr int mode_rounding(int mode, int kw) { return mode == kModeSR16 ? 2 : (mode == kModeSR && kw == 2) ? 3 : mode; }
 
@@ -485,9 +491,9 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
             const uint32_t rt = row_tile(vw, pos), kt = k_tile(vw, pos);
             const bool live = rt * kTile + lane_row < vw.R;
             const uint32_t blk_cur = blk;
-            uint8_t* code_dst = vw.codes + (uint64_t)blk_cur * 16u;
+            uint8_t* code_dst = vw.codes + (uint64_t)blk_cur * (mode_int4(MODE) ? 32u : 16u);
             uint8_t* scale_dst = vw.scales + (p.sf_native ? (rt * ((vw.k_blocks + 3) >> 2) + kt) * 512u + lane * 16 + q * 4 + part : blk_cur);
-            float* y_dst = MODE == kModeDump ? vw.y_out + (uint64_t)blk_cur * 32u : nullptr;
+            float* y_dst = mode_keeps_y(MODE) ? vw.y_out + (uint64_t)blk_cur * 32u : nullptr;
             // position of the next tile of this team (past the end: computed but not used)
             pos = advance_tile<DUAL>(p, pos, tile_of(it + kTeams));
             blk = first_block(pos);
@@ -521,13 +527,16 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
 #pragma unroll
                     for (int i = 0; i < 32; i += 2) mul2_rn(y[i], y[i + 1], cg, y[i], y[i + 1]);
                 }
-                if (MODE == kModeDump) {
-                    if (live) {
-                        float4* dst = reinterpret_cast<float4*>(y_dst + 32 * j);
+                if (mode_keeps_y(MODE) && live) {
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) dst[i] = make_float4(y[4 * i], y[4 * i + 1], y[4 * i + 2], y[4 * i + 3]);
-                    }
-                } else {
+                    for (int i = 0; i < 4; ++i) st_global_32B(y_dst + 32 * j + 8 * i, reinterpret_cast<const uint32_t*>(y) + 8 * i, p.wide_stores);
+                }
+                if constexpr (mode_int4(MODE)) {
+                    uint32_t bytes[8];
+                    quantize_block32_int4<MODE == kModeInt4SR>(y, rw, bytes, sb);
+                    if (live) st_global_32B(code_dst + 32 * j, bytes, p.wide_stores);
+                    sb_all |= sb << (8 * j);
+                } else if constexpr (MODE != kModeDump) {
                     quantize_block32_rw<mode_rounding(MODE, KW)>(y, rw, packed, sb, p.pipe);
                     if (live) *reinterpret_cast<uint4*>(code_dst + 16 * j) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
                     sb_all |= sb << (8 * j);
@@ -537,7 +546,8 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
                     for (int i = 0; i < 8; ++i) rw[i] = nx[i];
                 }
             }
-            if (MODE != kModeDump && live) {
+            if (MODE != kModeDump && (live || mode_int4(MODE))) {   // (MXINT4: rows that only fill the last tile are zero)
+                if (mode_int4(MODE) && !live) sb_all = 0;
                 // this thread's two or four consecutive bytes, in either scale layout
                 if (LITE) *reinterpret_cast<uint16_t*>(scale_dst) = (uint16_t)sb_all;
                 else *reinterpret_cast<uint32_t*>(scale_dst) = sb_all;
@@ -609,12 +619,13 @@ static cudaError_t quant_kernel_init(const void* k) {
 }
 
 cudaError_t quant_tc_init() {
-    const void* kernels[8] = {(const void*)quantize_tc_kernel<kModeSR, 1>, (const void*)quantize_tc_kernel<kModeRN, 1>,
-                              (const void*)quantize_tc_kernel<kModeDump, 1>, (const void*)quantize_tc_kernel<kModeSR16, 1>,
-                              (const void*)quantize_tc_kernel<kModeSR, 2>, (const void*)quantize_tc_kernel<kModeRN, 2>,
-                              (const void*)quantize_tc_kernel<kModeDump, 2>, (const void*)quantize_tc_kernel<kModeSR16, 2>};
-    for (int i = 0; i < 8; ++i) {
-        const cudaError_t e = i < 4 ? quant_kernel_init<false, 1>(kernels[i]) : quant_kernel_init<false, 2>(kernels[i]);
+    const void* kernels[10] = {(const void*)quantize_tc_kernel<kModeSR, 1>, (const void*)quantize_tc_kernel<kModeRN, 1>,
+                               (const void*)quantize_tc_kernel<kModeDump, 1>, (const void*)quantize_tc_kernel<kModeSR16, 1>,
+                               (const void*)quantize_tc_kernel<kModeInt4SR, 1>, (const void*)quantize_tc_kernel<kModeInt4RN, 1>,
+                               (const void*)quantize_tc_kernel<kModeSR, 2>, (const void*)quantize_tc_kernel<kModeRN, 2>,
+                               (const void*)quantize_tc_kernel<kModeDump, 2>, (const void*)quantize_tc_kernel<kModeSR16, 2>};
+    for (int i = 0; i < 10; ++i) {
+        const cudaError_t e = i < 6 ? quant_kernel_init<false, 1>(kernels[i]) : quant_kernel_init<false, 2>(kernels[i]);
         if (e != cudaSuccess) return e;
     }
     const void* dual[3] = {(const void*)quantize_tc_dual_kernel<kModeSR>, (const void*)quantize_tc_dual_kernel<kModeRN>,
@@ -639,6 +650,7 @@ cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cud
     if (dual && (n != 2 || lite || dump_y || a[0].g == 256 || a[0].custom_t != nullptr || a[0].x != a[1].x || a[0].rows != a[1].rows ||
                  a[0].cols != a[1].cols || a[0].ld != a[1].ld || a[0].reduce_dim != 1 || a[1].reduce_dim != 0 || a[0].rows % kTile != 0))
         return cudaErrorInvalidValue;
+    if (a[0].mxint4 && (n != 1 || dual || lite || dump_y || a[0].g == 256 || a[0].custom_t != nullptr || a[0].y_out == nullptr)) return cudaErrorInvalidValue;
     if (lite && (dump_y || a[0].g == 256 || a[0].custom_t != nullptr)) return cudaErrorInvalidValue;   // the small build: RHT with g <= 128, quantising
     QParams p;
     QMaps maps;
@@ -661,6 +673,7 @@ cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cud
     p.n_views = n;
     p.n_tiles = tiles;
     p.g = a[0].g; p.sf_native = a[0].sf_native; p.seed = a[0].seed;
+    p.wide_stores = ((reinterpret_cast<uintptr_t>(a[0].y_out) | (a[0].mxint4 ? reinterpret_cast<uintptr_t>(a[0].codes) : 0)) & 31u) == 0;
     p.custom_t = static_cast<const uint16_t*>(a[0].custom_t);
     if (p.custom_t != nullptr && p.g == 256) return cudaErrorInvalidValue;
     if (col_sums != nullptr && !dual) return cudaErrorInvalidValue;
@@ -693,10 +706,11 @@ cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cud
         w.d_minor = w.step % w.minor_count;
         if (dual) w.n_tiles = units;
     }
-    const bool wide = p.g == 256;
+    const bool wide = p.g == 256, mxint4 = a[0].mxint4;
     void (*kernel)(QMaps, QParams);
     if (dual) kernel = a[0].rounding == 0 ? quantize_tc_dual_kernel<kModeSR> : a[0].rounding == 2 ? quantize_tc_dual_kernel<kModeSR16> : quantize_tc_dual_kernel<kModeRN>;
     else if (lite) kernel = a[0].rounding == 0 ? quantize_tc_lite_kernel<kModeSR> : a[0].rounding == 2 ? quantize_tc_lite_kernel<kModeSR16> : quantize_tc_lite_kernel<kModeRN>;
+    else if (mxint4) kernel = a[0].rounding == 0 ? quantize_tc_kernel<kModeInt4SR, 1> : quantize_tc_kernel<kModeInt4RN, 1>;
     else if (dump_y) kernel = wide ? quantize_tc_kernel<kModeDump, 2> : quantize_tc_kernel<kModeDump, 1>;
     else if (a[0].rounding == 0) kernel = wide ? quantize_tc_kernel<kModeSR, 2> : quantize_tc_kernel<kModeSR, 1>;
     else if (a[0].rounding == 2) kernel = wide ? quantize_tc_kernel<kModeSR16, 2> : quantize_tc_kernel<kModeSR16, 1>;

@@ -142,18 +142,8 @@ __global__ void __launch_bounds__(kFp8Threads, 2) fp8_quantize_kernel(const __gr
 }
 
 // ---------------------------------------------------------------- MXINT4: integers -7..7 with one E8M0 scale per 32
-// E4M3 byte that holds the integer q in [0, 7] exactly (the tensor core reads the elements as E4M3).
-__device__ __forceinline__ uint32_t e4m3_of_small_int(uint32_t q) {
-    // 0, 1 = 1.0 2^0, 2, 3 = 1.5 2^1, 4, 5 = 1.25 2^2, 6 = 1.5 2^2, 7 = 1.75 2^2   (bias 7, three mantissa bits)
-    return (0x4E4C4A4844403800ull >> (8 * q)) & 0xFFu;
-}
-
-// One thread per MX block of 32 fp32 values.  Scale: the rule of Algorithms 1 / 2 with emax_elem = 2 (largest power of
-// two among the elements is 4).  SR (Algorithm 2): w = (3/4) |v| / X < 6, rounded on the integer grid with the dither
-// of Eq. 1-2 discretised to the element's 8-bit draw r: up iff 256 frac >= r + 1/2.  Exactly: u = floor(512 w) =
-// floor(3 * (128 |v| / X)), where 128 |v| / X is an exact power-of-two scaling and the product by 3 is rounded toward
-// zero (floor of a toward-zero rounding of a non-negative real equals the floor of the real); then q = u >> 9 and
-// up iff (u & 511) >= 2 r + 1.  RN (Algorithm 1): nearest integer, ties to even, saturating at 7.
+// The separate pass over transformed values (no transform, g = 256, reduce lengths the tensor-core transform does not take;
+// otherwise quantize_tc.cu rounds them where it has them): one thread per MX block.
 __global__ void mxint4_quantize_kernel(const float* __restrict__ y, int64_t R, int64_t K, int rounding, uint64_t seed, uint32_t stream_tag,
                                        uint8_t* __restrict__ codes, uint8_t* __restrict__ scales) {
     const int64_t nkb = K >> 5, blk = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -166,36 +156,14 @@ __global__ void mxint4_quantize_kernel(const float* __restrict__ y, int64_t R, i
         const float4 f = src[i];
         v[4 * i] = f.x; v[4 * i + 1] = f.y; v[4 * i + 2] = f.z; v[4 * i + 3] = f.w;
     }
-    float amax = 0.0f;
-#pragma unroll
-    for (int i = 0; i < 32; ++i) amax = fmaxf(amax, fabsf(v[i]));
-    const uint32_t byte = e8m0_from_amax(amax);
-    scales[sf_native_offset(r, kb, (nkb + 3) >> 2)] = (uint8_t)byte;
-    uint32_t out[8];
-    if (byte == 255u) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) out[i] = 0u;
+    uint32_t out[8], byte, rw[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+    if (rounding == 0) {
+        sr_draws32(seed, stream_tag, (uint64_t)(r * K + kb * 32), rw);
+        quantize_block32_int4<true>(v, rw, out, byte);
     } else {
-        const int e = (int)byte - 127;
-        uint32_t rw[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-        if (rounding == 0) sr_draws32(seed, stream_tag, (uint64_t)(r * K + kb * 32), rw);
-        const int sh = (rounding == 0 ? 7 : 0) - e;                      // |v| 2^sh, in two exact steps
-        const float p1 = pow2f_wide(sh / 2), p2 = pow2f_wide(sh - sh / 2);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            const float a = fabsf(v[i]) * p1 * p2;
-            uint32_t q;
-            if (rounding == 0) {
-                const uint32_t u = (uint32_t)__fmul_rz(a, 3.0f);         // floor(512 w), w < 6
-                const uint32_t rr = (rw[i >> 2] >> (8 * (i & 3))) & 0xFFu;
-                q = (u >> 9) + ((u & 511u) >= 2u * rr + 1u ? 1u : 0u);
-            } else {
-                q = (uint32_t)fminf(rintf(a), 7.0f);
-            }
-            const uint32_t code = e4m3_of_small_int(q) | ((__float_as_uint(v[i]) >> 24) & 0x80u);
-            if ((i & 3) == 0) out[i >> 2] = code; else out[i >> 2] |= code << (8 * (i & 3));
-        }
+        quantize_block32_int4<false>(v, rw, out, byte);
     }
+    scales[sf_native_offset(r, kb, (nkb + 3) >> 2)] = (uint8_t)byte;
     uint4* dst = reinterpret_cast<uint4*>(codes + r * K + kb * 32);
     dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
     dst[1] = make_uint4(out[4], out[5], out[6], out[7]);
@@ -247,6 +215,11 @@ cudaError_t launch_fp8_quantize(const Fp8QuantArgs* a, int n, uint16_t* partial,
 
 cudaError_t launch_mxint4_quantize(const float* y, int64_t R, int64_t K, int rounding, uint64_t seed, uint32_t stream_tag,
                                    uint8_t* codes, uint8_t* scales, cudaStream_t stream) {
+    // rows and K-blocks that only fill the last scale tiles are zero
+    if (R % 128 != 0 || K % 128 != 0) {
+        const cudaError_t e = cudaMemsetAsync(scales, 0, (size_t)((R + 127) / 128 * ((K + 127) / 128) * 512), stream);
+        if (e != cudaSuccess) return e;
+    }
     const int64_t blocks = R * (K >> 5);
     mxint4_quantize_kernel<<<(unsigned)((blocks + 127) / 128), 128, 0, stream>>>(y, R, K, rounding, seed, stream_tag, codes, scales);
     return cudaGetLastError();

@@ -54,3 +54,35 @@ def test_views_of_a_layer(b, n, m, dual, rounding, monkeypatch):
                + torch.arange(32, device="cuda").view(1, 1, 32, 1, 1)).expand_as(live) < R
         assert torch.equal(scales.view(live.shape)[row], want[1].view(live.shape)[row])
     assert gpu.mxfp4_device_status() == 0
+
+
+# MXINT4 in one launch with the transform: rows that fill no tile (their scale bytes are zero), buffers on 16-byte and on
+# 32-byte boundaries, against a pass over the transformed values in torch
+@pytest.mark.parametrize("rows,cols,reduce_dim", [(1, 128, 1), (130, 1280, 1), (384, 136, 0), (1000, 2048, 1)])
+@pytest.mark.parametrize("shift", [0, 16])
+@pytest.mark.parametrize("rounding", [0, 1])
+def test_mxint4_in_one_launch(rows, cols, reduce_dim, shift, rounding):
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(rows + cols)
+    x = torch.randn((rows, cols), generator=gen, device="cuda").bfloat16()
+    R, K = (rows, cols) if reduce_dim == 1 else (cols, rows)
+    codes = torch.full((R * K + 32,), 0xAA, dtype=torch.uint8, device="cuda")[shift:shift + R * K].view(R, K)
+    y = torch.full((R * K + 8,), float("nan"), device="cuda")[shift // 4:shift // 4 + R * K].view(R, K)
+    scales = torch.full((gpu.mxfp4_scale_bytes(R, K),), 0xAA, dtype=torch.uint8, device="cuda")
+    stream = torch.cuda.current_stream().cuda_stream
+    assert gpu.lib().mxfp4_int4_quantize(x.data_ptr(), rows, cols, cols, reduce_dim, 64, rounding, 5, 3, codes.data_ptr(), scales.data_ptr(),
+                                         y.data_ptr(), stream) == 0
+    assert gpu.mxfp4_device_status() == 0
+    assert torch.equal(y, gpu.mxfp4_rht(x, reduce_dim, 64, 5))
+    tiles = scales.view(-1, K // 128, 32, 4, 4).permute(0, 3, 2, 1, 4).reshape(-1, K // 32)
+    assert torch.all(tiles[R:] == 0)
+    exponent = torch.frexp(y.view(R, -1, 32).abs().amax(2))[1] - 3                     # floor(log2 amax) - 2
+    assert torch.equal(tiles[:R].int(), (exponent + 127).clamp(min=0))
+    q = codes.view(torch.float8_e4m3fn).double().view(R, -1, 32)
+    w = y.double().view(R, -1, 32) / torch.exp2(tiles[:R].double() - 127.0).unsqueeze(2) * (1.0 if rounding else 0.75)
+    if rounding:
+        assert torch.equal(q, w.round().clamp(-7.0, 7.0))
+    else:
+        assert torch.all((q - w).abs() < 1.0) and torch.all(q == q.round()) and abs(float((q - w).mean())) < 0.05
