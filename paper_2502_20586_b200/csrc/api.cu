@@ -419,7 +419,7 @@ struct Overlap {
 };
 mxfp4_status quantize_operands_impl(const void* dY, const void* X, const void* W, int64_t b, int64_t m, int64_t n, int g, int rounding,
                                     uint64_t seed, uint8_t* const c[4], uint8_t* const s[4], cudaStream_t stream, Overlap* ov = nullptr,
-                                    float* col_sums = nullptr, bool* col_sums_done = nullptr) {
+                                    const mx::BandSums* bias = nullptr, bool* bias_done = nullptr) {
     QuantArgs q[4] = {
         {dY, b, m, m, 1, g, rounding, seed, 1u, c[0], s[0], 1, nullptr},   // dY   [b, K = m]
         {W, m, n, n, 0, g, rounding, seed, 2u, c[1], s[1], 1, nullptr},    // W^T  [n, K = m]
@@ -450,12 +450,14 @@ mxfp4_status quantize_operands_impl(const void* dY, const void* X, const void* W
     // (worth a second launch only when dL/dy is large: below 2^25 elements, or when the column sums are not wanted from
     // it either, the four views go as one tile list in one launch, which is what the small layers' short kernels prefer)
     const int dual_mode = dual_setting();
-    if (all_tc && g != 256 && !force_lite() && (dual_mode == 2 || (dual_mode == 1 && (b * m >= (int64_t(1) << 25) || col_sums != nullptr)))) {
+    if (all_tc && g != 256 && !force_lite() && (dual_mode == 2 || (dual_mode == 1 && (b * m >= (int64_t(1) << 25) || bias != nullptr)))) {
         // dL/dy feeds lines 3 and 5: its two views come from ONE read of it; W^T and X^T in a second launch
         const QuantArgs dy[2] = {q[0], q[2]}, wx[2] = {q[1], q[3]};
+        // (the bias gradient's two passes ride along: band sums of dY in the first launch, their sum in the second)
+        float* col_sums = bias != nullptr ? const_cast<float*>(bias->partial) : nullptr;
         if (cuda_status(mx::launch_quantize_tc_group(dy, 2, false, stream, false, true, col_sums), "quantiser launch (both views of dY)") != MXFP4_OK) return MXFP4_ERR_CUDA;
-        if (col_sums != nullptr && col_sums_done != nullptr) *col_sums_done = true;     // the bias gradient's first pass rode along
-        return cuda_status(mx::launch_quantize_tc_group(wx, 2, false, stream), "quantiser launch (W, X)");
+        if (bias_done != nullptr) *bias_done = bias != nullptr;
+        return cuda_status(mx::launch_quantize_tc_group(wx, 2, false, stream, false, false, nullptr, bias), "quantiser launch (W, X)");
     }
     if (all_tc)                                     // the four views of the call in one launch
         return cuda_status(mx::launch_quantize_tc_group(q, 4, false, stream, g != 256 && force_lite()), "grouped quantiser launch");
@@ -523,8 +525,9 @@ mxfp4_status linear_backward_impl(const void* dY, const void* X, const void* W, 
     // Every tensor map is encoded before the first launch, so an encoding failure leaves nothing enqueued.
     if ((st = plan.encode(together)) != MXFP4_OK) return st;
     float* bias_partial = db != nullptr ? reinterpret_cast<float*>(base + bias_off) : nullptr;
+    const mx::BandSums bias{bias_partial, db, m, (int)(b / 128), accumulate};
     bool bias_fused = false;
-    if ((st = quantize_operands_impl(dY, X, W, b, m, n, g, rounding, seed, c, s, stream, &ov, bias_partial, &bias_fused)) != MXFP4_OK) {
+    if ((st = quantize_operands_impl(dY, X, W, b, m, n, g, rounding, seed, c, s, stream, &ov, db != nullptr ? &bias : nullptr, &bias_fused)) != MXFP4_OK) {
         if (ov.forked && (cudaEventRecord(ov.fj->join, ov.fj->side) != cudaSuccess || cudaStreamWaitEvent(stream, ov.fj->join, 0) != cudaSuccess)) return MXFP4_ERR_CUDA;
         return st;
     }
@@ -540,11 +543,9 @@ mxfp4_status linear_backward_impl(const void* dY, const void* X, const void* W, 
         st = plan.launch_one(0, stream);
         if (st == MXFP4_OK) st = plan.launch_one(1, stream);
     }
-    // dL/db = 1 dL/dy (problem statement): column sums of dY, after the GEMMs on the caller's stream
-    // (when the dual-view quantiser launch has already summed every 128-row band of dY, only the bands remain to be added)
-    if (st == MXFP4_OK && db != nullptr)
-        st = bias_fused ? cuda_status(mx::launch_bias_finish(bias_partial, m, (int)(b / 128), accumulate, db, stream), "bias gradient launch")
-                        : cuda_status(mx::launch_bias_grad(dY, b, m, m, accumulate, db, bias_partial, stream), "bias gradient launch");
+    // dL/db = 1 dL/dy (problem statement): column sums of dY, unless the quantiser launches have made them on their way
+    if (st == MXFP4_OK && db != nullptr && !bias_fused)
+        st = cuda_status(mx::launch_bias_grad(dY, b, m, m, accumulate, db, bias_partial, stream), "bias gradient launch");
     return st;
 }
 }  // namespace

@@ -95,6 +95,7 @@ struct QParams {
     bool wide_stores;          // y_out (and MXINT4 codes) start on 32-byte boundaries
     const uint16_t* custom_t;  // bf16 [g, g] row-major transform matrix given by the caller, or null (then diag(S) H_g / sqrt(g))
     uint64_t seed;
+    BandSums finish;           // partial == nullptr: none (see kernels.h)
     float* col_sums;           // DUAL launches: partial column sums [x rows / 128][x cols] of x in fp32 (bias gradient), or null
     PipeConsts pipe;           // see quant_math.cuh: constants kept opaque to the compiler
     PhiloxKeys keys;           // the ten Philox round keys of `seed` (key schedule only; the rounds run on the device)
@@ -379,6 +380,25 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
             *reinterpret_cast<float2*>(dst) = make_float2(s0, s1);
         }
         if (!ok && lane == 0) *abort_flag = 1;
+    } else if (!DUAL && !LITE && p.finish.partial != nullptr) {
+        // ------------------------------------------------------------------ warps 2, 3: the bands of the launch before, added up
+        // One thread per column, bands in order: a fixed summation order.  Bound by the latency of its loads, four in flight; as
+        // a kernel of its own after the GEMMs this took 4 to 5 us and a launch gap.
+        const float* partial = p.finish.partial;
+        const uint32_t m = (uint32_t)p.finish.m, end = m * (uint32_t)p.finish.bands;      // below 2^29: operands are below 2^36 elements
+#pragma unroll 1
+        for (uint32_t c = blockIdx.x * 64u + (threadIdx.x - 64u); c < m; c += gridDim.x * 64u) {
+            float sum = p.finish.accumulate ? p.finish.db[c] : 0.f;
+            uint32_t k = c;
+#pragma unroll 1
+            for (; k + 3u * m < end; k += 4u * m) {
+                const float v0 = partial[k], v1 = partial[k + m], v2 = partial[k + 2u * m], v3 = partial[k + 3u * m];
+                sum += v0; sum += v1; sum += v2; sum += v3;
+            }
+#pragma unroll 1
+            for (; k < end; k += m) sum += partial[k];
+            p.finish.db[c] = sum;
+        }
     }
     } else {
         // ------------------------------------------------------------------ epilogue (warp groups 1..4)
@@ -644,7 +664,8 @@ cudaError_t quant_tc_init() {
 }
 
 // Quantise n (1..kQuantMaxViews) eligible operand views that share g, seed, rounding and scale layout in one launch.
-cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cudaStream_t stream, bool lite, bool dual, float* col_sums) {
+cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cudaStream_t stream, bool lite, bool dual, float* col_sums,
+                                     const BandSums* finish) {
     if (n < 1 || n > kQuantMaxViews) return cudaErrorInvalidValue;
     // dual: a[0] and a[1] are the row-wise and the transposed view of one tensor, whose tiles are then loaded once for both
     if (dual && (n != 2 || lite || dump_y || a[0].g == 256 || a[0].custom_t != nullptr || a[0].x != a[1].x || a[0].rows != a[1].rows ||
@@ -678,6 +699,8 @@ cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cud
     if (p.custom_t != nullptr && p.g == 256) return cudaErrorInvalidValue;
     if (col_sums != nullptr && !dual) return cudaErrorInvalidValue;
     p.col_sums = col_sums;
+    if (finish != nullptr && (dual || lite)) return cudaErrorInvalidValue;
+    p.finish = finish != nullptr ? *finish : BandSums{nullptr, nullptr, 0, 0, 0};
     p.pipe = make_pipe_consts();
     {   // Philox key schedule: key_i = key_0 + i * (0x9E3779B9, 0xBB67AE85)
         uint32_t k0 = (uint32_t)p.seed, k1 = (uint32_t)(p.seed >> 32);
