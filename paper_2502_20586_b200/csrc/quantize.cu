@@ -43,34 +43,50 @@ __device__ __forceinline__ void rht_in_place(float (&v)[32], uint32_t sign_bits,
 
 // ------------------------------------------------------------------------------------------------ rowwise
 // Thread t of the grid owns MX block B = t: row B / (cols/32), columns [32 (B % (cols/32)), +32).
-template <int G, bool DUMP_Y>
+// Bound by memory with nearest rounding: 16384 x 2048, g = 0 16.7 -> 14.6 us (SR 22.8 -> 20.8), 16384 x 16384 117 -> 111, with:
+// Index: uint32_t where the tensor has fewer than 2^31 blocks (a 64-bit division costs more instructions than rounding the
+// block), else uint64_t.  `wide`: every row starts on a 32-byte boundary, so a block is two 32-byte loads of whole sectors.
+__device__ __forceinline__ void load_32B(const void* src, uint4& a, uint4& b, bool wide) {
+    if (wide) {
+        asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(src));
+    } else {
+        a = __ldg(reinterpret_cast<const uint4*>(src));
+        b = __ldg(reinterpret_cast<const uint4*>(src) + 1);
+    }
+}
+
+template <int G, bool DUMP_Y, typename Index>
 __global__ void __launch_bounds__(256) quantize_rowwise_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols,
                                                                int64_t ld, int rounding, uint64_t seed, uint32_t stream_tag,
                                                                uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
-                                                               int sf_native, float* __restrict__ y_out) {
-    const int64_t nkb = cols >> 5;
-    const int64_t B = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool valid = B < rows * nkb;
-    const int64_t row = valid ? B / nkb : 0;
-    const int64_t kb = valid ? B - row * nkb : 0;
+                                                               int sf_native, float* __restrict__ y_out, bool wide) {
+    const Index nkb = (Index)(cols >> 5);
+    const Index B = (Index)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool valid = B < (Index)rows * nkb;
+    const Index row = valid ? B / nkb : 0;
+    const Index kb = valid ? B - row * nkb : 0;
     const int lane = threadIdx.x & 31;
 
     float v[32];
     if (valid) {
-        const uint4* src = reinterpret_cast<const uint4*>(x + row * ld + kb * 32);
+        const __nv_bfloat16* src = x + (int64_t)row * ld + (int64_t)kb * 32;
+        uint4 q[4];
+        load_32B(src, q[0], q[1], wide);
+        load_32B(src + 16, q[2], q[3], wide);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) unpack_bf16x8(__ldg(src + i), v + 8 * i);
+        for (int i = 0; i < 4; ++i) unpack_bf16x8(q[i], v + 8 * i);
     } else {
 #pragma unroll
         for (int i = 0; i < 32; ++i) v[i] = 0.0f;
     }
-    if (G != 0) {
-        const uint32_t sb = sign_word(seed, (int)(kb & (G / 32 - 1)));
+    if constexpr (G != 0) {
+        const uint32_t sb = sign_word(seed, (int)(kb & (Index)(G / 32 - 1)));
         rht_in_place<G>(v, sb, lane, 1);
     }
     if (!valid) return;
     if (DUMP_Y) {
-        float4* dst = reinterpret_cast<float4*>(y_out + B * 32);
+        float4* dst = reinterpret_cast<float4*>(y_out + (int64_t)B * 32);
 #pragma unroll
         for (int i = 0; i < 8; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
         return;
@@ -78,7 +94,7 @@ __global__ void __launch_bounds__(256) quantize_rowwise_kernel(const __nv_bfloat
     uint32_t packed[4], sbyte;
     quantize_block32(v, rounding, seed, stream_tag, (uint64_t)B * 32u, packed, sbyte);
     reinterpret_cast<uint4*>(codes)[B] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-    const int64_t so = sf_native ? sf_native_offset(row, kb, (nkb + 3) >> 2) : B;
+    const int64_t so = sf_native ? sf_native_offset((int64_t)row, (int64_t)kb, (int64_t)((nkb + 3) >> 2)) : (int64_t)B;
     scales[so] = (uint8_t)sbyte;
 }
 
@@ -159,9 +175,10 @@ static cudaError_t launch(const QuantArgs& a, cudaStream_t stream) {
     if (a.reduce_dim == 1) {
         const int64_t nblocks = a.rows * (a.cols / 32);
         const unsigned grid = (unsigned)((nblocks + 255) / 256);
-#define MX_ROW(G_)                                                                                            \
-    quantize_rowwise_kernel<G_, DUMP_Y><<<grid, 256, 0, stream>>>(x, a.rows, a.cols, a.ld, a.rounding, a.seed, \
-                                                                   a.stream_tag, a.codes, a.scales, a.sf_native, a.y_out)
+        const bool wide = ((reinterpret_cast<uintptr_t>(x) | (uintptr_t)(a.ld * 2)) & 31u) == 0, small = nblocks < (int64_t(1) << 31);
+#define MX_ROW(G_)                                                                                                                   \
+    (small ? quantize_rowwise_kernel<G_, DUMP_Y, uint32_t> : quantize_rowwise_kernel<G_, DUMP_Y, uint64_t>)<<<grid, 256, 0, stream>>>( \
+        x, a.rows, a.cols, a.ld, a.rounding, a.seed, a.stream_tag, a.codes, a.scales, a.sf_native, a.y_out, wide)
         switch (a.g) {
             case 0: MX_ROW(0); break;
             case 32: MX_ROW(32); break;

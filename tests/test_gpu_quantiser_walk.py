@@ -86,3 +86,21 @@ def test_mxint4_in_one_launch(rows, cols, reduce_dim, shift, rounding):
         assert torch.equal(q, w.round().clamp(-7.0, 7.0))
     else:
         assert torch.all((q - w).abs() < 1.0) and torch.all(q == q.round()) and abs(float((q - w).mean())) < 0.05
+
+
+# The CUDA-core row-wise quantiser with rows on 32-byte boundaries and off them (pitch, base) gives the same bytes
+@pytest.mark.parametrize("rows,cols", [(1, 32), (7, 96), (300, 1056)])
+@pytest.mark.parametrize("rounding", [0, 1, 2])
+def test_row_alignment(rows, cols, rounding):
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(rows)
+    x = torch.randn((rows, cols), generator=gen, device="cuda").bfloat16()
+    want = gpu.mxfp4_rht_sr_quantize(x, 1, 0, 3, 2, rounding)
+    for pitch, start in ((cols + 8, 0), (cols + 16, 8), (cols + 16, 0)):
+        y = torch.empty((rows * pitch + 16,), dtype=torch.bfloat16, device="cuda").as_strided((rows, cols), (pitch, 1), start)
+        y.copy_(x)
+        got = gpu.mxfp4_rht_sr_quantize(y, 1, 0, 3, 2, rounding, gpu.SF_LINEAR)
+        assert torch.equal(got[0], want[0])
+        assert torch.equal(got[1], gpu.mxfp4_rht_sr_quantize(x, 1, 0, 3, 2, rounding, gpu.SF_LINEAR)[1])
