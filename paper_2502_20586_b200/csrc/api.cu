@@ -447,10 +447,12 @@ mxfp4_status quantize_operands_impl(const void* dY, const void* X, const void* W
         return cuda_status(mx::launch_quantize_tc_group(tail, 2, false, ov->fj->side, true), "small quantiser launch (second product)");
     }
     if (ov != nullptr) ov->first = -1;
-    // (worth a second launch only when dL/dy is large: below 2^25 elements, or when the column sums are not wanted from
-    // it either, the four views go as one tile list in one launch, which is what the small layers' short kernels prefer)
+    // One read of dL/dy for its two views needs a launch of its own (W and X follow in a second), and its units of two tiles
+    // spread less evenly: the four views as one tile list are faster until the read saved outweighs that.  Operands of a
+    // layer, one list / one read: 8192 x 1024 x 4096 39 / 49 us, 16384 x 8192 x 2048 106 / 117, 16384 x 4096 x 4096 103 / 112,
+    // 16384 x 2048 x 8192 152 / 154, 16384 x 4096 x 16384 329 / 327 (and a third less read from DRAM): from 2^28 elements on.
     const int dual_mode = dual_setting();
-    if (all_tc && g != 256 && !force_lite() && (dual_mode == 2 || (dual_mode == 1 && (b * m >= (int64_t(1) << 25) || bias != nullptr)))) {
+    if (all_tc && g != 256 && !force_lite() && (dual_mode == 2 || (dual_mode == 1 && (b * m >= (int64_t(1) << 28) || bias != nullptr)))) {
         // dL/dy feeds lines 3 and 5: its two views come from ONE read of it; W^T and X^T in a second launch
         const QuantArgs dy[2] = {q[0], q[2]}, wx[2] = {q[1], q[3]};
         // (the bias gradient's two passes ride along: band sums of dY in the first launch, their sum in the second)
