@@ -123,8 +123,8 @@ bool force_lite() {
     return e != nullptr && e[0] == '1';
 }
 
-// MXFP4_DUAL_DY: 1 (default) = one read of dL/dy for its two views where that pays (large layers, or a bias gradient
-// wanted); 0 = always separate tile lists (two reads); 2 = always one read.
+// MXFP4_DUAL_DY: 1 (default) = one read of dL/dy for its two views where that pays (2^28 elements and more; a bias
+// gradient's column sums ride along either way); 0 = always separate tile lists, sums by a pass of their own; 2 = always one read.
 int dual_setting() {
     const char* e = getenv("MXFP4_DUAL_DY");
     if (e == nullptr || e[0] == '\0') return 1;
@@ -259,7 +259,9 @@ struct GemmPlan {
         return g[i].use_pair ? cuda_status(mx::launch_gemm_pair(&g[i], 1, tile_n, stream), "pair GEMM launch")
                              : cuda_status(mx::launch_gemm(g[i], stream), "GEMM launch");
     }
-    mxfp4_status launch_both(cudaStream_t stream) const { return cuda_status(mx::launch_gemm_pair(g, 2, tile_n, stream), "pair GEMM launch (two products)"); }
+    mxfp4_status launch_both(cudaStream_t stream, const mx::BandSums* bias) const {
+        return cuda_status(mx::launch_gemm_pair(g, 2, tile_n, stream, bias), "pair GEMM launch (two products)");
+    }
 };
 
 mxfp4_status gemm_impl(const uint8_t* A_codes, const uint8_t* A_scales, const uint8_t* B_codes, const uint8_t* B_scales, int64_t M,
@@ -419,7 +421,7 @@ struct Overlap {
 };
 mxfp4_status quantize_operands_impl(const void* dY, const void* X, const void* W, int64_t b, int64_t m, int64_t n, int g, int rounding,
                                     uint64_t seed, uint8_t* const c[4], uint8_t* const s[4], cudaStream_t stream, Overlap* ov = nullptr,
-                                    const mx::BandSums* bias = nullptr, bool* bias_done = nullptr) {
+                                    float* col_sums = nullptr, bool* col_sums_done = nullptr) {
     QuantArgs q[4] = {
         {dY, b, m, m, 1, g, rounding, seed, 1u, c[0], s[0], 1, nullptr},   // dY   [b, K = m]
         {W, m, n, n, 0, g, rounding, seed, 2u, c[1], s[1], 1, nullptr},    // W^T  [n, K = m]
@@ -452,14 +454,17 @@ mxfp4_status quantize_operands_impl(const void* dY, const void* X, const void* W
     // layer, one list / one read: 8192 x 1024 x 4096 39 / 49 us, 16384 x 8192 x 2048 106 / 117, 16384 x 4096 x 4096 103 / 112,
     // 16384 x 2048 x 8192 152 / 154, 16384 x 4096 x 16384 329 / 327 (and a third less read from DRAM): from 2^28 elements on.
     const int dual_mode = dual_setting();
-    if (all_tc && g != 256 && !force_lite() && (dual_mode == 2 || (dual_mode == 1 && (b * m >= (int64_t(1) << 28) || bias != nullptr)))) {
+    if (all_tc && g != 256 && !force_lite() && (dual_mode == 2 || (dual_mode == 1 && b * m >= (int64_t(1) << 28)))) {
         // dL/dy feeds lines 3 and 5: its two views come from ONE read of it; W^T and X^T in a second launch
         const QuantArgs dy[2] = {q[0], q[2]}, wx[2] = {q[1], q[3]};
-        // (the bias gradient's two passes ride along: band sums of dY in the first launch, their sum in the second)
-        float* col_sums = bias != nullptr ? const_cast<float*>(bias->partial) : nullptr;
+        // (the bias gradient's first pass rides along: band sums of dY)
         if (cuda_status(mx::launch_quantize_tc_group(dy, 2, false, stream, false, true, col_sums), "quantiser launch (both views of dY)") != MXFP4_OK) return MXFP4_ERR_CUDA;
-        if (bias_done != nullptr) *bias_done = bias != nullptr;
-        return cuda_status(mx::launch_quantize_tc_group(wx, 2, false, stream, false, false, nullptr, bias), "quantiser launch (W, X)");
+        if (col_sums_done != nullptr) *col_sums_done = col_sums != nullptr;
+        return cuda_status(mx::launch_quantize_tc_group(wx, 2, false, stream), "quantiser launch (W, X)");
+    }
+    if (all_tc && g != 256 && !force_lite() && col_sums != nullptr && dual_mode != 0) {      // one launch, and the band sums with it
+        *col_sums_done = true;
+        return cuda_status(mx::launch_quantize_tc_group(q, 4, false, stream, false, false, col_sums), "grouped quantiser launch");
     }
     if (all_tc)                                     // the four views of the call in one launch
         return cuda_status(mx::launch_quantize_tc_group(q, 4, false, stream, g != 256 && force_lite()), "grouped quantiser launch");
@@ -529,7 +534,7 @@ mxfp4_status linear_backward_impl(const void* dY, const void* X, const void* W, 
     float* bias_partial = db != nullptr ? reinterpret_cast<float*>(base + bias_off) : nullptr;
     const mx::BandSums bias{bias_partial, db, m, (int)(b / 128), accumulate};
     bool bias_fused = false;
-    if ((st = quantize_operands_impl(dY, X, W, b, m, n, g, rounding, seed, c, s, stream, &ov, db != nullptr ? &bias : nullptr, &bias_fused)) != MXFP4_OK) {
+    if ((st = quantize_operands_impl(dY, X, W, b, m, n, g, rounding, seed, c, s, stream, &ov, together ? bias_partial : nullptr, &bias_fused)) != MXFP4_OK) {
         if (ov.forked && (cudaEventRecord(ov.fj->join, ov.fj->side) != cudaSuccess || cudaStreamWaitEvent(stream, ov.fj->join, 0) != cudaSuccess)) return MXFP4_ERR_CUDA;
         return st;
     }
@@ -540,12 +545,12 @@ mxfp4_status linear_backward_impl(const void* dY, const void* X, const void* W, 
         if (!joined) return MXFP4_ERR_CUDA;
         if (st == MXFP4_OK) st = plan.launch_one(1 - ov.first, stream);
     } else if (together) {
-        st = plan.launch_both(stream);
+        st = plan.launch_both(stream, bias_fused ? &bias : nullptr);
     } else {
         st = plan.launch_one(0, stream);
         if (st == MXFP4_OK) st = plan.launch_one(1, stream);
     }
-    // dL/db = 1 dL/dy (problem statement): column sums of dY, unless the quantiser launches have made them on their way
+    // dL/db = 1 dL/dy (problem statement): column sums of dY, unless the launches above have made them on their way
     if (st == MXFP4_OK && db != nullptr && !bias_fused)
         st = cuda_status(mx::launch_bias_grad(dY, b, m, m, accumulate, db, bias_partial, stream), "bias gradient launch");
     return st;

@@ -116,6 +116,7 @@ struct ParamsP {
     ProblemP prob[2];
     int n0, n1;                                             // tiles of the two products
     int rest, early;
+    BandSums bias;                                          // partial == nullptr: none
 };
 struct MapsP {
     CUtensorMap a[2], b[2], sfa[2], sfb[2], c[2];
@@ -343,6 +344,25 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
                 while (tile_i < walk.count && kt >= num_kt) { kt -= num_kt; num_kt = steps_of(++tile_i); }
             }
             if (!ok && lane == 0) *abort_flag = 1;
+        } else if (KIND == kMxf4 && !LITE && p.bias.partial != nullptr) {
+            // The second CTA of a pair issues nothing: its two warps add up the bands of dY's column sums (the quantiser launch
+            // before this one made them), a thread per column, bands in order.  Bound by the latency of its loads, hidden by
+            // the GEMM; as a kernel of its own behind it this took 4 to 5 us and a launch gap.
+            const float* partial = p.bias.partial;
+            const uint32_t m = (uint32_t)p.bias.m, end = m * (uint32_t)p.bias.bands;       // below 2^29: operands are below 2^36 elements
+#pragma unroll 1
+            for (uint32_t c = (blockIdx.x >> 1) * 64u + (uint32_t)(warp - 1) * 32u + (uint32_t)lane; c < m; c += (gridDim.x >> 1) * 64u) {
+                float sum = p.bias.accumulate ? p.bias.db[c] : 0.f;
+                uint32_t k = c;
+#pragma unroll 1
+                for (; k + 3u * m < end; k += 4u * m) {
+                    const float v0 = partial[k], v1 = partial[k + m], v2 = partial[k + 2u * m], v3 = partial[k + 3u * m];
+                    sum += v0; sum += v1; sum += v2; sum += v3;
+                }
+#pragma unroll 1
+                for (; k < end; k += m) sum += partial[k];
+                p.bias.db[c] = sum;
+            }
         }
     } else {
         // ------------------------------------------------------------------ scale loader (both CTAs)
@@ -603,7 +623,7 @@ int gemm_pair_tile_n(const GemmArgs* a, int n) {
     return time[1] < time[0] ? 128 : 256;
 }
 
-cudaError_t launch_gemm_pair(const GemmArgs* a, int n, int pn, cudaStream_t stream) {
+cudaError_t launch_gemm_pair(const GemmArgs* a, int n, int pn, cudaStream_t stream, const BandSums* bias) {
     if (n < 1 || n > 2 || (pn != 128 && pn != 256) || (a[0].lite && (n != 1 || pn != 256))) return cudaErrorInvalidValue;
     int pairs = 0;
     const cudaError_t e = pair_count(&pairs);
@@ -623,6 +643,8 @@ cudaError_t launch_gemm_pair(const GemmArgs* a, int n, int pn, cudaStream_t stre
     if (tiles[0] + tiles[1] < pairs) pairs = tiles[0] + tiles[1];
     const Spread s = spread_tiles(tiles[0], tiles[1], cost, pairs);
     p.n0 = tiles[0]; p.n1 = tiles[1]; p.rest = s.rest; p.early = s.early;
+    if (bias != nullptr && a[0].lite) return cudaErrorInvalidValue;
+    p.bias = bias != nullptr ? *bias : BandSums{};
     const uint32_t smem = a[0].lite ? LiteCfg::kSmem : pn == 128 ? PairCfg<kMxf4, false, 128>::kSmem : PairCfg<kMxf4, false, 256>::kSmem;
     void (*kernel)(MapsP, ParamsP) = a[0].lite ? gemm_mxf4_pair_lite_kernel : pn == 128 ? gemm_mxf4_pair_kernel<128> : gemm_mxf4_pair_kernel<256>;
     return launch_pairs(kernel, pairs, smem, maps, p, stream);

@@ -32,17 +32,17 @@ cudaError_t launch_quantize_tc(const QuantArgs& a, bool dump_y, cudaStream_t str
 constexpr int kQuantMaxViews = 4;
 // lite: the small-footprint build (g <= 128) that can share an SM with the small build of the pair GEMM.
 // dual: n = 2, a[0] / a[1] = the row-wise and the transposed view of ONE tensor (both extents multiples of 128): every tile of it is read once.
-// col_sums (dual only, may be null): fp32 [rows / 128, cols] receives the column sums of every 128-row band of that tensor.
-// finish (neither dual nor lite, may be null): db [m] = (accumulate ? db : 0) + the rows of partial [bands, m] added in order, by
-// warps that are idle otherwise (the col_sums of the launch before this one).
-struct BandSums {
-    const float* partial;
-    float* db;
-    int64_t m;
-    int bands, accumulate;
-};
+// col_sums (full-size build, g <= 128, may be null): fp32 [rows / 128, cols] receives the column sums of every 128-row band of a[0]'s
+// tensor (reduce_dim 1, rows a multiple of 128).
 cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cudaStream_t stream, bool lite = false, bool dual = false,
-                                     float* col_sums = nullptr, const BandSums* finish = nullptr);
+                                     float* col_sums = nullptr);
+// Second pass of the bias gradient: db [m] = (accumulate ? db : 0) + the rows of partial [bands, m] added in order.
+struct BandSums {
+    const float* partial = nullptr;
+    float* db = nullptr;
+    int64_t m = 0;
+    int bands = 0, accumulate = 0;
+};
 
 cudaError_t launch_quantize(const QuantArgs& a, cudaStream_t stream);
 cudaError_t launch_rht_dump(const QuantArgs& a, cudaStream_t stream);
@@ -142,7 +142,8 @@ cudaError_t launch_gemm(const GemmArgs& a, cudaStream_t stream);
 cudaError_t gemm_init();            // one-time: opt in to large dynamic shared memory
 // One product, or two independent ones in one launch; tile_n = what gemm_pair_tile_n says for them (the B maps' boxes depend on it).
 int gemm_pair_tile_n(const GemmArgs* a, int n);
-cudaError_t launch_gemm_pair(const GemmArgs* a, int n, int tile_n, cudaStream_t stream);
+// `bias` (may be null): warps that are idle otherwise add up the band sums.
+cudaError_t launch_gemm_pair(const GemmArgs* a, int n, int tile_n, cudaStream_t stream, const BandSums* bias = nullptr);
 cudaError_t gemm_pair_init();
 
 }  // namespace mx

@@ -95,8 +95,7 @@ struct QParams {
     bool wide_stores;          // y_out (and MXINT4 codes) start on 32-byte boundaries
     const uint16_t* custom_t;  // bf16 [g, g] row-major transform matrix given by the caller, or null (then diag(S) H_g / sqrt(g))
     uint64_t seed;
-    BandSums finish;           // partial == nullptr: none (see kernels.h)
-    float* col_sums;           // DUAL launches: partial column sums [x rows / 128][x cols] of x in fp32 (bias gradient), or null
+    float* col_sums;           // partial column sums [x rows / 128][x cols] of view 0's x in fp32 (bias gradient), or null
     PipeConsts pipe;           // see quant_math.cuh: constants kept opaque to the compiler
     PhiloxKeys keys;           // the ten Philox round keys of `seed` (key schedule only; the rounds run on the device)
 };
@@ -208,7 +207,7 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
 
     if (threadIdx.x == 0) {
         // a stage is free when its transforms have read it (one commit) and, with column sums on, the two summing warps too
-        const uint32_t n_readers = (DUAL && p.col_sums != nullptr) ? 3u : 1u;
+        const uint32_t n_readers = (KW == 1 && !LITE && p.col_sums != nullptr) ? 3u : 1u;
         for (int s = 0; s < kStagesQ; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], n_readers); }
         for (int b = 0; b < kAccBufs; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], (KW == 2 || LITE) ? 8 : 4); }
         *abort_flag = 0;
@@ -350,20 +349,25 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
             }
         }
         if (!ok && lane == 0) *abort_flag = 1;
-    } else if (DUAL && p.col_sums != nullptr) {
+    } else if (KW == 1 && !LITE && p.col_sums != nullptr) {
         // ------------------------------------------------------------------ warps 2, 3: column sums of the x tile (dL/db = 1 dL/dy)
         // The tile is in shared memory anyway: warp w sums columns 64 w .. 64 w + 63 (one TMA box), a lane two adjacent
         // columns (one 32-bit word per row; the 128-byte swizzle permutes 16-byte chunks inside a row, so a warp's 32
         // words of a row still fall into 32 different banks), rows in order: a fixed summation order.  One partial sum
-        // per (128-row band of x, column); a second kernel adds the bands in order.
+        // per (128-row band of x, column); the GEMM launch adds the bands in order.  (A launch of several views: only the
+        // tiles of view 0, the row-wise view of dY, are summed; the others pass.)
         const int w = warp - 2;
         uint32_t is = 0;
         bool ok = true;
-        for (uint32_t u = blockIdx.x; 2u * u < num_tiles; u += gridDim.x, ++is) {
+        for (uint32_t u = blockIdx.x; (DUAL ? 2u * u : u) < num_tiles; u += gridDim.x, ++is) {
             const int s = is % kStagesQ;
             ok = mbar_wait(&full_bar[s], (is / kStagesQ) & 1, abort_flag);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
+            if (!DUAL && u >= p.view[0].n_tiles) {
+                if (lane == 0) mbar_arrive(&empty_bar[s]);
+                continue;
+            }
             const uint8_t* box = smem + s * kTileBytes + w * kBoxBytes;
             float s0 = 0.f, s1 = 0.f;
 #pragma unroll 8
@@ -374,31 +378,12 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty_bar[s]);                   // this warp is done with the stage
-            const TilePos pos = locate_tile<DUAL>(p, 2u * u);
+            const TilePos pos = locate_tile<DUAL>(p, DUAL ? 2u * u : u);
             const uint32_t xr = row_tile(p.view[0], pos), xc = k_tile(p.view[0], pos);
             float* dst = p.col_sums + (int64_t)xr * (32 * (int64_t)p.view[0].k_blocks) + (int64_t)xc * kTile + w * 64 + 2 * lane;
             *reinterpret_cast<float2*>(dst) = make_float2(s0, s1);
         }
         if (!ok && lane == 0) *abort_flag = 1;
-    } else if (!DUAL && !LITE && p.finish.partial != nullptr) {
-        // ------------------------------------------------------------------ warps 2, 3: the bands of the launch before, added up
-        // One thread per column, bands in order: a fixed summation order.  Bound by the latency of its loads, four in flight; as
-        // a kernel of its own after the GEMMs this took 4 to 5 us and a launch gap.
-        const float* partial = p.finish.partial;
-        const uint32_t m = (uint32_t)p.finish.m, end = m * (uint32_t)p.finish.bands;      // below 2^29: operands are below 2^36 elements
-#pragma unroll 1
-        for (uint32_t c = blockIdx.x * 64u + (threadIdx.x - 64u); c < m; c += gridDim.x * 64u) {
-            float sum = p.finish.accumulate ? p.finish.db[c] : 0.f;
-            uint32_t k = c;
-#pragma unroll 1
-            for (; k + 3u * m < end; k += 4u * m) {
-                const float v0 = partial[k], v1 = partial[k + m], v2 = partial[k + 2u * m], v3 = partial[k + 3u * m];
-                sum += v0; sum += v1; sum += v2; sum += v3;
-            }
-#pragma unroll 1
-            for (; k < end; k += m) sum += partial[k];
-            p.finish.db[c] = sum;
-        }
     }
     } else {
         // ------------------------------------------------------------------ epilogue (warp groups 1..4)
@@ -664,8 +649,7 @@ cudaError_t quant_tc_init() {
 }
 
 // Quantise n (1..kQuantMaxViews) eligible operand views that share g, seed, rounding and scale layout in one launch.
-cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cudaStream_t stream, bool lite, bool dual, float* col_sums,
-                                     const BandSums* finish) {
+cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cudaStream_t stream, bool lite, bool dual, float* col_sums) {
     if (n < 1 || n > kQuantMaxViews) return cudaErrorInvalidValue;
     // dual: a[0] and a[1] are the row-wise and the transposed view of one tensor, whose tiles are then loaded once for both
     if (dual && (n != 2 || lite || dump_y || a[0].g == 256 || a[0].custom_t != nullptr || a[0].x != a[1].x || a[0].rows != a[1].rows ||
@@ -697,10 +681,9 @@ cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cud
     p.wide_stores = ((reinterpret_cast<uintptr_t>(a[0].y_out) | (a[0].mxint4 ? reinterpret_cast<uintptr_t>(a[0].codes) : 0)) & 31u) == 0;
     p.custom_t = static_cast<const uint16_t*>(a[0].custom_t);
     if (p.custom_t != nullptr && p.g == 256) return cudaErrorInvalidValue;
-    if (col_sums != nullptr && !dual) return cudaErrorInvalidValue;
+    // column sums: of view 0's tensor, read row-wise in whole 128-row bands
+    if (col_sums != nullptr && (lite || dump_y || a[0].g == 256 || a[0].mxint4 || a[0].reduce_dim != 1 || a[0].rows % kTile != 0)) return cudaErrorInvalidValue;
     p.col_sums = col_sums;
-    if (finish != nullptr && (dual || lite)) return cudaErrorInvalidValue;
-    p.finish = finish != nullptr ? *finish : BandSums{nullptr, nullptr, 0, 0, 0};
     p.pipe = make_pipe_consts();
     {   // Philox key schedule: key_i = key_0 + i * (0x9E3779B9, 0xBB67AE85)
         uint32_t k0 = (uint32_t)p.seed, k1 = (uint32_t)(p.seed >> 32);
