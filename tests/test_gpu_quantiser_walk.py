@@ -104,3 +104,22 @@ def test_row_alignment(rows, cols, rounding):
         got = gpu.mxfp4_rht_sr_quantize(y, 1, 0, 3, 2, rounding, gpu.SF_LINEAR)
         assert torch.equal(got[0], want[0])
         assert torch.equal(got[1], gpu.mxfp4_rht_sr_quantize(x, 1, 0, 3, 2, rounding, gpu.SF_LINEAR)[1])
+
+
+# The bias gradient's two passes inside the launches of a backward call: band sums in the one-list and in the one-read form,
+# added up by the GEMM launch; against fp64, overwriting and accumulating
+@pytest.mark.parametrize("b,n,m", [(128, 264, 128), (640, 8, 1152), (2048, 1000, 5120)])
+@pytest.mark.parametrize("dual", ["0", "1", "2"])
+def test_bias_gradient_inside_the_launches(b, n, m, dual, monkeypatch):
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    monkeypatch.setenv("MXFP4_DUAL_DY", dual)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(b + m)
+    dY, X, W = (torch.randn(s, generator=gen, device="cuda").bfloat16() for s in ((b, m), (b, n), (m, n)))
+    _, dW, db = gpu.mxfp4_linear_backward_ex(dY, X, W, 64, 5, gpu.ROUND_SR, gpu.OUT_FP32, with_bias=True)
+    want, bound = dY.double().sum(0), b * 2.0 ** -24 * dY.double().abs().sum(0)      # fp32 sums in any order
+    assert torch.all((db.double() - want).abs() <= bound)
+    gpu.mxfp4_linear_backward_ex(dY, X, W, 64, 6, gpu.ROUND_SR, gpu.OUT_FP32, dW=dW, db=db, accumulate=True)
+    assert torch.all((db.double() - 2.0 * want).abs() <= 4.0 * bound)
+    assert gpu.mxfp4_device_status() == 0
