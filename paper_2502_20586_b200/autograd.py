@@ -19,8 +19,6 @@ class MxFp4LinearFunction(torch.autograd.Function):
         if fp8_forward:     # Section 4.1: E4M3 forward pass (one scale per tensor), the library's own kernels
             y = mx.mxfp4_linear_forward_fp8(x.reshape(-1, x.shape[-1]).contiguous(), weight.contiguous(), mx.OUT_BF16)
             y = y.view(*x.shape[:-1], weight.shape[0])
-        elif bias is not None and bias.dim() == 1 and bias.dtype == x.dtype == weight.dtype:
-            return torch.nn.functional.linear(x, weight, bias)     # the bias in the product's epilogue: one rounding, no second pass over y
         else:
             y = x @ weight.t()
         return y if bias is None else y + bias

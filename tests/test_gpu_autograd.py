@@ -39,6 +39,26 @@ def test_backward_is_the_library_call_and_estimates_the_gradient(torch_gpu):
     assert mx.mxfp4_device_status() == 0
 
 
+# a bias that is not zero, added to the rounded product; against fp64 with the two bf16 roundings and the fp32 sums as the bound
+@pytest.mark.parametrize("lead", [(256,), (2, 128)])
+def test_biased_bf16_forward(torch_gpu, lead):
+    torch = torch_gpu
+    from paper_2502_20586_b200.autograd import MxFp4Linear
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    layer = MxFp4Linear(264, 384, bias=True, g=64)
+    with torch.no_grad():
+        layer.bias.copy_(torch.randn(384, device="cuda", generator=gen))
+    x = torch.randn(*lead, 264, device="cuda", generator=gen).to(torch.bfloat16)
+    y = layer(x)
+    w, b = layer.weight.detach(), layer.bias.detach()
+    assert y.dtype == torch.bfloat16 and torch.equal(y, x @ w.t() + b)
+    product = x.double() @ w.double().t()
+    exact = product + b.double()
+    half_ulp = 2.0 ** -9
+    bound = half_ulp * ((1 + half_ulp) * product.abs() + exact.abs()) + 264 * 2.0 ** -23 * (x.double().abs() @ w.double().abs().t())
+    assert torch.all((y.double() - exact).abs() <= bound)
+
+
 def test_seeds_advance_and_the_mean_gradient_converges(torch_gpu):
     """SR makes the backward unbiased (Lemma 3.1): the mean over T calls approaches the exact gradient like T^-1/2."""
     torch = torch_gpu
