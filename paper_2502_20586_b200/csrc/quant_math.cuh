@@ -449,8 +449,13 @@ __device__ __forceinline__ void quantize_block32(const float (&y)[32], int round
 // Byte offset of the scale of (row r, 32-block k) in the tcgen05 scale-factor tiling: 128-row x 4-block
 // tiles of 512 bytes, tile (r/128, k/4) at ((r/128) * n_ktiles + k/4) * 512, inside a tile
 // (r % 32) * 16 + ((r % 128) / 32) * 4 + k % 4.
-__device__ __forceinline__ int64_t sf_native_offset(int64_t r, int64_t k, int64_t n_ktiles) {
+__host__ __device__ __forceinline__ int64_t sf_native_offset(int64_t r, int64_t k, int64_t n_ktiles) {
     return ((r >> 7) * n_ktiles + (k >> 2)) * 512 + (r & 31) * 16 + ((r & 127) >> 5) * 4 + (k & 3);
+}
+// The same for the first of a row's four scales in tile `tile`, row 32 quadrant + lane of it.  Tile indices fit 32 bits, byte
+// offsets do not: rows are padded to 128, so an operand of few rows passes 2^23 tiles within the element limit.
+__host__ __device__ __forceinline__ uint64_t sf_row_offset(uint32_t tile, uint32_t quadrant, uint32_t lane) {
+    return (uint64_t)tile * 512u + lane * 16u + quadrant * 4u;
 }
 
 }  // namespace mx

@@ -436,7 +436,7 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
                 const bool live = rt * kTile + lane_row < vw.R;
                 const uint32_t blk_cur = blk;
                 uint8_t* code_dst = vw.codes + (uint64_t)blk_cur * 16u;
-                uint8_t* scale_dst = vw.scales + (p.sf_native ? (rt * ((vw.k_blocks + 3) >> 2) + 2 * kt + hh) * 512u + lane * 16 + q * 4 : blk_cur);
+                uint8_t* scale_dst = vw.scales + (p.sf_native ? sf_row_offset(rt * ((vw.k_blocks + 3) >> 2) + 2 * kt + hh, q, lane) : blk_cur);
                 float* y_dst = MODE == kModeDump ? vw.y_out + (uint64_t)blk_cur * 32u : nullptr;
                 pos = advance_tile<DUAL>(p, pos, tile_of(it + kTeams));
                 blk = first_block(pos);
@@ -497,7 +497,7 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
             const bool live = rt * kTile + lane_row < vw.R;
             const uint32_t blk_cur = blk;
             uint8_t* code_dst = vw.codes + (uint64_t)blk_cur * (mode_int4(MODE) ? 32u : 16u);
-            uint8_t* scale_dst = vw.scales + (p.sf_native ? (rt * ((vw.k_blocks + 3) >> 2) + kt) * 512u + lane * 16 + q * 4 + part : blk_cur);
+            uint8_t* scale_dst = vw.scales + (p.sf_native ? sf_row_offset(rt * ((vw.k_blocks + 3) >> 2) + kt, q, lane) + part : blk_cur);
             float* y_dst = mode_keeps_y(MODE) ? vw.y_out + (uint64_t)blk_cur * 32u : nullptr;
             // position of the next tile of this team (past the end: computed but not used)
             pos = advance_tile<DUAL>(p, pos, tile_of(it + kTeams));

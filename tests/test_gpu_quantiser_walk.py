@@ -123,3 +123,36 @@ def test_bias_gradient_inside_the_launches(b, n, m, dual, monkeypatch):
     gpu.mxfp4_linear_backward_ex(dY, X, W, 64, 6, gpu.ROUND_SR, gpu.OUT_FP32, dW=dW, db=db, accumulate=True)
     assert torch.all((db.double() - 2.0 * want).abs() <= 4.0 * bound)
     assert gpu.mxfp4_device_status() == 0
+
+
+# An operand of eight rows with more than 2^23 scale tiles (its scales fill more than 4 GB), against the same quantiser on the
+# operand's first and last columns: nearest rounding, so the bytes do not depend on where a block lies
+@pytest.mark.parametrize("kind,reduce_dim,g", [("mxfp4", 1, 64), ("mxfp4", 0, 32), ("mxfp4", 1, 256), ("mxint4", 1, 128)])
+def test_more_than_four_gigabytes_of_scales(kind, reduce_dim, g):
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    if torch.cuda.mem_get_info()[0] < (90 << 30):
+        pytest.skip("needs 90 GB of device memory")
+    K = (1 << 30) + 256
+
+    def quantise(x):
+        if kind == "mxint4":
+            return gpu.mxfp4_int4_quantize(x, reduce_dim, g, 3, 2, gpu.ROUND_RN)[:2]
+        return gpu.mxfp4_rht_sr_quantize(x, reduce_dim, g, 3, 2, gpu.ROUND_RN)
+
+    x = torch.zeros((8, K) if reduce_dim == 1 else (K, 8), dtype=torch.bfloat16, device="cuda")
+    ends = [x.narrow(reduce_dim, 0, 1024), x.narrow(reduce_dim, 1 << 30, 256)]
+    for i, end in enumerate(ends):
+        end.copy_(_small_integers(tuple(end.shape), i + 1) * (1 << 4 * i))
+    codes, scales = quantise(x)
+    assert gpu.mxfp4_device_status() == 0
+    tiles = scales.view(-1, 32, 4, 4)[:, :8, 0, :]                       # the eight rows' bytes of every tile
+    per_tile = codes.shape[1] // (K // 128)
+    for end, t0 in ((ends[0], 0), (ends[1], 1 << 23)):
+        want, want_scales = quantise(end.contiguous())
+        n = want_scales.numel() // 512
+        assert torch.equal(tiles[t0:t0 + n], want_scales.view(-1, 32, 4, 4)[:, :8, 0, :])
+        assert torch.equal(codes[:, t0 * per_tile:(t0 + n) * per_tile], want)
+    assert not torch.any(tiles[8:1 << 23])
+    del x, ends, codes, scales, tiles, end
+    torch.cuda.empty_cache()
