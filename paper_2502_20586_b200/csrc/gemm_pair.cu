@@ -309,8 +309,8 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
                 const uint32_t buf = tile_i % kAccBufs, acc = tmem_acc + buf * PN;
                 if (kt == 0) {
                     if (!(ok = __all_sync(0xffffffffu, mbar_wait_spin(&tmem_empty[buf], ((tile_i / kAccBufs) & 1) ^ 1, abort_flag)))) break;
-                    tc_fence_after_sync();
                 }
+                tc_fence_after_sync();                       // the other warp's MMAs on this accumulator come before mine, in every step
                 const uint32_t hi2 = 2u << 30;
                 const bool last = kt == num_kt - 1;
                 auto D = [&](uint32_t lo) { return ((uint64_t)desc_hi << 32) | lo; };
