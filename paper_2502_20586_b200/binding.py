@@ -100,6 +100,14 @@ def _ptr(t) -> int:
     return 0 if t is None else t.data_ptr()
 
 
+def _empty(like, shape, dtype):
+    """A plain tensor on the device of ``like``.  ``new_empty`` spares the device object (2.2 -> 1.7 us, timed on
+    CPU tensors), but returns a subclass for a subclass."""
+    if type(like) is torch.Tensor:
+        return like.new_empty(shape, dtype=dtype)
+    return torch.empty(shape, dtype=dtype, device=like.device)
+
+
 def lib():
     """The raw ctypes handle (tests use it to probe error codes with arbitrary arguments)."""
     return _lib
@@ -195,11 +203,11 @@ def mxfp4_linear_backward_fused(dY, X, W, g: int, seed: int, rounding: int = ROU
         assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()
     dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
     if dX is None:
-        dX = dY.new_empty((b, n), dtype=dt)
+        dX = _empty(dY, (b, n), dt)
     if dW is None:
-        dW = dY.new_empty((m, n), dtype=dt)
+        dW = _empty(dY, (m, n), dt)
     if workspace is None:
-        workspace = dY.new_empty(mxfp4_linear_backward_workspace(b, m, n), dtype=torch.uint8)
+        workspace = _empty(dY, mxfp4_linear_backward_workspace(b, m, n), torch.uint8)
     _check(_lib.mxfp4_linear_backward_fused(_ptr(dY), _ptr(X), _ptr(W), b, m, n, g, rounding, seed, _ptr(dX), _ptr(dW),
                                             out_dtype, _ptr(workspace), workspace.numel(), _stream()))
     return dX, dW
@@ -213,7 +221,7 @@ def mxfp4_quantize_operands(dY, X, W, g: int, seed: int, rounding: int = ROUND_S
     for t in (dY, X, W):
         assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()
     if workspace is None:
-        workspace = dY.new_empty(mxfp4_linear_backward_workspace(b, m, n), dtype=torch.uint8)
+        workspace = _empty(dY, mxfp4_linear_backward_workspace(b, m, n), torch.uint8)
     _check(_lib.mxfp4_quantize_operands(_ptr(dY), _ptr(X), _ptr(W), b, m, n, g, rounding, seed, _ptr(workspace), workspace.numel(),
                                         _stream()))
     off = (_sz * 8)()
@@ -247,12 +255,12 @@ def mxfp4_linear_backward(dY, X, W, g: int, seed: int, rounding: int = ROUND_SR,
         assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()
     dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
     if dX is None:
-        dX = dY.new_empty((b, n), dtype=dt)
+        dX = _empty(dY, (b, n), dt)
     if dW is None:
-        dW = dY.new_empty((m, n), dtype=dt)
+        dW = _empty(dY, (m, n), dt)
     need = mxfp4_linear_backward_workspace(b, m, n)
     if workspace is None:
-        workspace = dY.new_empty(need, dtype=torch.uint8)
+        workspace = _empty(dY, need, torch.uint8)
     _check(_lib.mxfp4_linear_backward(_ptr(dY), _ptr(X), _ptr(W), b, m, n, g, rounding, seed, _ptr(dX), _ptr(dW),
                                       out_dtype, _ptr(workspace), workspace.numel(), _stream()))
     return dX, dW
@@ -272,16 +280,16 @@ def mxfp4_linear_backward_ex(dY, X, W, g: int, seed: int, rounding: int = ROUND_
         assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()
     dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
     if dX is None:
-        dX = dY.new_empty((b, n), dtype=dt)
+        dX = _empty(dY, (b, n), dt)
     if dW is None:
         assert not accumulate, "accumulation needs an existing dW"
-        dW = dY.new_empty((m, n), dtype=dt)
+        dW = _empty(dY, (m, n), dt)
     if db is None and with_bias:
         assert not accumulate, "accumulation needs an existing db"
         db = torch.empty((m,), dtype=torch.float32, device=dY.device)
     need = mxfp4_linear_backward_ex_workspace(b, m, n, db is not None)
     if workspace is None:
-        workspace = dY.new_empty(need, dtype=torch.uint8)
+        workspace = _empty(dY, need, torch.uint8)
     _check(_lib.mxfp4_linear_backward_ex(_ptr(dY), _ptr(X), _ptr(W), b, m, n, g, rounding, seed, _ptr(dX), _ptr(dW),
                                          _ptr(db) if db is not None else None, out_dtype, 1 if accumulate else 0,
                                          _ptr(workspace), workspace.numel(), _stream()))
@@ -302,9 +310,9 @@ def mxfp4_linear_backward_static(dY, X, W, g: int, seed: int, rounding: int = RO
         assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()
     dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
     if dX is None:
-        dX = dY.new_empty((b, n), dtype=dt)
+        dX = _empty(dY, (b, n), dt)
     if dW is None:
-        dW = dY.new_empty((m, n), dtype=dt)
+        dW = _empty(dY, (m, n), dt)
     _check(_lib.mxfp4_linear_backward_static(_ptr(dY), _ptr(X), _ptr(W), b, m, n, g, rounding, seed, _ptr(dX), _ptr(dW),
                                              out_dtype, _stream()))
     return dX, dW
