@@ -54,8 +54,10 @@ def test_biased_bf16_forward(torch_gpu, lead):
     assert y.dtype == torch.bfloat16 and torch.equal(y, x @ w.t() + b)
     product = x.double() @ w.double().t()
     exact = product + b.double()
-    half_ulp = 2.0 ** -9
-    bound = half_ulp * ((1 + half_ulp) * product.abs() + exact.abs()) + 264 * 2.0 ** -23 * (x.double().abs() @ w.double().abs().t())
+    # bf16 has eight significant bits: one rounding is off by at most u = 2^-8 of the value.  The product is rounded once (u |p|),
+    # the sum of the rounded product and the bias once more (u (|exact| + u |p|)); 264 fp32 additions, doubled for those two factors.
+    u = 2.0 ** -8
+    bound = u * product.abs() + u * (exact.abs() + u * product.abs()) + 264 * 2.0 ** -23 * (x.double().abs() @ w.double().abs().t())
     assert torch.all((y.double() - exact).abs() <= bound)
 
 
