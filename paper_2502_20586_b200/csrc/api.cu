@@ -202,7 +202,8 @@ void attach_input_map(QuantArgs& a) {
 mxfp4_status make_output_map(CUtensorMap* map, void* C, int64_t M, int64_t N, int64_t ldc, bool fp32) {
     const int64_t es = fp32 ? 4 : 2;
     const cuuint64_t dims[2] = {(cuuint64_t)N, (cuuint64_t)M};
-    const cuuint64_t strides[1] = {(cuuint64_t)(ldc * es)};
+    // (of a single row the pitch is any number the caller likes; a tensor map takes 40 bits)
+    const cuuint64_t strides[1] = {(cuuint64_t)((M > 1 ? ldc : round_up(N, 8)) * es)};
     const cuuint32_t box[2] = {(cuuint32_t)(64 / es), 32};
     const cuuint32_t elem_strides[2] = {1, 1};
     return encode_status(g_rt.encode(map, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, C, dims, strides,

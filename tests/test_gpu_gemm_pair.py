@@ -98,3 +98,18 @@ def test_eight_bit_products(gpu, M, N, K, kind, fp32):
     # fp32 sums (and one rounding of the scale and of the product) of K terms; bf16 output: half a unit in the last place more
     bound = 16 * 2.0 ** -24 * size + (0.0 if fp32 else 2.0 ** -8) * want.abs()
     assert torch.all((got.double() - want).abs() <= bound + 1e-30)
+
+
+# one output row: its pitch means nothing and may be larger than a tensor map can hold
+@pytest.mark.parametrize("ldc", [264, 1 << 20, 1 << 40])
+def test_pitch_of_a_single_row(gpu, ldc):
+    import torch
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(1)
+    a, b = ((torch.randn((rows, 256), generator=gen, device="cuda") * 8).to(torch.float8_e4m3fn).view(torch.uint8) for rows in (1, 264))
+    one = torch.ones(2, device="cuda")
+    want = gpu.mxfp4_fp8_gemm(a, one, b, one, gpu.OUT_FP32)
+    got = torch.full((1, 264), float("nan"), device="cuda")
+    assert gpu.lib().mxfp4_fp8_gemm(a.data_ptr(), one.data_ptr(), b.data_ptr(), one.data_ptr(), 1, 264, 256, got.data_ptr(), ldc, gpu.OUT_FP32,
+                                    torch.cuda.current_stream().cuda_stream) == 0
+    assert gpu.mxfp4_device_status() == 0 and torch.equal(got, want)
