@@ -594,7 +594,7 @@ def run_gpu(args):
                        "frac_of_nominal_9pf": value / world / NOMINAL_FP4_TFLOPS, "timed_region_s": ms * args.steps * 1e-3,
                        "step_as_separate_calls_ms": calls_ms},
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h, "ms_per_step": ms_e2e},
-            "gpu_launches": args.steps * sum(3 if l.b * l.m >= (1 << 28) else 2 for l in layers),   # per layer: one or two quantiser launches + one for both GEMMs
+            "gpu_launches": args.steps * sum(3 if l.b * l.m >= mx.ONE_READ_ELEMENTS else 2 for l in layers),   # per layer: one or two quantiser launches + one for both GEMMs
             "clocks": clocks,
             "roofline": None if gemm_tflops is None else {
                          "kernel": "gemm_mxf4_pair_kernel", "bound": "tensor", "achieved": gemm_tflops, "peak": fp4_peak, "unit": "TFLOP/s",

@@ -129,6 +129,10 @@ MXFP4_API mxfp4_status mxfp4_gemm(const uint8_t* A_codes, const uint8_t* A_scale
                         int64_t M, int64_t N, int64_t K, int sf_layout, float alpha,
                         void* C, int64_t ldc, int out_dtype, void* cuda_stream);
 
+/* Elements of dY from which on one launch reads it once for its two views and a second one takes W and X; below, one launch
+ * takes the four views. */
+#define MXFP4_ONE_READ_ELEMENTS (1ll << 28)
+
 /* Bytes of device workspace mxfp4_linear_backward needs for these shapes (codes + scales of the four
  * quantised operands). */
 MXFP4_API size_t mxfp4_linear_backward_workspace(int64_t b, int64_t m, int64_t n);

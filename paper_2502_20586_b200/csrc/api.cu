@@ -24,7 +24,7 @@ struct Runtime {
     std::once_flag once;
     mxfp4_status status = MXFP4_OK;
     EncodeTiledFn encode = nullptr;
-    bool gemm_pair = true;       // CTA-pair GEMM (gemm_pair.cu); MXFP4_GEMM_PAIR=0 selects the 1-CTA kernel (gemm.cu)
+    bool gemm_pair = true;       // CTA-pair GEMM (gemm_pair.cu); MXFP4_GEMM_PAIR=0 selects the 1-CTA kernel (gemm.cu) for MXFP4 products
     std::mutex mu;
     static constexpr int kMaxDevices = 64;
     mxfp4_status dev_status[kMaxDevices];
@@ -123,7 +123,7 @@ bool force_lite() {
     return e != nullptr && e[0] == '1';
 }
 
-// MXFP4_DUAL_DY: 1 (default) = one read of dL/dy for its two views where that pays (2^28 elements and more; a bias
+// MXFP4_DUAL_DY: 1 (default) = one read of dL/dy for its two views where that pays (MXFP4_ONE_READ_ELEMENTS; a bias
 // gradient's column sums ride along either way); 0 = always separate tile lists, sums by a pass of their own; 2 = always one read.
 int dual_setting() {
     const char* e = getenv("MXFP4_DUAL_DY");
@@ -452,10 +452,14 @@ mxfp4_status quantize_operands_impl(const void* dY, const void* X, const void* W
     if (ov != nullptr) ov->first = -1;
     // One read of dL/dy for its two views needs a launch of its own (W and X follow in a second), and its units of two tiles
     // spread less evenly: the four views as one tile list are faster until the read saved outweighs that.  Operands of a
-    // layer, one list / one read: 8192 x 1024 x 4096 39 / 49 us, 16384 x 8192 x 2048 106 / 117, 16384 x 4096 x 4096 103 / 112,
-    // 16384 x 2048 x 8192 152 / 154, 16384 x 4096 x 16384 329 / 327 (and a third less read from DRAM): from 2^28 elements on.
+    // layer, tokens x in x out, g = 128, one list / one read in us.  SR, below 2^28 elements of dL/dy: 8192 x 1024 x 4096
+    // 39 / 49, 16384 x 8192 x 2048 106 / 117, 16384 x 4096 x 4096 103 / 112, 16384 x 2048 x 8192 156 / 154.  At 2^28:
+    // 16384 x 1024 x 16384 308 / 302, 16384 x 4096 x 16384 375 / 380, 32768 x 4096 x 8192 435 / 440, 65536 x 1024 x 4096 366 / 370;
+    // at 2^29 32768 x 4096 x 16384 841 / 819, 16384 x 4096 x 32768 696 / 688; at 2^30 65536 x 4096 x 16384 1363 / 1294.  Nearest
+    // rounding gains more (16384 x 4096 x 16384 326 / 312, 32768 x 4096 x 16384 632 / 617), SR16 as well (353 / 340, 701 / 660).  Whole
+    // calls differ by less than their repeats.  So 2^28 is where the two tie with SR and the others gain 2 - 6 %.
     const int dual_mode = dual_setting();
-    if (all_tc && g != 256 && !force_lite() && (dual_mode == 2 || (dual_mode == 1 && b * m >= (int64_t(1) << 28)))) {
+    if (all_tc && g != 256 && !force_lite() && (dual_mode == 2 || (dual_mode == 1 && b * m >= MXFP4_ONE_READ_ELEMENTS))) {
         // dL/dy feeds lines 3 and 5: its two views come from ONE read of it; W^T and X^T in a second launch
         const QuantArgs dy[2] = {q[0], q[2]}, wx[2] = {q[1], q[3]};
         // (the bias gradient's first pass rides along: band sums of dY)

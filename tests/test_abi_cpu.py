@@ -45,6 +45,13 @@ def test_scale_bytes_and_workspace(lib):
     assert lib.mxfp4_linear_backward_workspace(0, m, n) == 0
 
 
+def test_constants_of_the_header_are_those_of_the_binding(lib):
+    header = open(os.path.join(ROOT, "include", "mxfp4.h")).read()
+    for name, value in (("STATIC_WORKSPACE_BYTES", lib.STATIC_WORKSPACE_BYTES), ("ONE_READ_ELEMENTS", lib.ONE_READ_ELEMENTS)):
+        base, shift = re.search(rf"#define MXFP4_{name} \((\d+)\w* << (\d+)\)", header).groups()
+        assert int(base) << int(shift) == value
+
+
 def test_argument_validation_needs_no_device(lib):
     raw = lib.lib()
     P = 0x1000                                    # a fake, 16-byte aligned, never dereferenced pointer
