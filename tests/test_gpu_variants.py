@@ -101,7 +101,7 @@ def _int4_codes_from_e4m3(codes):
     return (np.abs(v).astype(np.uint8) | (np.signbit(v).astype(np.uint8) << 3))
 
 
-@pytest.mark.parametrize("g", [0, 64, 128])
+@pytest.mark.parametrize("g", [0, 32, 64, 128, 256])
 @pytest.mark.parametrize("reduce_dim,shape", [(1, (130, 1280)), (0, (768, 136)), (1, (3, 32))])
 @pytest.mark.parametrize("rounding", [0, 1])
 def test_int4_quantiser_bit_exact_on_gpu_values(gpu, ref, g, reduce_dim, shape, rounding):
