@@ -21,25 +21,28 @@
 //                stores (or reduce-adds when accumulating).
 // A-row scales are per CTA; every CTA needs the scales of all 256 B rows.
 //
-// What bounds it: the tensor pipe in the steady state (539 cycles a K-step, four MMAs of 137 by their nominal rate)
-// and the board's power (1.36 - 1.57 GHz in a long launch); per tile about 1100 cycles in which the pipe stands still,
-// since TMEM has no room for a second 256-column accumulator beside the scale slots.  Two things got it there:
-//   - issue.  From a lane-0 branch an MMA took its thread 92 cycles, a scale copy 60, a commit 109 (descriptors go to
-//     uniform registers one by one), 660 cycles a step with two threads.  With warp-uniform control flow and an elected
-//     lane the issuers wait for operands instead.  Back to back, before -> now: 16384 x 4096 x 16384 382 -> 349 us (alone
-//     372 -> 333: 6.6 PFLOP/s), 16384 x 4096 x 4096 105 -> 97, 1024 x 1024 x 8192 16.2 -> 12.5.  One issuing warp without
-//     the baton: 376, 103, 16.5;
+// What bounds it: the tensor pipe in the steady state (0.34 us a K-step of a pair tile; the same MMAs on operands that stay in
+// shared memory, fp4_ceiling.cu, take 0.34 us at the 7.4 PFLOP/s they measure) and the board's power (1.36 - 1.57 GHz in a long
+// launch); per tile 0.65 us in which the pipe stands still, since TMEM has no room for a second 256-column accumulator beside the
+// scale slots.  Two things got it there:
+//   - issue.  From a lane-0 branch the descriptors of every MMA, scale copy and commit go to uniform registers one by one, and
+//     two issuing threads did not keep up with the pipe.  With warp-uniform control flow and an elected lane the issuers wait
+//     for operands instead.  Back to back, before -> now: 16384 x 4096 x 16384 382 -> 349 us (alone 372 -> 333: 6.6 PFLOP/s),
+//     16384 x 4096 x 4096 105 -> 97, 1024 x 1024 x 8192 16.2 -> 12.5.  One issuing warp without the baton: 376, 103, 16.5;
 //   - the hand-over.  Eight warps take the accumulator out unconverted, in place of four that had to convert the first
 //     half before reading the second, and for fp32 stored every 32 columns before reading the next: 16384 x 8192 x 2048
-//     bf16 125 -> 115 us, fp32 197 -> 143 (537 MB written: the store bounds it; a second staging buffer, stores without
-//     the evict-first hint, and 32-byte stores straight from the registers gained nothing).
+//     bf16 125 -> 115 us, fp32 197 -> 143 (537 MB written, but memory is not the bound: a fill of that buffer takes 74 us, the
+//     same product with K = 128 84, with K = 2048 135 on that box.  Per pair tile the fp32 stores take about 3.0 us and the MMAs
+//     2.7, and they overlap in part only; a second staging buffer, stores without the evict-first hint, and 32-byte stores
+//     straight from the registers gained nothing).
 // A 256 x 384 pair tile (two N = 192 MMAs from one A) was slower everywhere: 391 -> 414 us at K = 16384, 106 -> 115 at 4096
 // (before the issue change).
 //
 // The 8-bit products (FP8 forward pass, MXINT4; enum Kind) run on the same roles: a one-CTA kernel of 128 x 256 tiles with
 // one accumulator and stores from registers served them before.  E4M3 16384 x 4096 x 4096: 221 -> 168 us (3.3 PFLOP/s,
 // twice the measured bf16 rate), 8192 x 3072 x 1024 50 -> 23, 16 x 4096 x 4096 16.5 -> 11.4; MXINT4
-// 16384 x 4096 x 4096 245 -> 178, 1024 x 1024 x 8192 34 -> 20.
+// 16384 x 4096 x 4096 245 -> 178, 1024 x 1024 x 8192 34 -> 20.  It was the better one for few rows and many columns, where
+// half of every pair idles (16 x 20480 x 4096: E4M3 23 -> 28 us, MXINT4 23 -> 37; 16 x 65536 x 4096 58 -> 62).
 #include <cuda_bf16.h>
 
 #include <cstdlib>

@@ -43,20 +43,10 @@ __device__ __forceinline__ void sr_draws32(uint64_t seed, uint32_t stream_tag, u
     rw[4] = b.x; rw[5] = b.y; rw[6] = b.z; rw[7] = b.w;
 }
 
-// Same draws with the ten round keys expanded once per thread (they depend on the seed only).
+// Same draws with the ten round keys given (they depend on the seed only and come with the kernel's parameters).
 struct PhiloxKeys {
     uint32_t k0[10], k1[10];
 };
-__device__ __forceinline__ PhiloxKeys philox_expand_keys(uint64_t seed) {
-    PhiloxKeys ks;
-    uint32_t a = (uint32_t)seed, b = (uint32_t)(seed >> 32);
-#pragma unroll
-    for (int i = 0; i < 10; ++i) {
-        ks.k0[i] = a; ks.k1[i] = b;
-        a += 0x9E3779B9u; b += 0xBB67AE85u;
-    }
-    return ks;
-}
 __device__ __forceinline__ uint4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, const PhiloxKeys& ks) {
 #pragma unroll
     for (int i = 0; i < 10; ++i) {

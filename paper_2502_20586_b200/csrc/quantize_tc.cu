@@ -21,17 +21,17 @@
 //
 //   warp 0        TMA producer (two 64-column x 128-row boxes per tile, 128-byte swizzle, 4-stage ring)
 //   warp 1        MMA issuer (8 K=16 MMAs per tile into one of four 128-column TMEM accumulators)
-//   warps 2, 3    idle: they complete warp group 0, which hands registers (setmaxnreg) to the epilogue groups
+//   warps 2, 3    column sums of dY when a bias gradient is wanted, else idle; they complete warp group 0, which hands
+//                 registers (setmaxnreg) to the epilogue groups
 //   warps 4..15   epilogue, three groups of four warps on alternate tiles: warp = TMEM lane quadrant, a thread owns one
 //                 output row of the tile: tcgen05.ld 32 columns at a time, scale / SR / pack / store per MX block
 //                 (g = 256: four groups, warps 4..19)
 //
 // What bounds it: the rounding arithmetic of the epilogue warps (10 instructions per element), as long as the issuer
-// keeps up.  It did not: MMAs issued from a lane-0 branch cost 150 cycles each beside busy epilogue warps (descriptors
-// moved to uniform registers every time), 1200 of the 2100 cycles of a tile, and every epilogue warp waited a third of its
-// time for an accumulator.  Warp-uniform issue with one elected lane, 32-bit MX-block arithmetic per tile, two fp32 products
-// per instruction and three groups with a spare accumulator instead of four without one, 16384 x 16384 views, before ->
-// now: SR row-wise 140 -> 123 us, g = 64 133 -> 117, transposing 141 -> 139, g = 256 152 -> 132, SR16 131 -> 111 (6.1 TB/s),
+// keeps up.  It did not: MMAs issued from a lane-0 branch have their descriptors moved to uniform registers every time, and
+// every epilogue warp waited for an accumulator.  Warp-uniform issue with one elected lane, 32-bit MX-block arithmetic per
+// tile, two fp32 products per instruction and three groups with a spare accumulator instead of four without one,
+// 16384 x 16384 views, before -> now: SR row-wise 140 -> 123 us, g = 64 133 -> 117, transposing 141 -> 139, g = 256 152 -> 132, SR16 131 -> 111 (6.1 TB/s),
 // RN 112 -> 108; the operands of a backward call, 16384 x 4096 x 16384 341 -> 300, 8192 x 1024 x 4096 56 -> 48, 8192 x 1024
 // x 1024 18.6 -> 16.0.
 // Every mbarrier wait is bounded; on expiry the CTA records a status word and unwinds.
@@ -386,19 +386,18 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
         if (!ok && lane == 0) *abort_flag = 1;
     }
     } else {
-        // ------------------------------------------------------------------ epilogue (warp groups 1..4)
+        // ------------------------------------------------------------------ epilogue (the warp groups after the first)
         reg_alloc<Cfg::kRegsEpi>();
-        // Four groups of four warps take alternate tiles; inside a group a warp owns one TMEM lane quadrant, i.e. a
-        // thread owns one output row of the tile: four MX blocks, 64 bytes of codes, 4 scale bytes.  The SR draws of a
-        // block are computed while the block before it is rounded (for a tile's first block: at the end of the tile
-        // before); they depend only on element indices.
+        // Groups of four warps (FULL: three, four for g = 256; LITE: two) take alternate tiles or share them, see below; inside
+        // a group a warp owns one TMEM lane quadrant, i.e. a thread owns one output row of the tile: four MX blocks, 64 bytes of
+        // codes, 4 scale bytes.  The SR draws of a block are computed while the block before it is rounded (for a tile's first
+        // block: at the end of the tile before); they depend only on element indices.
         const int e = warp - 4;
         const int q = warp & 3;                      // TMEM lane quadrant this warp may read
         const int grp = e >> 2;
         const float cg = p.custom_t != nullptr ? 1.0f : p.g == 32 ? 0.17677669529663687f : p.g == 128 ? 0.08838834764831845f : 1.0f;
-        // FULL: the groups take alternate tiles.  LITE: both groups take every tile of the CTA, group 0 the row's MX
-        // blocks 0 and 1, group 1 blocks 2 and 3.
-        // A team takes every kTeams-th tile of the CTA.  FULL: a group is a team, a thread handles all four blocks of its row.
+        // A team takes every kTeams-th tile of the CTA.  FULL: a group is a team (g = 256: two groups are, one for each half of
+        // the 256-chunk), a thread handles all four blocks of its row.
         // LITE: the two groups share every tile, group 0 the row's MX blocks 0 and 1, group 1 blocks 2 and 3.
         constexpr int kTeams = KW == 2 ? 2 : LITE ? 1 : kEpiGroups;
         constexpr int kBlocksPerThread = LITE ? 2 : 4;
