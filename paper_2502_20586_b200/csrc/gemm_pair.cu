@@ -22,7 +22,7 @@
 // A-row scales are per CTA; every CTA needs the scales of all 256 B rows.
 //
 // What bounds it: the tensor pipe in the steady state (0.34 us a K-step of a pair tile; the same MMAs on operands that stay in
-// shared memory, fp4_ceiling.cu, take 0.34 us at the 7.4 PFLOP/s they measure) and the board's power (1.36 - 1.57 GHz in a long
+// shared memory, fp4_ceiling.cu, take 0.31 us in a burst, 0.35 sustained: 8.1 and 7.1 PFLOP/s) and the board's power (1.36 - 1.57 GHz in a long
 // launch); per tile 0.65 us in which the pipe stands still, since TMEM has no room for a second 256-column accumulator beside the
 // scale slots.  Two things got it there:
 //   - issue.  From a lane-0 branch the descriptors of every MMA, scale copy and commit go to uniform registers one by one, and

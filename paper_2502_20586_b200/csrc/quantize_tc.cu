@@ -27,7 +27,7 @@
 //                 output row of the tile: tcgen05.ld 32 columns at a time, scale / SR / pack / store per MX block
 //                 (g = 256: four groups, warps 4..19)
 //
-// What bounds it: the rounding arithmetic of the epilogue warps (10 instructions per element), as long as the issuer
+// What bounds it: the rounding arithmetic of the epilogue warps (9.4 instructions per element), as long as the issuer
 // keeps up.  It did not: MMAs issued from a lane-0 branch have their descriptors moved to uniform registers every time, and
 // every epilogue warp waited for an accumulator.  Warp-uniform issue with one elected lane, 32-bit MX-block arithmetic per
 // tile, two fp32 products per instruction and three groups with a spare accumulator instead of four without one,
