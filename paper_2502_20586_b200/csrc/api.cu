@@ -65,7 +65,7 @@ mxfp4_status runtime_init() {
         if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) st = MXFP4_ERR_CUDA;
         else if (major != 10) st = MXFP4_ERR_DEVICE;
         else if (mx::gemm_init() != cudaSuccess || mx::gemm_pair_init() != cudaSuccess || mx::quant_tc_init() != cudaSuccess ||
-                 mx::gemm_fused_init() != cudaSuccess)
+                 mx::gemm_fused_init() != cudaSuccess || mx::gemm_f8_init() != cudaSuccess)
             st = MXFP4_ERR_CUDA;
         g_rt.dev_status[dev] = st;
         g_rt.dev_done[dev] = true;
@@ -651,11 +651,15 @@ mxfp4_status gemm8_impl(const uint8_t* A, const uint8_t* B, const uint8_t* sfa, 
                         int64_t M, int64_t N, int64_t K, float alpha, void* C, int64_t ldc, int out_dtype, cudaStream_t stream) {
     mx::Gemm8Args a;
     a.block_scaled = sfa != nullptr;
-    a.scale_a = sa; a.scale_b = sb;
+    a.sfa = sfa; a.sfb = sfb; a.scale_a = sa; a.scale_b = sb;
     a.M = M; a.N = N; a.K = K; a.alpha = alpha; a.C = C; a.ldc = ldc; a.out_fp32 = out_dtype == MXFP4_OUT_FP32;
-    const int tile_n = mx::gemm_f8_tile_n(a);
     mxfp4_status st = make_bytes_map(&a.tmap_a, A, M, K, 128);
     if (st != MXFP4_OK) return st;
+    if (mx::gemm_f8_one_cta(a)) {
+        if ((st = make_bytes_map(&a.tmap_b, B, N, K, 256)) != MXFP4_OK) return st;
+        return cuda_status(mx::launch_gemm_f8_one_cta(a, stream), "8-bit GEMM launch (one CTA a tile)");
+    }
+    const int tile_n = mx::gemm_f8_tile_n(a);
     if ((st = make_bytes_map(&a.tmap_b, B, N, K, tile_n / 2)) != MXFP4_OK) return st;
     if (a.block_scaled) {
         if ((st = make_scales_map(&a.tmap_sfa, sfa, M, K, 1)) != MXFP4_OK) return st;
@@ -744,7 +748,7 @@ mxfp4_status mxfp4_device_status(void* cuda_stream) {
     if (cudaStreamSynchronize(static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess) return MXFP4_ERR_CUDA;
     unsigned int word = 0;
     cudaError_t (*const fetch[])(unsigned int*) = {mx::fetch_gemm_status, mx::fetch_gemm_pair_status, mx::fetch_quant_tc_status,
-                                                   mx::fetch_fp4_ceiling_status, mx::fetch_gemm_fused_status};
+                                                   mx::fetch_fp4_ceiling_status, mx::fetch_gemm_fused_status, mx::fetch_gemm_f8_status};
     for (auto f : fetch) {
         unsigned int w = 0;
         if (f(&w) != cudaSuccess) return MXFP4_ERR_CUDA;

@@ -41,8 +41,7 @@
 // The 8-bit products (FP8 forward pass, MXINT4; enum Kind) run on the same roles: a one-CTA kernel of 128 x 256 tiles with
 // one accumulator and stores from registers served them before.  E4M3 16384 x 4096 x 4096: 221 -> 168 us (3.3 PFLOP/s,
 // twice the measured bf16 rate), 8192 x 3072 x 1024 50 -> 23, 16 x 4096 x 4096 16.5 -> 11.4; MXINT4
-// 16384 x 4096 x 4096 245 -> 178, 1024 x 1024 x 8192 34 -> 20.  It was the better one for few rows and many columns, where
-// half of every pair idles (16 x 20480 x 4096: E4M3 23 -> 28 us, MXINT4 23 -> 37; 16 x 65536 x 4096 58 -> 62).
+// 16384 x 4096 x 4096 245 -> 178, 1024 x 1024 x 8192 34 -> 20.  It still serves few rows and many columns (gemm_f8.cu).
 #include <cuda_bf16.h>
 
 #include <cstdlib>

@@ -101,15 +101,17 @@ cudaError_t launch_gemm_fused(const FusedGemmArgs& a, cudaStream_t stream);
 cudaError_t gemm_fused_init();
 cudaError_t fetch_gemm_fused_status(unsigned int* word);
 
-// GEMM on 8-bit element containers (gemm_pair.cu): E4M3 operands with per-tensor scales (FP8 forward pass), or E4M3
+// GEMM on 8-bit element containers (gemm_pair.cu, and gemm_f8.cu for few rows and many columns): E4M3 operands with per-tensor scales (FP8 forward pass), or E4M3
 // containers of MXINT4 integers with one UE8M0 scale per 32 elements (native scale layout, K % 128 == 0).
 struct Gemm8Args {
     CUtensorMap tmap_a;   // bytes [M, K], box 128 B x 128 rows, 128-byte swizzle
-    CUtensorMap tmap_b;   // bytes [N, K], box 128 B x tile_n / 2 rows
-    CUtensorMap tmap_c;   // output, as in GemmArgs
+    CUtensorMap tmap_b;   // bytes [N, K], box 128 B x tile_n / 2 rows (one-CTA kernel: 256 rows)
+    CUtensorMap tmap_c;   // output, as in GemmArgs (pair kernel)
     bool block_scaled;
     CUtensorMap tmap_sfa; // block_scaled: scale tiles (native layout) as [row tiles * K tiles, 512 bytes], box = one tile
     CUtensorMap tmap_sfb;
+    const uint8_t* sfa;   // block_scaled: the same scales for the one-CTA kernel
+    const uint8_t* sfb;
     const float* scale_a; // plain: device pointers to the per-tensor scales; C = A B^T / (scale_a scale_b)
     const float* scale_b;
     int64_t M, N, K;
@@ -120,6 +122,10 @@ struct Gemm8Args {
 };
 int gemm_f8_tile_n(const Gemm8Args& a);            // from M, N, K
 cudaError_t launch_gemm_f8(const Gemm8Args& a, int tile_n, cudaStream_t stream);
+bool gemm_f8_one_cta(const Gemm8Args& a);          // from M, N: the one-CTA kernel is the better one
+cudaError_t launch_gemm_f8_one_cta(const Gemm8Args& a, cudaStream_t stream);
+cudaError_t gemm_f8_init();
+cudaError_t fetch_gemm_f8_status(unsigned int* word);
 
 // Element-wise kernels of the extensions (variants.cu).
 // Per-tensor E4M3 quantisation of one or two tensors: scale[0] = 448 / amax(x) (1 for an all-zero tensor), scale[1] = amax,

@@ -1,4 +1,4 @@
-// Element-wise kernels of the two extensions of the recipe (the GEMMs are in gemm_pair.cu):
+// Element-wise kernels of the two extensions of the recipe (the GEMMs are in gemm_pair.cu and gemm_f8.cu):
 //   - per-tensor E4M3 quantisation for the FP8 forward pass (Section 4.1; supplementary FP8 results);
 //   - MXINT4 elements (Section 3, opening remark): Algorithm 1 / 2 with 4-bit integers in place of E2M1.
 #include <cuda_bf16.h>

@@ -113,3 +113,33 @@ def test_pitch_of_a_single_row(gpu, ldc):
     assert gpu.lib().mxfp4_fp8_gemm(a.data_ptr(), one.data_ptr(), b.data_ptr(), one.data_ptr(), 1, 264, 256, got.data_ptr(), ldc, gpu.OUT_FP32,
                                     torch.cuda.current_stream().cuda_stream) == 0
     assert gpu.mxfp4_device_status() == 0 and torch.equal(got, want)
+
+
+# at most 128 rows: one column tile more than pairs is where the one-CTA kernel takes over; the same bits as the pairs give for
+# the halves of the columns
+@pytest.mark.parametrize("M,N,K", [(1, 18952, 128), (128, 18952, 256), (17, 37896, 384), (100, 75784, 128)])
+@pytest.mark.parametrize("kind", ["fp8", "int4"])
+@pytest.mark.parametrize("fp32", [False, True])
+def test_few_rows_and_many_columns(gpu, M, N, K, kind, fp32):
+    import torch
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(M + N + K)
+    out = gpu.OUT_FP32 if fp32 else gpu.OUT_BF16
+    a, b = ((torch.randn((rows, K), generator=gen, device="cuda") * 8).to(torch.float8_e4m3fn) for rows in (M, N))
+    if kind == "int4":
+        a, b = (t.float().clamp(-7, 7).round().to(torch.float8_e4m3fn) for t in (a, b))
+    ca, cb = a.view(torch.uint8), b.view(torch.uint8)
+    sa, sb = (_operand(gen, rows, K)[1] if kind == "int4" else torch.tensor([s, 0.0], device="cuda") for rows, s in ((M, 3.0), (N, 0.25)))
+    whole = torch.full((M, N + 8), float("nan"), dtype=torch.float32 if fp32 else torch.bfloat16, device="cuda")[:, :N]
+
+    def product(c0, c1, C):
+        if kind == "fp8":
+            return gpu.mxfp4_fp8_gemm(ca, sa, cb[c0:c1], sb, out, C_out=C)
+        return gpu.mxfp4_int4_gemm(ca, sa, cb[c0:c1], sb[c0 // 128 * (K // 128) * 512:], 1.0, out, C_out=C)
+
+    product(0, N, whole)
+    assert gpu.mxfp4_device_status() == 0
+    for c0 in range(0, N, 16384):
+        c1 = min(N, c0 + 16384)
+        assert torch.equal(whole[:, c0:c1], product(c0, c1, None))
+    assert gpu.mxfp4_device_status() == 0
