@@ -90,7 +90,8 @@ def _check(code: int):
 
 
 def _stream() -> int:
-    """Handle of the current stream of the current device, without building a Stream object around it (3.2 -> 0.3 us a call)."""
+    """Handle of the current stream of the current device, without building a Stream object around it (3.2 -> 0.3 us a call).
+    Both functions are private to torch: ``torch.cuda.current_stream().cuda_stream`` says the same."""
     if not torch.cuda.is_initialized():
         torch.cuda.init()
     return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
@@ -101,8 +102,8 @@ def _ptr(t) -> int:
 
 
 def _empty(like, shape, dtype):
-    """A plain tensor on the device of ``like``.  ``new_empty`` spares the device object (2.2 -> 1.7 us, timed on
-    CPU tensors), but returns a subclass for a subclass."""
+    """A plain tensor on the device of ``like``.  ``new_empty`` spares the device object (2.4 -> 1.9 us), but returns a
+    subclass for a subclass."""
     if type(like) is torch.Tensor:
         return like.new_empty(shape, dtype=dtype)
     return torch.empty(shape, dtype=dtype, device=like.device)
