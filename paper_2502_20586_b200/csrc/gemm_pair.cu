@@ -32,7 +32,7 @@
 //   - the hand-over.  Eight warps take the accumulator out unconverted, in place of four that had to convert the first
 //     half before reading the second, and for fp32 stored every 32 columns before reading the next: 16384 x 8192 x 2048
 //     bf16 125 -> 115 us, fp32 197 -> 143 (537 MB written, but memory is not the bound: a fill of that buffer takes 74 us, the
-//     same product with K = 128 84, with K = 2048 135 on that box.  Per pair tile the fp32 stores take about 3.0 us and the MMAs
+//     same product with K = 128 84, with K = 2048 135 beside them.  Per pair tile the fp32 stores take about 3.0 us and the MMAs
 //     2.7, and they overlap in part only; a second staging buffer, stores without the evict-first hint, and 32-byte stores
 //     straight from the registers gained nothing).
 // A 256 x 384 pair tile (two N = 192 MMAs from one A) was slower everywhere: 391 -> 414 us at K = 16384, 106 -> 115 at 4096
