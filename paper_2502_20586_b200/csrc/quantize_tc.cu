@@ -92,7 +92,7 @@ struct QParams {
     int n_views;
     uint32_t n_tiles;          // over all views
     int g, sf_native;
-    bool wide_stores;          // y_out (and MXINT4 codes) start on 32-byte boundaries
+    bool wide_stores;          // y_out and every view's codes start on 32-byte boundaries
     const uint16_t* custom_t;  // bf16 [g, g] row-major transform matrix given by the caller, or null (then diag(S) H_g / sqrt(g))
     uint64_t seed;
     float* col_sums;           // partial column sums [x rows / 128][x cols] of view 0's x in fp32 (bias gradient), or null
@@ -181,6 +181,19 @@ template <bool FOLD>
 __device__ __forceinline__ void view_draws32(const PhiloxKeys& ks, const QView& vw, uint32_t blk, uint32_t (&rw)[8]) {
     if (FOLD) sr_draws32_view(ks, vw.pv, blk, rw);
     else sr_draws32_block(ks, vw.stream_tag, blk, rw);
+}
+
+// Codes of block j of a thread's row: two blocks go out together, 32 bytes, a whole L2 sector where the operand starts on one.
+// A block at a time wrote every sector in two halves: 16384 x 16384 SR transposing 140 -> 124 us, row-wise 126 -> 124, RN 118.5 -> 105
+// (the memory's rate) and 109 -> 105; the operands of 16384 x 4096 x 16384 324 -> 308.
+__device__ __forceinline__ void store_codes(uint8_t* dst, int j, const uint32_t (&packed)[4], uint32_t (&kept)[4], bool wide) {
+    if ((j & 1) == 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) kept[i] = packed[i];
+    } else {
+        const uint32_t both[8] = {kept[0], kept[1], kept[2], kept[3], packed[0], packed[1], packed[2], packed[3]};
+        st_global_32B(dst + 16 * (j - 1), both, wide);
+    }
 }
 
 // KW = 128-wide k-tiles per entry of the tile list: 1, or 2 for g = 256 (a tile then spans one 256-chunk).
@@ -446,7 +459,7 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
                 if (!ok) break;
                 tc_fence_after_sync();
                 const uint32_t ta = tmem_base + ((uint32_t)(q * 32) << 16) + b0 * kTile;
-                uint32_t sb_all = 0;
+                uint32_t sb_all = 0, kept[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     uint32_t nx[8], packed[4], sb = 0;
@@ -478,7 +491,7 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
                         }
                     } else {
                         quantize_block32_rw<mode_rounding(MODE, KW)>(y, rw, packed, sb, p.pipe);
-                        if (live) *reinterpret_cast<uint4*>(code_dst + 16 * j) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+                        if (live) store_codes(code_dst, j, packed, kept, p.wide_stores);
                         sb_all |= sb << (8 * j);
                     }
                     if (mode_draws(MODE)) {
@@ -507,7 +520,7 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
             if (!ok) break;
             tc_fence_after_sync();
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + b * kTile + 32 * part;
-            uint32_t sb_all = 0;
+            uint32_t sb_all = 0, kept[4];
 #pragma unroll
             for (int j = 0; j < kBlocksPerThread; ++j) {
                 uint32_t raw[32], nx[8], packed[4], sb = 0;
@@ -542,7 +555,7 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
                     sb_all |= sb << (8 * j);
                 } else if constexpr (MODE != kModeDump) {
                     quantize_block32_rw<mode_rounding(MODE, KW)>(y, rw, packed, sb, p.pipe);
-                    if (live) *reinterpret_cast<uint4*>(code_dst + 16 * j) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+                    if (live) store_codes(code_dst, j, packed, kept, p.wide_stores);
                     sb_all |= sb << (8 * j);
                 }
                 if (mode_draws(MODE)) {
@@ -677,7 +690,9 @@ cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cud
     p.n_views = n;
     p.n_tiles = tiles;
     p.g = a[0].g; p.sf_native = a[0].sf_native; p.seed = a[0].seed;
-    p.wide_stores = ((reinterpret_cast<uintptr_t>(a[0].y_out) | (a[0].mxint4 ? reinterpret_cast<uintptr_t>(a[0].codes) : 0)) & 31u) == 0;
+    uintptr_t stores = reinterpret_cast<uintptr_t>(a[0].y_out);
+    for (int v = 0; v < n; ++v) stores |= reinterpret_cast<uintptr_t>(a[v].codes);
+    p.wide_stores = (stores & 31u) == 0;
     p.custom_t = static_cast<const uint16_t*>(a[0].custom_t);
     if (p.custom_t != nullptr && p.g == 256) return cudaErrorInvalidValue;
     // column sums: of view 0's tensor, read row-wise in whole 128-row bands
