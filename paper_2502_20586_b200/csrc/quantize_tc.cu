@@ -49,6 +49,20 @@ constexpr uint32_t kBoxBytes = 64 * 2 * 128;        // one TMA box: 64 bf16 colu
 constexpr uint32_t kTileBytes = 2 * kBoxBytes;      // 32 KB
 constexpr uint32_t kTBytes = 2 * kBoxBytes;         // transform matrix, 128 x 128 bf16
 
+// What the epilogue has to know of a tile.  The producer thread, which works out where the tile lies in any case, leaves it in
+// shared memory: each epilogue thread did the same arithmetic for every tile of its own.
+struct __align__(16) TileInfo {
+    uint8_t* codes;            // codes of the tile's first row
+    uint8_t* scales;           // native layout: the tile's 512 bytes; linear: scales of its first row
+    uint32_t blk;              // index in the view of the first row's first MX block
+    uint32_t k_blocks;         // MX blocks from one row to the next
+    uint32_t rows;             // rows of the tile that exist
+    uint32_t view;
+};
+// The producer is at most kStages tiles ahead of the MMA issuer and that one kAccBufs ahead of an epilogue group which has not
+// read its accumulator out: sixteen entries are never overwritten before they are read.
+constexpr uint32_t kInfoSlots = 16;
+
 // Two builds of the kernel.  FULL owns its SM: a 4-stage ring, four TMEM accumulators, three epilogue warp groups on
 // alternate tiles (g = 256: two teams of two groups, each with its pair of accumulators).  LITE is sized to run beside the small build of the pair GEMM (gemm_pair.cu) on the same SM, so that
 // the operands of one product are quantised while the other product's GEMM keeps the FP4 pipe busy: one 32 KB stage,
@@ -61,7 +75,9 @@ struct QCfg {
     static constexpr int kTmemCols = LITE ? 128 : 512;
     static constexpr int kEpiGroups = LITE ? 2 : KW == 2 ? 4 : 3;       // epilogue warp groups (one warp per TMEM lane quadrant)
     static constexpr int kEpiWarps = 4 * kEpiGroups;
-    static constexpr uint32_t kSmem = kStages * kTileBytes + (LITE ? 1 : 2) * kTBytes + 1024 + 256;   // FULL: two transform matrices for g = 256
+    static constexpr int kTransforms = KW;                               // g = 256: two half-transforms
+    static constexpr uint32_t kSmem = kStages * kTileBytes + kTransforms * kTBytes + kInfoSlots * (uint32_t)sizeof(TileInfo) + 1024 + 512;
+    static_assert((2 * kStages + 2 * kAccBufs + (int)kInfoSlots) * 8 + 8 <= 512, "barriers");
     // Register hand-over (setmaxnreg): warp group 0 shrinks to kRegsLight, the epilogue groups grow to kRegsEpi.  The
     // increase can only draw on what the CTA itself holds, i.e. threads x registers-per-thread at launch: the init
     // routine checks that budget against the compiled kernel, because an increase that cannot be met waits forever.
@@ -78,10 +94,8 @@ struct QView {                 // one operand view: output operand [R, K] read f
     uint32_t n_tiles;          // r_tiles * k_tiles
     uint32_t minor_count;      // tiles along the fast direction of the view's tile order (see locate_tile)
     uint32_t lg_band;          // log2 of the tiles across the fast direction that are walked side by side (TilePos)
-    uint32_t step, d_major, d_minor;   // an epilogue team's stride through the tile list, whole and split by minor_count
     int reduce_dim;            // 1: K runs along x columns (x tile is the K-major operand); 0: along x rows (MN-major)
     uint32_t stream_tag;
-    PhiloxViewConsts pv;       // index-independent part of the first three Philox rounds for this view's draws (operands < 2^36 elements)
     uint8_t* codes;
     uint8_t* scales;
     float* y_out;              // transform dump only
@@ -92,7 +106,7 @@ struct QParams {
     int n_views;
     uint32_t n_tiles;          // over all views
     int g, sf_native;
-    bool wide_stores;          // y_out and every view's codes start on 32-byte boundaries
+    bool wide_stores;          // y_out and the codes of every view start on 32-byte boundaries
     const uint16_t* custom_t;  // bf16 [g, g] row-major transform matrix given by the caller, or null (then diag(S) H_g / sqrt(g))
     uint64_t seed;
     float* col_sums;           // partial column sums [x rows / 128][x cols] of view 0's x in fp32 (bias gradient), or null
@@ -138,30 +152,17 @@ __device__ __forceinline__ uint32_t along_minor(const QView& vw, const TilePos& 
 __device__ __forceinline__ uint32_t across_minor(const QView& vw, const TilePos& pos) { return (pos.major << vw.lg_band) | (pos.minor & ((1u << vw.lg_band) - 1u)); }
 __device__ __forceinline__ uint32_t row_tile(const QView& vw, const TilePos& pos) { return vw.reduce_dim == 1 ? across_minor(vw, pos) : along_minor(vw, pos); }
 __device__ __forceinline__ uint32_t k_tile(const QView& vw, const TilePos& pos) { return vw.reduce_dim == 1 ? along_minor(vw, pos) : across_minor(vw, pos); }
-// The next tile of an epilogue team (t_next in the list; past its end: any valid position, not used): additions only
-// while the walk stays inside the view.
-template <bool DUAL>
-__device__ __forceinline__ TilePos advance_tile(const QParams& p, const TilePos& cur, uint32_t t_next) {
-    const QView& vw = p.view[cur.v];
-    TilePos pos = cur;
-    if (DUAL) {                               // three tiles on: one or two units, the other view
-        const uint32_t units = cur.v == 0 ? 1u : 2u;
-        pos.local += units * vw.step;
-        if (pos.local >= vw.n_tiles) return locate_tile<DUAL>(p, t_next < p.n_tiles ? t_next : 0u);
-        pos.v = 1 - cur.v;
-        for (uint32_t i = 0; i < units; ++i) {
-            pos.major += vw.d_major;
-            pos.minor += vw.d_minor;
-            if (pos.minor >= vw.minor_count) { pos.minor -= vw.minor_count; ++pos.major; }
-        }
-        return pos;
-    }
-    pos.local += vw.step;
-    if (pos.local >= vw.n_tiles) return locate_tile<DUAL>(p, t_next < p.n_tiles ? t_next : 0u);
-    pos.major += vw.d_major;
-    pos.minor += vw.d_minor;
-    if (pos.minor >= vw.minor_count) { pos.minor -= vw.minor_count; ++pos.major; }
-    return pos;
+template <int KW, bool INT4>
+__device__ __forceinline__ void describe_tile(const QParams& p, const TilePos& pos, TileInfo& out) {
+    const QView& vw = p.view[pos.v];
+    const uint32_t rt = row_tile(vw, pos), kt = k_tile(vw, pos) * KW;
+    const uint32_t blk = rt * (uint32_t)kTile * vw.k_blocks + kt * 4u;
+    out.codes = vw.codes + (uint64_t)blk * (INT4 ? 32u : 16u);
+    out.scales = vw.scales + (p.sf_native ? sf_row_offset(rt * ((vw.k_blocks + 3) >> 2) + kt, 0, 0) : (uint64_t)blk);
+    out.blk = blk;
+    out.k_blocks = vw.k_blocks;
+    out.rows = vw.R - rt * (uint32_t)kTile;
+    out.view = (uint32_t)pos.v;
 }
 
 // kModeInt4*: MXINT4 elements, one byte each, together with the transformed values that were rounded (g <= 128): what a pass
@@ -171,17 +172,8 @@ enum { kModeSR = 0, kModeRN = 1, kModeDump = 2, kModeSR16 = 3, kModeInt4SR = 4, 
 constexpr bool mode_draws(int mode) { return mode == kModeSR || mode == kModeSR16 || mode == kModeInt4SR; }
 constexpr bool mode_int4(int mode) { return mode == kModeInt4SR || mode == kModeInt4RN; }
 constexpr bool mode_keeps_y(int mode) { return mode == kModeDump || mode_int4(mode); }
-// template argument of quantize_block32_rw; the g = 256 kernel (kw = 2) rounds SR through the convert instruction (same codes, fewer registers)
-constexpr int mode_rounding(int mode, int kw) { return mode == kModeSR16 ? 2 : (mode == kModeSR && kw == 2) ? 3 : mode; }
-
-// The 32 draws of MX block `blk` (of the view: element index / 32).  FOLD: with the view's precomputed constants (fewer
-// instructions, five more live values: pays where registers are not the limit, i.e. in the SR16 kernel; the integer SR
-// path and the g = 256 kernel lose with it).
-template <bool FOLD>
-__device__ __forceinline__ void view_draws32(const PhiloxKeys& ks, const QView& vw, uint32_t blk, uint32_t (&rw)[8]) {
-    if (FOLD) sr_draws32_view(ks, vw.pv, blk, rw);
-    else sr_draws32_block(ks, vw.stream_tag, blk, rw);
-}
+// template argument of quantize_block32_rw
+constexpr int mode_rounding(int mode) { return mode == kModeSR16 ? 2 : mode; }
 
 // Codes of block j of a thread's row: two blocks go out together, 32 bytes, a whole L2 sector where the operand starts on one.
 // A block at a time wrote every sector in two halves: 16384 x 16384 SR transposing 140 -> 124 us, row-wise 126 -> 124, RN 118.5 -> 105
@@ -195,6 +187,8 @@ __device__ __forceinline__ void store_codes(uint8_t* dst, int j, const uint32_t 
         st_global_32B(dst + 16 * (j - 1), both, wide);
     }
 }
+// Tiles (units) that a round-robin deal of n gives this CTA.
+__device__ __forceinline__ uint32_t tiles_of_cta(uint32_t n) { return blockIdx.x < n ? (n - blockIdx.x + gridDim.x - 1u) / gridDim.x : 0u; }
 
 // KW = 128-wide k-tiles per entry of the tile list: 1, or 2 for g = 256 (a tile then spans one 256-chunk).
 template <int MODE, int KW, bool LITE, bool DUAL>
@@ -206,23 +200,25 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* smem_t = smem + kStagesQ * kTileBytes;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem_t + (LITE ? 1 : 2) * kTBytes);
+    TileInfo* info = reinterpret_cast<TileInfo*>(smem_t + Cfg::kTransforms * kTBytes);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(info + kInfoSlots);
     uint64_t* full_bar = bars;                          // [kStagesQ]  TMA -> MMA
     uint64_t* empty_bar = bars + kStagesQ;              // [kStagesQ]  MMA -> TMA
     uint64_t* acc_full = bars + 2 * kStagesQ;           // [kAccBufs]  MMA -> epilogue
     uint64_t* acc_empty = bars + 2 * kStagesQ + kAccBufs;   // [kAccBufs]  epilogue -> MMA
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStagesQ + 2 * kAccBufs);
+    uint64_t* info_full = acc_empty + kAccBufs;         // [kInfoSlots] producer -> epilogue
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(info_full + kInfoSlots);
     volatile uint32_t* abort_flag = tmem_slot + 1;
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp-uniform, and known to be)
     const uint32_t num_tiles = p.n_tiles;
-    constexpr bool kFold = MODE == kModeSR16 && KW == 1;
 
     if (threadIdx.x == 0) {
         // a stage is free when its transforms have read it (one commit) and, with column sums on, the two summing warps too
         const uint32_t n_readers = (KW == 1 && !LITE && p.col_sums != nullptr) ? 3u : 1u;
         for (int s = 0; s < kStagesQ; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], n_readers); }
         for (int b = 0; b < kAccBufs; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], (KW == 2 || LITE) ? 8 : 4); }
+        for (uint32_t i = 0; i < kInfoSlots; ++i) mbar_init(&info_full[i], 1);
         *abort_flag = 0;
         mbar_fence_init();
         for (int v = 0; v < p.n_views; ++v) prefetch_tensormap(&maps.x[v]);
@@ -276,11 +272,11 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
         if (lane == 0) {
-            uint32_t it = 0;
+            uint32_t it = 0, n_info = 0;
             bool ok = true;
             // DUAL: one load per unit (two logical tiles), in the coordinates of its row-wise view
             for (uint32_t t = DUAL ? 2u * blockIdx.x : blockIdx.x; t < num_tiles && ok; t += (DUAL ? 2u : 1u) * gridDim.x) {
-                const TilePos pos = locate_tile<DUAL>(p, t);
+                TilePos pos = locate_tile<DUAL>(p, t);
                 // x coordinates: (column, row).  reduce_dim 1: output rows = x rows, k = x columns; else swapped.
                 const bool rowwise = p.view[pos.v].reduce_dim == 1;
 #pragma unroll
@@ -293,6 +289,13 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
                     mbar_expect_tx(&full_bar[s], kTileBytes);
                     tma_load_2d(st, &maps.x[pos.v], &full_bar[s], cx, cy);
                     tma_load_2d(st + kBoxBytes, &maps.x[pos.v], &full_bar[s], cx + 64, cy);
+                }
+                if (!ok) break;
+#pragma unroll
+                for (int h = 0; h < (DUAL ? 2 : 1); ++h, ++n_info) {
+                    if (DUAL) pos.v = h;
+                    describe_tile<KW, mode_int4(MODE)>(p, pos, info[n_info % kInfoSlots]);
+                    mbar_arrive(&info_full[n_info % kInfoSlots]);
                 }
             }
             if (!ok) *abort_flag = 1;
@@ -403,8 +406,8 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
         reg_alloc<Cfg::kRegsEpi>();
         // Groups of four warps (FULL: three, four for g = 256; LITE: two) take alternate tiles or share them, see below; inside
         // a group a warp owns one TMEM lane quadrant, i.e. a thread owns one output row of the tile: four MX blocks, 64 bytes of
-        // codes, 4 scale bytes.  The SR draws of a block are computed while the block before it is rounded (for a tile's first
-        // block: at the end of the tile before); they depend only on element indices.
+        // codes, 4 scale bytes.  The SR draws of a block depend on element indices only and are computed while the accumulator is
+        // on its way to the registers.
         const int e = warp - 4;
         const int q = warp & 3;                      // TMEM lane quadrant this warp may read
         const int grp = e >> 2;
@@ -416,50 +419,36 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
         constexpr int kBlocksPerThread = LITE ? 2 : 4;
         const uint32_t part = KW == 2 ? 4u * (grp & 1) : LITE ? 2u * grp : 0u;    // first MX block of the row this thread handles
         const uint32_t lane_row = (uint32_t)(q * 32 + lane);
+        const uint32_t scale_off = (uint32_t)sf_row_offset(KW == 2 ? grp & 1 : 0, q, lane) + (KW == 2 ? 0u : part);   // native layout, from the tile's first byte
         bool ok = true;
+        auto wait = [&](uint64_t* bar, uint32_t parity) { return ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)); };
 
-        auto first_block = [&](const TilePos& pos) -> uint32_t {         // index of this thread's first MX block
-            const QView& vw = p.view[pos.v];
-            return (row_tile(vw, pos) * (uint32_t)kTile + lane_row) * vw.k_blocks + k_tile(vw, pos) * (4u * KW) + part;
-        };
-
-        // logical tile of this CTA's i-th accumulator: tiles are dealt out round-robin; in a DUAL launch whole units are
-        // (two consecutive logical tiles, one per view), so that both transforms of a unit read the same stage
-        auto tile_of = [&](uint32_t i) -> uint32_t {
-            return DUAL ? 2u * (blockIdx.x + (i >> 1) * gridDim.x) + (i & 1u) : blockIdx.x + i * gridDim.x;
-        };
-        uint32_t it = KW == 2 ? (uint32_t)(grp >> 1) : LITE ? 0u : (uint32_t)grp;
-        uint32_t t = tile_of(it);
-        TilePos pos = locate_tile<DUAL>(p, t < num_tiles ? t : 0u);
-        uint32_t blk = first_block(pos);
-        uint32_t rw[8];
-        if (mode_draws(MODE)) view_draws32<kFold>(p.keys, p.view[pos.v], blk, rw);
-        if (KW == 2) {
-            // g = 256: a tile is one 256-chunk of 128 rows; its two k-tiles went through T_0 and T_1 into the accumulator
-            // pair (b0, b0 + 1): u = A_lo T_0, v = A_hi T_1.  The transformed values are y[0..127] = u + v and
-            // y[128..255] = u - v (H_256 = [[H, H], [H, -H]]).  Tiles alternate between the two accumulator pairs; pair
-            // pr is drained by groups 2 pr (the u + v half) and 2 pr + 1 (the u - v half), so every barrier is used by
-            // the same warps each time and its phases alternate for them.
-            const int pr = grp >> 1, hh = grp & 1;
-            for (; t < num_tiles; it += kTeams, t = tile_of(it)) {
-                const int b0 = 2 * pr;
-                const QView& vw = p.view[pos.v];
-                const uint32_t rt = row_tile(vw, pos), kt = k_tile(vw, pos);
-                const bool live = rt * kTile + lane_row < vw.R;
-                const uint32_t blk_cur = blk;
-                uint8_t* code_dst = vw.codes + (uint64_t)blk_cur * 16u;
-                uint8_t* scale_dst = vw.scales + (p.sf_native ? sf_row_offset(rt * ((vw.k_blocks + 3) >> 2) + 2 * kt + hh, q, lane) : blk_cur);
-                float* y_dst = MODE == kModeDump ? vw.y_out + (uint64_t)blk_cur * 32u : nullptr;
-                pos = advance_tile<DUAL>(p, pos, tile_of(it + kTeams));
-                blk = first_block(pos);
-                const QView& vw_next = p.view[pos.v];
+        // i-th accumulator of the CTA.  Tiles are dealt out round-robin; in a DUAL launch whole units are (two consecutive tiles,
+        // one per view), so that both transforms of a unit read the same stage.
+        const uint32_t n_mine = DUAL ? 2u * tiles_of_cta(num_tiles >> 1) : tiles_of_cta(num_tiles);
+        for (uint32_t it = KW == 2 ? (uint32_t)(grp >> 1) : LITE ? 0u : (uint32_t)grp; it < n_mine; it += kTeams) {
+            if (!wait(&info_full[it % kInfoSlots], (it / kInfoSlots) & 1)) break;
+            const TileInfo ti = info[it % kInfoSlots];
+            const QView& vw = p.view[ti.view];
+            const bool live = lane_row < ti.rows;
+            const uint32_t row_blk = lane_row * ti.k_blocks + part, blk = ti.blk + row_blk;   // this thread's first MX block
+            uint8_t* code_dst = ti.codes + (uint64_t)row_blk * (mode_int4(MODE) ? 32u : 16u);
+            uint8_t* scale_dst = ti.scales + (p.sf_native ? scale_off : row_blk);
+            float* y_dst = mode_keeps_y(MODE) ? vw.y_out + (uint64_t)blk * 32u : nullptr;
+            uint32_t sb_all = 0, kept[4];
+            if constexpr (KW == 2) {
+                // g = 256: a tile is one 256-chunk of 128 rows; its two k-tiles went through T_0 and T_1 into the accumulator
+                // pair (b0, b0 + 1): u = A_lo T_0, v = A_hi T_1.  The transformed values are y[0..127] = u + v and
+                // y[128..255] = u - v (H_256 = [[H, H], [H, -H]]).  Tiles alternate between the two accumulator pairs; pair
+                // pr is drained by groups 2 pr (the u + v half) and 2 pr + 1 (the u - v half), so every barrier is used by
+                // the same warps each time and its phases alternate for them.
+                const int b0 = 2 * (grp >> 1), hh = grp & 1;
                 const uint32_t ph = (it >> 1) & 1;                               // this pair's (it / 2)-th use
-                ok = mbar_wait(&acc_full[b0], ph, abort_flag) && mbar_wait(&acc_full[b0 + 1], ph, abort_flag);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
+                uint32_t rw[8];
+                if (mode_draws(MODE)) sr_draws32_block(p.keys, vw.stream_tag, blk, rw);
+                if (!wait(&acc_full[b0], ph) || !wait(&acc_full[b0 + 1], ph)) break;
                 tc_fence_after_sync();
                 const uint32_t ta = tmem_base + ((uint32_t)(q * 32) << 16) + b0 * kTile;
-                uint32_t sb_all = 0, kept[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     uint32_t nx[8], packed[4], sb = 0;
@@ -479,10 +468,7 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
                         __syncwarp();
                         if (lane == 0) { mbar_arrive(&acc_empty[b0]); mbar_arrive(&acc_empty[b0 + 1]); }
                     }
-                    if (mode_draws(MODE)) {
-                        if (j < 3) view_draws32<kFold>(p.keys, vw, blk_cur + (j + 1), nx);
-                        else view_draws32<kFold>(p.keys, vw_next, blk, nx);
-                    }
+                    if (mode_draws(MODE) && j < 3) sr_draws32_block(p.keys, vw.stream_tag, blk + (j + 1), nx);   // beside the rounding of this block
                     if (MODE == kModeDump) {
                         if (live) {
                             float4* dst = reinterpret_cast<float4*>(y_dst + 32 * j);
@@ -490,84 +476,64 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
                             for (int i = 0; i < 8; ++i) dst[i] = make_float4(y[4 * i], y[4 * i + 1], y[4 * i + 2], y[4 * i + 3]);
                         }
                     } else {
-                        quantize_block32_rw<mode_rounding(MODE, KW)>(y, rw, packed, sb, p.pipe);
+                        quantize_block32_rw<mode_rounding(MODE)>(y, rw, packed, sb, p.pipe);
                         if (live) store_codes(code_dst, j, packed, kept, p.wide_stores);
                         sb_all |= sb << (8 * j);
                     }
-                    if (mode_draws(MODE)) {
+                    if (mode_draws(MODE) && j < 3) {
 #pragma unroll
                         for (int i = 0; i < 8; ++i) rw[i] = nx[i];
                     }
                 }
                 if (MODE != kModeDump && live) *reinterpret_cast<uint32_t*>(scale_dst) = sb_all;
-            }
-        } else
-        for (; t < num_tiles; it += kTeams, t = tile_of(it)) {
-            const int b = it % kAccBufs;
-            const QView& vw = p.view[pos.v];
-            const uint32_t rt = row_tile(vw, pos), kt = k_tile(vw, pos);
-            const bool live = rt * kTile + lane_row < vw.R;
-            const uint32_t blk_cur = blk;
-            uint8_t* code_dst = vw.codes + (uint64_t)blk_cur * (mode_int4(MODE) ? 32u : 16u);
-            uint8_t* scale_dst = vw.scales + (p.sf_native ? sf_row_offset(rt * ((vw.k_blocks + 3) >> 2) + kt, q, lane) + part : blk_cur);
-            float* y_dst = mode_keeps_y(MODE) ? vw.y_out + (uint64_t)blk_cur * 32u : nullptr;
-            // position of the next tile of this team (past the end: computed but not used)
-            pos = advance_tile<DUAL>(p, pos, tile_of(it + kTeams));
-            blk = first_block(pos);
-            const QView& vw_next = p.view[pos.v];
-            ok = mbar_wait(&acc_full[b], (it / kAccBufs) & 1, abort_flag);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            tc_fence_after_sync();
-            const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + b * kTile + 32 * part;
-            uint32_t sb_all = 0, kept[4];
+            } else {
+                const int b = it % kAccBufs;
+                if (!wait(&acc_full[b], (it / kAccBufs) & 1)) break;
+                tc_fence_after_sync();
+                const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + b * kTile + 32 * part;
 #pragma unroll
-            for (int j = 0; j < kBlocksPerThread; ++j) {
-                uint32_t raw[32], nx[8], packed[4], sb = 0;
-                float y[32];
-                tmem_ld_32x32b_x32(taddr + 32 * j, raw);
-                if (mode_draws(MODE)) {                         // while the load is under way
-                    if (j < kBlocksPerThread - 1) view_draws32<kFold>(p.keys, vw, blk_cur + (j + 1), nx);
-                    else view_draws32<kFold>(p.keys, vw_next, blk, nx);
-                    tmem_ld_wait_after(nx);
-                } else {
-                    tmem_ld_wait();
-                }
-                if (j == kBlocksPerThread - 1) {                // the accumulator is free once it has been read
-                    tc_fence_before_sync();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&acc_empty[b]);
-                }
+                for (int j = 0; j < kBlocksPerThread; ++j) {
+                    uint32_t raw[32], rw[8], packed[4], sb = 0;
+                    float y[32];
+                    tmem_ld_32x32b_x32(taddr + 32 * j, raw);
+                    if (mode_draws(MODE)) {                         // while the load is under way
+                        sr_draws32_block(p.keys, vw.stream_tag, blk + j, rw);
+                        tmem_ld_wait_after(rw);
+                    } else {
+                        tmem_ld_wait();
+                    }
+                    if (j == kBlocksPerThread - 1) {                // the accumulator is free once it has been read
+                        tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&acc_empty[b]);
+                    }
 #pragma unroll
-                for (int i = 0; i < 32; ++i) y[i] = __uint_as_float(raw[i]);
-                if (cg != 1.0f) {                               // g = 32, 128: 1/sqrt(g) is not a power of two (for g = 64 it is folded into T)
+                    for (int i = 0; i < 32; ++i) y[i] = __uint_as_float(raw[i]);
+                    if (cg != 1.0f) {                               // g = 32, 128: 1/sqrt(g) is not a power of two (for g = 64 it is folded into T)
 #pragma unroll
-                    for (int i = 0; i < 32; i += 2) mul2_rn(y[i], y[i + 1], cg, y[i], y[i + 1]);
-                }
-                if (mode_keeps_y(MODE) && live) {
+                        for (int i = 0; i < 32; i += 2) mul2_rn(y[i], y[i + 1], cg, y[i], y[i + 1]);
+                    }
+                    if (mode_keeps_y(MODE) && live) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) st_global_32B(y_dst + 32 * j + 8 * i, reinterpret_cast<const uint32_t*>(y) + 8 * i, p.wide_stores);
+                        for (int i = 0; i < 4; ++i) st_global_32B(y_dst + 32 * j + 8 * i, reinterpret_cast<const uint32_t*>(y) + 8 * i, p.wide_stores);
+                    }
+                    if constexpr (mode_int4(MODE)) {
+                        uint32_t bytes[8];
+                        quantize_block32_int4<MODE == kModeInt4SR>(y, rw, bytes, sb);
+                        if (live) st_global_32B(code_dst + 32 * j, bytes, p.wide_stores);
+                        sb_all |= sb << (8 * j);
+                    } else if constexpr (MODE != kModeDump) {
+                        quantize_block32_rw<mode_rounding(MODE)>(y, rw, packed, sb, p.pipe);
+                        if (live) store_codes(code_dst, j, packed, kept, p.wide_stores);
+                        sb_all |= sb << (8 * j);
+                    }
                 }
-                if constexpr (mode_int4(MODE)) {
-                    uint32_t bytes[8];
-                    quantize_block32_int4<MODE == kModeInt4SR>(y, rw, bytes, sb);
-                    if (live) st_global_32B(code_dst + 32 * j, bytes, p.wide_stores);
-                    sb_all |= sb << (8 * j);
-                } else if constexpr (MODE != kModeDump) {
-                    quantize_block32_rw<mode_rounding(MODE, KW)>(y, rw, packed, sb, p.pipe);
-                    if (live) store_codes(code_dst, j, packed, kept, p.wide_stores);
-                    sb_all |= sb << (8 * j);
+                if (MODE != kModeDump && (live || mode_int4(MODE))) {   // (MXINT4: rows that only fill the last tile are zero)
+                    if (mode_int4(MODE) && !live) sb_all = 0;
+                    // this thread's two or four consecutive bytes, in either scale layout
+                    if (LITE) *reinterpret_cast<uint16_t*>(scale_dst) = (uint16_t)sb_all;
+                    else *reinterpret_cast<uint32_t*>(scale_dst) = sb_all;
                 }
-                if (mode_draws(MODE)) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) rw[i] = nx[i];
-                }
-            }
-            if (MODE != kModeDump && (live || mode_int4(MODE))) {   // (MXINT4: rows that only fill the last tile are zero)
-                if (mode_int4(MODE) && !live) sb_all = 0;
-                // this thread's two or four consecutive bytes, in either scale layout
-                if (LITE) *reinterpret_cast<uint16_t*>(scale_dst) = (uint16_t)sb_all;
-                else *reinterpret_cast<uint32_t*>(scale_dst) = sb_all;
             }
         }
         if (!ok && lane == 0) *abort_flag = 1;
@@ -706,7 +672,6 @@ cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cud
             k0 += 0x9E3779B9u; k1 += 0xBB67AE85u;
         }
     }
-    for (int v = 0; v < kQuantMaxViews; ++v) p.view[v].pv = philox_view_consts(p.keys, p.view[v].stream_tag);
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -720,10 +685,6 @@ cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cud
         const uint32_t across = w.reduce_dim == 1 ? w.r_tiles : w.k_tiles;
         if (dual || w.reduce_dim == 0) while (w.lg_band < 2 && (across >> w.lg_band) % 2 == 0) ++w.lg_band;
         w.minor_count = (w.reduce_dim == 1 ? w.k_tiles : w.r_tiles) << w.lg_band;
-        // an epilogue team's stride (kTeams tiles of its CTA; DUAL: one unit, see advance_tile)
-        w.step = (lite || dual ? 1u : p.g == 256 ? 2u : (uint32_t)QCfg<false, 1>::kEpiGroups) * grid;
-        w.d_major = w.step / w.minor_count;
-        w.d_minor = w.step % w.minor_count;
         if (dual) w.n_tiles = units;
     }
     const bool wide = p.g == 256, mxint4 = a[0].mxint4;
@@ -738,7 +699,7 @@ cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cud
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid); cfg.stream = stream;
     cfg.blockDim = dim3(lite ? LiteQCfg::kThreads : wide ? QCfg<false, 2>::kThreads : QCfg<false, 1>::kThreads);
-    cfg.dynamicSmemBytes = lite ? LiteQCfg::kSmem : QCfg<false, 1>::kSmem;
+    cfg.dynamicSmemBytes = lite ? LiteQCfg::kSmem : wide ? QCfg<false, 2>::kSmem : QCfg<false, 1>::kSmem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
