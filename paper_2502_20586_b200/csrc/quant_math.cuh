@@ -106,19 +106,23 @@ __device__ __forceinline__ float inv_sqrt_g(int g) {
 
 // ---------------------------------------------------------------- transform operand of the tensor-core RHT
 // bf16 entry (n, k) of the transform operand, stored N x K (K-major): T[k][n] = S_k H_g[k][n] inside a g-chunk.
-// g = 256 (Sylvester: H_256 = [[H_128, H_128], [H_128, -H_128]]): entry (n, k) of the half-transform h, T_h[k][n] =
-// S_{128 h + k} H_128[k][n] / 16; the epilogue combines u = A_lo T_0 and v = A_hi T_1 into u + v and u - v.
-__device__ __forceinline__ uint32_t transform_entry_256(int n, int k, const uint32_t (&sign)[4]) {
-    const uint32_t neg = ((sign[k >> 5] >> (k & 31)) ^ (uint32_t)__popc(k & n)) & 1u;
-    return 0x3D80u | (neg << 15);                                         // 1/16 = exact 1/sqrt(256)
-}
-
 __device__ __forceinline__ uint32_t transform_entry(int n, int k, int g, const uint32_t (&sign)[4]) {
     if ((n ^ k) & ~(g - 1)) return 0u;                                   // different g-chunks
     const int kk = k & (g - 1);
     const uint32_t neg = ((sign[kk >> 5] >> (kk & 31)) ^ (uint32_t)__popc(k & n & (g - 1))) & 1u;
     const uint32_t mag = g == 64 ? 0x3E00u : 0x3F80u;                    // 1/8 (exact 1/sqrt(64)) or 1
     return mag | (neg << 15);
+}
+// Eight entries of a row at once, k = 8 c .. 8 c + 7 of row n of diag(S) H (g <= 128, or a half-transform of g = 256: H_256 =
+// [[H_128, H_128], [H_128, -H_128]], T_h[k][n] = S_{128 h + k} H_128[k][n] / 16; the epilogue combines u = A_lo T_0 and v = A_hi T_1
+// into u + v and u - v).  The signs are one byte: (-1)^popc(k & n) for k's low three bits is a Walsh pattern of n's, the rest
+// of k flips all eight or none, S flips each.  `mag`: the bf16 magnitude, twice.  An entry at a time took each quantiser launch a microsecond.
+__device__ __forceinline__ void hadamard_row8(int n, int c, const uint4& sign, uint32_t mag, uint32_t (&w)[4]) {
+    const uint32_t lo = (c & 4) ? sign.y : sign.x, hi = (c & 4) ? sign.w : sign.z;
+    uint32_t neg = ((c & 8) ? hi : lo) >> (8 * (c & 3));
+    neg ^= ((n & 1) ? 0xAAu : 0u) ^ ((n & 2) ? 0xCCu : 0u) ^ ((n & 4) ? 0xF0u : 0u) ^ ((__popc((c << 3) & n) & 1) ? 0xFFu : 0u);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) w[j] = mag | ((neg << (15 - 2 * j)) & 0x8000u) | ((neg << (30 - 2 * j)) & 0x80000000u);
 }
 
 // ---------------------------------------------------------------- scale rule and encoders

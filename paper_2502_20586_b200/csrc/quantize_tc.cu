@@ -230,28 +230,24 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
     {
         if (KW == 1 && p.custom_t != nullptr) pdl_wait();                // the matrix may come from the kernel before this one
         // Transform operand, written in the 128-byte-swizzled K-major layout the MMA descriptor expects:
-        // entry (n, k) at box (k / 64), row n (128 B pitch), 16-byte chunk ((k % 64) / 8) ^ (n % 8).
+        // entry (n, k) at box (k / 64), row n (128 B pitch), 16-byte chunk ((k % 64) / 8) ^ (n % 8).  Only the g x g block at the
+        // origin is read (g = 256: the two 128 x 128 half-transforms).
+        const int lg_c = p.g == 32 ? 2 : p.g == 64 ? 3 : 4;                  // chunks of eight k to a row: 2^lg_c
 #pragma unroll
         for (int h = 0; h < KW; ++h) {                                   // KW = 2: sign bits 128 h .. 128 h + 127 come from Philox call h
-            const uint4 o = philox4x32_10((uint32_t)h, 0u, 0u, 0u, (uint32_t)p.seed, (uint32_t)(p.seed >> 32));
-            const uint32_t sign[4] = {o.x, o.y, o.z, o.w};
-            for (int task = threadIdx.x; task < 128 * 16; task += kThreadsQ) {
-                const int n = task >> 4, c = task & 15;                  // c: 16-byte chunk = 8 consecutive k
+            const uint4 sign = philox4x32_10((uint32_t)h, 0u, 0u, 0u, (uint32_t)p.seed, (uint32_t)(p.seed >> 32));
+            const uint32_t mag = KW == 2 ? 0x3D803D80u : p.g == 64 ? 0x3E003E00u : 0x3F803F80u;    // 1/16, 1/8: exact 1/sqrt(g); else 1
+            for (int task = threadIdx.x; task < 8 << (2 * lg_c); task += kThreadsQ) {
+                const int n = task >> lg_c, c = task & ((1 << lg_c) - 1);
                 uint32_t w[4];
+                if (KW == 1 && p.custom_t != nullptr) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int k0 = c * 8 + 2 * j;
-                    if (KW == 1 && p.custom_t != nullptr) {
-                        // entry (n, k) of the operand = T[k % g][n % g] inside a g-chunk, 0 across chunks (Section 3.2: any orthogonal matrix)
-                        const int gm = p.g - 1;
-                        const bool same = ((n ^ k0) & ~gm) == 0;              // k0 and k0 + 1 lie in the same chunk (g is even)
-                        const uint32_t lo = same ? p.custom_t[(k0 & gm) * p.g + (n & gm)] : 0u;
-                        const uint32_t hi = same ? p.custom_t[((k0 + 1) & gm) * p.g + (n & gm)] : 0u;
-                        w[j] = lo | (hi << 16);
-                    } else {
-                        w[j] = KW == 2 ? (transform_entry_256(n, k0, sign) | (transform_entry_256(n, k0 + 1, sign) << 16))
-                                       : (transform_entry(n, k0, p.g, sign) | (transform_entry(n, k0 + 1, p.g, sign) << 16));
+                    for (int j = 0; j < 4; ++j) {                        // entry (n, k) of the operand = T[k][n] (Section 3.2: any orthogonal matrix)
+                        const int k = c * 8 + 2 * j;
+                        w[j] = p.custom_t[k * p.g + n] | ((uint32_t)p.custom_t[(k + 1) * p.g + n] << 16);
                     }
+                } else {
+                    hadamard_row8(n, c, sign, mag, w);
                 }
                 const uint32_t off = (uint32_t)(c >> 3) * kBoxBytes + (uint32_t)n * 128u + (uint32_t)(((c & 7) ^ (n & 7)) << 4);
                 *reinterpret_cast<uint4*>(smem_t + h * kTBytes + off) = make_uint4(w[0], w[1], w[2], w[3]);
