@@ -178,9 +178,11 @@ __device__ __forceinline__ void tc_mma_mxf8_pair(uint32_t d_tmem, uint64_t a_des
         : "memory");
 }
 
-template <Kind KIND, bool LITE, int PN>
+// SPLIT: two pairs of a 4-CTA cluster share ONE output tile, each with half of its K-steps (see split_pays and the epilogue).
+template <Kind KIND, bool LITE, int PN, bool SPLIT = false>
 __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP& p) {
     using Cfg = PairCfg<KIND, LITE, PN>;
+    static_assert(!SPLIT || (PN == 128 && KIND != kMxf4), "split products: 8-bit kinds, 128-wide tiles");
     constexpr int kStagesP = Cfg::kStages, kAccBufs = Cfg::kAccBufs;
     constexpr uint32_t kStageB = Cfg::kStageB, kSfSlotB = Cfg::kSfSlotB;
     extern __shared__ uint8_t smem_raw[];
@@ -197,8 +199,13 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
     volatile uint32_t* abort_flag = tmem_slot + 2;
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp-uniform, and known to be)
-    const uint32_t rank = cluster_ctarank();                // 0 = leader
-    const TileWalk walk(p, (int)(blockIdx.x >> 1), (int)(gridDim.x >> 1));
+    const uint32_t rank = cluster_ctarank() & 1u;           // in the pair: 0 = leader
+    const uint32_t half_k = SPLIT ? cluster_ctarank() >> 1 : 0u;                 // this pair's half of the K-steps
+    constexpr int kLgCtas = SPLIT ? 2 : 1;
+    const TileWalk walk(p, (int)(blockIdx.x >> kLgCtas), (int)(gridDim.x >> kLgCtas));
+    // K-steps of a tile that are this pair's: all of them, or the first or second half
+    auto first_step = [&](int num_kt) { return SPLIT && half_k != 0 ? (num_kt + 1) >> 1 : 0; };
+    auto end_step = [&](int num_kt) { return SPLIT && half_k == 0 ? (num_kt + 1) >> 1 : num_kt; };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStagesP; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
@@ -249,10 +256,10 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
             for (uint32_t tl = 0; tl < walk.count && ok; ++tl) {
                 int mt, nt;
                 const int w = walk.locate(p, tl, mt, nt);
-                const int num_kt = p.prob[w].num_kt;
+                const int end_kt = end_step(p.prob[w].num_kt);
                 const CUtensorMap *map_a = &maps.a[w], *map_b = &maps.b[w];
                 const int a_rt = 2 * mt + (int)rank;                            // this CTA's 128-row tile of A
-                for (int kt = 0; kt < num_kt; ++kt, ++it) {
+                for (int kt = first_step(p.prob[w].num_kt); kt < end_kt; ++kt, ++it) {
                     const int s = it % kStagesP;
                     if (!(ok = mbar_wait(&empty_bar[s], ((it / kStagesP) & 1) ^ 1, abort_flag))) break;
                     uint8_t* st = smem + s * kStageB;
@@ -280,7 +287,10 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
             const uint32_t a_lo0 = (uint32_t)desc0;
             const uint32_t me = warp == 1 ? 0u : 1u;
             uint32_t s = me % kStagesP, ph = 0, tile_i = 0, n = 0;
-            auto steps_of = [&](uint32_t tile) { return p.prob[(int)tile < walk.n_first ? 0 : 1].num_kt; };
+            auto steps_of = [&](uint32_t tile) {
+                const int all = p.prob[(int)tile < walk.n_first ? 0 : 1].num_kt;
+                return end_step(all) - first_step(all);
+            };
             int kt = (int)me, num_kt = steps_of(0);
             while (tile_i < walk.count && kt >= num_kt) { kt -= num_kt; num_kt = steps_of(++tile_i); }
             bool ok = true;
@@ -336,8 +346,8 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
                     }
                     tc_fence_before_sync();
                     mbar_arrive(&turn[me ^ 1]);                                    // pass the baton
-                    tc_commit_pair(&empty_bar[s]);                                 // frees the operand stage and the scale slot
-                    if (last) tc_commit_pair(&tmem_full[buf]);
+                    tc_commit_pair(&empty_bar[s], 2u * half_k);                    // frees the operand stage and the scale slot
+                    if (last) tc_commit_pair(&tmem_full[buf], 2u * half_k);
                 }
                 __syncwarp();
                 s += 2;
@@ -376,10 +386,10 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
             for (uint32_t tl = 0; tl < walk.count && ok; ++tl) {
                 int mt, nt;
                 const int w = walk.locate(p, tl, mt, nt);
-                const int num_kt = p.prob[w].num_kt, nkc = p.prob[w].nkc;
+                const int end_kt = end_step(p.prob[w].num_kt), nkc = p.prob[w].nkc;
                 const CUtensorMap *map_a = &maps.sfa[w], *map_b = &maps.sfb[w];
                 const int32_t a_row = (2 * mt + (int)rank) * nkc, b_row = nt * (PN / 128) * nkc;
-                for (int kt = 0; kt < num_kt; ++kt, ++it) {
+                for (int kt = first_step(p.prob[w].num_kt); kt < end_kt; ++kt, ++it) {
                     const int s = it % kStagesP;
                     if (!(ok = mbar_wait(&empty_bar[s], ((it / kStagesP) & 1) ^ 1, abort_flag))) break;
                     uint8_t* dst = sf_ring + s * kSfSlotB;
@@ -391,6 +401,11 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
             }
             if (!ok) *abort_flag = 1;
         }
+    }
+    if (SPLIT) {                                            // the two barriers of the exchange below
+        __syncwarp();
+        cluster_sync_all();
+        cluster_sync_all();
     }
     } else {
         // ------------------------------------------------------------------ epilogue (both CTAs, own 128 rows)
@@ -420,6 +435,63 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
                 bulk_commit_group();
             }
         };
+        if constexpr (SPLIT) {
+            // One tile a cluster.  CTA r of either pair holds the same 128 rows x 128 columns, summed over half of K.  Pair 0
+            // finishes the first 64 columns, pair 1 the others: each sends what the other finishes into that CTA's operand ring, which
+            // is idle by then (first barrier: every MMA of all four CTAs is done), and adds what it gets (second barrier: it is
+            // there).  One fp32 addition, the same whichever side makes it.  A warp takes 32 columns of its lane quadrant.
+            int mt, nt;
+            walk.locate(p, 0, mt, nt);
+            const ProblemP& pr = p.prob[0];
+            const CUtensorMap* map = &maps.c[0];
+            ok = __all_sync(0xffffffffu, mbar_wait_spin(&tmem_full[0], 0, abort_flag));
+            tc_fence_after_sync();
+            cluster_sync_all();
+            uint32_t mine[32];
+            const uint32_t taddr = tmem_acc + ((uint32_t)(q * 32) << 16) + 32 * half;
+            // 16 bytes of a row at a time, a warp's 32 rows side by side
+            const uint32_t slot = smem_u32(smem) + (uint32_t)(half * 8 * 128 + q * 32 + lane) * 16u;
+            if (ok) {
+                uint32_t other[32];
+                tmem_ld_32x32b_x32(taddr + 64 * (1 - half_k), other);
+                tmem_ld_32x32b_x32(taddr + 64 * half_k, mine);
+                tmem_ld_wait();
+                const uint32_t dst = peer_smem(slot, (1 - half_k) * 2 + rank);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) st_peer_16B(dst + i * 2048, other[4 * i], other[4 * i + 1], other[4 * i + 2], other[4 * i + 3]);
+            }
+            cluster_sync_all();
+            if (ok) {
+                const float alpha = KIND == kF8 ? 1.0f / (*pr.scale_a * *pr.scale_b) : pr.alpha;
+                const int64_t row0 = (int64_t)mt * PM + (int64_t)rank * 128 + q * 32, col = (int64_t)nt * PN + 64 * half_k + 32 * half;
+                float v[32];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float4 o = *reinterpret_cast<const float4*>(smem + (slot - smem_u32(smem)) + i * 2048);
+                    v[4 * i] = (__uint_as_float(mine[4 * i]) + o.x) * alpha;
+                    v[4 * i + 1] = (__uint_as_float(mine[4 * i + 1]) + o.y) * alpha;
+                    v[4 * i + 2] = (__uint_as_float(mine[4 * i + 2]) + o.z) * alpha;
+                    v[4 * i + 3] = (__uint_as_float(mine[4 * i + 3]) + o.w) * alpha;
+                }
+                const bool in_range = row0 < pr.M && col < pr.N;
+                uint32_t o[16];
+                if (pr.out_fp32) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(v[16 * h + j]);
+                        put(o, map, pr.accumulate != 0, (int32_t)col + 16 * h, (int32_t)row0, in_range && col + 16 * h < pr.N);
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+                        o[j] = *reinterpret_cast<const uint32_t*>(&h);
+                    }
+                    put(o, map, false, (int32_t)col, (int32_t)row0, in_range);
+                }
+            }
+        } else
         for (uint32_t tl = kAccBufs == 2 ? half : 0; tl < walk.count; tl += kAccBufs) {
             int mt, nt;
             const int w = walk.locate(p, tl, mt, nt);
@@ -502,6 +574,12 @@ gemm_8bit_pair_kernel(const __grid_constant__ MapsP maps, const __grid_constant_
     gemm_pair_body<KIND, false, PN>(maps, p);
 }
 
+template <Kind KIND>
+__global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(kThreadsP, 1)
+gemm_split_kernel(const __grid_constant__ MapsP maps, const __grid_constant__ ParamsP p) {
+    gemm_pair_body<KIND, false, 128, true>(maps, p);
+}
+
 // The small-footprint build (see PairCfg): same roles, same arithmetic, same accumulation order.
 using LiteCfg = PairCfg<kMxf4, true, 256>;
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(LiteCfg::kLaunchRegs)
@@ -535,6 +613,8 @@ cudaError_t gemm_pair_init() {
     if (e == cudaSuccess) e = pair_kernel_init<PairCfg<kF8, false, 128>>(gemm_8bit_pair_kernel<kF8, 128>);
     if (e == cudaSuccess) e = pair_kernel_init<PairCfg<kMxf8, false, 256>>(gemm_8bit_pair_kernel<kMxf8, 256>);
     if (e == cudaSuccess) e = pair_kernel_init<PairCfg<kMxf8, false, 128>>(gemm_8bit_pair_kernel<kMxf8, 128>);
+    if (e == cudaSuccess) e = pair_kernel_init<PairCfg<kF8, false, 128>>(gemm_split_kernel<kF8>);
+    if (e == cudaSuccess) e = pair_kernel_init<PairCfg<kMxf8, false, 128>>(gemm_split_kernel<kMxf8>);
     return e != cudaSuccess ? e : pair_kernel_init<LiteCfg>(gemm_mxf4_pair_lite_kernel);
 }
 
@@ -566,6 +646,16 @@ Spread spread_tiles(int n0, int n1, const double (&cost)[2], int pairs) {
 double tile_cost(int pn, int64_t K) {
     const double steps = (double)ceil_div(K, 256);
     return pn == 256 ? 0.34 * steps + 0.65 : 0.245 * steps + 0.3;
+}
+
+// Whether an 8-bit product goes out with two pairs to a tile (SPLIT): its 128-wide tiles leave half of the pairs idle (32 clusters
+// of four SMs fit the chip's GPCs at once), and half of its K-steps take longer than the exchange, about 2 us.  Whole tiles / split
+// in us, 1024 x 1024 (512 x 2048, 2048 x 512 and 130 x 4096 the same within 0.2): MXINT4 K = 1024 6.6 / 7.4, 2048 8.3 / 8.3, 4096
+// 11.7 / 10.1, 8192 18.3 / 13.9; E4M3 6.7 / 7.3, 8.4 / 8.2, 11.8 / 10.0, 18.4 / 13.7.  MXFP4 products keep whole tiles: with twice the elements to a K-step they would
+// gain from K = 8192 on only (11.7 / 10.4), and their bits stay those of the one launch a backward call makes.
+constexpr int kSplitClusters = 32, kSplitSteps = 24;
+bool split_pays(int64_t M, int64_t N, int64_t steps) {
+    return (int64_t)ceil_div(M, PM) * ceil_div(N, 128) <= kSplitClusters && steps >= kSplitSteps;
 }
 
 void fill_problem(ProblemP& p, const GemmArgs& a, int pn) {
@@ -658,6 +748,7 @@ cudaError_t launch_gemm_pair(const GemmArgs* a, int n, int pn, cudaStream_t stre
 int gemm_f8_tile_n(const Gemm8Args& a) {
     int pairs = 0;
     if (pair_count(&pairs) != cudaSuccess) return 256;
+    if (split_pays(a.M, a.N, a.K >> 7)) return 128;
     const double steps = (double)(a.K >> 7), cost[2] = {0.36 * steps + 0.1, 0.245 * steps + 0.1};
     double time[2];
     for (int i = 0; i < 2; ++i) time[i] = ceil_div((int64_t)ceil_div(a.M, PM) * ceil_div(a.N, i == 0 ? 256 : 128), pairs) * cost[i];
@@ -684,6 +775,11 @@ cudaError_t launch_gemm_f8(const Gemm8Args& a, int pn, cudaStream_t stream) {
     p.rest = p.n0 % pairs;
     maps.a[0] = a.tmap_a; maps.b[0] = a.tmap_b; maps.c[0] = a.tmap_c;
     if (a.block_scaled) { maps.sfa[0] = a.tmap_sfa; maps.sfb[0] = a.tmap_sfb; }
+    if (pn == 128 && split_pays(a.M, a.N, q.num_kt)) {
+        p.rest = 0;
+        return launch_pairs(a.block_scaled ? gemm_split_kernel<kMxf8> : gemm_split_kernel<kF8>, 2 * p.n0,
+                            a.block_scaled ? PairCfg<kMxf8, false, 128>::kSmem : PairCfg<kF8, false, 128>::kSmem, maps, p, stream);
+    }
     if (a.block_scaled)
         return pn == 128 ? launch_pairs(gemm_8bit_pair_kernel<kMxf8, 128>, pairs, PairCfg<kMxf8, false, 128>::kSmem, maps, p, stream)
                          : launch_pairs(gemm_8bit_pair_kernel<kMxf8, 256>, pairs, PairCfg<kMxf8, false, 256>::kSmem, maps, p, stream);

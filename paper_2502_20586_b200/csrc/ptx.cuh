@@ -296,6 +296,15 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint64_t* bar, uint32_t rank
         "mbarrier.arrive.shared::cluster.b64 _, [r];\n\t}"
         ::"r"(smem_u32(bar)), "r"(rank) : "memory");
 }
+// Address of the same shared-memory location in CTA `rank` of the cluster, and a 16-byte store there.
+__device__ __forceinline__ uint32_t peer_smem(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_peer_16B(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
 // 2-D tiled load into THIS CTA's shared memory whose completion bytes are counted on the mbarrier of the pair's
 // leader (even-ranked) CTA: clearing bit 24 of a shared-window address names the leader's copy.  Each CTA fetches
 // its own tiles; nothing is broadcast.
@@ -328,10 +337,10 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t cols)
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
 }
 // Arrive, in both CTAs of the pair, on the mbarrier at this shared-memory offset once all tcgen05 operations issued
-// so far by this thread have completed.
-__device__ __forceinline__ void tc_commit_pair(uint64_t* bar) {
+// so far by this thread have completed.  `leader`: the rank of the pair's even CTA in its cluster.
+__device__ __forceinline__ void tc_commit_pair(uint64_t* bar, uint32_t leader = 0) {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
+                 ::"r"(smem_u32(bar)), "h"((uint16_t)(3u << leader)) : "memory");
 }
 // Same completion tracking, arriving on the issuing CTA's barrier only.
 __device__ __forceinline__ void tc_commit_pair_local(uint64_t* bar) {

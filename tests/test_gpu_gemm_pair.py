@@ -100,6 +100,15 @@ def test_eight_bit_products(gpu, M, N, K, kind, fp32):
     assert torch.all((got.double() - want).abs() <= bound + 1e-30)
 
 
+# two pairs to a tile, each half of the K-steps: the fewest steps that split, an odd number of them, the most tiles, ragged edges
+# (the bounds are those of whole tiles: one addition more)
+@pytest.mark.parametrize("M,N,K", [(1, 8, 3072), (129, 136, 3200), (1000, 1016, 8192), (130, 4096, 3072)])
+@pytest.mark.parametrize("kind", ["fp8", "int4"])
+@pytest.mark.parametrize("fp32", [False, True])
+def test_eight_bit_products_over_two_pairs(gpu, M, N, K, kind, fp32):
+    test_eight_bit_products(gpu, M, N, K, kind, fp32)
+
+
 # one output row: its pitch means nothing and may be larger than a tensor map can hold
 @pytest.mark.parametrize("ldc", [264, 1 << 20, 1 << 40])
 def test_pitch_of_a_single_row(gpu, ldc):
