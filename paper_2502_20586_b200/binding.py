@@ -298,7 +298,7 @@ def mxfp4_linear_backward_ex(dY, X, W, g: int, seed: int, rounding: int = ROUND_
 
 
 STATIC_WORKSPACE_BYTES = 8 << 20
-ONE_READ_ELEMENTS = 1 << 28      # MXFP4_ONE_READ_ELEMENTS: a layer's operands take two quantiser launches from here on, one below
+ONE_READ_ELEMENTS = 1 << 28      # MXFP4_ONE_READ_ELEMENTS: a layer's operands take two quantiser launches from here on (ROUND_RN: from an eighth of it), one below
 
 
 def mxfp4_linear_backward_static(dY, X, W, g: int, seed: int, rounding: int = ROUND_SR, out_dtype: int = OUT_BF16,

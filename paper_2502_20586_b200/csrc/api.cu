@@ -458,8 +458,13 @@ mxfp4_status quantize_operands_impl(const void* dY, const void* X, const void* W
     // at 2^29 32768 x 4096 x 16384 841 / 819, 16384 x 4096 x 32768 696 / 688; at 2^30 65536 x 4096 x 16384 1363 / 1294.  Nearest
     // rounding gains more (16384 x 4096 x 16384 326 / 312, 32768 x 4096 x 16384 632 / 617), SR16 as well (353 / 340, 701 / 660).  Whole
     // calls differ by less than their repeats.  So 2^28 is where the two tie with SR and the others gain 2 - 6 %.
+    // (Those figures are from before codes were stored 32 bytes at a time, which took 5 - 10 % off both forms; the lines stay where they
+    // are for the stochastic modes.)  Nearest rounding, whose arithmetic is cheap, is bound by the read in one list and gains from
+    // 2^25 on: whole calls, list / one read, 4096 x 1024 x 4096 31.8 / 34.5, 8192 x 1024 x 4096 62.6 / 58.9, 16384 x 8192 x 2048 288 / 281,
+    // 16384 x 4096 x 4096 270 / 257; operands of 16384 x 2048 x 8192 125 / 97, 16384 x 4096 x 16384 257 / 210.
     const int dual_mode = dual_setting();
-    if (all_tc && g != 256 && !force_lite() && (dual_mode == 2 || (dual_mode == 1 && b * m >= MXFP4_ONE_READ_ELEMENTS))) {
+    const int64_t one_read = rounding == MXFP4_ROUND_RN ? MXFP4_ONE_READ_ELEMENTS >> 3 : MXFP4_ONE_READ_ELEMENTS;
+    if (all_tc && g != 256 && !force_lite() && (dual_mode == 2 || (dual_mode == 1 && b * m >= one_read))) {
         // dL/dy feeds lines 3 and 5: its two views come from ONE read of it; W^T and X^T in a second launch
         const QuantArgs dy[2] = {q[0], q[2]}, wx[2] = {q[1], q[3]};
         // (the bias gradient's first pass rides along: band sums of dY)
