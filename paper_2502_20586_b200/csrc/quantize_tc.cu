@@ -20,20 +20,25 @@
 // three launch / prologue / drain gaps per layer.
 //
 //   warp 0        TMA producer (two 64-column x 128-row boxes per tile, 128-byte swizzle, 4-stage ring)
-//   warp 1        MMA issuer (8 K=16 MMAs per tile into one of four 128-column TMEM accumulators)
+//   warp 1        MMA issuer (8 K=16 MMAs per tile, N = g, into one of four 128-column TMEM accumulators)
 //   warps 2, 3    column sums of dY when a bias gradient is wanted, else idle; they complete warp group 0, which hands
 //                 registers (setmaxnreg) to the epilogue groups
 //   warps 4..15   epilogue, three groups of four warps on alternate tiles: warp = TMEM lane quadrant, a thread owns one
 //                 output row of the tile: tcgen05.ld 32 columns at a time, scale / SR / pack / store per MX block
 //                 (g = 256: four groups, warps 4..19)
 //
-// What bounds it: the rounding arithmetic of the epilogue warps (9.4 instructions per element), as long as the issuer
-// keeps up.  It did not: MMAs issued from a lane-0 branch have their descriptors moved to uniform registers every time, and
-// every epilogue warp waited for an accumulator.  Warp-uniform issue with one elected lane, 32-bit MX-block arithmetic per
-// tile, two fp32 products per instruction and three groups with a spare accumulator instead of four without one,
-// 16384 x 16384 views, before -> now: SR row-wise 140 -> 123 us, g = 64 133 -> 117, transposing 141 -> 139, g = 256 152 -> 132, SR16 131 -> 111 (6.1 TB/s),
-// RN 112 -> 108; the operands of a backward call, 16384 x 4096 x 16384 341 -> 300, 8192 x 1024 x 4096 56 -> 48, 8192 x 1024
-// x 1024 18.6 -> 16.0.
+// What bounds it: SR by the epilogue's logic pipe and, in calls that last, by the board's power (950 - 1000 W at 1.4 - 1.7 GHz: time is
+// energy, an instruction per element about a hundredth of a call); RN and SR16 by the memory.  What brought it there:
+//   - issue.  MMAs issued from a lane-0 branch have their descriptors moved to uniform registers every time, and every epilogue
+//     warp waited for an accumulator; a converged warp with one elected lane, and three epilogue groups with a spare accumulator instead of
+//     four without one;
+//   - whole sectors of codes in one store (store_codes), SR through the convert (quantize_block32_rw), tiles described once
+//     (TileInfo), MMAs without T's zero blocks, T eight entries at a time (hadamard_row8).
+// 16384 x 16384 views, before the last five -> now: SR row-wise 124 -> 116 us, transposing 140 -> 116, g = 64 118 / 138 -> 108, g = 256 132 -> 128,
+// SR16 111 / 130 -> 107, RN 108 / 119 -> 105 (6.5 TB/s); the operands of a backward call, 16384 x 4096 x 4096 105 -> 95, 8192 x 1024 x 4096 38.5 -> 35.
+// Slower were: the block loop rolled up (SR 127), four groups with accumulators handed back by halves (128), TMEM loads a block
+// ahead (134), part of the Philox rounds folded into constants of the view (more moves than it saved: 96 instructions a block for 85), a fifth
+// stage (RN 110).
 // Every mbarrier wait is bounded; on expiry the CTA records a status word and unwinds.
 #include <cuda_bf16.h>
 
@@ -106,6 +111,7 @@ struct QParams {
     int n_views;
     uint32_t n_tiles;          // over all views
     int g, sf_native;
+    bool x_passes;             // x is read past the L2 cache's ordinary lines (see launch_quantize_tc_group)
     bool wide_stores;          // y_out and the codes of every view start on 32-byte boundaries
     const uint16_t* custom_t;  // bf16 [g, g] row-major transform matrix given by the caller, or null (then diag(S) H_g / sqrt(g))
     uint64_t seed;
@@ -270,6 +276,7 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
         if (lane == 0) {
             uint32_t it = 0, n_info = 0;
             bool ok = true;
+            const uint64_t evict_first = l2_policy_evict_first();
             // DUAL: one load per unit (two logical tiles), in the coordinates of its row-wise view
             for (uint32_t t = DUAL ? 2u * blockIdx.x : blockIdx.x; t < num_tiles && ok; t += (DUAL ? 2u : 1u) * gridDim.x) {
                 TilePos pos = locate_tile<DUAL>(p, t);
@@ -283,8 +290,13 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
                     const int32_t cx = (int32_t)((rowwise ? kt : rt) * kTile), cy = (int32_t)((rowwise ? rt : kt) * kTile);
                     uint8_t* st = smem + s * kTileBytes;
                     mbar_expect_tx(&full_bar[s], kTileBytes);
-                    tma_load_2d(st, &maps.x[pos.v], &full_bar[s], cx, cy);
-                    tma_load_2d(st + kBoxBytes, &maps.x[pos.v], &full_bar[s], cx + 64, cy);
+                    if (p.x_passes) {
+                        tma_load_2d_hint(st, &maps.x[pos.v], &full_bar[s], cx, cy, evict_first);
+                        tma_load_2d_hint(st + kBoxBytes, &maps.x[pos.v], &full_bar[s], cx + 64, cy, evict_first);
+                    } else {
+                        tma_load_2d(st, &maps.x[pos.v], &full_bar[s], cx, cy);
+                        tma_load_2d(st + kBoxBytes, &maps.x[pos.v], &full_bar[s], cx + 64, cy);
+                    }
                 }
                 if (!ok) break;
 #pragma unroll
@@ -657,6 +669,10 @@ cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cud
     for (int v = n; v < kQuantMaxViews; ++v) { p.view[v] = p.view[0]; p.view[v].tile_begin = 0xFFFFFFFFu; maps.x[v] = maps.x[0]; }
     p.n_views = n;
     p.n_tiles = tiles;
+    // A launch that moves more than the L2 cache holds (2 bytes read and 17/32 written an element, 126 MB) marks x's lines as the
+    // first to go, so that codes are still there when the GEMM reads them: whole calls 8192 x 1024 x 4096 66.3 -> 64.5 us, larger ones
+    // between equal and 2 % faster.  Smaller launches keep x, which the next launch may read again (8192 x 1024 x 1024 marked: 28.0 -> 28.6).
+    p.x_passes = (double)tiles * (kTile * kTile * (a[0].g == 256 ? 2 : 1)) * 2.53125 > 126e6;
     p.g = a[0].g; p.sf_native = a[0].sf_native; p.seed = a[0].seed;
     uintptr_t stores = reinterpret_cast<uintptr_t>(a[0].y_out);
     for (int v = 0; v < n; ++v) stores |= reinterpret_cast<uintptr_t>(a[v].codes);
