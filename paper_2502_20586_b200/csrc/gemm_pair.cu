@@ -199,7 +199,7 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
     volatile uint32_t* abort_flag = tmem_slot + 2;
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp-uniform, and known to be)
-    const uint32_t rank = cluster_ctarank() & 1u;           // in the pair: 0 = leader
+    const uint32_t rank = SPLIT ? cluster_ctarank() & 1u : cluster_ctarank();    // in the pair: 0 = leader
     const uint32_t half_k = SPLIT ? cluster_ctarank() >> 1 : 0u;                 // this pair's half of the K-steps
     constexpr int kLgCtas = SPLIT ? 2 : 1;
     const TileWalk walk(p, (int)(blockIdx.x >> kLgCtas), (int)(gridDim.x >> kLgCtas));
