@@ -47,21 +47,23 @@ __device__ __forceinline__ void rht_in_place(float (&v)[32], uint32_t sign_bits,
 // Bound by memory with nearest rounding: 16384 x 2048, g = 0 16.7 -> 14.6 us (SR 22.8 -> 20.8), 16384 x 16384 117 -> 111, with:
 // Index: uint32_t where the tensor has fewer than 2^31 blocks (a 64-bit division costs more instructions than rounding the
 // block), else uint64_t.  `wide`: every row starts on a 32-byte boundary, so a block is two 32-byte loads of whole sectors.
+// The kernels of this file may start while the kernel that writes x still runs (pdl_wait): x is read by ordinary loads that stay
+// behind the wait, through pointers that are not `restrict`; never through the read-only path.
 __device__ __forceinline__ void load_32B(const void* src, uint4& a, uint4& b, bool wide) {
     if (wide) {
-        asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-            : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(src));
+        asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(src) : "memory");
     } else {
-        a = __ldg(reinterpret_cast<const uint4*>(src));
-        b = __ldg(reinterpret_cast<const uint4*>(src) + 1);
+        a = reinterpret_cast<const uint4*>(src)[0];
+        b = reinterpret_cast<const uint4*>(src)[1];
     }
 }
 
 template <int G, bool DUMP_Y, typename Index>
-__global__ void __launch_bounds__(256) quantize_rowwise_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols,
+__global__ void __launch_bounds__(256) quantize_rowwise_kernel(const __nv_bfloat16* x, int64_t rows, int64_t cols,
                                                                int64_t ld, int rounding, uint64_t seed, uint32_t stream_tag,
-                                                               uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
-                                                               int sf_native, float* __restrict__ y_out, bool wide, bool chain) {
+                                                               uint8_t* codes, uint8_t* scales,
+                                                               int sf_native, float* y_out, bool wide, bool chain) {
     if (chain) pdl_launch_dependents();
     pdl_wait();
     const Index nkb = (Index)(cols >> 5);
@@ -110,10 +112,10 @@ constexpr int kTrRows = 256;
 constexpr int kTrCols = 64;
 
 template <int G, bool DUMP_Y>
-__global__ void __launch_bounds__(256) quantize_transpose_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols,
+__global__ void __launch_bounds__(256) quantize_transpose_kernel(const __nv_bfloat16* x, int64_t rows, int64_t cols,
                                                                  int64_t ld, int rounding, uint64_t seed, uint32_t stream_tag,
-                                                                 uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
-                                                                 int sf_native, float* __restrict__ y_out, bool chain) {
+                                                                 uint8_t* codes, uint8_t* scales,
+                                                                 int sf_native, float* y_out, bool chain) {
     __shared__ __align__(16) uint32_t tile[kTrRows * 32];
     if (chain) pdl_launch_dependents();
     pdl_wait();
@@ -128,7 +130,7 @@ __global__ void __launch_bounds__(256) quantize_transpose_kernel(const __nv_bflo
         const int c = tid & 7;
         uint4 q = make_uint4(0u, 0u, 0u, 0u);
         if (row0 + r < rows && col0 + c * 8 < cols)
-            q = __ldg(reinterpret_cast<const uint4*>(x + (row0 + r) * ld + col0 + c * 8));
+            q = *reinterpret_cast<const uint4*>(x + (row0 + r) * ld + col0 + c * 8);
         const int rot = (c + (r >> 5)) & 7;
         *reinterpret_cast<uint4*>(&tile[r * 32 + rot * 4]) = q;
     }

@@ -106,6 +106,44 @@ def test_row_alignment(rows, cols, rounding):
         assert torch.equal(got[1], gpu.mxfp4_rht_sr_quantize(x, 1, 0, 3, 2, rounding, gpu.SF_LINEAR)[1])
 
 
+# The CUDA-core quantisers start while the product that writes their input still runs (few tiles, so SMs are free, and a long
+# K): the bytes are those of a run that waits between the two
+@pytest.mark.parametrize("reduce_dim", [0, 1])
+@pytest.mark.parametrize("g", [0, 32])
+@pytest.mark.parametrize("pad", [0, 8])
+def test_product_quantised_by_the_next_launch(reduce_dim, g, pad):
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    M, N, K = 288, 544, 16384                                            # no reduce length that the tensor-core quantiser takes
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(g + pad)
+    a = [torch.randint(0, 256, (M, K // 2), generator=gen, device="cuda", dtype=torch.uint8) for _ in range(2)]
+    b = torch.randint(0, 256, (N, K // 2), generator=gen, device="cuda", dtype=torch.uint8)
+    ones = [torch.full((gpu.mxfp4_scale_bytes(rows, K),), 127, dtype=torch.uint8, device="cuda") for rows in (M, N)]
+    C = torch.zeros((M, N + pad), dtype=torch.bfloat16, device="cuda")[:, :N]
+
+    def product(i):
+        gpu.mxfp4_gemm(a[i], ones[0], b, ones[1], 1.0, gpu.OUT_BF16, C_out=C)
+
+    def quantise():
+        return gpu.mxfp4_rht_sr_quantize(C, reduce_dim, g, 3, 2, gpu.ROUND_SR, gpu.SF_LINEAR)
+
+    want = []
+    for i in range(2):
+        product(i)
+        torch.cuda.synchronize()
+        want.append(quantise())
+        torch.cuda.synchronize()
+    assert not torch.equal(want[0][0], want[1][0])
+    got = []
+    for i in range(40):
+        product(i % 2)
+        got.append(quantise())
+    assert gpu.mxfp4_device_status() == 0
+    for i, (codes, scales) in enumerate(got):
+        assert torch.equal(codes, want[i % 2][0]) and torch.equal(scales, want[i % 2][1]), i
+
+
 # The bias gradient's two passes inside the launches of a backward call: band sums in the one-list and in the one-read form,
 # added up by the GEMM launch; against fp64, overwriting and accumulating
 @pytest.mark.parametrize("b,n,m", [(128, 264, 128), (640, 8, 1152), (2048, 1000, 5120)])
