@@ -305,7 +305,7 @@ cudaError_t launch_gemm_f8_one_cta(const Gemm8Args& a, cudaStream_t stream) {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, a.block_scaled ? gemm_f8_kernel<true> : gemm_f8_kernel<false>, a.tmap_a, a.tmap_b, p);
+    return launch_result(cudaLaunchKernelEx(&cfg, a.block_scaled ? gemm_f8_kernel<true> : gemm_f8_kernel<false>, a.tmap_a, a.tmap_b, p));
 }
 
 }  // namespace mx

@@ -694,7 +694,7 @@ cudaError_t launch_pairs(void (*kernel)(MapsP, ParamsP), int pairs, uint32_t sme
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, maps, p);
+    return launch_result(cudaLaunchKernelEx(&cfg, kernel, maps, p));
 }
 }  // namespace
 

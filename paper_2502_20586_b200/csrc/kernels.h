@@ -6,6 +6,12 @@
 
 namespace mx {
 
+// What a launch returned, taken out of the runtime's record if it is an error: checks after later launches are not to find it again.
+inline cudaError_t launch_result(cudaError_t e) {
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
 struct QuantArgs {
     const void* x;        // bf16 [rows, cols], leading dimension ld
     int64_t rows, cols, ld;

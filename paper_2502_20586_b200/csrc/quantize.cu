@@ -187,7 +187,7 @@ static cudaError_t launch_after(void (*kernel)(Params...), dim3 grid, cudaStream
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = chain ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+    return launch_result(cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...));
 }
 
 template <bool DUMP_Y>

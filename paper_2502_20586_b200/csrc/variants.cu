@@ -209,8 +209,8 @@ cudaError_t launch_fp8_quantize(const Fp8QuantArgs* a, int n, uint16_t* partial,
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, dense ? fp8_amax_kernel<true> : fp8_amax_kernel<false>, p);
-    return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, dense ? fp8_quantize_kernel<true> : fp8_quantize_kernel<false>, p);
+    const cudaError_t e = launch_result(cudaLaunchKernelEx(&cfg, dense ? fp8_amax_kernel<true> : fp8_amax_kernel<false>, p));
+    return e != cudaSuccess ? e : launch_result(cudaLaunchKernelEx(&cfg, dense ? fp8_quantize_kernel<true> : fp8_quantize_kernel<false>, p));
 }
 
 cudaError_t launch_mxint4_quantize(const float* y, int64_t R, int64_t K, int rounding, uint64_t seed, uint32_t stream_tag,

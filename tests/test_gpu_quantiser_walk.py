@@ -144,6 +144,17 @@ def test_product_quantised_by_the_next_launch(reduce_dim, g, pad):
         assert torch.equal(codes, want[i % 2][0]) and torch.equal(scales, want[i % 2][1]), i
 
 
+# A launch that is refused (here: more bands of rows than a grid holds) is the call's error and no other's
+def test_refused_launch_leaves_no_error_behind():
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    x = torch.zeros((256 << 16, 8), dtype=torch.bfloat16, device="cuda")
+    with pytest.raises(gpu.MxFp4Error):
+        gpu.mxfp4_rht_sr_quantize(x, 0, 0, 3, 2, gpu.ROUND_RN)
+    codes, scales, _ = gpu.mxfp4_int4_quantize(x[:256], 0, 0, 3, 2, gpu.ROUND_RN)     # looks for a launch error after its last kernel
+    assert gpu.mxfp4_device_status() == 0 and not torch.any(codes) and not torch.any(scales)
+
+
 # The bias gradient's two passes inside the launches of a backward call: band sums in the one-list and in the one-read form,
 # added up by the GEMM launch; against fp64, overwriting and accumulating
 @pytest.mark.parametrize("b,n,m", [(128, 264, 128), (640, 8, 1152), (2048, 1000, 5120)])
