@@ -142,7 +142,7 @@ def test_quantizer_is_deterministic_and_tags_differ(gpu):
 
 
 def test_quantizer_huge_and_tiny_magnitudes(gpu, ref):
-    """Scale clamps and the wide-exponent path: blocks near 2^100 and near the subnormals."""
+    """Scale clamps: blocks near 2^100 and near the subnormals."""
     rng = np.random.default_rng(8)
     x = rng.standard_normal((64, 256)).astype(np.float32)
     x[:16] *= 2.0 ** 100
@@ -155,6 +155,27 @@ def test_quantizer_huge_and_tiny_magnitudes(gpu, ref):
         _, rc, rs = ref.rht_quantize(xb, 0, rounding, 3, 1)
         assert np.array_equal(scales, rs)
         assert np.array_equal(codes, rc)
+
+
+@pytest.mark.parametrize("rounding", [0, 1, 2])
+def test_quantizer_up_to_the_largest_numbers(gpu, ref, rounding):
+    """One row for each of the scale bytes 226 .. 252, the last with the largest bf16 numbers, in both directions; and through
+    the tensor cores, where integers times a power of two keep every sum exact."""
+    rng = np.random.default_rng(21)
+    x = rng.uniform(1.0, 255.0 / 128.0, (27, 256)) * 2.0 ** -rng.integers(0, 8, (27, 256)) * rng.choice([-1.0, 1.0], (27, 256))
+    x[:, ::32] = 255.0 / 128.0
+    xb = wl.to_bf16_bits((x * 2.0 ** (np.arange(27.0)[:, None] + 101.0)).astype(np.float32))
+    for reduce_dim, bits in ((1, xb), (0, np.ascontiguousarray(np.pad(xb, ((0, 5), (0, 0))).T))):
+        codes, scales = _quant_gpu(gpu, bits, reduce_dim, 0, 3, 1, rounding, gpu.SF_LINEAR)
+        _, rc, rs = ref.rht_quantize(bits, 0, rounding, 3, 1, transpose=(reduce_dim == 0))
+        assert np.array_equal(rs[:27], np.broadcast_to(np.arange(226, 253)[:, None], (27, 8)))
+        assert np.array_equal(scales, rs) and np.array_equal(codes, rc)
+    wide = rng.integers(-8, 9, (64, 256)) * 2.0 ** rng.integers(100, 119, (64, 1))
+    bits = wl.to_bf16_bits(wide.astype(np.float32))
+    codes, scales = _quant_gpu(gpu, bits, 1, 64, 3, 1, rounding, gpu.SF_LINEAR)
+    _, rc, rs = ref.rht_quantize(bits, 64, rounding, 3, 1)
+    assert rs.min() < 228 and rs.max() > 240
+    assert np.array_equal(scales, rs) and np.array_equal(codes, rc)
 
 
 # ------------------------------------------------------------------------------------------------ GEMM
