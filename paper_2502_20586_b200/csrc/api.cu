@@ -431,6 +431,7 @@ mxfp4_status quantize_operands_impl(const void* dY, const void* X, const void* W
     };
     bool all_tc = true;
     for (int i = 0; i < 4; ++i) {
+        q[i].layer = true;
         if (i == 2) { q[2].tmap_x = q[0].tmap_x; q[2].has_tmap = q[0].has_tmap; }   // the same tensor; both reduce lengths are multiples of 128
         else attach_input_map(q[i]);
         all_tc = all_tc && mx::quant_tc_eligible(q[i]);

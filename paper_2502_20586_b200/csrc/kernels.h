@@ -27,8 +27,26 @@ struct QuantArgs {
     CUtensorMap tmap_x;   // x as [rows, cols] bf16, box 64 cols x 128 rows, 128-byte swizzle (tensor-core path)
     bool has_tmap;
     const void* custom_t = nullptr;   // bf16 [g, g] row-major: transform matrix given by the caller instead of diag(S) H_g / sqrt(g) (tensor-core path, g <= 128)
+    bool layer = false;     // one of the four operand views of a layer's backward call: the call's products read its codes next
     bool mxint4 = false;    // MXINT4 codes (one byte per element) and y_out in one pass (tensor-core path, g <= 128, rounding 0 or 1, native scales)
 };
+
+// Whether a launch of the tensor-core quantiser marks x's lines as the first to leave L2, so that codes are still there when a
+// GEMM reads them.  Counted are 2 bytes read and 17/32 written an element of every view.
+// The views of a backward call: where that is more than L2 holds (126 MB).  Whole calls of 8192 tokens, 1024 in, not marked / marked, SR, RN, SR16
+// in us: 3072 out (157 MB) 53.9, 49.4, 51.0 / 52.3, 47.5, 49.3; 4096 out (202 MB) 65.6, 59.8, 63.5 / 64.0, 58.5, 62.9; larger layers the same
+// within their repeats.  Below the line: 1024 out (66 MB) 28.6, 25.0, 27.4 / 29.0, 25.4, 27.5; 8192 x 512 x 2304 (105 MB) RN 32.4 / 33.2.  Two
+// views from one read count twice: every line is read once in any case.  2^25 elements (103 MB moved, 170 counted) RN 8192 x 1024 x 4096 60.5 / 57.6.
+// One view, quantised by a call of its own: only up to 180 MB, since x may be read again next and a marked stream of several times L2's
+// size is slower.  RN in us, the view alone, both views in turn, a product with 2048 rows: 8192 x 6144 (127 MB) 23.4, 46.0, 73.0 / 20.2, 43.4, 68.5;
+// 8192 x 8192 (170) 29.3, 58.4, 90.0 / 25.5, 60.4, 87.8; 10240 x 8192 (212) 35.3, 70.8, 107.4 / 30.6, 76.4, 105.7; 16384 x 8192 (340) 54.7, 109, 151 / 59.0, 121,
+// 156; 16384 x 16384 104, 207, 305 / 117, 235, 310.  Not where the transformed values are written (dump of 8192 x 6144: 57.5 / 60.0).
+inline bool quant_input_leaves_l2(const QuantArgs* a, int n) {
+    double bytes = 0.0;
+    for (int v = 0; v < n; ++v) bytes += (double)a[v].rows * (double)a[v].cols * 2.53125;
+    if (a[0].layer) return bytes > 126e6;
+    return n == 1 && a[0].y_out == nullptr && bytes > 126e6 && bytes <= 180e6;
+}
 
 // Tensor-core transform path (quantize_tc.cu): g in {32, 64, 128} and reduce length a multiple of 128.
 bool quant_tc_eligible(const QuantArgs& a);

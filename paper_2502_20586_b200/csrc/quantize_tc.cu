@@ -111,7 +111,7 @@ struct QParams {
     int n_views;
     uint32_t n_tiles;          // over all views
     int g, sf_native;
-    bool x_passes;             // x is read past the L2 cache's ordinary lines (see launch_quantize_tc_group)
+    bool x_passes;             // x's lines are the first to leave L2 (quant_input_leaves_l2)
     bool wide_stores;          // y_out and the codes of every view start on 32-byte boundaries
     const uint16_t* custom_t;  // bf16 [g, g] row-major transform matrix given by the caller, or null (then diag(S) H_g / sqrt(g))
     uint64_t seed;
@@ -669,10 +669,7 @@ cudaError_t launch_quantize_tc_group(const QuantArgs* a, int n, bool dump_y, cud
     for (int v = n; v < kQuantMaxViews; ++v) { p.view[v] = p.view[0]; p.view[v].tile_begin = 0xFFFFFFFFu; maps.x[v] = maps.x[0]; }
     p.n_views = n;
     p.n_tiles = tiles;
-    // A launch that moves more than the L2 cache holds (2 bytes read and 17/32 written an element, 126 MB) marks x's lines as the
-    // first to go, so that codes are still there when the GEMM reads them: whole calls 8192 x 1024 x 4096 66.3 -> 64.5 us, larger ones
-    // between equal and 2 % faster.  Smaller launches keep x, which the next launch may read again (8192 x 1024 x 1024 marked: 28.0 -> 28.6).
-    p.x_passes = (double)tiles * (kTile * kTile * (a[0].g == 256 ? 2 : 1)) * 2.53125 > 126e6;
+    p.x_passes = quant_input_leaves_l2(a, n);
     p.g = a[0].g; p.sf_native = a[0].sf_native; p.seed = a[0].seed;
     uintptr_t stores = reinterpret_cast<uintptr_t>(a[0].y_out);
     for (int v = 0; v < n; ++v) stores |= reinterpret_cast<uintptr_t>(a[v].codes);
