@@ -197,6 +197,11 @@ def aggregate_value(flops_per_rank: float, world: int, ms: float) -> float:
 
 
 # ------------------------------------------------------------------------------------------------ GPU arm
+def launches_per_step(layers, one_read_elements: int) -> int:
+    """Kernels of one step: per layer one quantiser launch, or two where dY is read once for its two views, and one for both GEMMs."""
+    return sum(3 if l.b * l.m >= one_read_elements else 2 for l in layers)
+
+
 def run_gpu(args):
     import torch
     import torch.distributed as dist
@@ -594,7 +599,7 @@ def run_gpu(args):
                        "frac_of_nominal_9pf": value / world / NOMINAL_FP4_TFLOPS, "timed_region_s": ms * args.steps * 1e-3,
                        "step_as_separate_calls_ms": calls_ms},
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h, "ms_per_step": ms_e2e},
-            "gpu_launches": args.steps * sum(3 if l.b * l.m >= mx.ONE_READ_ELEMENTS else 2 for l in layers),   # per layer: one or two quantiser launches + one for both GEMMs
+            "gpu_launches": args.steps * launches_per_step(layers, mx.one_read_elements(rnd)),
             "clocks": clocks,
             "roofline": None if gemm_tflops is None else {
                          "kernel": "gemm_mxf4_pair_kernel", "bound": "tensor", "achieved": gemm_tflops, "peak": fp4_peak, "unit": "TFLOP/s",

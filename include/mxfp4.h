@@ -130,8 +130,9 @@ MXFP4_API mxfp4_status mxfp4_gemm(const uint8_t* A_codes, const uint8_t* A_scale
                         void* C, int64_t ldc, int out_dtype, void* cuda_stream);
 
 /* Elements of dY from which on one launch reads it once for its two views and a second one takes W and X; below, one launch
- * takes the four views.  (MXFP4_ROUND_RN: from an eighth of that on.) */
+ * takes the four views.  _RN: with MXFP4_ROUND_RN, else the first. */
 #define MXFP4_ONE_READ_ELEMENTS (1ll << 28)
+#define MXFP4_ONE_READ_ELEMENTS_RN (1ll << 25)
 
 /* Bytes of device workspace mxfp4_linear_backward needs for these shapes (codes + scales of the four
  * quantised operands). */

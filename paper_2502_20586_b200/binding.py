@@ -298,7 +298,13 @@ def mxfp4_linear_backward_ex(dY, X, W, g: int, seed: int, rounding: int = ROUND_
 
 
 STATIC_WORKSPACE_BYTES = 8 << 20
-ONE_READ_ELEMENTS = 1 << 28      # MXFP4_ONE_READ_ELEMENTS: a layer's operands take two quantiser launches from here on (ROUND_RN: from an eighth of it), one below
+ONE_READ_ELEMENTS = 1 << 28       # MXFP4_ONE_READ_ELEMENTS: from here on a layer's operands take two quantiser launches, below one
+ONE_READ_ELEMENTS_RN = 1 << 25    # MXFP4_ONE_READ_ELEMENTS_RN: the same with ROUND_RN
+
+
+def one_read_elements(rounding: int) -> int:
+    """Elements of dY [b, m] from which on ``mxfp4_linear_backward`` reads it once for both views, by a launch of its own (g <= 128)."""
+    return ONE_READ_ELEMENTS_RN if rounding == ROUND_RN else ONE_READ_ELEMENTS
 
 
 def mxfp4_linear_backward_static(dY, X, W, g: int, seed: int, rounding: int = ROUND_SR, out_dtype: int = OUT_BF16,

@@ -123,7 +123,7 @@ bool force_lite() {
     return e != nullptr && e[0] == '1';
 }
 
-// MXFP4_DUAL_DY: 1 (default) = one read of dL/dy for its two views where that pays (MXFP4_ONE_READ_ELEMENTS; a bias
+// MXFP4_DUAL_DY: 1 (default) = one read of dL/dy for its two views where that pays (MXFP4_ONE_READ_ELEMENTS, _RN; a bias
 // gradient's column sums ride along either way); 0 = always separate tile lists, sums by a pass of their own; 2 = always one read.
 int dual_setting() {
     const char* e = getenv("MXFP4_DUAL_DY");
@@ -452,19 +452,17 @@ mxfp4_status quantize_operands_impl(const void* dY, const void* X, const void* W
     }
     if (ov != nullptr) ov->first = -1;
     // One read of dL/dy for its two views needs a launch of its own (W and X follow in a second), and its units of two tiles
-    // spread less evenly: the four views as one tile list are faster until the read saved outweighs that.  Operands of a
-    // layer, tokens x in x out, g = 128, one list / one read in us.  SR, below 2^28 elements of dL/dy: 8192 x 1024 x 4096
-    // 39 / 49, 16384 x 8192 x 2048 106 / 117, 16384 x 4096 x 4096 103 / 112, 16384 x 2048 x 8192 156 / 154.  At 2^28:
-    // 16384 x 1024 x 16384 308 / 302, 16384 x 4096 x 16384 375 / 380, 32768 x 4096 x 8192 435 / 440, 65536 x 1024 x 4096 366 / 370;
-    // at 2^29 32768 x 4096 x 16384 841 / 819, 16384 x 4096 x 32768 696 / 688; at 2^30 65536 x 4096 x 16384 1363 / 1294.  Nearest
-    // rounding gains more (16384 x 4096 x 16384 326 / 312, 32768 x 4096 x 16384 632 / 617), SR16 as well (353 / 340, 701 / 660).  Whole
-    // calls differ by less than their repeats.  So 2^28 is where the two tie with SR and the others gain 2 - 6 %.
-    // (Those figures are from before codes were stored 32 bytes at a time, which took 5 - 10 % off both forms; the lines stay where they
-    // are for the stochastic modes.)  Nearest rounding, whose arithmetic is cheap, is bound by the read in one list and gains from
-    // 2^25 on: whole calls, list / one read, 4096 x 1024 x 4096 31.8 / 34.5, 8192 x 1024 x 4096 62.6 / 58.9, 16384 x 8192 x 2048 288 / 281,
-    // 16384 x 4096 x 4096 270 / 257; operands of 16384 x 2048 x 8192 125 / 97, 16384 x 4096 x 16384 257 / 210.
+    // spread less evenly: the four views as one tile list are faster until the read saved outweighs that.  The stochastic modes are bound by
+    // arithmetic and gain from 2^28 elements of dL/dy on, nearest rounding, which is bound by memory, from 2^25.  Whole calls in us, tokens x in x
+    // out, list / one read, SR, RN, SR16; g = 64 in the first two, else 128:
+    //   2^24  4096 x 1024 x 4096    37.6 / 42.9    32.3 / 34.4    36.0 / 39.8      2^28  16384 x 1024 x 16384  498 / 500      453 / 370      494 / 490
+    //   2^25  8192 x 1024 x 4096    64.6 / 71.4    62.0 / 57.3    63.6 / 69.3            16384 x 4096 x 16384  1178 / 1177    1091 / 999     1147 / 1124
+    //         16384 x 8192 x 2048   335 / 347      327 / 332      340 / 347              32768 x 4096 x 8192   1201 / 1206    1157 / 1098    1184 / 1173
+    //   2^26  16384 x 4096 x 4096   325 / 336      317 / 307      311 / 316        2^29  32768 x 4096 x 16384  2382 / 2348    2346 / 2187    2284 / 2268
+    //   2^27  16384 x 2048 x 8192   344 / 351      338 / 303      368 / 370
+    // The operands alone: 16384 x 4096 x 16384 350 / 347, 308 / 222, 303 / 296; 8192 x 1024 x 4096 34.7 / 38.6, 30.9 / 29.9, 31.9 / 34.6.
     const int dual_mode = dual_setting();
-    const int64_t one_read = rounding == MXFP4_ROUND_RN ? MXFP4_ONE_READ_ELEMENTS >> 3 : MXFP4_ONE_READ_ELEMENTS;
+    const int64_t one_read = rounding == MXFP4_ROUND_RN ? MXFP4_ONE_READ_ELEMENTS_RN : MXFP4_ONE_READ_ELEMENTS;
     if (all_tc && g != 256 && !force_lite() && (dual_mode == 2 || (dual_mode == 1 && b * m >= one_read))) {
         // dL/dy feeds lines 3 and 5: its two views come from ONE read of it; W^T and X^T in a second launch
         const QuantArgs dy[2] = {q[0], q[2]}, wx[2] = {q[1], q[3]};

@@ -47,9 +47,19 @@ def test_scale_bytes_and_workspace(lib):
 
 def test_constants_of_the_header_are_those_of_the_binding(lib):
     header = open(os.path.join(ROOT, "include", "mxfp4.h")).read()
-    for name, value in (("STATIC_WORKSPACE_BYTES", lib.STATIC_WORKSPACE_BYTES), ("ONE_READ_ELEMENTS", lib.ONE_READ_ELEMENTS)):
+    for name, value in (("STATIC_WORKSPACE_BYTES", lib.STATIC_WORKSPACE_BYTES), ("ONE_READ_ELEMENTS", lib.ONE_READ_ELEMENTS),
+                        ("ONE_READ_ELEMENTS_RN", lib.ONE_READ_ELEMENTS_RN)):
         base, shift = re.search(rf"#define MXFP4_{name} \((\d+)\w* << (\d+)\)", header).groups()
         assert int(base) << int(shift) == value
+
+
+def test_launches_that_the_benchmark_counts(lib):
+    """FC1 of the 345M model has 2^25 elements of dY: two quantiser launches with nearest rounding, one with the stochastic modes."""
+    import bench
+    from paper_2502_20586_b200.workloads import Linear
+    layers = [Linear("fc1", 8192, 1024, 4096), Linear("below", 8192, 1024, 4032), Linear("large", 16384, 4096, 16384)]
+    for rounding, want in ((lib.ROUND_SR, 2 + 2 + 3), (lib.ROUND_RN, 3 + 2 + 3), (lib.ROUND_SR16, 2 + 2 + 3)):
+        assert bench.launches_per_step(layers, lib.one_read_elements(rounding)) == want
 
 
 def test_argument_validation_needs_no_device(lib):

@@ -56,6 +56,29 @@ def test_views_of_a_layer(b, n, m, dual, rounding, monkeypatch):
     assert gpu.mxfp4_device_status() == 0
 
 
+# Nearest rounding reads dY once from 2^25 elements on: at the line and just below, the default against both forms asked for
+@pytest.mark.parametrize("b", [8192, 8064])
+def test_default_form_around_one_read(b, monkeypatch):
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    n, m = 264, 4096
+    assert (b * m >= gpu.one_read_elements(gpu.ROUND_RN)) == (b == 8192)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(b)
+    dY, X, W = (torch.randn(s, generator=gen, device="cuda").bfloat16() for s in ((b, m), (b, n), (m, n)))
+    out = {}
+    for form in ("1", "0", "2"):
+        monkeypatch.setenv("MXFP4_DUAL_DY", form)
+        workspace = torch.zeros(gpu.mxfp4_linear_backward_workspace(b, m, n), dtype=torch.uint8, device="cuda")
+        gpu.mxfp4_quantize_operands(dY, X, W, 64, 9, gpu.ROUND_RN, workspace=workspace)
+        out[form] = (workspace, *gpu.mxfp4_linear_backward_ex(dY, X, W, 64, 9, gpu.ROUND_RN, gpu.OUT_FP32, with_bias=True))
+        assert gpu.mxfp4_device_status() == 0
+    for form in ("0", "2"):
+        assert all(torch.equal(got, want) for got, want in zip(out["1"][:3], out[form][:3]))
+    assert torch.equal(out["1"][3], out["2"][3])                         # band sums either way; form 0 sums in a pass of its own
+    assert torch.all((out["1"][3].double() - dY.double().sum(0)).abs() <= b * 2.0 ** -24 * dY.double().abs().sum(0))
+
+
 # MXINT4 in one launch with the transform: rows that fill no tile (their scale bytes are zero), buffers on 16-byte and on
 # 32-byte boundaries, against a pass over the transformed values in torch
 @pytest.mark.parametrize("rows,cols,reduce_dim", [(1, 128, 1), (130, 1280, 1), (384, 136, 0), (1000, 2048, 1)])
