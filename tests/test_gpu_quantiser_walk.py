@@ -79,6 +79,28 @@ def test_default_form_around_one_read(b, monkeypatch):
     assert torch.all((out["1"][3].double() - dY.double().sum(0)).abs() <= b * 2.0 ** -24 * dY.double().abs().sum(0))
 
 
+# Codes that start on a 16-byte and on no 32-byte boundary go out in 16-byte stores: the same bytes, and none beyond them
+@pytest.mark.parametrize("rows,cols,reduce_dim", [(3, 256, 1), (130, 1280, 1), (512, 136, 0), (2048, 1000, 0)])
+@pytest.mark.parametrize("g", [0, 32, 64, 128, 256])
+@pytest.mark.parametrize("rounding", [0, 1, 2])
+def test_codes_on_sixteen_bytes(rows, cols, reduce_dim, g, rounding):
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(rows + g)
+    x = torch.randn((rows, cols), generator=gen, device="cuda").bfloat16()
+    want, want_scales = gpu.mxfp4_rht_sr_quantize(x, reduce_dim, g, 3, 2, rounding, gpu.SF_LINEAR)
+    assert want.data_ptr() % 32 == 0
+    for start in (16, 48):
+        buffer = torch.full((want.numel() + 96,), 0xAA, dtype=torch.uint8, device="cuda")
+        codes = buffer[start:start + want.numel()].view(want.shape)
+        assert codes.data_ptr() % 32 == 16
+        _, scales = gpu.mxfp4_rht_sr_quantize(x, reduce_dim, g, 3, 2, rounding, gpu.SF_LINEAR, codes=codes)
+        assert torch.equal(codes, want) and torch.equal(scales, want_scales)
+        assert torch.all(buffer[:start] == 0xAA) and torch.all(buffer[start + want.numel():] == 0xAA)
+    assert gpu.mxfp4_device_status() == 0
+
+
 # MXINT4 in one launch with the transform: rows that fill no tile (their scale bytes are zero), buffers on 16-byte and on
 # 32-byte boundaries, against a pass over the transformed values in torch
 @pytest.mark.parametrize("rows,cols,reduce_dim", [(1, 128, 1), (130, 1280, 1), (384, 136, 0), (1000, 2048, 1)])
