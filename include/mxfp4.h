@@ -253,7 +253,9 @@ MXFP4_API mxfp4_status mxfp4_linear_backward_static(const void* dY, const void* 
  *   E4M3(fp32(x * scale[0])), round-to-nearest-even, saturating at +-448.  Two kernels, no host synchronisation.
  * mxfp4_fp8_gemm: C [M, N] = (sum_k A[i, k] B[j, k]) / (A_scale[0] B_scale[0]); A [M, K], B [N, K] E4M3 bytes, K-major,
  *   K % 128 == 0, N % 8 == 0; the scales are DEVICE pointers (as written by mxfp4_fp8_quantize); fp32 accumulation on the
- *   tensor cores (tcgen05 kind::f8f6f4); C bf16 or fp32, leading dimension ldc.
+ *   tensor cores (tcgen05 kind::f8f6f4); C bf16 or fp32, leading dimension ldc.  The order of the fp32 sum depends on M, N and K
+ *   alone, so equal calls give equal bits; with K >= 3072 and at most 32 tiles of 256 x 128 the sum is made in two halves of
+ *   K, so the last bits of a row may differ from those of the same row in a larger product.
  * mxfp4_linear_forward_fp8: y [b, m] = x [b, n] W [m, n]^T through the two calls above; n % 128 == 0, m % 8 == 0;
  *   workspace of mxfp4_linear_forward_fp8_workspace(b, n, m) bytes, 256-byte aligned (codes of both operands, scales).
  * Errors as for the other calls (MXFP4_ERR_NULL / _SHAPE / _ALIGN / _MODE / _WORKSPACE / _CUDA).
@@ -279,7 +281,8 @@ MXFP4_API mxfp4_status mxfp4_linear_forward_fp8(const void* x, const void* W, in
  *   aligned, caller-owned) receives the transformed values on the way.  Scale bytes that only fill the last tiles
  *   are set to zero.
  * mxfp4_int4_gemm: C [M, N] = alpha sum_k q_A X_A q_B X_B on the tensor cores (tcgen05 kind::mxf8f6f4, one scale per
- *   32 elements); K % 128 == 0, N % 8 == 0; alpha = 16/9 undoes two 3/4 pre-scales as in Algorithm 3.
+ *   32 elements); K % 128 == 0, N % 8 == 0; alpha = 16/9 undoes two 3/4 pre-scales as in Algorithm 3.  Order of the sum: as
+ *   for mxfp4_fp8_gemm.
  */
 MXFP4_API mxfp4_status mxfp4_int4_quantize(const void* x, int64_t rows, int64_t cols, int64_t ld, int reduce_dim, int g, int rounding,
                                            uint64_t seed, uint32_t stream_tag, uint8_t* codes, uint8_t* scales, float* y_scratch,

@@ -352,7 +352,8 @@ def mxfp4_fp8_quantize(x: torch.Tensor, codes=None, scale=None):
 
 
 def mxfp4_fp8_gemm(A_codes, A_scale, B_codes, B_scale, out_dtype: int = OUT_BF16, C_out=None):
-    """C [M, N] = A B^T / (A_scale[0] B_scale[0]) with E4M3 operands [M, K], [N, K]."""
+    """C [M, N] = A B^T / (A_scale[0] B_scale[0]) with E4M3 operands [M, K], [N, K].  Small products of a long K sum it in two
+    halves (mxfp4.h): the last bits of a row may then differ from those of the same row in a larger product."""
     M, K = A_codes.shape
     N = B_codes.shape[0]
     if C_out is None:
@@ -392,7 +393,7 @@ def mxfp4_int4_quantize(x: torch.Tensor, reduce_dim: int, g: int, seed: int, str
 
 
 def mxfp4_int4_gemm(A_codes, A_scales, B_codes, B_scales, alpha: float = 1.0, out_dtype: int = OUT_BF16, C_out=None):
-    """C [M, N] = alpha * sum_k (q X)_A (q X)_B for MXINT4 operands [M, K], [N, K] (one byte per element)."""
+    """C [M, N] = alpha * sum_k (q X)_A (q X)_B for MXINT4 operands [M, K], [N, K] (one byte per element); sums as in ``mxfp4_fp8_gemm``."""
     M, K = A_codes.shape
     N = B_codes.shape[0]
     if C_out is None:

@@ -41,7 +41,8 @@
 // The 8-bit products (FP8 forward pass, MXINT4; enum Kind) run on the same roles: a one-CTA kernel of 128 x 256 tiles with
 // one accumulator and stores from registers served them before.  E4M3 16384 x 4096 x 4096: 221 -> 168 us (3.3 PFLOP/s,
 // twice the measured bf16 rate), 8192 x 3072 x 1024 50 -> 23, 16 x 4096 x 4096 16.5 -> 11.4; MXINT4
-// 16384 x 4096 x 4096 245 -> 178, 1024 x 1024 x 8192 34 -> 20.  It still serves few rows and many columns (gemm_f8.cu).
+// 16384 x 4096 x 4096 245 -> 178, 1024 x 1024 x 8192 34 -> 20.  Since then the issue above and the split products: 168 - 172, 20.3, 10.0 and 167, 13.2.
+// The one-CTA kernel still serves few rows and many columns (gemm_f8.cu).
 #include <cuda_bf16.h>
 
 #include <cstdlib>
@@ -60,10 +61,10 @@ constexpr uint32_t kEpiB = 8 * kEpiBuf;
 constexpr uint32_t kBarB = 256;
 constexpr int kThreadsP = 12 * 32;
 
-// Three builds of the kernel.  PN = 256 (256 x 256 pair tile): six operand stages (all 227 KB of shared memory), one
+// Four builds of the kernel.  PN = 256 (256 x 256 pair tile): six operand stages (all 227 KB of shared memory), one
 // 512-column TMEM allocation, every register of the SM.  PN = 128 (256 x 128): eight stages, and TMEM room for two
 // accumulators, so that a tile's MMAs run while the tile before is taken out; see gemm_pair_tile_n() for when it is the better
-// one.  LITE (PN = 256) leaves room for a second, independent kernel on the same SM (the tensor-core quantiser's small
+// one, and for its SPLIT form, of 8-bit products only, split_pays().  LITE (PN = 256) leaves room for a second, independent kernel on the same SM (the tensor-core quantiser's small
 // build, quantize_tc.cu, which quantises the OTHER product's operands meanwhile): four stages, TMEM taken as 256 + 128
 // columns, 104 registers per thread at launch.
 // Operand kinds: E2M1 with one UE8M0 scale per 32 elements (the method's GEMM); E4M3 with one scale per tensor (FP8 forward
@@ -650,9 +651,11 @@ double tile_cost(int pn, int64_t K) {
 
 // Whether an 8-bit product goes out with two pairs to a tile (SPLIT): its 128-wide tiles leave half of the pairs idle (32 clusters
 // of four SMs fit the chip's GPCs at once), and half of its K-steps take longer than the exchange, about 2 us.  Whole tiles / split
-// in us, 1024 x 1024 (512 x 2048, 2048 x 512 and 130 x 4096 the same within 0.2): MXINT4 K = 1024 6.6 / 7.4, 2048 8.3 / 8.3, 4096
-// 11.7 / 10.1, 8192 18.3 / 13.9; E4M3 6.7 / 7.3, 8.4 / 8.2, 11.8 / 10.0, 18.4 / 13.7.  MXFP4 products keep whole tiles: with twice the elements to a K-step they would
-// gain from K = 8192 on only (11.7 / 10.4), and their bits stay those of the one launch a backward call makes.
+// in us, 1024 x 1024 (512 x 2048 and 130 x 4096 the same within 0.3): MXINT4 K = 3072 8.9 / 8.8, 4096 10.5 / 9.8, 8192 17.1 / 13.2; E4M3 8.9 / 8.7, 10.6 / 9.5,
+// 17.1 / 12.8.  Below the line split lost: MXINT4 K = 1024 6.6 / 7.4, 2048 8.3 / 8.3 (as separate calls, a microsecond more each).
+// What it costs: the sum over K is then one of two halves, so the last bits of a row of an 8-bit product depend on how many rows and
+// columns are computed with it, as they do in no product of whole tiles (mxfp4.h says so).  MXFP4 products keep whole tiles: a backward
+// call's bits are those of its products one by one, and with twice the elements to a K-step they would gain from K = 8192 on only (11.7 / 10.4).
 constexpr int kSplitClusters = 32, kSplitSteps = 24;
 bool split_pays(int64_t M, int64_t N, int64_t steps) {
     return (int64_t)ceil_div(M, PM) * ceil_div(N, 128) <= kSplitClusters && steps >= kSplitSteps;
@@ -743,8 +746,8 @@ cudaError_t launch_gemm_pair(const GemmArgs* a, int n, int pn, cudaStream_t stre
 }
 
 // Columns of a pair tile for an 8-bit product: the width with which the last pair is done first.  Measured per tile: 0.36 us
-// a K-step + 0.1 (256 wide), 0.245 + 0.1 (128 wide).  128 wins where 256-wide tiles leave pairs idle (16 x 4096 x 4096:
-// 15.0 -> 11.4 us, 1024 x 1024 x 8192 26 -> 20), 256 elsewhere (16384 x 4096 x 4096: 168 us against 221).
+// a K-step + 0.1 (256 wide), 0.245 + 0.1 (128 wide).  E4M3, 256 / 128 wide: 128 wins where 256-wide tiles leave pairs idle (16 x 4096 x
+// 4096 13.8 / 10.2 us, 1024 x 1024 x 2048 9.8 / 7.3), 256 elsewhere (8192 x 3072 x 1024 20.3 / 26.9, 16384 x 4096 x 4096 170 / 236).
 int gemm_f8_tile_n(const Gemm8Args& a) {
     int pairs = 0;
     if (pair_count(&pairs) != cudaSuccess) return 256;

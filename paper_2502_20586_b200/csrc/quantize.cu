@@ -176,8 +176,10 @@ __global__ void __launch_bounds__(256) quantize_transpose_kernel(const __nv_bflo
 
 // ---------------------------------------------------------------------------------------------- launchers
 // Programmatic dependent launch (`chain`), as for the tensor-core kernels: the two quantisers and the GEMM of a small product come up
-// in the last wave of one another.  g = 0, both quantisers and the GEMM, RN / SR: 256 x 512 x 512 14.4 / 14.4 -> 10.2 / 10.6 us, 1024 x 1024 x 2048
-// 16.4 / 16.4 -> 12.7 / 14.6, 4096 x 2048 x 2048 23.9 / 26.7 -> 20.5 / 23.1 (2^18 blocks); 16384 x 8192 x 2048 (2^20 and 2^19) lost, 187.4 -> 191.1.
+// in the last wave of one another.  g = 0, both quantisers and the GEMM, fp32 result, RN / SR, without -> with, replayed as a graph: 256 x 512 x
+// 512 9.6 / 10.2 -> 8.3 / 8.9 us, 1024 x 1024 x 2048 11.6 / 12.8 -> 10.7 / 13.0, 4096 x 2048 x 2048 19.5 / 22.5 -> 18.1 / 21.0 (2^18 and 2^17 blocks; as separate
+// calls 24.2 / 27 -> 19.3 / 22.2).  Above the line nothing to gain: 8192 x 4096 x 2048 with its larger quantiser chained or not 48.2 / 52.3, 47.2 / 52.2;
+// 16384 x 8192 x 2048 155 - 158 / 185 - 189 in either form.
 constexpr int64_t kChainBlocks = int64_t(1) << 18;
 template <typename... Params, typename... Args>
 static cudaError_t launch_after(void (*kernel)(Params...), dim3 grid, cudaStream_t stream, bool chain, Args... args) {

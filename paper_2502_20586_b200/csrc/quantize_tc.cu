@@ -34,8 +34,9 @@
 //     four without one;
 //   - whole sectors of codes in one store (store_codes), SR through the convert (quantize_block32_rw), tiles described once
 //     (TileInfo), MMAs without T's zero blocks, T eight entries at a time (hadamard_row8).
-// 16384 x 16384 views, before the last five -> now: SR row-wise 124 -> 116 us, transposing 140 -> 116, g = 64 118 / 138 -> 108, g = 256 132 -> 128,
-// SR16 111 / 130 -> 107, RN 108 / 119 -> 105 (6.5 TB/s); the operands of a backward call, 16384 x 4096 x 4096 105 -> 95, 8192 x 1024 x 4096 38.5 -> 35.
+// 16384 x 16384 views, before the last five -> now, in bursts: SR row-wise 124 -> 112 us, transposing 140 -> 113, g = 64 118 / 138 -> 107, g = 256
+// 132 -> 125, SR16 111 / 130 -> 103 - 105, RN 108 / 119 -> 105 (6.5 TB/s); the operands of a backward call, 16384 x 4096 x 4096 105 -> 95 - 102 (g = 128),
+// 8192 x 1024 x 4096 38.5 -> 35 (g = 64).
 // Slower were: the block loop rolled up (SR 127), four groups with accumulators handed back by halves (128), TMEM loads a block
 // ahead (134), part of the Philox rounds folded into constants of the view (more moves than it saved: 96 instructions a block for 85), a fifth
 // stage (RN 110).
@@ -328,8 +329,9 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
             const uint64_t adesc = rowwise ? make_smem_desc(a_addr, 16, 1024, 2) : make_smem_desc(a_addr, kBoxBytes, 1024, 2);
             const uint32_t a_half = rowwise ? kBoxBytes >> 4 : 4 * 2048 >> 4, a_step = rowwise ? 32 >> 4 : 2048 >> 4;
             // T is block-diagonal with equal blocks: chunk c of the tile's 128 / g takes its own columns of A against the first block.
-            // (With the zero blocks multiplied as well the tensor cores did two or four times the work, at the board's power limit:
-            // g = 64, operands of 8192 x 1024 x 4096 41.0 -> 39.8 us, nearest rounding 32.6 -> 31.6; 16384 x 16384 SR 110 -> 108.)
+            // (With the zero blocks multiplied as well the tensor cores did two or four times the work, at the board's power limit.  g = 64,
+            // when that changed and other parts still took longer: operands of 8192 x 1024 x 4096 41.0 -> 39.8 us (now 35), nearest rounding
+            // 32.6 -> 31.6 (now 30 - 31); 16384 x 16384 SR 110 -> 108.)
 #pragma unroll
             for (uint32_t ks = 0; ks < 8; ++ks) {
                 const uint32_t c = ks >> lg_steps, kc = ks & ((1u << lg_steps) - 1u);
@@ -592,7 +594,7 @@ bool quant_tc_eligible(const QuantArgs& a) {
     const int64_t K = a.reduce_dim == 1 ? a.cols : a.rows;
     const int64_t R = a.reduce_dim == 1 ? a.rows : a.cols;
     const int64_t tiles = ((R + kTile - 1) / kTile) * (K / kTile);          // tile indices are 32-bit in the kernel
-    // the element index that keys the SR draws stays below 2^36 (the kernel folds a zero high counter word into its constants)
+    // below 2^36 elements the index of a block's two Philox calls fits the low counter word
     return (a.g == 32 || a.g == 64 || a.g == 128 || a.g == 256) && K % kTile == 0 && tiles < (int64_t(1) << 28) && a.has_tmap &&
            R * K < (int64_t(1) << 36);
 }
