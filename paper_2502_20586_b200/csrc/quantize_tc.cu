@@ -194,6 +194,14 @@ __device__ __forceinline__ void store_codes(uint8_t* dst, int j, const uint32_t 
         st_global_32B(dst + 16 * (j - 1), both, wide);
     }
 }
+// sum += the eight bf16 values of v, each widened exactly and added in fp32 (one instruction an element).
+__device__ __forceinline__ void add_bf16x8(float (&sum)[8], const uint4& v) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.f32.bf16 %0, lo, %0;\n\tadd.f32.bf16 %1, hi, %1;\n\t}"
+            : "+f"(sum[2 * i]), "+f"(sum[2 * i + 1]) : "r"(w[i]));
+}
 // Tiles (units) that a round-robin deal of n gives this CTA.
 __device__ __forceinline__ uint32_t tiles_of_cta(uint32_t n) { return blockIdx.x < n ? (n - blockIdx.x + gridDim.x - 1u) / gridDim.x : 0u; }
 
@@ -359,6 +367,7 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
                 }
             }
         } else {
+            const bool sums = KW == 1 && !LITE && p.col_sums != nullptr;
             for (uint32_t t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
                 int v = 0;
 #pragma unroll
@@ -375,6 +384,7 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
                         transform(s_addr + s * kTileBytes, rowwise, h, b);
                         tc_commit(&empty_bar[s]);
                         tc_commit(&acc_full[b]);
+                        if (sums && v != 0) mbar_arrive(&empty_bar[s], 2);   // in place of the two summing warps, which only read view 0
                     }
                     __syncwarp();
                 }
@@ -383,37 +393,52 @@ __device__ __forceinline__ void quantize_tc_body(const QMaps& maps, const QParam
         if (!ok && lane == 0) *abort_flag = 1;
     } else if (KW == 1 && !LITE && p.col_sums != nullptr) {
         // ------------------------------------------------------------------ warps 2, 3: column sums of the x tile (dL/db = 1 dL/dy)
-        // The tile is in shared memory anyway: warp w sums columns 64 w .. 64 w + 63 (one TMA box), a lane two adjacent
-        // columns (one 32-bit word per row; the 128-byte swizzle permutes 16-byte chunks inside a row, so a warp's 32
-        // words of a row still fall into 32 different banks), rows in order: a fixed summation order.  One partial sum
-        // per (128-row band of x, column); the GEMM launch adds the bands in order.  (A launch of several views: only the
-        // tiles of view 0, the row-wise view of dY, are summed; the others pass.)
+        // The tile is in shared memory anyway: warp w sums columns 64 w .. 64 w + 63 (one TMA box).  A lane takes eight adjacent columns
+        // (one 16-byte chunk, moved by the 128-byte swizzle; eight lanes read a whole row, so no bank conflicts) of every fourth row, rows
+        // in order; the four row groups are added pairwise: a fixed summation order.  One partial sum per (128-row band of x, column);
+        // the GEMM launch adds the bands in order.  (A launch of several views: only the tiles of view 0, the row-wise view of dY, are
+        // summed; for the others, which follow, the MMA issuer counts these warps' arrivals.)
+        // These two warps set the pace of view 0's tiles when they take long over one (each shares its scheduler with three epilogue warps):
+        // two columns a lane, 128 rows in a chain of additions and widening by shift and mask took 9 us of a call of 4096 x 2048 x 6144, and
+        // the other views' tiles passed through their hands as well.  Calls with db (without), before -> now, SR, fp32 results: 4096 x 2048 x
+        // 6144 86.0 -> 79.8 us (77.3), 8192 x 1024 x 4096 78.1 -> 70.3 (67.4), 8192 x 1024 x 1024 36.6 -> 33.9 (32.6), 4224 x 1000 x 1408 27.5 -> 25.3 (24.8).
         const int w = warp - 2;
+        const uint32_t chunk = (uint32_t)lane & 7u, rg = (uint32_t)lane >> 3;
+        const uint32_t off0 = rg * 128u + ((chunk ^ rg) << 4), off1 = (rg + 4u) * 128u + ((chunk ^ (rg + 4u)) << 4);   // rows rg and rg + 4
         uint32_t is = 0;
         bool ok = true;
-        for (uint32_t u = blockIdx.x; (DUAL ? 2u * u : u) < num_tiles; u += gridDim.x, ++is) {
+        for (uint32_t u = blockIdx.x; u < (DUAL ? num_tiles >> 1 : p.view[0].n_tiles); u += gridDim.x, ++is) {
             const int s = is % kStagesQ;
             ok = mbar_wait(&full_bar[s], (is / kStagesQ) & 1, abort_flag);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
-            if (!DUAL && u >= p.view[0].n_tiles) {
-                if (lane == 0) mbar_arrive(&empty_bar[s]);
-                continue;
-            }
             const uint8_t* box = smem + s * kTileBytes + w * kBoxBytes;
-            float s0 = 0.f, s1 = 0.f;
-#pragma unroll 8
-            for (int r = 0; r < kTile; ++r) {
-                const uint32_t v = *reinterpret_cast<const uint32_t*>(box + r * 128 + ((((lane >> 2) ^ (r & 7)) << 4) | ((lane & 3) << 2)));
-                s0 += __uint_as_float(v << 16);
-                s1 += __uint_as_float(v & 0xFFFF0000u);
+            float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+            for (int r = 0; r < kTile; r += 8) {
+                const uint4 a = *reinterpret_cast<const uint4*>(box + r * 128 + off0), b = *reinterpret_cast<const uint4*>(box + r * 128 + off1);
+                add_bf16x8(sum, a);
+                add_bf16x8(sum, b);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty_bar[s]);                   // this warp is done with the stage
+            // rows: groups 0 and 1, 2 and 3, then the two pairs; a lane ends up with two of its chunk's eight columns
+            const bool odd = (rg & 1u) != 0, high = (rg & 2u) != 0;
+            float half[4], quarter[2];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float got = __shfl_xor_sync(0xffffffffu, odd ? sum[i] : sum[4 + i], 8);
+                half[i] = (odd ? sum[4 + i] : sum[i]) + got;
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float got = __shfl_xor_sync(0xffffffffu, high ? half[i] : half[2 + i], 16);
+                quarter[i] = (high ? half[2 + i] : half[i]) + got;
+            }
             const TilePos pos = locate_tile<DUAL>(p, DUAL ? 2u * u : u);
             const uint32_t xr = row_tile(p.view[0], pos), xc = k_tile(p.view[0], pos);
-            float* dst = p.col_sums + (int64_t)xr * (32 * (int64_t)p.view[0].k_blocks) + (int64_t)xc * kTile + w * 64 + 2 * lane;
-            *reinterpret_cast<float2*>(dst) = make_float2(s0, s1);
+            float* dst = p.col_sums + (int64_t)xr * (32 * (int64_t)p.view[0].k_blocks) + (int64_t)xc * kTile + w * 64 + 8 * chunk + (odd ? 4 : 0) + (high ? 2 : 0);
+            *reinterpret_cast<float2*>(dst) = make_float2(quarter[0], quarter[1]);
         }
         if (!ok && lane == 0) *abort_flag = 1;
     }

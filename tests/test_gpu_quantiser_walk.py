@@ -219,6 +219,22 @@ def test_bias_gradient_inside_the_launches(b, n, m, dual, monkeypatch):
     assert gpu.mxfp4_device_status() == 0
 
 
+# Band sums of values whose fp32 sums are exact in any order (the largest and smallest bf16 exponents of small integers, subnormal
+# ones among them), and of infinities and NaN
+@pytest.mark.parametrize("scale", [2.0 ** -133, 2.0 ** -126, 1.0, 2.0 ** 100])
+@pytest.mark.parametrize("b,m,dual", [(128, 128, "0"), (384, 1152, "0"), (384, 1152, "2")])
+def test_band_sums_are_exact(scale, b, m, dual, monkeypatch):
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    monkeypatch.setenv("MXFP4_DUAL_DY", "1" if dual == "0" else dual)              # (0 sums in a pass of its own)
+    dY = (_small_integers((b, m), 5).double() * scale).to(torch.bfloat16)
+    assert torch.equal(dY.double(), _small_integers((b, m), 5).double() * scale)
+    dY[5, 3], dY[b - 1, m - 1], dY[7, 64], dY[9, 64] = float("inf"), float("nan"), float("inf"), -float("inf")
+    X, W = (torch.zeros(s, dtype=torch.bfloat16, device="cuda") for s in ((b, 8), (m, 8)))
+    db = gpu.mxfp4_linear_backward_ex(dY, X, W, 64, 5, gpu.ROUND_SR, gpu.OUT_FP32, with_bias=True)[2]
+    assert torch.equal(db.double().nan_to_num(7.0, 8.0, 9.0), dY.double().sum(0).nan_to_num(7.0, 8.0, 9.0))
+
+
 # An operand of eight rows with more than 2^23 scale tiles (its scales fill more than 4 GB), against the same quantiser on the
 # operand's first and last columns: nearest rounding, so the bytes do not depend on where a block lies
 @pytest.mark.parametrize("kind,reduce_dim,g", [("mxfp4", 1, 64), ("mxfp4", 0, 32), ("mxfp4", 1, 256), ("mxint4", 1, 128)])
