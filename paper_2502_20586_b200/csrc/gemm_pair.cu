@@ -251,26 +251,31 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
     reg_dealloc<Cfg::kRegsLight>();
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer (both CTAs)
-        if (lane == 0) {
-            uint32_t it = 0;
-            bool ok = true;
-            for (uint32_t tl = 0; tl < walk.count && ok; ++tl) {
-                int mt, nt;
-                const int w = walk.locate(p, tl, mt, nt);
-                const int end_kt = end_step(p.prob[w].num_kt);
-                const CUtensorMap *map_a = &maps.a[w], *map_b = &maps.b[w];
-                const int a_rt = 2 * mt + (int)rank;                            // this CTA's 128-row tile of A
-                for (int kt = first_step(p.prob[w].num_kt); kt < end_kt; ++kt, ++it) {
-                    const int s = it % kStagesP;
-                    if (!(ok = mbar_wait(&empty_bar[s], ((it / kStagesP) & 1) ^ 1, abort_flag))) break;
+        // The whole warp walks the loop and one elected lane issues, here and in the scale loader, as the MMA issuers do: from a lane-0 branch,
+        // with divisions by the ring's size, a step's loads took 425 cycles of this thread, more than a 128-wide tile's MMAs (256), and the ring
+        // filled as slowly at every start; now 240.  Before -> now: 1024 x 1024 x 8192 11.7 -> 11.2 us, 256 x 512 x 512 5.2 -> 5.0,
+        // 16384 x 4096 x 4096 98 -> 96.5, 16384 x 8192 x 2048 111 -> 108.5; backward 8192 x 1024 x 1024 29.1 -> 27.9.
+        uint32_t s = 0, ph = 1;
+        bool ok = true;
+        for (uint32_t tl = 0; tl < walk.count && ok; ++tl) {
+            int mt, nt;
+            const int w = walk.locate(p, tl, mt, nt);
+            const int end_kt = end_step(p.prob[w].num_kt);
+            const CUtensorMap *map_a = &maps.a[w], *map_b = &maps.b[w];
+            const int32_t a_row = (2 * mt + (int)rank) * 128, b_row = nt * PN + (int)rank * (PN / 2);   // this CTA's rows of A, half of B's
+            for (int kt = first_step(p.prob[w].num_kt); kt < end_kt; ++kt) {
+                if (!(ok = __all_sync(0xffffffffu, mbar_wait(&empty_bar[s], ph, abort_flag)))) break;
+                if (elect_one()) {
                     uint8_t* st = smem + s * kStageB;
                     if (rank == 0) mbar_expect_tx(&full_bar[s], 2 * (kStageB + kSfSlotB));   // operands and scales of both CTAs
-                    tma_load_2d_pair(st, map_a, &full_bar[s], kt * kGemmBKBytes, a_rt * 128);
-                    tma_load_2d_pair(st + kAB, map_b, &full_bar[s], kt * kGemmBKBytes, nt * PN + (int)rank * (PN / 2));
+                    tma_load_2d_pair(st, map_a, &full_bar[s], kt * kGemmBKBytes, a_row);
+                    tma_load_2d_pair(st + kAB, map_b, &full_bar[s], kt * kGemmBKBytes, b_row);
                 }
+                __syncwarp();
+                if (++s == (uint32_t)kStagesP) { s = 0; ph ^= 1; }
             }
-            if (!ok) *abort_flag = 1;
         }
+        if (!ok && lane == 0) *abort_flag = 1;
     } else if (warp == 1 || warp == 2) {
         // ------------------------------------------------------------------ MMA issuers (leader CTA only)
         // Two warps take the steps in turn (even steps warp 1, odd steps warp 2): while one issues its MMAs, the other has
@@ -381,8 +386,8 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
         // ------------------------------------------------------------------ scale loader (both CTAs)
         // One box = the one or two 512-byte scale tiles of a 128-row tile for this K-step (box rows past the operand read zeros; a
         // box that runs over the end of an odd K reads the next row tile's first, which no MMA uses).
-        if (lane == 0 && KIND != kF8) {
-            uint32_t it = 0;
+        if (KIND != kF8) {
+            uint32_t s = 0, ph = 1;
             bool ok = true;
             for (uint32_t tl = 0; tl < walk.count && ok; ++tl) {
                 int mt, nt;
@@ -390,17 +395,20 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
                 const int end_kt = end_step(p.prob[w].num_kt), nkc = p.prob[w].nkc;
                 const CUtensorMap *map_a = &maps.sfa[w], *map_b = &maps.sfb[w];
                 const int32_t a_row = (2 * mt + (int)rank) * nkc, b_row = nt * (PN / 128) * nkc;
-                for (int kt = first_step(p.prob[w].num_kt); kt < end_kt; ++kt, ++it) {
-                    const int s = it % kStagesP;
-                    if (!(ok = mbar_wait(&empty_bar[s], ((it / kStagesP) & 1) ^ 1, abort_flag))) break;
-                    uint8_t* dst = sf_ring + s * kSfSlotB;
-                    tma_load_2d_pair(dst, map_a, &full_bar[s], 0, a_row + Cfg::kSfTiles * kt);
+                for (int kt = first_step(p.prob[w].num_kt); kt < end_kt; ++kt) {
+                    if (!(ok = __all_sync(0xffffffffu, mbar_wait(&empty_bar[s], ph, abort_flag)))) break;
+                    if (elect_one()) {
+                        uint8_t* dst = sf_ring + s * kSfSlotB;
+                        tma_load_2d_pair(dst, map_a, &full_bar[s], 0, a_row + Cfg::kSfTiles * kt);
 #pragma unroll
-                    for (int j = 0; j < PN / 128; ++j)
-                        tma_load_2d_pair(dst + Cfg::kSfaB * (1 + j), map_b, &full_bar[s], 0, b_row + j * nkc + Cfg::kSfTiles * kt);
+                        for (int j = 0; j < PN / 128; ++j)
+                            tma_load_2d_pair(dst + Cfg::kSfaB * (1 + j), map_b, &full_bar[s], 0, b_row + j * nkc + Cfg::kSfTiles * kt);
+                    }
+                    __syncwarp();
+                    if (++s == (uint32_t)kStagesP) { s = 0; ph ^= 1; }
                 }
             }
-            if (!ok) *abort_flag = 1;
+            if (!ok && lane == 0) *abort_flag = 1;
         }
     }
     if (SPLIT) {                                            // the two barriers of the exchange below
