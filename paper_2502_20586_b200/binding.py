@@ -14,6 +14,10 @@ if not os.path.exists(LIB_PATH):
     raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2502_20586_b200.build` "
                       "(there is no CPU fallback)")
 _lib = C.CDLL(LIB_PATH)
+try:
+    from . import _host_calls
+except ImportError as e:
+    raise ImportError("the native host calls are missing: build them with `python -m paper_2502_20586_b200.build`") from e
 
 OK = 0
 ROUND_SR, ROUND_RN, ROUND_SR16 = 0, 1, 2
@@ -70,6 +74,8 @@ _lib.mxfp4_device_status.restype = _int
 _lib.mxfp4_status_string.argtypes = [_int]
 _lib.mxfp4_status_string.restype = C.c_char_p
 
+_host_calls.bind(C.cast(_lib.mxfp4_linear_backward_ex_workspace, _vp).value, C.cast(_lib.mxfp4_linear_backward_ex, _vp).value)
+
 EXPORTS = ["mxfp4_rht_sr_quantize", "mxfp4_rht", "mxfp4_gemm", "mxfp4_linear_backward_workspace",
            "mxfp4_linear_backward", "mxfp4_linear_backward_static", "mxfp4_scale_bytes", "mxfp4_device_status", "mxfp4_status_string",
            "mxfp4_fp4_ceiling", "mxfp4_linear_backward_ex_workspace", "mxfp4_linear_backward_ex", "mxfp4_gemm_fused",
@@ -107,6 +113,17 @@ def _empty(like, shape, dtype):
     if type(like) is torch.Tensor:
         return like.new_empty(shape, dtype=dtype)
     return torch.empty(shape, dtype=dtype, device=like.device)
+
+
+_PLAIN = {torch.Tensor, torch.nn.Parameter}
+
+
+def _plain(*tensors) -> bool:
+    """Whether the native host call (csrc/host_calls.cpp) takes these: tensors of no subclass, or None."""
+    for t in tensors:
+        if t is not None and type(t) not in _PLAIN:
+            return False
+    return True
 
 
 def lib():
@@ -250,6 +267,10 @@ def mxfp4_linear_backward_workspace(b: int, m: int, n: int) -> int:
 def mxfp4_linear_backward(dY, X, W, g: int, seed: int, rounding: int = ROUND_SR, out_dtype: int = OUT_BF16,
                           dX=None, dW=None, workspace=None):
     """Algorithm 3: dY [b, m], X [b, n], W [m, n] bf16 (contiguous)  ->  (dX [b, n], dW [m, n])."""
+    if dY is not None and X is not None and W is not None and _plain(dY, X, W, dX, dW, workspace):
+        status, dX, dW, _ = _host_calls.backward(dY, X, W, g, seed, rounding, out_dtype, dX, dW, None, False, False, workspace)
+        _check(status)
+        return dX, dW
     b, m = dY.shape
     _, n = X.shape
     for t in (dY, X, W):
@@ -275,6 +296,10 @@ def mxfp4_linear_backward_ex(dY, X, W, g: int, seed: int, rounding: int = ROUND_
                              dX=None, dW=None, db=None, with_bias: bool = False, accumulate: bool = False, workspace=None):
     """Algorithm 3 plus the bias gradient (fp32 [m], column sums of dY) and accumulation into fp32 dW / db.
     Returns (dX, dW, db) with db None unless with_bias or db is given."""
+    if dY is not None and X is not None and W is not None and _plain(dY, X, W, dX, dW, db, workspace):
+        status, dX, dW, db = _host_calls.backward(dY, X, W, g, seed, rounding, out_dtype, dX, dW, db, with_bias, accumulate, workspace)
+        _check(status)
+        return dX, dW, db
     b, m = dY.shape
     _, n = X.shape
     for t in (dY, X, W):

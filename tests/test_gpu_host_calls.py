@@ -1,0 +1,94 @@
+"""The native host call of a layer's backward (csrc/host_calls.cpp) against the Python one, which serves tensors of a subclass: the same
+bits, buffers, streams and refusals."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _layer(b=256, n=264, m=384):
+    import torch
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(b + n + m)
+    return [torch.randn(s, generator=gen, device="cuda").bfloat16() for s in ((b, m), (b, n), (m, n))]
+
+
+def _tagged(t):
+    import torch
+
+    class Tagged(torch.Tensor):
+        pass
+    return t.as_subclass(Tagged)
+
+
+@pytest.mark.parametrize("seed", [0, -1, 2 ** 64 - 1, 2 ** 64 + 5])
+@pytest.mark.parametrize("out_dtype", [0, 1])
+@pytest.mark.parametrize("with_bias", [False, True])
+def test_both_host_paths_give_the_same(seed, out_dtype, with_bias):
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    dY, X, W = _layer()
+    want = gpu.mxfp4_linear_backward_ex(_tagged(dY), X, W, 64, seed, 0, out_dtype, with_bias=with_bias)
+    got = gpu.mxfp4_linear_backward_ex(dY.requires_grad_(True), X, torch.nn.Parameter(W), 64, seed, 0, out_dtype, with_bias=with_bias)
+    plain = gpu.mxfp4_linear_backward(dY, X, W, 64, seed, 0, out_dtype)
+    for a, b in zip(want, got):
+        assert (a is None and b is None) or (type(b) is torch.Tensor and a.dtype == b.dtype and torch.equal(a, b) and not b.requires_grad)
+    assert torch.equal(plain[0], want[0]) and torch.equal(plain[1], want[1])
+    with torch.cuda.stream(torch.cuda.Stream()):
+        side = gpu.mxfp4_linear_backward(dY, X, W, 64, seed, 0, out_dtype, dX=torch.empty_like(want[0]), dW=torch.empty_like(want[1]))
+        torch.cuda.current_stream().synchronize()
+    assert torch.equal(side[0], want[0]) and torch.equal(side[1], want[1]) and gpu.mxfp4_device_status() == 0
+
+
+def test_buffers_of_the_caller_come_back():
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    dY, X, W = _layer()
+    dX, dW, db = (torch.zeros(s, device="cuda") for s in ((256, 264), (384, 264), (384,)))
+    ws = torch.empty(gpu.mxfp4_linear_backward_ex_workspace(256, 384, 264, True), dtype=torch.uint8, device="cuda")
+    out = gpu.mxfp4_linear_backward_ex(dY, X, W, 64, 3, 0, 1, dX=dX, dW=dW, db=db, accumulate=True, workspace=ws)
+    assert out[0] is dX and out[1] is dW and out[2] is db
+    ref = gpu.mxfp4_linear_backward_ex(dY, X, W, 64, 3, 0, 1, with_bias=True)
+    assert torch.equal(ref[0], dX) and torch.equal(ref[1], dW) and torch.equal(ref[2], db)      # accumulated onto zeros
+
+
+def test_refusals():
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    dY, X, W = _layer()
+    for bad in ((dY.float(), X, W), (dY, X.cpu(), W), (dY, X, W.t()), (dY[:, ::2], X, W)):
+        with pytest.raises(AssertionError):
+            gpu.mxfp4_linear_backward(*bad, 64, 0)
+    with pytest.raises(ValueError):
+        gpu.mxfp4_linear_backward(dY.view(2, 128, 384), X, W, 64, 0)
+    with pytest.raises(AssertionError):
+        gpu.mxfp4_linear_backward_ex(dY, X, W, 64, 0, 0, 1, accumulate=True)
+    with pytest.raises(gpu.MxFp4Error) as e:
+        gpu.mxfp4_linear_backward(dY, X, W, 48, 0)
+    assert e.value.code == 4
+    with pytest.raises(gpu.MxFp4Error) as e:
+        gpu.mxfp4_linear_backward(dY, X, W, 64, 0, workspace=torch.empty(16, dtype=torch.uint8, device="cuda"))
+    assert e.value.code == 6
+    with pytest.raises(TypeError):
+        gpu.mxfp4_linear_backward(dY, X, W, 64.0, 0)
+    with pytest.raises(RuntimeError):                        # a batched tensor has no memory of its own
+        torch.vmap(lambda d: gpu.mxfp4_linear_backward(d, X, W, 64, 0)[0])(dY[None])
+    del dY, X, W
+    free = torch.cuda.mem_get_info()[0]
+    wide = torch.empty(1, dtype=torch.bfloat16, device="cuda").expand(1 << 20, 1 << 20)         # expanded: not contiguous
+    with pytest.raises(AssertionError):
+        gpu.mxfp4_linear_backward(wide, wide, wide, 64, 0)
+    assert torch.cuda.mem_get_info()[0] >= free - (64 << 20) and gpu.mxfp4_device_status() == 0
+
+
+def test_out_of_memory_is_an_exception():
+    """The results of a small input that do not fit the device: torch's own exception, and the library keeps working."""
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    n = 1 << 27                                              # dX of 2^21 x 2^27 would be 2^49 bytes
+    dY = torch.zeros((1 << 21, 128), dtype=torch.bfloat16, device="cuda")
+    X = torch.zeros((1, n), dtype=torch.bfloat16, device="cuda")        # (only its width is looked at before the results are allocated)
+    with pytest.raises(torch.OutOfMemoryError):
+        gpu.mxfp4_linear_backward(dY, X, X[:, :128].contiguous(), 64, 0)
+    dY, X, W = _layer()
+    gpu.mxfp4_linear_backward(dY, X, W, 64, 0)
+    assert gpu.mxfp4_device_status() == 0
