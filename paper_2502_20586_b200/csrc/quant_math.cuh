@@ -258,11 +258,14 @@ __device__ __forceinline__ void quantize_block32_rw(const float (&y)[32], const 
 // Quantise 32 consecutive fp32 values to MXINT4: integers -7..7 as E4M3 bytes (the tensor core reads them as E4M3) + one
 // E8M0 byte.  Scale: the rule of Algorithms 1 / 2 with emax_elem = 2 (largest power of two among the elements is 4).
 //   SR (Algorithm 2): w = (3/4) |v| / X < 6, rounded on the integer grid with the dither of Eq. 1-2 discretised to the
-//     element's 8-bit draw r: up iff 256 frac >= r + 1/2.  Exactly: a = 128 |v| / X is a power-of-two scaling, one fused
-//     multiply-add toward zero forms 2^23 + floor(3 a) = 2^23 + floor(512 w), and adding 511 - 2 r carries into bit 9
-//     exactly when the low nine bits are at least 2 r + 1: the rounded integer stands in bits 9..11.
-//   RN (Algorithm 1): nearest integer, ties to even, saturating at 7; 2^23 + a rounded to nearest holds it in its low bits.
-// Four integers at a time are the selectors of one byte permute of the table of E4M3 bytes 0, 1, .. 7.
+//     element's 8-bit draw r: up iff 256 frac >= r + 1/2, so the result is floor(w + (511 - 2 r) / 512).  Exactly: one fused
+//     multiply-add toward zero forms 2^14 + (511 - 2 r) / 512 + w in units of 1/512 (the first two are such units, so the truncation
+//     is w's), and the integer stands in bits 9..11.  3/4 / X is a normal fp32 for every finite block.
+//   RN (Algorithm 1): nearest integer, ties to even, saturating at 7; 2^23 + |v| / X rounded to nearest holds it in its low bits.
+//     (|v| / X is exact, or so small that it rounds to 0 either way.)
+// The byte of each result that holds its integer is gathered, the four integers become the selectors of one byte permute of the table
+// of E4M3 bytes 0, 1, .. 7.  About 8 instructions an element; with two scalings, a shift, a mask and an insertion for each integer 11 (SR,
+// values and codes of 512 x 4096 7.8 -> 7.3 us, 1024 x 8192 20.9 -> 20.7, 8192 x 8192 91.5 -> 88.4; RN 6.9 -> 6.4, 19.2 -> 19.4, 85.7 -> 85.7).
 template <bool SR>
 __device__ __forceinline__ void quantize_block32_int4(const float (&v)[32], const uint32_t (&rw)[8], uint32_t (&out)[8], uint32_t& scale_byte) {
     scale_byte = e8m0_from_amax(block_amax(v));
@@ -271,20 +274,21 @@ __device__ __forceinline__ void quantize_block32_int4(const float (&v)[32], cons
         for (int i = 0; i < 8; ++i) out[i] = 0u;
         return;
     }
-    const int sh = (SR ? 7 : 0) - ((int)scale_byte - 127);              // |v| 2^sh, in two exact steps
-    const float p1 = pow2f_wide(sh / 2), p2 = pow2f_wide(sh - sh / 2);
+    // 3/4 * 2^-e or 2^-e
+    const float c = __uint_as_float(SR ? ((253u << 23) | 0x400000u) - (scale_byte << 23) : (254u - scale_byte) << 23);
 #pragma unroll
     for (int w = 0; w < 8; ++w) {
-        uint32_t sel = 0u, sign[4];
+        uint32_t u[4], sign[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const float y = v[4 * w + j], a = fabsf(y) * p1 * p2;
-            uint32_t q;
-            if (SR) q = ((__float_as_uint(__fmaf_rz(a, 3.0f, 8388608.0f)) + 511u - 2u * ((rw[w] >> (8 * j)) & 0xFFu)) >> 9) & 7u;
-            else q = __float_as_uint(__fadd_rn(fminf(a, 7.0f), 8388608.0f)) & 7u;
-            sel |= q << (4 * j);
+            const float y = v[4 * w + j];
+            if (SR) u[j] = __float_as_uint(__fmaf_rz(fabsf(y), c, __uint_as_float(0x468001FFu - 2u * ((rw[w] >> (8 * j)) & 0xFFu))));
+            else u[j] = __float_as_uint(__fadd_rn(fminf(fabsf(y) * c, 7.0f), 8388608.0f));
             sign[j] = __float_as_uint(y);
         }
+        const uint32_t b01 = __byte_perm(u[0], u[1], SR ? 0x0051 : 0x0040), b23 = __byte_perm(u[2], u[3], SR ? 0x0051 : 0x0040);
+        const uint32_t b = __byte_perm(b01, b23, 0x5410), q = (SR ? b >> 1 : b) & 0x07070707u;
+        const uint32_t sel = __byte_perm(q | (q >> 4), 0u, 0x4420);      // one integer a nibble
         const uint32_t s01 = __byte_perm(sign[0], sign[1], 0x0073), s23 = __byte_perm(sign[2], sign[3], 0x0073);   // top bytes
         out[w] = __byte_perm(0x44403800u, 0x4E4C4A48u, sel) | (__byte_perm(s01, s23, 0x5410) & 0x80808080u);
     }
