@@ -127,6 +127,28 @@ def test_int4_quantiser_bit_exact_on_gpu_values(gpu, ref, g, reduce_dim, shape, 
     assert np.array_equal(_int4_codes_from_e4m3(codes.cpu().numpy()), oc)
 
 
+# A block for every exponent that a scale can have, subnormal blocks and the largest finite ones among them; in each, ties of the integer
+# grid, values just beside them, zeros of both signs and values far below the scale
+@pytest.mark.parametrize("g,top", [(0, 127), (64, 119)])                       # (a transform of 64 can be eight times the largest element)
+@pytest.mark.parametrize("rounding", [0, 1])
+def test_int4_rounding_at_every_scale(gpu, ref, g, top, rounding):
+    rng = np.random.default_rng(g + rounding)
+    exps = np.arange(-133, top + 1)
+    v = rng.integers(-255, 256, (exps.size, 128)).astype(np.float64) / 128.0     # eight bits: exact in bf16 where the exponent allows
+    v[:, ::7] = np.clip(np.round(v[:, ::7] * 4.0) / 4.0, -1.75, 1.75)
+    v[:, 5::32] *= 2.0 ** -30
+    v[:, 9::32], v[:, 10::32], v[:, 0] = 0.0, -0.0, 1.984375
+    x = (np.ldexp(v, exps[:, None])).astype(np.float32).view(np.uint32) >> 16
+    codes, scales, y = gpu.mxfp4_int4_quantize(_dev(x.astype(np.uint16)), 1, g, 55, 3, rounding)
+    assert gpu.mxfp4_device_status() == 0
+    y = y.cpu().numpy()
+    assert np.isfinite(y).all()
+    oc, os_ = ref.mxint4_quantize(y, rounding, 55, 3)
+    assert os_.min() == 0 and os_.max() >= top + 127 - 4
+    assert np.array_equal(hp.sf_native_to_linear(scales.cpu().numpy(), *y.shape), os_)
+    assert np.array_equal(_int4_codes_from_e4m3(codes.cpu().numpy()), oc)
+
+
 @pytest.mark.parametrize("M,N,K", [(128, 256, 128), (200, 264, 640), (1, 8, 128), (384, 1032, 2176)])
 def test_int4_gemm_matches_fp64_product(gpu, ref, M, N, K):
     import torch
