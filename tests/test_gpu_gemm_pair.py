@@ -42,6 +42,25 @@ def test_tile_walk(gpu, M, N, K, fp32):
     assert torch.all((got.double() - want).abs() <= tol * (a.abs() @ b.abs().t() if fp32 else want.abs()) + 1e-30)
 
 
+# One tile to a pair, whose columns the two epilogue groups share in the 8-bit builds, against the same rows in a product of several tiles to
+# a pair, whose groups take whole tiles: the same bits.  128-wide tiles and (E4M3) 256-wide ones, ragged rows and columns
+@pytest.mark.parametrize("rows,more,N,K", [(200, 9000, 264, 256), (257, 19000, 136, 384), (512, 12000, 1000, 128)])
+@pytest.mark.parametrize("out", [0, 1])
+def test_single_tile_of_a_pair(gpu, rows, more, N, K, out):
+    import torch
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(rows + N + K)
+    ca, sa, _ = _operand(gen, more, K)
+    cb, sb, _ = _operand(gen, N, K)
+    few = sa[:(rows + 127) // 128 * ((K + 127) // 128) * 512]
+    assert torch.equal(gpu.mxfp4_gemm(ca[:rows], few, cb, sb, 1.5, out), gpu.mxfp4_gemm(ca, sa, cb, sb, 1.5, out)[:rows])
+    a, b = (torch.randint(0, 0x60, (n, K), generator=gen, device="cuda", dtype=torch.uint8) for n in (more, N * 4))      # E4M3, finite
+    one = torch.ones(2, device="cuda")
+    assert torch.equal(gpu.mxfp4_fp8_gemm(a[:rows], one, b, one, out), gpu.mxfp4_fp8_gemm(a, one, b, one, out)[:rows])
+    assert torch.equal(gpu.mxfp4_int4_gemm(a[:rows], few, b[:N], sb, 1.5, out), gpu.mxfp4_int4_gemm(a, sa, b[:N], sb, 1.5, out)[:rows])
+    assert gpu.mxfp4_device_status() == 0
+
+
 # The two products of a backward call go out as one launch: tile counts below and above the number of pairs (74), equal
 # and unequal K, a first product that leaves some pairs with one tile more than the rest, both tile widths, ragged edges.
 @pytest.mark.parametrize("b,n,m", [(256, 512, 512), (384, 8, 256), (8192, 1024, 1024), (8192, 1024, 3072), (4224, 1000, 1408), (1024, 4096, 4096),
