@@ -200,6 +200,29 @@ def test_refused_launch_leaves_no_error_behind():
     assert gpu.mxfp4_device_status() == 0 and not torch.any(codes) and not torch.any(scales)
 
 
+# As many tiles as the chip has SMs (half tiles to the epilogue groups) and one more (whole tiles): the rows that both have, row-wise and
+# transposing, in either scale layout, a last tile of a few rows
+@pytest.mark.parametrize("K,g", [(128, 64), (256, 128), (512, 32)])
+@pytest.mark.parametrize("rounding", [0, 2])
+@pytest.mark.parametrize("layout", [0, 1])
+def test_half_tiles(K, g, rounding, layout):
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rows = sms // (K // 128) * 128
+    x = _small_integers((rows + 128, K), K + g)
+    whole, scales = gpu.mxfp4_rht_sr_quantize(x, 1, g, 7, 3, rounding, layout)
+    for n in (rows, rows - 100, 40):
+        for y, dim in ((x[:n], 1), (x[:n].t()[:, :n // 8 * 8].contiguous(), 0)):
+            codes, s = gpu.mxfp4_rht_sr_quantize(y, dim, g, 7, 3, rounding, layout)
+            n_rows = codes.shape[0]
+            assert torch.equal(codes, whole[:n_rows])
+            per = K // 32 if layout == gpu.SF_LINEAR else K * 4                      # scales of a row, of a tile of 128 rows
+            full = n_rows if layout == gpu.SF_LINEAR else n_rows // 128
+            assert torch.equal(s[:full * per], scales[:full * per])
+    assert gpu.mxfp4_device_status() == 0
+
+
 # The bias gradient's two passes inside the launches of a backward call: band sums in the one-list and in the one-read form,
 # added up by the GEMM launch; against fp64, overwriting and accumulating
 @pytest.mark.parametrize("b,n,m", [(128, 264, 128), (640, 8, 1152), (2048, 1000, 5120)])
