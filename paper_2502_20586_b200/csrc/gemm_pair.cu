@@ -179,11 +179,6 @@ __device__ __forceinline__ void tc_mma_mxf8_pair(uint32_t d_tmem, uint64_t a_des
         : "memory");
 }
 
-template <int N>
-struct Count {                                              // a number known at compile time, as an argument
-    static constexpr int value = N;
-};
-
 // SPLIT: two pairs of a 4-CTA cluster share ONE output tile, each with half of its K-steps (see split_pays and the epilogue).
 template <Kind KIND, bool LITE, int PN, bool SPLIT = false>
 __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP& p) {
@@ -428,11 +423,6 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
         // the groups take alternate tiles, each its own accumulator.
         const int q = warp & 3, half = (warp - 4) >> 2;
         uint8_t* stage = epi_ring + (warp - 4) * kEpiBuf;
-        // One tile to this pair (8-bit builds): the groups share it, half of its columns each, instead of one taking it and the other nothing.
-        // Whole E4M3 forward passes, tokens x out x in: 1000 x 4096 x 1024 17.4 -> 17.0 us, 2000 x 2048 x 1024 15.2 -> 14.8, 4096 x 1024 x 2048 22.1 ->
-        // 21.6.  Not the MXFP4 builds: a backward call of 256 x 512 x 512 gained (9.75 -> 9.4), 8192 x 1024 x 1024 (28.65 -> 28.9) and 1024 x 1024 x 8192
-        // (29.0 -> 30.2), where some pairs have one tile and others several, lost.
-        const bool shared = KIND != kMxf4 && kAccBufs == 2 && walk.count == 1;
         const uint64_t pol_c = l2_policy_evict_first();         // the output is not read again here: let the operands keep L2
         bool ok = true;
         // One staged block: 16 registers = 64 bytes of this lane's row, columns [col, col + 64 B), into this warp's buffer
@@ -510,34 +500,77 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
                     put(o, map, false, (int32_t)col, (int32_t)row0, in_range);
                 }
             }
+        } else if (KIND != kMxf4 && kAccBufs == 2 && walk.count == 1) {
+            // One tile to this pair (8-bit builds): the groups share it, half of its columns each, instead of one taking it and the other nothing.
+            // Whole E4M3 forward passes, tokens x out x in: 1000 x 4096 x 1024 17.4 -> 16.8 us, 2000 x 2048 x 1024 15.2 -> 14.7, 4096 x 1024 x 2048
+            // 22.1 -> 21.6.  Code of its own: woven into the loop below it cost the other builds (backward 8192 x 1024 x 1024 27.9 -> 28.3).  Not the
+            // MXFP4 builds: a backward call of 256 x 512 x 512 gained (9.75 -> 9.4), 8192 x 1024 x 1024 (28.65 -> 28.9) and 1024 x 1024 x 8192
+            // (29.0 -> 30.2), where some pairs have one tile and others several, lost.
+            int mt, nt;
+            walk.locate(p, 0, mt, nt);
+            const ProblemP& pr = p.prob[0];
+            const CUtensorMap* map = &maps.c[0];
+            ok = __all_sync(0xffffffffu, mbar_wait_spin(&tmem_full[0], 0, abort_flag));
+            if (ok) {
+                tc_fence_after_sync();
+                constexpr int kChunks = PN / 64;                     // of 32 columns
+                const int64_t row0 = (int64_t)mt * PM + (int64_t)rank * 128 + q * 32, col0 = (int64_t)nt * PN + half * (PN / 2);
+                const float alpha = KIND == kF8 ? 1.0f / (*pr.scale_a * *pr.scale_b) : pr.alpha;
+                uint32_t r[kChunks][32];
+#pragma unroll
+                for (int c = 0; c < kChunks; ++c) tmem_ld_32x32b_x32(tmem_acc + ((uint32_t)(q * 32) << 16) + half * (PN / 2) + c * 32, r[c]);
+                tmem_ld_wait();
+#pragma unroll
+                for (int c = 0; c < kChunks; ++c) {
+                    const int64_t col = col0 + c * 32;
+                    const bool in_range = row0 < pr.M && col < pr.N;
+                    uint32_t o[16];
+                    if (pr.out_fp32) {
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) o[j] = __float_as_uint(__uint_as_float(r[c][16 * h + j]) * alpha);
+                            put(o, map, false, (int32_t)col + 16 * h, (int32_t)row0, in_range && col + 16 * h < pr.N);
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(r[c][2 * j]) * alpha,
+                                                                           __uint_as_float(r[c][2 * j + 1]) * alpha);
+                            o[j] = *reinterpret_cast<const uint32_t*>(&h);
+                        }
+                        put(o, map, false, (int32_t)col, (int32_t)row0, in_range);
+                    }
+                }
+            }
         } else
-        for (uint32_t tl = kAccBufs == 2 && !shared ? half : 0; tl < walk.count; tl += kAccBufs) {
+        for (uint32_t tl = kAccBufs == 2 ? half : 0; tl < walk.count; tl += kAccBufs) {
             int mt, nt;
             const int w = walk.locate(p, tl, mt, nt);
             const ProblemP& pr = p.prob[w];
             const CUtensorMap* map = &maps.c[w];
-            const uint32_t buf = tl % kAccBufs;
+            const uint32_t buf = kAccBufs == 2 ? half : 0;
             ok = __all_sync(0xffffffffu, mbar_wait_spin(&tmem_full[buf], (tl / kAccBufs) & 1, abort_flag));
             if (!ok) break;
             tc_fence_after_sync();
             const int64_t row0 = (int64_t)mt * PM + (int64_t)rank * 128 + q * 32;
+            const uint32_t taddr = tmem_acc + ((uint32_t)(q * 32) << 16) + half * Cfg::kWarpCols;   // (two accumulators: its own, kWarpCols = PN)
             constexpr int kBatches = Cfg::kWarpCols / 32 / Cfg::kBatch;
-            const int from = kAccBufs == 1 || shared ? half * (PN / 2) : 0;      // this warp's first column of the tile
-            const uint32_t taddr = tmem_acc + ((uint32_t)(q * 32) << 16) + buf * PN + from;
             const float alpha = KIND == kF8 ? 1.0f / (*pr.scale_a * *pr.scale_b) : pr.alpha;
-            // `chunks` x 32 columns: all of them into registers, then out
-            auto take = [&](auto chunks, uint32_t src, int64_t colb, bool hand_back) {
-                uint32_t r[chunks.value][32];
+#pragma unroll 1
+            for (int hb = 0; hb < kBatches; ++hb) {
+                uint32_t r[Cfg::kBatch][32];
 #pragma unroll
-                for (int c = 0; c < chunks.value; ++c) tmem_ld_32x32b_x32(src + c * 32, r[c]);
+                for (int c = 0; c < Cfg::kBatch; ++c) tmem_ld_32x32b_x32(taddr + (hb * Cfg::kBatch + c) * 32, r[c]);
                 tmem_ld_wait();
-                if (hand_back) {                         // the accumulator is in registers: the next tile's MMAs may start
+                if (hb == kBatches - 1) {                // the accumulator is in registers: the next tile's MMAs may start
                     tc_fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive_cluster(&tmem_empty[buf], 0);
                 }
+                const int64_t colb = (int64_t)nt * PN + (kAccBufs == 1 ? half * Cfg::kWarpCols : 0) + hb * Cfg::kBatch * 32;
 #pragma unroll
-                for (int c = 0; c < chunks.value; ++c) {
+                for (int c = 0; c < Cfg::kBatch; ++c) {
                     const int64_t col = colb + c * 32;
                     const bool in_range = row0 < pr.M && col < pr.N;
                     uint32_t o[16];
@@ -558,13 +591,6 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
                         put(o, map, false, (int32_t)col, (int32_t)row0, in_range);
                     }
                 }
-            };
-            const int64_t col0 = (int64_t)nt * PN + from;
-            if (KIND != kMxf4 && kAccBufs == 2 && shared) {
-                take(Count<PN / 64>(), taddr, col0, false);
-            } else {
-#pragma unroll 1
-                for (int hb = 0; hb < kBatches; ++hb) take(Count<Cfg::kBatch>(), taddr + hb * Cfg::kBatch * 32, col0 + hb * Cfg::kBatch * 32, hb == kBatches - 1);
             }
         }
         if (lane == 0) bulk_wait_group<0>();                         // every store has left shared memory and is visible
