@@ -41,6 +41,16 @@ bool integer(PyObject* o, uint64_t* out) {
     return *out != ~uint64_t(0) || PyErr_Occurred() == nullptr;
 }
 
+// Other Python threads run while one of these lives, an exception included.  It goes around the allocations as well as the library: one
+// that the caching allocator has no block for frees others and waits for the GPU, where a host callback may need the interpreter.
+struct NoGil {
+    PyThreadState* thread = PyEval_SaveThread();
+    NoGil() = default;
+    NoGil(const NoGil&) = delete;
+    NoGil& operator=(const NoGil&) = delete;
+    ~NoGil() { PyEval_RestoreThread(thread); }
+};
+
 // backward(dY, X, W, g, seed, rounding, out_dtype, dX, dW, db, with_bias, accumulate, workspace) -> (status, dX, dW, db): Algorithm 3.
 // None for dX, dW, db (with_bias) or workspace: made here.
 PyObject* backward(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
@@ -72,23 +82,22 @@ PyObject* backward(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
     const auto like = dY.options().requires_grad(false);
     auto given = [&](int i) { return args[i] == Py_None ? at::Tensor() : THPVariable_Unpack(args[i]); };
     at::Tensor dX = given(7), dW = given(8), db = given(9), workspace = given(12);
-    const auto result = like.dtype((int)out_dtype == 1 ? at::kFloat : at::kBFloat16);
-    if (!dX.defined()) dX = at::empty({b, n}, result);
     if (accumulate != 0 && (!dW.defined() || (with_bias != 0 && !db.defined()))) {
         PyErr_SetString(PyExc_AssertionError, "accumulation needs an existing dW, and db");
         return nullptr;
     }
-    if (!dW.defined()) dW = at::empty({m, n}, result);
-    if (with_bias != 0 && !db.defined()) db = at::empty({m}, like.dtype(at::kFloat));
-    if (!workspace.defined()) workspace = at::empty({(int64_t)g_workspace(b, m, n, db.defined() ? 1 : 0)}, like.dtype(at::kByte));
-    const void *p_dY = dY.data_ptr(), *p_X = X.data_ptr(), *p_W = W.data_ptr();
-    void *p_dX = dX.data_ptr(), *p_dW = dW.data_ptr(), *p_db = db.defined() ? db.data_ptr() : nullptr, *p_ws = workspace.data_ptr();
-    void* stream = c10::cuda::getCurrentCUDAStream().stream();
     int status;
-    Py_BEGIN_ALLOW_THREADS
-    status = g_backward(p_dY, p_X, p_W, b, m, n, (int)g, (int)rounding, seed, p_dX, p_dW, static_cast<float*>(p_db), (int)out_dtype, accumulate, p_ws,
-                        (size_t)workspace.numel(), stream);
-    Py_END_ALLOW_THREADS
+    {
+        const NoGil others_run;
+        const auto result = like.dtype((int)out_dtype == 1 ? at::kFloat : at::kBFloat16);
+        if (!dX.defined()) dX = at::empty({b, n}, result);
+        if (!dW.defined()) dW = at::empty({m, n}, result);
+        if (with_bias != 0 && !db.defined()) db = at::empty({m}, like.dtype(at::kFloat));
+        if (!workspace.defined()) workspace = at::empty({(int64_t)g_workspace(b, m, n, db.defined() ? 1 : 0)}, like.dtype(at::kByte));
+        status = g_backward(dY.data_ptr(), X.data_ptr(), W.data_ptr(), b, m, n, (int)g, (int)rounding, seed, dX.data_ptr(), dW.data_ptr(),
+                            db.defined() ? static_cast<float*>(db.data_ptr()) : nullptr, (int)out_dtype, accumulate, workspace.data_ptr(),
+                            (size_t)workspace.numel(), c10::cuda::getCurrentCUDAStream().stream());
+    }
     PyObject* out[4] = {PyLong_FromLong(status), nullptr, nullptr, nullptr};
     const at::Tensor* made[3] = {&dX, &dW, &db};
     for (int i = 0; i < 3; ++i) {

@@ -92,3 +92,45 @@ def test_out_of_memory_is_an_exception():
     dY, X, W = _layer()
     gpu.mxfp4_linear_backward(dY, X, W, 64, 0)
     assert gpu.mxfp4_device_status() == 0
+
+
+def test_other_threads_run_while_a_call_allocates():
+    """A result for which the caching allocator first has to free blocks, which waits for the GPU (a torch kernel of about half a
+    second): another Python thread keeps running all the while."""
+    import threading
+    import time
+
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    torch.cuda.empty_cache()                                                    # no room left over from another test's segments
+    dY, X, W = (torch.zeros(s, dtype=torch.bfloat16, device="cuda") for s in ((4096, 128), (4096, 4096), (128, 4096)))
+    dW = torch.empty((128, 4096), device="cuda")
+    workspace = torch.empty(gpu.mxfp4_linear_backward_workspace(4096, 128, 4096), dtype=torch.uint8, device="cuda")
+    call = lambda: gpu.mxfp4_linear_backward(dY, X, W, 64, 0, gpu.ROUND_SR, gpu.OUT_FP32, dW=dW, workspace=workspace)[0]
+    call()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    blocks = [torch.empty(48 << 20, dtype=torch.uint8, device="cuda") for _ in range(2)]      # dX takes 64 MB: neither will do
+    del blocks
+    ticks, stop = [], threading.Event()
+
+    def tick():
+        while not stop.is_set():
+            ticks.append(time.perf_counter())
+            time.sleep(0.001)
+    other = threading.Thread(target=tick)
+    torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + (16 << 20)) / torch.cuda.mem_get_info()[1])
+    try:
+        other.start()
+        torch.cuda._sleep(10 ** 9)
+        start = time.perf_counter()
+        dX = call()
+        end = time.perf_counter()
+    finally:
+        stop.set()
+        other.join()
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    seen = [start, *(t for t in ticks if start < t < end), end]
+    assert end - start > 0.2                                                    # the call did wait
+    assert max(b - a for a, b in zip(seen, seen[1:])) < 0.5 * (end - start)
+    assert not torch.any(dX) and gpu.mxfp4_device_status() == 0
