@@ -10,6 +10,8 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmxfp4_b200.so")
 HOST = os.path.join(HERE, "_host_calls.so")
 HOST_SOURCE = os.path.join(CSRC, "host_calls.cpp")
+INCLUDE = os.path.join(os.path.dirname(HERE), "include")
+HEADER = os.path.join(INCLUDE, "mxfp4.h")
 SOURCES = ["api.cu", "gemm.cu", "gemm_pair.cu", "gemm_fused.cu", "quantize.cu", "quantize_tc.cu", "static_workspace.cu", "fp4_ceiling.cu", "bias_grad.cu", "gemm_f8.cu", "variants.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden", "--expt-relaxed-constexpr"]
@@ -19,22 +21,30 @@ def _stale() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".cpp")] + [os.path.join(HERE, "..", "include", "mxfp4.h")]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".cpp")] + [HEADER]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
-def build_host(force: bool = False) -> str:
-    """The binding's host calls: C++ against the headers and libraries of the torch that imports them."""
-    if not force and os.path.exists(HOST) and os.path.getmtime(HOST) >= os.path.getmtime(HOST_SOURCE):
-        return HOST
+def _host_stale() -> bool:
+    return not os.path.exists(HOST) or any(os.path.getmtime(d) > os.path.getmtime(HOST) for d in (HOST_SOURCE, HEADER))
+
+
+def host_command(out: str, include: str = INCLUDE) -> list:
+    """The compiler's command line for the host calls: C++ against the headers and libraries of the torch that imports them."""
     import torch
     root = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
-    include = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
-               os.path.join(cuda, "include")]
-    subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-                    f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}", *(f"-I{d}" for d in include), HOST_SOURCE, "-o", HOST + ".tmp",
-                    "-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"], check=True)
+    dirs = [include, os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
+            os.path.join(cuda, "include")]
+    return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}", *(f"-I{d}" for d in dirs), HOST_SOURCE, "-o", out,
+            "-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+
+
+def build_host(force: bool = False) -> str:
+    if not force and not _host_stale():
+        return HOST
+    subprocess.run(host_command(HOST + ".tmp"), check=True)
     os.replace(HOST + ".tmp", HOST)
     return HOST
 

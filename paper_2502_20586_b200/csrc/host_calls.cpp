@@ -15,20 +15,19 @@
 
 #include <cstdint>
 
+#include "mxfp4.h"
+
 namespace {
 
-// Entry points of the library, as binding.py has loaded it (include/mxfp4.h).
-typedef size_t (*WorkspaceFn)(int64_t b, int64_t m, int64_t n, int with_bias);
-typedef int (*BackwardFn)(const void* dY, const void* X, const void* W, int64_t b, int64_t m, int64_t n, int g, int rounding, uint64_t seed, void* dX,
-                          void* dW, float* db, int out_dtype, int accumulate, void* workspace, size_t workspace_bytes, void* stream);
-WorkspaceFn g_workspace = nullptr;
-BackwardFn g_backward = nullptr;
+// Entry points of the library, as binding.py has loaded it.
+decltype(&mxfp4_linear_backward_ex_workspace) g_workspace = nullptr;
+decltype(&mxfp4_linear_backward_ex) g_backward = nullptr;
 
 PyObject* bind(PyObject*, PyObject* args) {
     unsigned long long workspace = 0, backward = 0;
     if (!PyArg_ParseTuple(args, "KK", &workspace, &backward)) return nullptr;
-    g_workspace = reinterpret_cast<WorkspaceFn>(workspace);
-    g_backward = reinterpret_cast<BackwardFn>(backward);
+    g_workspace = reinterpret_cast<decltype(g_workspace)>(workspace);
+    g_backward = reinterpret_cast<decltype(g_backward)>(backward);
     Py_RETURN_NONE;
 }
 
@@ -86,7 +85,7 @@ PyObject* backward(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
         PyErr_SetString(PyExc_AssertionError, "accumulation needs an existing dW, and db");
         return nullptr;
     }
-    int status;
+    mxfp4_status status;
     {
         const NoGil others_run;
         const auto result = like.dtype((int)out_dtype == 1 ? at::kFloat : at::kBFloat16);
