@@ -8,6 +8,8 @@ import os
 
 import torch
 
+from . import build as _build
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libmxfp4_b200.so")
 if not os.path.exists(LIB_PATH):
@@ -17,7 +19,10 @@ _lib = C.CDLL(LIB_PATH)
 try:
     from . import _host_calls
 except ImportError as e:
-    raise ImportError("the native host calls are missing: build them with `python -m paper_2502_20586_b200.build`") from e
+    raise ImportError(f"the native host calls do not load ({e}): build them with `python -m paper_2502_20586_b200.build`") from e
+if getattr(_host_calls, "built_for", None) != _build.host_stamp():
+    raise ImportError(f"the native host calls are {getattr(_host_calls, 'built_for', 'an earlier build')}, this is {_build.host_stamp()}: "
+                      "build them with `python -m paper_2502_20586_b200.build`")
 
 OK = 0
 ROUND_SR, ROUND_RN, ROUND_SR16 = 0, 1, 2

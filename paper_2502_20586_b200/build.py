@@ -1,5 +1,5 @@
 """Compile the CUDA library in-tree for sm_100a, ``paper_2502_20586_b200/libmxfp4_b200.so``, and the native host calls of the binding,
-``_host_calls.so``."""
+``_host_calls`` with the file name of this Python's extension modules."""
 import os
 import subprocess
 import sys
@@ -8,7 +8,8 @@ import sysconfig
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmxfp4_b200.so")
-HOST = os.path.join(HERE, "_host_calls.so")
+HOST = os.path.join(HERE, "_host_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
+HOST_UNTAGGED = os.path.join(HERE, "_host_calls.so")                     # any Python would load this: an earlier build's goes
 HOST_SOURCE = os.path.join(CSRC, "host_calls.cpp")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 HEADER = os.path.join(INCLUDE, "mxfp4.h")
@@ -25,8 +26,17 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def host_stamp() -> str:
+    """What the host calls are compiled against, besides their sources: inline code of torch's headers works on the running torch's objects."""
+    import torch
+    return f"host calls for torch {torch.__version__}, C++11 ABI {int(torch.compiled_with_cxx11_abi())}, {sys.implementation.cache_tag}"
+
+
 def _host_stale() -> bool:
-    return not os.path.exists(HOST) or any(os.path.getmtime(d) > os.path.getmtime(HOST) for d in (HOST_SOURCE, HEADER))
+    if not os.path.exists(HOST) or any(os.path.getmtime(d) > os.path.getmtime(HOST) for d in (HOST_SOURCE, HEADER)):
+        return True
+    with open(HOST, "rb") as f:
+        return host_stamp().encode() + b"\0" not in f.read()
 
 
 def host_command(out: str, include: str = INCLUDE) -> list:
@@ -37,7 +47,7 @@ def host_command(out: str, include: str = INCLUDE) -> list:
     dirs = [include, os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
             os.path.join(cuda, "include")]
     return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}", *(f"-I{d}" for d in dirs), HOST_SOURCE, "-o", out,
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}", f'-DMXFP4_HOST_STAMP="{host_stamp()}"', *(f"-I{d}" for d in dirs), HOST_SOURCE, "-o", out,
             "-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
 
 
@@ -46,6 +56,8 @@ def build_host(force: bool = False) -> str:
         return HOST
     subprocess.run(host_command(HOST + ".tmp"), check=True)
     os.replace(HOST + ".tmp", HOST)
+    if HOST_UNTAGGED != HOST and os.path.exists(HOST_UNTAGGED):
+        os.remove(HOST_UNTAGGED)
     return HOST
 
 

@@ -123,4 +123,9 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_host_calls", nullptr, -1, methods
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__host_calls() { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__host_calls() {
+    PyObject* m = PyModule_Create(&module);
+    // the torch and Python whose headers are compiled in here (build.py): binding.py compares it with the running ones
+    if (m != nullptr && PyModule_AddStringConstant(m, "built_for", MXFP4_HOST_STAMP) != 0) Py_CLEAR(m);
+    return m;
+}

@@ -2,8 +2,10 @@
 import os
 import re
 import subprocess
+import sys
 
 import pytest
+import torch
 
 from paper_2502_20586_b200 import build
 
@@ -19,6 +21,7 @@ def compiled(monkeypatch, tmp_path):
         os.utime(copy, (1000, 1000))
         monkeypatch.setattr(build, name, str(copy))
     monkeypatch.setattr(build, "HOST", str(host))
+    monkeypatch.setattr(build, "HOST_UNTAGGED", str(tmp_path / "_host_calls.so"))
     started = []
 
     def run(command, check):
@@ -34,6 +37,25 @@ def test_built_again_when_what_it_is_made_of_is_newer(compiled, newer):
         os.utime(getattr(build, newer), (4e9, 4e9))
     build.build_host()
     assert len(compiled) == (newer is not None)
+
+
+@pytest.mark.parametrize("what", ["torch", "python"])
+def test_built_again_for_another_torch_or_python(compiled, monkeypatch, what):
+    if what == "torch":
+        monkeypatch.setattr(torch, "__version__", "99.0")
+    else:
+        monkeypatch.setattr(build.sys.implementation, "cache_tag", "cpython-99")
+    open(build.HOST_UNTAGGED, "wb").close()
+    build.build_host()
+    assert len(compiled) == 1 and not os.path.exists(build.HOST_UNTAGGED)
+
+
+@pytest.mark.parametrize("version,said", [("torch.__version__", None), ("'99.0'", "torch 99.0")])
+def test_the_import_refuses_a_build_for_another_torch(version, said):
+    code = f"import torch; torch.__version__ = {version}\nfrom paper_2502_20586_b200 import binding"
+    done = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=os.path.dirname(build.INCLUDE))
+    assert (done.returncode != 0) == (said is not None)
+    assert said is None or ("ImportError" in done.stderr and said in done.stderr and "paper_2502_20586_b200.build" in done.stderr)
 
 
 def test_a_changed_prototype_does_not_compile(tmp_path):
