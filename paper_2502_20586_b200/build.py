@@ -43,12 +43,10 @@ def host_command(out: str, include: str = INCLUDE) -> list:
     """The compiler's command line for the host calls: C++ against the headers and libraries of the torch that imports them."""
     import torch
     root = os.path.dirname(torch.__file__)
-    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
-    dirs = [include, os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
-            os.path.join(cuda, "include")]
+    dirs = [include, os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"]]
     return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
             f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}", f'-DMXFP4_HOST_STAMP="{host_stamp()}"', *(f"-I{d}" for d in dirs), HOST_SOURCE, "-o", out,
-            "-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+            "-L" + os.path.join(root, "lib"), "-lc10", "-ltorch_cpu", "-ltorch_python"]
 
 
 def build_host(force: bool = False) -> str:

@@ -9,7 +9,7 @@
 #include <Python.h>
 
 #include <ATen/ops/empty.h>
-#include <c10/cuda/CUDAStream.h>
+#include <c10/core/impl/VirtualGuardImpl.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -38,6 +38,12 @@ bool integer(PyObject* o, uint64_t* out) {
     *out = PyLong_AsUnsignedLongLongMask(i);
     Py_DECREF(i);
     return *out != ~uint64_t(0) || PyErr_Occurred() == nullptr;
+}
+
+// The current device's current stream, by torch's interface for any device: this module needs no CUDA library of torch's to load.
+void* current_stream() {
+    const c10::impl::VirtualGuardImpl cuda(c10::DeviceType::CUDA);
+    return cuda.getStreamNativeHandle(cuda.getStream(cuda.getDevice()));
 }
 
 // Other Python threads run while one of these lives, an exception included.  It goes around the allocations as well as the library: one
@@ -95,7 +101,7 @@ PyObject* backward(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
         if (!workspace.defined()) workspace = at::empty({(int64_t)g_workspace(b, m, n, db.defined() ? 1 : 0)}, like.dtype(at::kByte));
         status = g_backward(dY.data_ptr(), X.data_ptr(), W.data_ptr(), b, m, n, (int)g, (int)rounding, seed, dX.data_ptr(), dW.data_ptr(),
                             db.defined() ? static_cast<float*>(db.data_ptr()) : nullptr, (int)out_dtype, accumulate, workspace.data_ptr(),
-                            (size_t)workspace.numel(), c10::cuda::getCurrentCUDAStream().stream());
+                            (size_t)workspace.numel(), current_stream());
     }
     PyObject* out[4] = {PyLong_FromLong(status), nullptr, nullptr, nullptr};
     const at::Tensor* made[3] = {&dX, &dW, &db};

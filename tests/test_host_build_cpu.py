@@ -65,3 +65,9 @@ def test_a_changed_prototype_does_not_compile(tmp_path):
     (tmp_path / "mxfp4.h").write_text(changed)
     done = subprocess.run([*build.host_command(os.devnull, str(tmp_path)), "-fsyntax-only"], capture_output=True, text=True)
     assert done.returncode != 0 and "too many arguments" in done.stderr
+
+
+def test_links_no_cuda_library_of_torchs():
+    """A torch that was built without CUDA imports the binding too (its calls then refuse every tensor)."""
+    libraries = [flag for flag in build.host_command("out") if flag.startswith("-l")]
+    assert "-lc10" in libraries and not any("cuda" in flag for flag in libraries)
