@@ -4,6 +4,7 @@ Every step of the method runs in the CUDA kernels behind ``libmxfp4_b200.so``; t
 memory and streams.  There is no CPU fallback: if the library has not been built this module fails to import.
 """
 import ctypes as C
+import operator
 import os
 
 import torch
@@ -123,8 +124,22 @@ def _empty(like, shape, dtype):
 _PLAIN = {torch.Tensor, torch.nn.Parameter}
 
 
+class ArgumentError(C.ArgumentError, TypeError):
+    """An argument that ctypes does not take as the integer it should be."""
+
+
+def _integer(value, ctype) -> int:
+    """An integer argument as ctypes takes it: one of Python's, whatever has an index, or one of ctypes' own of this type."""
+    try:
+        ctype.from_param(value)
+        value = getattr(value, "_as_parameter_", value)
+        return operator.index(value.value if isinstance(value, ctype) else value)
+    except TypeError as e:
+        raise ArgumentError(str(e)) from None
+
+
 def _plain(*tensors) -> bool:
-    """Whether the native host call (csrc/host_calls.cpp) takes these: tensors of no subclass, or None."""
+    """Whether the native host call (csrc/host_calls.cpp) takes these: tensors of no subclass, or None.  ``_backward`` has its steps for the rest."""
     for t in tensors:
         if t is not None and type(t) not in _PLAIN:
             return False
@@ -273,24 +288,12 @@ def mxfp4_linear_backward(dY, X, W, g: int, seed: int, rounding: int = ROUND_SR,
                           dX=None, dW=None, workspace=None):
     """Algorithm 3: dY [b, m], X [b, n], W [m, n] bf16 (contiguous)  ->  (dX [b, n], dW [m, n])."""
     if dY is not None and X is not None and W is not None and _plain(dY, X, W, dX, dW, workspace):
-        status, dX, dW, _ = _host_calls.backward(dY, X, W, g, seed, rounding, out_dtype, dX, dW, None, False, False, workspace)
-        _check(status)
-        return dX, dW
-    b, m = dY.shape
-    _, n = X.shape
-    for t in (dY, X, W):
-        assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()
-    dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
-    if dX is None:
-        dX = _empty(dY, (b, n), dt)
-    if dW is None:
-        dW = _empty(dY, (m, n), dt)
-    need = mxfp4_linear_backward_workspace(b, m, n)
-    if workspace is None:
-        workspace = _empty(dY, need, torch.uint8)
-    _check(_lib.mxfp4_linear_backward(_ptr(dY), _ptr(X), _ptr(W), b, m, n, g, rounding, seed, _ptr(dX), _ptr(dW),
-                                      out_dtype, _ptr(workspace), workspace.numel(), _stream()))
-    return dX, dW
+        done = _host_calls.backward(dY, X, W, g, seed, rounding, out_dtype, dX, dW, None, False, False, workspace)
+        if done is not None:
+            status, dX, dW, _ = done
+            _check(status)
+            return dX, dW
+    return _backward(dY, X, W, g, seed, rounding, out_dtype, dX, dW, None, False, False, workspace)[:2]
 
 
 def mxfp4_linear_backward_ex_workspace(b: int, m: int, n: int, with_bias: bool) -> int:
@@ -302,13 +305,21 @@ def mxfp4_linear_backward_ex(dY, X, W, g: int, seed: int, rounding: int = ROUND_
     """Algorithm 3 plus the bias gradient (fp32 [m], column sums of dY) and accumulation into fp32 dW / db.
     Returns (dX, dW, db) with db None unless with_bias or db is given."""
     if dY is not None and X is not None and W is not None and _plain(dY, X, W, dX, dW, db, workspace):
-        status, dX, dW, db = _host_calls.backward(dY, X, W, g, seed, rounding, out_dtype, dX, dW, db, with_bias, accumulate, workspace)
-        _check(status)
-        return dX, dW, db
+        done = _host_calls.backward(dY, X, W, g, seed, rounding, out_dtype, dX, dW, db, with_bias, accumulate, workspace)
+        if done is not None:
+            status, dX, dW, db = done
+            _check(status)
+            return dX, dW, db
+    return _backward(dY, X, W, g, seed, rounding, out_dtype, dX, dW, db, with_bias, accumulate, workspace)
+
+
+def _backward(dY, X, W, g, seed, rounding, out_dtype, dX, dW, db, with_bias, accumulate, workspace):
+    """The steps of the native host call for what that does not take: tensors of a subclass, integers of ctypes."""
     b, m = dY.shape
     _, n = X.shape
     for t in (dY, X, W):
         assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()
+    g, seed, rounding, out_dtype = _integer(g, _int), _integer(seed, _u64), _integer(rounding, _int), _integer(out_dtype, _int)
     dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
     if dX is None:
         dX = _empty(dY, (b, n), dt)

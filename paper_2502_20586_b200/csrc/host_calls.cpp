@@ -31,8 +31,9 @@ PyObject* bind(PyObject*, PyObject* args) {
     Py_RETURN_NONE;
 }
 
-// An integer argument as ctypes passes it: any Python integer, its low bits.
+// Whether an argument is an integer by itself, and if so its low bits, as ctypes takes them.
 bool integer(PyObject* o, uint64_t* out) {
+    if (!PyIndex_Check(o)) return false;
     PyObject* i = PyNumber_Index(o);
     if (i == nullptr) return false;
     *out = PyLong_AsUnsignedLongLongMask(i);
@@ -57,7 +58,7 @@ struct NoGil {
 };
 
 // backward(dY, X, W, g, seed, rounding, out_dtype, dX, dW, db, with_bias, accumulate, workspace) -> (status, dX, dW, db): Algorithm 3.
-// None for dX, dW, db (with_bias) or workspace: made here.
+// None for dX, dW, db (with_bias) or workspace: made here.  The result is None where g, seed, rounding or out_dtype is no integer by itself.
 PyObject* backward(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
     HANDLE_TH_ERRORS
     if (n_args != 13) {
@@ -80,7 +81,10 @@ PyObject* backward(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
             return nullptr;
         }
     uint64_t g, seed, rounding, out_dtype;
-    if (!integer(args[3], &g) || !integer(args[4], &seed) || !integer(args[5], &rounding) || !integer(args[6], &out_dtype)) return nullptr;
+    if (!integer(args[3], &g) || !integer(args[4], &seed) || !integer(args[5], &rounding) || !integer(args[6], &out_dtype)) {
+        if (PyErr_Occurred() != nullptr) return nullptr;
+        Py_RETURN_NONE;                                               // ctypes may know what to do with it
+    }
     const int with_bias = PyObject_IsTrue(args[10]), accumulate = PyObject_IsTrue(args[11]);
     if (with_bias < 0 || accumulate < 0) return nullptr;
     const int64_t b = dY.size(0), m = dY.size(1), n = X.size(1);

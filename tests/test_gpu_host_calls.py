@@ -134,3 +134,35 @@ def test_other_threads_run_while_a_call_allocates():
     assert end - start > 0.2                                                    # the call did wait
     assert max(b - a for a, b in zip(seen, seen[1:])) < 0.5 * (end - start)
     assert not torch.any(dX) and gpu.mxfp4_device_status() == 0
+
+
+class _Parameter:
+    """An argument as ctypes lets a class of the caller's pass for one."""
+    def __init__(self, value):
+        self._as_parameter_ = value
+
+
+# Integers in every form that ctypes takes for one, and forms that it does not: by either host path
+@pytest.mark.parametrize("subclass", [False, True])
+def test_integers_of_every_kind(subclass):
+    import ctypes
+
+    import numpy as np
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    dY, X, W = _layer()
+    want = gpu.mxfp4_linear_backward(dY, X, W, 64, 5, gpu.ROUND_SR, gpu.OUT_FP32)
+    if subclass:
+        dY = _tagged(dY)
+    i, u = ctypes.c_int, ctypes.c_uint64
+    for ints in ((i(64), u(5), i(0), i(1)), (64, u(5), 0, i(1)), (np.int64(64), np.uint64(5), False, True), (_Parameter(64), 5, 0, _Parameter(i(1)))):
+        got = gpu.mxfp4_linear_backward_ex(dY, X, W, *ints, with_bias=True)
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+        assert torch.equal(gpu.mxfp4_linear_backward(dY, X, W, *ints)[1], want[1])
+    for ints in ((64.0, 5, 0, 1), (64, "5", 0, 1), (64, 5, None, 1), (64, 5, 0, ctypes.c_float(1)), (ctypes.c_long(64), 5, 0, 1)):
+        for error in (TypeError, ctypes.ArgumentError):
+            with pytest.raises(error):
+                gpu.mxfp4_linear_backward(dY, X, W, *ints)
+            with pytest.raises(error):
+                gpu.mxfp4_linear_backward_ex(dY, X, W, *ints)
+    assert gpu.mxfp4_device_status() == 0
