@@ -130,6 +130,8 @@ class ArgumentError(C.ArgumentError, TypeError):
 
 def _integer(value, ctype) -> int:
     """An integer argument as ctypes takes it: one of Python's, whatever has an index, or one of ctypes' own of this type."""
+    if type(value) is int:
+        return value
     try:
         ctype.from_param(value)
         value = getattr(value, "_as_parameter_", value)
@@ -144,6 +146,25 @@ def _plain(*tensors) -> bool:
         if t is not None and type(t) not in _PLAIN:
             return False
     return True
+
+
+def _layer(dY, X, W, dX, dW, db, workspace, dtype):
+    """b, m and n of a layer's tensors dY [b, m], X [b, n], W [m, n], which the library gets with their addresses, and so with those of the
+    buffers that the caller has for dX, dW (of ``dtype``), db and scratch: none may be smaller than b, m and n say or laid out otherwise."""
+    if dY is not None and X is not None and W is not None and db is None and _plain(dY, X, W, dX, dW, workspace):
+        return _host_calls.layer(dY, X, W, dX, dW, workspace, dtype is torch.float32)
+    b, m = dY.shape
+    rows, n = X.shape
+    for t in (dY, X, W):
+        assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()
+    device, shape = dY.device, W.shape
+    assert rows == b and (shape == (m, n) or (len(shape) != 2 and W.numel() == m * n)) and X.device == device and W.device == device, \
+        "dY [b, m], X [b, n] and W [m, n] on one GPU are expected"
+    for t, elements, columns, kind in ((dX, b * n, n, dtype), (dW, m * n, n, dtype), (db, m, None, torch.float32), (workspace, 0, None, None)):
+        assert not isinstance(t, torch.Tensor) or (
+            t.device == device and t.is_contiguous() and t.numel() >= elements and (kind is None or t.dtype == kind) and
+            (columns is None or t.dim() != 2 or t.shape[1] == columns)), "a buffer has another type or device, is not contiguous or too small"
+    return b, m, n
 
 
 def lib():
@@ -235,11 +256,8 @@ def mxfp4_gemm_fused(x, reduce_dim: int, g: int, seed: int, stream_tag: int, rou
 def mxfp4_linear_backward_fused(dY, X, W, g: int, seed: int, rounding: int = ROUND_SR, out_dtype: int = OUT_BF16,
                                 dX=None, dW=None, workspace=None):
     """Algorithm 3 with dY / dY^T transformed and quantised inside the two GEMM kernels (fused-producer variant)."""
-    b, m = dY.shape
-    _, n = X.shape
-    for t in (dY, X, W):
-        assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()
     dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
+    b, m, n = _layer(dY, X, W, dX, dW, None, workspace, dt)
     if dX is None:
         dX = _empty(dY, (b, n), dt)
     if dW is None:
@@ -254,10 +272,7 @@ def mxfp4_linear_backward_fused(dY, X, W, g: int, seed: int, rounding: int = ROU
 def mxfp4_quantize_operands(dY, X, W, g: int, seed: int, rounding: int = ROUND_SR, workspace=None):
     """Algorithm 3 lines 3-6 in one launch.  Returns [(codes, scales)] for Q1..Q4 as views into the workspace
     (codes [R, K/2] u8, scales flat u8 in the native layout), ready for mxfp4_gemm."""
-    b, m = dY.shape
-    _, n = X.shape
-    for t in (dY, X, W):
-        assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()
+    b, m, n = _layer(dY, X, W, None, None, None, workspace, None)
     if workspace is None:
         workspace = _empty(dY, mxfp4_linear_backward_workspace(b, m, n), torch.uint8)
     _check(_lib.mxfp4_quantize_operands(_ptr(dY), _ptr(X), _ptr(W), b, m, n, g, rounding, seed, _ptr(workspace), workspace.numel(),
@@ -315,23 +330,19 @@ def mxfp4_linear_backward_ex(dY, X, W, g: int, seed: int, rounding: int = ROUND_
 
 def _backward(dY, X, W, g, seed, rounding, out_dtype, dX, dW, db, with_bias, accumulate, workspace):
     """The steps of the native host call for what that does not take: tensors of a subclass, integers of ctypes."""
-    b, m = dY.shape
-    _, n = X.shape
-    for t in (dY, X, W):
-        assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()
     g, seed, rounding, out_dtype = _integer(g, _int), _integer(seed, _u64), _integer(rounding, _int), _integer(out_dtype, _int)
     dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
+    b, m, n = _layer(dY, X, W, dX, dW, db, workspace, dt)
+    assert not accumulate or (dW is not None and (db is not None or not with_bias)), "accumulation needs an existing dW, and db"
+    like = next((t for t in (X, W) if type(t) is torch.Tensor), dY)              # (whatever is asked of a subclass goes through its own hooks)
     if dX is None:
-        dX = _empty(dY, (b, n), dt)
+        dX = _empty(like, (b, n), dt)
     if dW is None:
-        assert not accumulate, "accumulation needs an existing dW"
-        dW = _empty(dY, (m, n), dt)
+        dW = _empty(like, (m, n), dt)
     if db is None and with_bias:
-        assert not accumulate, "accumulation needs an existing db"
-        db = torch.empty((m,), dtype=torch.float32, device=dY.device)
-    need = mxfp4_linear_backward_ex_workspace(b, m, n, db is not None)
+        db = _empty(like, (m,), torch.float32)
     if workspace is None:
-        workspace = _empty(dY, need, torch.uint8)
+        workspace = _empty(like, mxfp4_linear_backward_ex_workspace(b, m, n, db is not None), torch.uint8)
     _check(_lib.mxfp4_linear_backward_ex(_ptr(dY), _ptr(X), _ptr(W), b, m, n, g, rounding, seed, _ptr(dX), _ptr(dW),
                                          _ptr(db) if db is not None else None, out_dtype, 1 if accumulate else 0,
                                          _ptr(workspace), workspace.numel(), _stream()))
@@ -353,11 +364,8 @@ def mxfp4_linear_backward_static(dY, X, W, g: int, seed: int, rounding: int = RO
     """mxfp4_linear_backward for callers that cannot provide scratch memory: the library's own fixed array
     (STATIC_WORKSPACE_BYTES per GPU) holds the quantised operands.  Pass dX and dW to make the call itself
     allocation-free; shapes that need more scratch than the array raise MxFp4Error(6)."""
-    b, m = dY.shape
-    _, n = X.shape
-    for t in (dY, X, W):
-        assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()
     dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
+    b, m, n = _layer(dY, X, W, dX, dW, None, None, dt)
     if dX is None:
         dX = _empty(dY, (b, n), dt)
     if dW is None:

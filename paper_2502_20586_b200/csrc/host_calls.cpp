@@ -14,6 +14,7 @@
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <cstdint>
+#include <initializer_list>
 
 #include "mxfp4.h"
 
@@ -57,6 +58,58 @@ struct NoGil {
     ~NoGil() { PyEval_RestoreThread(thread); }
 };
 
+bool refuse(PyObject* error, const char* why) {
+    PyErr_SetString(error, why);
+    return false;
+}
+
+// A tensor, or nothing for None.
+at::Tensor tensor_or_none(PyObject* o) { return o == Py_None ? at::Tensor() : THPVariable_Unpack(o); }
+
+bool are_tensors(PyObject* const* args, std::initializer_list<int> required, std::initializer_list<int> given) {
+    for (int i : required)
+        if (!THPVariable_Check(args[i])) return refuse(PyExc_TypeError, "a tensor is expected");
+    for (int i : given)
+        if (args[i] != Py_None && !THPVariable_Check(args[i])) return refuse(PyExc_TypeError, "a tensor is expected");
+    return true;
+}
+
+// The tensors of a layer's backward call and the buffers that the caller has for it.  The kernels get addresses and b, m and n: no tensor
+// may be smaller than these say, of another type or laid out otherwise.  binding.py's _layer says the same of tensors of a subclass.
+bool layer_fits(const at::Tensor& dY, const at::Tensor& X, const at::Tensor& W, const at::Tensor& dX, const at::Tensor& dW, const at::Tensor& db,
+                const at::Tensor& workspace, bool fp32) {
+    if (dY.dim() != 2 || X.dim() != 2) return refuse(PyExc_ValueError, "dY and X have two dimensions");
+    for (const at::Tensor* t : {&dY, &X, &W})
+        if (!t->is_cuda() || t->scalar_type() != at::kBFloat16 || !t->is_contiguous())
+            return refuse(PyExc_AssertionError, "contiguous bf16 tensors on the GPU are expected");
+    const int64_t b = dY.size(0), m = dY.size(1), n = X.size(1);
+    if (X.size(0) != b || W.numel() != m * n || (W.dim() == 2 && W.size(1) != n) || X.device() != dY.device() || W.device() != dY.device())
+        return refuse(PyExc_AssertionError, "dY [b, m], X [b, n] and W [m, n] on one GPU are expected");
+    auto in_place = [&](const at::Tensor& t) { return !t.defined() || (t.device() == dY.device() && t.is_contiguous()); };
+    auto holds = [&](const at::Tensor& t, int64_t elements, at::ScalarType type) {
+        return !t.defined() || (in_place(t) && t.scalar_type() == type && t.numel() >= elements);
+    };
+    auto rows_of_n = [&](const at::Tensor& t) { return !t.defined() || t.dim() != 2 || t.size(1) == n; };
+    const at::ScalarType result = fp32 ? at::kFloat : at::kBFloat16;
+    if (!holds(dX, b * n, result) || !rows_of_n(dX) || !holds(dW, m * n, result) || !rows_of_n(dW) || !holds(db, m, at::kFloat) || !in_place(workspace))
+        return refuse(PyExc_AssertionError, "a buffer has another type or device, is not contiguous or too small");
+    return true;
+}
+
+// layer(dY, X, W, dX, dW, workspace, fp32) -> (b, m, n), or the exception that the caller gets.
+PyObject* layer(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
+    HANDLE_TH_ERRORS
+    if (n_args != 7) {
+        PyErr_SetString(PyExc_TypeError, "layer: 7 arguments");
+        return nullptr;
+    }
+    if (!are_tensors(args, {0, 1, 2}, {3, 4, 5})) return nullptr;
+    const at::Tensor &dY = THPVariable_Unpack(args[0]), &X = THPVariable_Unpack(args[1]), &W = THPVariable_Unpack(args[2]);
+    if (!layer_fits(dY, X, W, tensor_or_none(args[3]), tensor_or_none(args[4]), at::Tensor(), tensor_or_none(args[5]), args[6] == Py_True)) return nullptr;
+    return Py_BuildValue("LLL", (long long)dY.size(0), (long long)dY.size(1), (long long)X.size(1));
+    END_HANDLE_TH_ERRORS
+}
+
 // backward(dY, X, W, g, seed, rounding, out_dtype, dX, dW, db, with_bias, accumulate, workspace) -> (status, dX, dW, db): Algorithm 3.
 // None for dX, dW, db (with_bias) or workspace: made here.  The result is None where g, seed, rounding or out_dtype is no integer by itself.
 PyObject* backward(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
@@ -65,21 +118,7 @@ PyObject* backward(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
         PyErr_SetString(PyExc_TypeError, "backward: 13 arguments");
         return nullptr;
     }
-    for (int i : {0, 1, 2, 7, 8, 9, 12})
-        if (!THPVariable_Check(args[i]) && (i < 3 || args[i] != Py_None)) {
-            PyErr_SetString(PyExc_TypeError, "backward: a tensor is expected");
-            return nullptr;
-        }
-    const at::Tensor &dY = THPVariable_Unpack(args[0]), &X = THPVariable_Unpack(args[1]), &W = THPVariable_Unpack(args[2]);
-    if (dY.dim() != 2 || X.dim() != 2) {
-        PyErr_SetString(PyExc_ValueError, "dY and X have two dimensions");
-        return nullptr;
-    }
-    for (const at::Tensor* t : {&dY, &X, &W})
-        if (!t->is_cuda() || t->scalar_type() != at::kBFloat16 || !t->is_contiguous()) {
-            PyErr_SetString(PyExc_AssertionError, "contiguous bf16 tensors on the GPU are expected");
-            return nullptr;
-        }
+    if (!are_tensors(args, {0, 1, 2}, {7, 8, 9, 12})) return nullptr;
     uint64_t g, seed, rounding, out_dtype;
     if (!integer(args[3], &g) || !integer(args[4], &seed) || !integer(args[5], &rounding) || !integer(args[6], &out_dtype)) {
         if (PyErr_Occurred() != nullptr) return nullptr;
@@ -87,18 +126,19 @@ PyObject* backward(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
     }
     const int with_bias = PyObject_IsTrue(args[10]), accumulate = PyObject_IsTrue(args[11]);
     if (with_bias < 0 || accumulate < 0) return nullptr;
-    const int64_t b = dY.size(0), m = dY.size(1), n = X.size(1);
-    const auto like = dY.options().requires_grad(false);
-    auto given = [&](int i) { return args[i] == Py_None ? at::Tensor() : THPVariable_Unpack(args[i]); };
-    at::Tensor dX = given(7), dW = given(8), db = given(9), workspace = given(12);
+    const at::Tensor &dY = THPVariable_Unpack(args[0]), &X = THPVariable_Unpack(args[1]), &W = THPVariable_Unpack(args[2]);
+    at::Tensor dX = tensor_or_none(args[7]), dW = tensor_or_none(args[8]), db = tensor_or_none(args[9]), workspace = tensor_or_none(args[12]);
+    const bool fp32 = (int)out_dtype == MXFP4_OUT_FP32;
+    if (!layer_fits(dY, X, W, dX, dW, db, workspace, fp32)) return nullptr;
     if (accumulate != 0 && (!dW.defined() || (with_bias != 0 && !db.defined()))) {
         PyErr_SetString(PyExc_AssertionError, "accumulation needs an existing dW, and db");
         return nullptr;
     }
+    const int64_t b = dY.size(0), m = dY.size(1), n = X.size(1);
     mxfp4_status status;
     {
         const NoGil others_run;
-        const auto result = like.dtype((int)out_dtype == 1 ? at::kFloat : at::kBFloat16);
+        const auto like = dY.options().requires_grad(false), result = like.dtype(fp32 ? at::kFloat : at::kBFloat16);
         if (!dX.defined()) dX = at::empty({b, n}, result);
         if (!dW.defined()) dW = at::empty({m, n}, result);
         if (with_bias != 0 && !db.defined()) db = at::empty({m}, like.dtype(at::kFloat));
@@ -126,6 +166,7 @@ PyObject* backward(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
 
 PyMethodDef methods[] = {
     {"bind", bind, METH_VARARGS, "addresses of mxfp4_linear_backward_ex_workspace and mxfp4_linear_backward_ex"},
+    {"layer", (PyCFunction)(void (*)(void))layer, METH_FASTCALL, "(b, m, n)"},
     {"backward", (PyCFunction)(void (*)(void))backward, METH_FASTCALL, "(status, dX, dW, db)"},
     {nullptr, nullptr, 0, nullptr},
 };

@@ -81,16 +81,66 @@ def test_refusals():
 
 
 def test_out_of_memory_is_an_exception():
-    """The results of a small input that do not fit the device: torch's own exception, and the library keeps working."""
+    """A result that does not fit what this process may take of the device: torch's own exception, and the library keeps working."""
     import torch
     from paper_2502_20586_b200 import binding as gpu
-    n = 1 << 27                                              # dX of 2^21 x 2^27 would be 2^49 bytes
-    dY = torch.zeros((1 << 21, 128), dtype=torch.bfloat16, device="cuda")
-    X = torch.zeros((1, n), dtype=torch.bfloat16, device="cuda")        # (only its width is looked at before the results are allocated)
-    with pytest.raises(torch.OutOfMemoryError):
-        gpu.mxfp4_linear_backward(dY, X, X[:, :128].contiguous(), 64, 0)
+    dY, X, W = _layer(4096, 8192, 128)
+    torch.cuda.empty_cache()
+    torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + (16 << 20)) / torch.cuda.mem_get_info()[1])
+    try:
+        with pytest.raises(torch.OutOfMemoryError):          # 128 MB, sixteen of which there are
+            gpu.mxfp4_linear_backward(dY, X, W, 64, 0, gpu.ROUND_SR, gpu.OUT_FP32)
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
     dY, X, W = _layer()
     gpu.mxfp4_linear_backward(dY, X, W, 64, 0)
+    assert gpu.mxfp4_device_status() == 0
+
+
+# Tensors and buffers that are smaller than the sizes say, or laid out or typed otherwise: refused by either host path before the library
+# is called, whose kernels would read and write past them
+@pytest.mark.parametrize("subclass", [False, True])
+def test_tensors_that_do_not_fit_are_refused(subclass):
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    dY, X, W = _layer()                                                          # b 256, n 264, m 384
+    make = lambda *size, dtype=torch.float32: torch.zeros(size, dtype=dtype, device="cuda")
+    bf16 = dict(dtype=torch.bfloat16)
+    tag = _tagged if subclass else (lambda t: t)
+    for x, w in ((X[:128], W), (X[:255], W), (make(384, 264, **bf16), W), (X, W[:256]), (X, make(264, 384, **bf16)), (X, make(384, 256, **bf16)), (X, W.view(-1)[8:])):
+        for call in (gpu.mxfp4_linear_backward, gpu.mxfp4_linear_backward_ex, gpu.mxfp4_linear_backward_static, gpu.mxfp4_linear_backward_fused,
+                     gpu.mxfp4_quantize_operands):
+            with pytest.raises(AssertionError):
+                call(tag(dY), x, w, 64, 0)
+    need = gpu.mxfp4_linear_backward_ex_workspace(256, 384, 264, True)
+    good = dict(dX=make(256, 264), dW=make(384, 264), db=make(384), workspace=make(need, dtype=torch.uint8))
+    bad = dict(dX=(make(255, 264), make(256, 264, **bf16), make(256, 272), make(264, 256).t(), make(256, 528)[:, ::2], make(256, 264).cpu(),
+                   make(1).expand(256, 264)),
+               dW=(make(383, 264), make(384, 264, **bf16), make(264, 384), make(264, 384).t(), make(384, 264).cpu()),
+               db=(make(383), make(384, **bf16), make(768)[::2], make(384).cpu()),
+               workspace=(make(2 * need, dtype=torch.uint8)[::2], make(1, dtype=torch.uint8).expand(need), torch.zeros(need, dtype=torch.uint8)))
+    for name, buffers in bad.items():
+        for t in buffers:
+            with pytest.raises(AssertionError):
+                gpu.mxfp4_linear_backward_ex(tag(dY), X, W, 64, 0, 0, gpu.OUT_FP32, accumulate=True, **{**good, name: t})
+            if name == "db":
+                continue
+            with pytest.raises(AssertionError):
+                gpu.mxfp4_linear_backward(tag(dY), X, W, 64, 0, 0, gpu.OUT_FP32, **{name: t})
+            for call in (gpu.mxfp4_linear_backward_static, gpu.mxfp4_linear_backward_fused):
+                if name != "workspace" or call is gpu.mxfp4_linear_backward_fused:
+                    with pytest.raises(AssertionError):
+                        call(tag(dY), X, W, 64, 0, 0, gpu.OUT_FP32, **{name: t})
+            if name == "workspace":
+                with pytest.raises(AssertionError):
+                    gpu.mxfp4_quantize_operands(tag(dY), X, W, 64, 0, workspace=t)
+    assert not any(torch.any(t) for t in good.values())                          # nothing ran
+    # larger buffers, and W or buffers of one dimension, serve as before: the results stand at the buffers' start
+    want = gpu.mxfp4_linear_backward_ex(dY, X, W, 64, 0, 0, gpu.OUT_FP32, with_bias=True)
+    flat = dict(dX=make(256 * 264 + 24), dW=make(400, 264), db=make(1, 400), workspace=make(need, dtype=torch.int32))
+    got = gpu.mxfp4_linear_backward_ex(tag(dY), X, W.view(-1), 64, 0, 0, gpu.OUT_FP32, **flat)
+    for a, t in zip(want, got):
+        assert torch.equal(t.view(-1)[:a.numel()], a.view(-1)) and not torch.any(t.view(-1)[a.numel():])
     assert gpu.mxfp4_device_status() == 0
 
 
