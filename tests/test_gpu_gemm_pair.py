@@ -43,21 +43,23 @@ def test_tile_walk(gpu, M, N, K, fp32):
 
 
 # One tile to a pair, whose columns the two epilogue groups share in the 8-bit builds, against the same rows in a product of several tiles to
-# a pair, whose groups take whole tiles: the same bits.  128-wide tiles and (E4M3) 256-wide ones, ragged rows and columns
-@pytest.mark.parametrize("rows,more,N,K", [(200, 9000, 264, 256), (257, 19000, 136, 384), (512, 12000, 1000, 128)])
+# a pair, whose groups take whole tiles: the same bits.  128-wide tiles, ragged rows and columns; 256-wide ones from 1000 rows on with
+# 8-bit products of 4096 and 4128 columns (128 and 132 tiles of 128 columns take two rounds of the 74 pairs, 64 and 68 of 256 columns one)
+@pytest.mark.parametrize("rows,more,N,K", [(200, 9000, 264, 256), (257, 19000, 136, 384), (512, 12000, 1000, 128), (1000, 9000, 1024, 384), (990, 9000, 1032, 256)])
 @pytest.mark.parametrize("out", [0, 1])
 def test_single_tile_of_a_pair(gpu, rows, more, N, K, out):
     import torch
     gen = torch.Generator(device="cuda")
     gen.manual_seed(rows + N + K)
     ca, sa, _ = _operand(gen, more, K)
-    cb, sb, _ = _operand(gen, N, K)
+    cb, sb, _ = _operand(gen, N * 4, K)
     few = sa[:(rows + 127) // 128 * ((K + 127) // 128) * 512]
-    assert torch.equal(gpu.mxfp4_gemm(ca[:rows], few, cb, sb, 1.5, out), gpu.mxfp4_gemm(ca, sa, cb, sb, 1.5, out)[:rows])
+    assert torch.equal(gpu.mxfp4_gemm(ca[:rows], few, cb[:N], sb, 1.5, out), gpu.mxfp4_gemm(ca, sa, cb[:N], sb, 1.5, out)[:rows])
     a, b = (torch.randint(0, 0x60, (n, K), generator=gen, device="cuda", dtype=torch.uint8) for n in (more, N * 4))      # E4M3, finite
     one = torch.ones(2, device="cuda")
     assert torch.equal(gpu.mxfp4_fp8_gemm(a[:rows], one, b, one, out), gpu.mxfp4_fp8_gemm(a, one, b, one, out)[:rows])
-    assert torch.equal(gpu.mxfp4_int4_gemm(a[:rows], few, b[:N], sb, 1.5, out), gpu.mxfp4_int4_gemm(a, sa, b[:N], sb, 1.5, out)[:rows])
+    for n in (N, N * 4):
+        assert torch.equal(gpu.mxfp4_int4_gemm(a[:rows], few, b[:n], sb, 1.5, out), gpu.mxfp4_int4_gemm(a, sa, b[:n], sb, 1.5, out)[:rows])
     assert gpu.mxfp4_device_status() == 0
 
 

@@ -2,6 +2,8 @@
 quantiser or a walk of another shape: the transform is exact on small integers, so codes and scales are equal bytes."""
 import pytest
 
+from tests import helpers as hp
+
 pytestmark = pytest.mark.gpu
 
 
@@ -201,25 +203,29 @@ def test_refused_launch_leaves_no_error_behind():
 
 
 # As many tiles as the chip has SMs (half tiles to the epilogue groups) and one more (whole tiles): the rows that both have, row-wise and
-# transposing, in either scale layout, a last tile of a few rows
+# transposing, in either scale layout, a last tile of a few rows; with the sign vector's transform and with a caller's matrix
 @pytest.mark.parametrize("K,g", [(128, 64), (256, 128), (512, 32)])
 @pytest.mark.parametrize("rounding", [0, 2])
 @pytest.mark.parametrize("layout", [0, 1])
-def test_half_tiles(K, g, rounding, layout):
+@pytest.mark.parametrize("given", [False, True])
+def test_half_tiles(K, g, rounding, layout, given):
     import torch
     from paper_2502_20586_b200 import binding as gpu
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     rows = sms // (K // 128) * 128
     x = _small_integers((rows + 128, K), K + g)
-    whole, scales = gpu.mxfp4_rht_sr_quantize(x, 1, g, 7, 3, rounding, layout)
+    T = _small_integers((g, g), g) / 8
+    quantise = lambda y, dim: gpu.mxfp4_transform_quantize(y, dim, T, 7, 3, rounding, layout) if given else \
+        gpu.mxfp4_rht_sr_quantize(y, dim, g, 7, 3, rounding, layout)
+    linear = lambda s, n: s.view(n, K // 32) if layout == gpu.SF_LINEAR else \
+        torch.from_numpy(hp.sf_native_to_linear(s.cpu().numpy(), n, K)).cuda()
+    whole, scales = quantise(x, 1)
+    scales = linear(scales, rows + 128)
     for n in (rows, rows - 100, 40):
         for y, dim in ((x[:n], 1), (x[:n].t()[:, :n // 8 * 8].contiguous(), 0)):
-            codes, s = gpu.mxfp4_rht_sr_quantize(y, dim, g, 7, 3, rounding, layout)
+            codes, s = quantise(y, dim)
             n_rows = codes.shape[0]
-            assert torch.equal(codes, whole[:n_rows])
-            per = K // 32 if layout == gpu.SF_LINEAR else K * 4                      # scales of a row, of a tile of 128 rows
-            full = n_rows if layout == gpu.SF_LINEAR else n_rows // 128
-            assert torch.equal(s[:full * per], scales[:full * per])
+            assert n_rows > n - 8 and torch.equal(codes, whole[:n_rows]) and torch.equal(linear(s, n_rows), scales[:n_rows])
     assert gpu.mxfp4_device_status() == 0
 
 
