@@ -1,7 +1,8 @@
-"""Thin Python binding of the C-ABI library (include/mxfp4.h): argument marshalling only.
+"""Thin Python binding of the C-ABI library (include/mxfp4.h): checks, the tensors that the caller did not bring, argument marshalling.
 
 Every step of the method runs in the CUDA kernels behind ``libmxfp4_b200.so``; torch is used for device
-memory and streams.  There is no CPU fallback: if the library has not been built this module fails to import.
+memory and streams.  A layer's backward call goes through one native function (csrc/host_calls.cpp), the others through ctypes.
+There is no CPU fallback: if the library or the host calls have not been built this module fails to import.
 """
 import ctypes as C
 import operator

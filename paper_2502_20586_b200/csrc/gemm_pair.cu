@@ -21,11 +21,11 @@
 //                stores (or reduce-adds when accumulating).
 // A-row scales are per CTA; every CTA needs the scales of all 256 B rows.
 //
-// What bounds it: the tensor pipe in the steady state (0.34 us a K-step of a pair tile; the same MMAs on operands that stay in
-// shared memory, fp4_ceiling.cu, take 0.31 us in a burst, 0.35 sustained: 8.1 and 7.1 PFLOP/s) and the board's power (1.36 - 1.57 GHz in a long
-// launch); per tile 0.65 us in which the pipe stands still, since TMEM has no room for a second 256-column accumulator beside the
-// scale slots.  (In cycles: a K-step 515 - 550, a tile's hand-over 1500 - 2300 with bf16 output, 3300 with fp32, 660 where the tile is not stored: the stores
-// and the next tile's loads share the way out of the SM.)  Two things got it there:
+// What bounds it, in cycles of the SM: the tensor pipe in the steady state (a K-step of a pair tile 515 - 550; the same MMAs on operands that
+// stay in shared memory 512.8, fp4_ceiling.cu: 8.1 PFLOP/s in a burst, 7.1 sustained), and per tile a hand-over in which the pipe stands still,
+// since TMEM has no room for a second 256-column accumulator beside the scale slots: 1500 - 2300 with bf16 output (1.0 - 1.5 us at 1.55 GHz), 3300
+// with fp32 (2.1 us at 1.6), 660 where the tile is not stored: the stores and the next tile's loads share the way out of the SM.  The clock is what the
+// board's power leaves: 1.44 - 1.6 GHz in the first launches of a run, 1.18 - 1.33 in a long one.  Two things got it there:
 //   - issue.  From a lane-0 branch the descriptors of every MMA, scale copy and commit go to uniform registers one by one, and
 //     two issuing threads did not keep up with the pipe.  With warp-uniform control flow and an elected lane the issuers wait
 //     for operands instead.  Back to back, before -> now: 16384 x 4096 x 16384 382 -> 349 us (alone 372 -> 333: 6.6 PFLOP/s),
@@ -255,7 +255,7 @@ __device__ __forceinline__ void gemm_pair_body(const MapsP& maps, const ParamsP&
         // The whole warp walks the loop and one elected lane issues, here and in the scale loader, as the MMA issuers do: from a lane-0 branch,
         // with divisions by the ring's size, a step's loads took 425 cycles of this thread, more than a 128-wide tile's MMAs (256), and the ring
         // filled as slowly at every start; now 240.  Before -> now: 1024 x 1024 x 8192 11.7 -> 11.2 us, 256 x 512 x 512 5.2 -> 5.0,
-        // 16384 x 4096 x 4096 98 -> 96.5, 16384 x 8192 x 2048 111 -> 108.5; backward 8192 x 1024 x 1024 29.1 -> 27.9.
+        // 16384 x 4096 x 4096 98 -> 96.5, 16384 x 8192 x 2048 111 -> 108.5 (bf16 output; with fp32 it did not move); backward 8192 x 1024 x 1024 29.1 -> 27.9.
         uint32_t s = 0, ph = 1;
         bool ok = true;
         for (uint32_t tl = 0; tl < walk.count && ok; ++tl) {
@@ -694,8 +694,10 @@ Spread spread_tiles(int n0, int n1, const double (&cost)[2], int pairs) {
     return best;
 }
 
-// Microseconds a pair spends on one tile of a launch that does not reach the board's power limit: measured per K-step, and
-// per tile what the hand-over of the accumulator (256) or the stores (128, two accumulators) add.
+// Microseconds a pair spends on one tile of a launch that does not reach the board's power limit, for comparing plans: per K-step, and
+// per tile what the hand-over of the accumulator (256) or the stores (128, two accumulators) add.  Fitted to the times of whole launches with bf16
+// output, which overlap a part of the hand-over (head of this file); fp32 output and addition, whose hand-over is about twice as long, are planned
+// with the same figures.
 double tile_cost(int pn, int64_t K) {
     const double steps = (double)ceil_div(K, 256);
     return pn == 256 ? 0.34 * steps + 0.65 : 0.245 * steps + 0.3;

@@ -685,8 +685,10 @@ cudaError_t quant_tc_init() {
 
 // Launches that give no CTA more than one tile: the groups take half of it each, where a tile otherwise waits for one group's four
 // blocks in a row.  256 x 512 x 512, operands 4.57 -> 4.23 us (SR), 4.35 -> 4.08 (SR16), 3.73 -> 3.80 (nearest rounding, whose blocks are short: not
-// there); whole calls with SR 10.1 -> 9.75.  With more tiles a group's own tile hides the others' and the halves only cost: 8192 x 1024 x 1024 14.7 ->
-// 15.5 (SR), 16384 x 4096 x 4096 96.4 -> 101.3.
+// there); whole calls with SR 10.1 -> 9.75.  Single views of K = 128, whole tiles / halves in us a launch: SR 16 tiles 4.13 / 3.70, 100 tiles 4.59 / 3.89,
+// 148 tiles 4.95 / 4.23; SR16 3.87 / 3.44, 4.15 / 3.68, 4.53 / 4.00.  The line is the mechanism's, short of where the two cross: with two or three tiles to a CTA the
+// halves still gain (296 tiles SR 5.45 / 5.31, SR16 5.28 / 4.95; 440 tiles 6.03 / 5.80, 5.64 / 5.35), with eleven a group's own tile hides the others' and
+// they cost: 8192 x 1024 x 1024 14.7 / 15.5 (SR), 16384 x 4096 x 4096 96.4 / 101.3.
 static bool quantise_by_halves(uint32_t tiles, int sms, int g, int rounding) { return tiles <= (uint32_t)sms && g != 256 && rounding != 1; }
 
 // Quantise n (1..kQuantMaxViews) eligible operand views that share g, seed, rounding and scale layout in one launch.
