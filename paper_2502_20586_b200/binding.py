@@ -419,10 +419,17 @@ def mxfp4_linear_forward_fp8(x, W, out_dtype: int = OUT_BF16, y=None, workspace=
     m = W.shape[0]
     for t in (x, W):
         assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()
+    assert W.numel() == m * n, "x [b, n] and W [m, n] are expected"
+    dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
     if y is None:
-        y = torch.empty((b, m), dtype=torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16, device=x.device)
+        y = _empty(x, (b, m), dt)
+    else:
+        assert y.is_cuda and y.dtype == dt and y.is_contiguous() and y.numel() >= b * m and (y.dim() != 2 or y.shape[1] == m), \
+            "y has another type or device, is not contiguous or too small"
     if workspace is None:
-        workspace = torch.empty(int(_lib.mxfp4_linear_forward_fp8_workspace(b, n, m)), dtype=torch.uint8, device=x.device)
+        workspace = _empty(x, int(_lib.mxfp4_linear_forward_fp8_workspace(b, n, m)), torch.uint8)
+    else:
+        assert workspace.is_cuda and workspace.is_contiguous(), "the workspace is not contiguous memory of the GPU"
     _check(_lib.mxfp4_linear_forward_fp8(_ptr(x), _ptr(W), b, n, m, _ptr(y), out_dtype, _ptr(workspace), workspace.numel(), _stream()))
     return y
 

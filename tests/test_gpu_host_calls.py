@@ -216,3 +216,22 @@ def test_integers_of_every_kind(subclass):
             with pytest.raises(error):
                 gpu.mxfp4_linear_backward_ex(dY, X, W, *ints)
     assert gpu.mxfp4_device_status() == 0
+
+
+def test_forward_tensors_that_do_not_fit_are_refused():
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    x, W = (torch.ones(s, dtype=torch.bfloat16, device="cuda") for s in ((200, 256), (136, 256)))
+    make = lambda *size, dtype=torch.float32: torch.zeros(size, dtype=dtype, device="cuda")
+    for w in (W[:, :128].contiguous(), make(136, 264, dtype=torch.bfloat16), make(136, dtype=torch.bfloat16)):
+        with pytest.raises(AssertionError):
+            gpu.mxfp4_linear_forward_fp8(x, w)
+    for y in (make(199, 136), make(200, 136, dtype=torch.bfloat16), make(136, 200).t(), make(200, 144), make(200, 136).cpu()):
+        with pytest.raises(AssertionError):
+            gpu.mxfp4_linear_forward_fp8(x, W, gpu.OUT_FP32, y=y)
+    for workspace in (make(1 << 20)[::2], torch.zeros(1 << 20, dtype=torch.uint8)):
+        with pytest.raises(AssertionError):
+            gpu.mxfp4_linear_forward_fp8(x, W, workspace=workspace)
+    y = make(200 * 136 + 8)
+    gpu.mxfp4_linear_forward_fp8(x, W.view(136, 16, 16), gpu.OUT_FP32, y=y, workspace=make(1 << 20, dtype=torch.uint8))
+    assert torch.all(y[:-8] == 256.0) and not torch.any(y[-8:]) and gpu.mxfp4_device_status() == 0
