@@ -141,6 +141,13 @@ def _integer(value, ctype) -> int:
         raise ArgumentError(str(e)) from None
 
 
+def _result_type(out_dtype):
+    """The type of the results that the library writes for ``out_dtype``, whose low 32 bits ctypes passes."""
+    if type(out_dtype) is not int:
+        out_dtype = _integer(out_dtype, _int)
+    return torch.float32 if out_dtype & 0xFFFFFFFF == OUT_FP32 else torch.bfloat16
+
+
 def _plain(*tensors) -> bool:
     """Whether the native host call (csrc/host_calls.cpp) takes these: tensors of no subclass, or None.  ``_backward`` has its steps for the rest."""
     for t in tensors:
@@ -234,7 +241,7 @@ def mxfp4_gemm(A_codes, A_scales, B_codes, B_scales, alpha: float = 1.0, out_dty
     N, K2b = B_codes.shape
     assert K2 == K2b
     if C_out is None:
-        C_out = torch.empty((M, N), dtype=torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16, device=A_codes.device)
+        C_out = torch.empty((M, N), dtype=_result_type(out_dtype), device=A_codes.device)
     _check(_lib.mxfp4_gemm(_ptr(A_codes), _ptr(A_scales), _ptr(B_codes), _ptr(B_scales), M, N, 2 * K2, SF_NATIVE,
                            alpha, _ptr(C_out), C_out.stride(0), out_dtype, _stream()))
     return C_out
@@ -248,7 +255,7 @@ def mxfp4_gemm_fused(x, reduce_dim: int, g: int, seed: int, stream_tag: int, rou
     M = rows if reduce_dim == 1 else cols
     N = B_codes.shape[0]
     if C_out is None:
-        C_out = torch.empty((M, N), dtype=torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16, device=x.device)
+        C_out = torch.empty((M, N), dtype=_result_type(out_dtype), device=x.device)
     _check(_lib.mxfp4_gemm_fused(_ptr(x), rows, cols, x.stride(0), reduce_dim, g, rounding, seed, stream_tag, _ptr(B_codes),
                                  _ptr(B_scales), N, alpha, _ptr(C_out), C_out.stride(0), out_dtype, _stream()))
     return C_out
@@ -257,7 +264,7 @@ def mxfp4_gemm_fused(x, reduce_dim: int, g: int, seed: int, stream_tag: int, rou
 def mxfp4_linear_backward_fused(dY, X, W, g: int, seed: int, rounding: int = ROUND_SR, out_dtype: int = OUT_BF16,
                                 dX=None, dW=None, workspace=None):
     """Algorithm 3 with dY / dY^T transformed and quantised inside the two GEMM kernels (fused-producer variant)."""
-    dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
+    dt = _result_type(out_dtype)
     b, m, n = _layer(dY, X, W, dX, dW, None, workspace, dt)
     if dX is None:
         dX = _empty(dY, (b, n), dt)
@@ -332,7 +339,7 @@ def mxfp4_linear_backward_ex(dY, X, W, g: int, seed: int, rounding: int = ROUND_
 def _backward(dY, X, W, g, seed, rounding, out_dtype, dX, dW, db, with_bias, accumulate, workspace):
     """The steps of the native host call for what that does not take: tensors of a subclass, integers of ctypes."""
     g, seed, rounding, out_dtype = _integer(g, _int), _integer(seed, _u64), _integer(rounding, _int), _integer(out_dtype, _int)
-    dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
+    dt = _result_type(out_dtype)
     b, m, n = _layer(dY, X, W, dX, dW, db, workspace, dt)
     assert not accumulate or (dW is not None and (db is not None or not with_bias)), "accumulation needs an existing dW, and db"
     like = next((t for t in (X, W) if type(t) is torch.Tensor), dY)              # (whatever is asked of a subclass goes through its own hooks)
@@ -365,7 +372,7 @@ def mxfp4_linear_backward_static(dY, X, W, g: int, seed: int, rounding: int = RO
     """mxfp4_linear_backward for callers that cannot provide scratch memory: the library's own fixed array
     (STATIC_WORKSPACE_BYTES per GPU) holds the quantised operands.  Pass dX and dW to make the call itself
     allocation-free; shapes that need more scratch than the array raise MxFp4Error(6)."""
-    dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
+    dt = _result_type(out_dtype)
     b, m, n = _layer(dY, X, W, dX, dW, None, None, dt)
     if dX is None:
         dX = _empty(dY, (b, n), dt)
@@ -407,7 +414,7 @@ def mxfp4_fp8_gemm(A_codes, A_scale, B_codes, B_scale, out_dtype: int = OUT_BF16
     M, K = A_codes.shape
     N = B_codes.shape[0]
     if C_out is None:
-        C_out = torch.empty((M, N), dtype=torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16, device=A_codes.device)
+        C_out = torch.empty((M, N), dtype=_result_type(out_dtype), device=A_codes.device)
     _check(_lib.mxfp4_fp8_gemm(_ptr(A_codes), _ptr(A_scale), _ptr(B_codes), _ptr(B_scale), M, N, K, _ptr(C_out), C_out.stride(0),
                                out_dtype, _stream()))
     return C_out
@@ -420,7 +427,7 @@ def mxfp4_linear_forward_fp8(x, W, out_dtype: int = OUT_BF16, y=None, workspace=
     for t in (x, W):
         assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()
     assert W.numel() == m * n, "x [b, n] and W [m, n] are expected"
-    dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
+    dt = _result_type(out_dtype)
     if y is None:
         y = _empty(x, (b, m), dt)
     else:
@@ -454,7 +461,7 @@ def mxfp4_int4_gemm(A_codes, A_scales, B_codes, B_scales, alpha: float = 1.0, ou
     M, K = A_codes.shape
     N = B_codes.shape[0]
     if C_out is None:
-        C_out = torch.empty((M, N), dtype=torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16, device=A_codes.device)
+        C_out = torch.empty((M, N), dtype=_result_type(out_dtype), device=A_codes.device)
     _check(_lib.mxfp4_int4_gemm(_ptr(A_codes), _ptr(A_scales), _ptr(B_codes), _ptr(B_scales), M, N, K, alpha, _ptr(C_out), C_out.stride(0),
                                 out_dtype, _stream()))
     return C_out

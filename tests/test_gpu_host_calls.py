@@ -218,6 +218,31 @@ def test_integers_of_every_kind(subclass):
     assert gpu.mxfp4_device_status() == 0
 
 
+# out_dtype in every form that stands for 1 to the library: results of four bytes an element from every call that makes them itself
+def test_every_form_of_fp32_makes_fp32_results():
+    import ctypes
+
+    import torch
+    from paper_2502_20586_b200 import binding as gpu
+    dY, X, W = _layer(m=512)
+    q = gpu.mxfp4_quantize_operands(dY, X, W, 64, 5)
+    a, b = gpu.mxfp4_int4_quantize(X[:, :256], 1, 64, 5)[:2], gpu.mxfp4_int4_quantize(W[:, :256], 1, 64, 5)[:2]
+    one = torch.ones(2, device="cuda")
+    calls = [lambda o: gpu.mxfp4_linear_backward(dY, X, W, 64, 5, 0, o), lambda o: gpu.mxfp4_linear_backward(_tagged(dY), X, W, 64, 5, 0, o),
+             lambda o: gpu.mxfp4_linear_backward_static(dY, X, W, 64, 5, 0, o), lambda o: gpu.mxfp4_linear_backward_fused(dY, X, W, 64, 5, 0, o),
+             lambda o: gpu.mxfp4_gemm(*q[0], *q[1], out_dtype=o), lambda o: gpu.mxfp4_gemm_fused(dY, 1, 64, 5, 0, 0, *q[1], out_dtype=o),
+             lambda o: gpu.mxfp4_linear_forward_fp8(X[:, :256].contiguous(), W[:, :256].contiguous(), o),
+             lambda o: gpu.mxfp4_fp8_gemm(a[0], one, b[0], one, o), lambda o: gpu.mxfp4_int4_gemm(*a, *b, out_dtype=o)]
+    flat = lambda r: [r] if isinstance(r, torch.Tensor) else list(r)
+    for call in calls:
+        want = flat(call(gpu.OUT_FP32))
+        for o in (True, ctypes.c_int(1), _Parameter(1), _Parameter(ctypes.c_int(1)), (1 << 32) + 1):
+            got = flat(call(o))
+            assert all(t.dtype == torch.float32 and torch.equal(t, w) for t, w in zip(got, want))
+        assert all(t.dtype == torch.bfloat16 for t in flat(call(ctypes.c_int(0))))
+    assert gpu.mxfp4_device_status() == 0
+
+
 def test_forward_tensors_that_do_not_fit_are_refused():
     import torch
     from paper_2502_20586_b200 import binding as gpu
